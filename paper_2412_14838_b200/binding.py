@@ -1,8 +1,10 @@
-"""ctypes view of libdkv.so: the same entry points as include/dkv.h, argument marshalling only.
+"""Python view of libdkv.so: the same entry points as include/dkv.h, argument marshalling only.
 
 Every step of the path runs inside the CUDA library; this module converts torch tensors (or raw
 integer addresses) to pointers, passes the current CUDA stream, and raises ``DkvError`` on a
-non-zero return code.  There is no CPU fallback: ``load()`` raises when the library is missing.
+non-zero return code.  The calls that a serving loop makes convert their arguments in native code
+(csrc/pycall.cpp, loaded as ``_dkv_pycall``), the others through ctypes.  There is no CPU fallback:
+``load()`` raises when the library is missing.
 """
 from __future__ import annotations
 
@@ -39,11 +41,12 @@ class DkvError(RuntimeError):
 
 
 _lib = None
+_call = None                     # the native half, csrc/pycall.cpp
 
 
 def load() -> ctypes.CDLL:
     """Load libdkv.so (built by ``paper_2412_14838_b200.build``); fail loudly if it is absent."""
-    global _lib
+    global _lib, _call
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -92,8 +95,17 @@ def load() -> ctypes.CDLL:
         fn.restype = ctypes.c_int
     lib.dkv_strerror.restype = ctypes.c_char_p
     lib.dkv_launch_count.restype = ctypes.c_int64
-    _lib = lib
+    import torch                 # noqa: F401  (the native half is linked with torch's libraries)
+    from . import _dkv_pycall
+    _lib, _call = lib, _dkv_pycall
     return lib
+
+
+def _native():
+    """The native half, loaded on first use."""
+    if _call is None:
+        load()
+    return _call
 
 
 def strerror(code: int) -> str:
@@ -111,22 +123,6 @@ def _ptr(x) -> Optional[int]:
     if hasattr(x, "ctypes"):
         return x.ctypes.data
     raise TypeError(f"cannot take the address of {type(x)}")
-
-
-def _stream(stream) -> Optional[int]:
-    if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream or None
-    if isinstance(stream, int):
-        return stream or None
-    return stream.cuda_stream or None
-
-
-def _ptr_array(items: Sequence) -> ctypes.Array:
-    arr = (ctypes.c_void_p * len(items))()
-    for i, it in enumerate(items):
-        arr[i] = _ptr(it)
-    return arr
 
 
 def _check(code: int, what: str) -> None:
@@ -165,57 +161,51 @@ def dkv_destroy(ctx: int) -> None:
 
 
 def dkv_reset(ctx: int, stream=None) -> None:
-    _check(load().dkv_reset(ctx, _stream(stream)), "dkv_reset")
+    _check(_native().reset(ctx, stream), "dkv_reset")
 
 
 def dkv_score(ctx: int, layer: int, q_win, k, scores_out=None, stream=None) -> None:
-    _check(load().dkv_score(ctx, layer, _ptr(q_win), _ptr(k), _ptr(scores_out), _stream(stream)), "dkv_score")
+    _check(_native().score(ctx, layer, q_win, k, scores_out, stream), "dkv_score")
 
 
 def dkv_score_static(cfg: DkvConfig, q_win, k, scores_out, stream=None) -> None:
     """Score one layer without a context and without any device allocation (see include/dkv.h)."""
-    _check(load().dkv_score_static(ctypes.byref(cfg), _ptr(q_win), _ptr(k), _ptr(scores_out), _stream(stream)),
-           "dkv_score_static")
+    _check(_native().score_static(ctypes.addressof(cfg), q_win, k, scores_out, stream), "dkv_score_static")
 
 
 def dkv_score_lse(ctx: int, layer: int, q_win, k, lse, scores_out=None, stream=None) -> None:
     """Score one layer in a single sweep, given the window rows' log-sum-exp fp32 [Bt, Hq, ws] (see include/dkv.h)."""
-    _check(load().dkv_score_lse(ctx, layer, _ptr(q_win), _ptr(k), _ptr(lse), _ptr(scores_out), _stream(stream)),
-           "dkv_score_lse")
+    _check(_native().score_lse(ctx, layer, q_win, k, lse, scores_out, stream), "dkv_score_lse")
 
 
 def dkv_set_scores(ctx: int, layer: int, scores, stream=None) -> None:
-    _check(load().dkv_set_scores(ctx, layer, _ptr(scores), _stream(stream)), "dkv_set_scores")
+    _check(_native().set_scores(ctx, layer, scores, stream), "dkv_set_scores")
 
 
 def dkv_select_topk(ctx: int, layer: int, idx_out=None, rank_out=None, stream=None) -> None:
-    _check(load().dkv_select_topk(ctx, layer, _ptr(idx_out), _ptr(rank_out), _stream(stream)), "dkv_select_topk")
+    _check(_native().select_topk(ctx, layer, idx_out, rank_out, stream), "dkv_select_topk")
 
 
 def dkv_rebudget(ctx: int, upto_layer: int, counts_out=None, stream=None) -> None:
-    _check(load().dkv_rebudget(ctx, upto_layer, _ptr(counts_out), _stream(stream)), "dkv_rebudget")
+    _check(_native().rebudget(ctx, upto_layer, counts_out, stream), "dkv_rebudget")
 
 
 def dkv_compact(ctx: int, layer: int, k_src, v_src, kb, vb, len_out=None, stream=None) -> None:
-    _check(load().dkv_compact(ctx, layer, _ptr(k_src), _ptr(v_src), _ptr(kb), _ptr(vb), _ptr(len_out),
-                              _stream(stream)), "dkv_compact")
+    _check(_native().compact(ctx, layer, k_src, v_src, kb, vb, len_out, stream), "dkv_compact")
 
 
 def dkv_compact_all(ctx: int, upto_layer: int, kb: Sequence, vb: Sequence, stream=None) -> None:
-    _check(load().dkv_compact_all(ctx, upto_layer, _ptr_array(kb), _ptr_array(vb), _stream(stream)),
-           "dkv_compact_all")
+    _check(_native().compact_all(ctx, upto_layer, kb, vb, stream), "dkv_compact_all")
 
 
 def dkv_run_prefill_pass(ctx: int, q_win: Sequence, k: Sequence, v: Sequence, kb: Sequence, vb: Sequence,
                          stream=None) -> None:
-    _check(load().dkv_run_prefill_pass(ctx, _ptr_array(q_win), _ptr_array(k), _ptr_array(v), _ptr_array(kb),
-                                       _ptr_array(vb), _stream(stream)), "dkv_run_prefill_pass")
+    _check(_native().run_prefill_pass(ctx, q_win, k, v, kb, vb, stream), "dkv_run_prefill_pass")
 
 
 def dkv_run_prefill_pass_host(ctx: int, q_win: Sequence, k: Sequence, v: Sequence, kb: Sequence, vb: Sequence,
                               counts_out=None) -> None:
-    _check(load().dkv_run_prefill_pass_host(ctx, _ptr_array(q_win), _ptr_array(k), _ptr_array(v), _ptr_array(kb),
-                                            _ptr_array(vb), _ptr(counts_out)), "dkv_run_prefill_pass_host")
+    _check(_native().run_prefill_pass_host(ctx, q_win, k, v, kb, vb, counts_out), "dkv_run_prefill_pass_host")
 
 
 def dkv_host_pass_bytes(ctx: int):
@@ -228,30 +218,28 @@ def dkv_host_pass_bytes(ctx: int):
 def dkv_run_prefill_pass_lse(ctx: int, q_win: Sequence, k: Sequence, v: Sequence, lse: Sequence, kb: Sequence,
                              vb: Sequence, stream=None) -> None:
     """The pass with every layer scored in one sweep from the window rows' log-denominators (see include/dkv.h)."""
-    _check(load().dkv_run_prefill_pass_lse(ctx, _ptr_array(q_win), _ptr_array(k), _ptr_array(v), _ptr_array(lse),
-                                           _ptr_array(kb), _ptr_array(vb), _stream(stream)), "dkv_run_prefill_pass_lse")
+    _check(_native().run_prefill_pass_lse(ctx, q_win, k, v, lse, kb, vb, stream), "dkv_run_prefill_pass_lse")
 
 
 DKV_POLICY_UNIFORM, DKV_POLICY_PYRAMID = 0, 1
 
 
 def dkv_apply_policy(ctx: int, policy: int, counts_out=None, stream=None) -> None:
-    _check(load().dkv_apply_policy(ctx, policy, _ptr(counts_out), _stream(stream)), "dkv_apply_policy")
+    _check(_native().apply_policy(ctx, policy, counts_out, stream), "dkv_apply_policy")
 
 
 def dkv_select_positions(ctx: int, layer: int, n_sink: int, n_recent: int, stream=None) -> None:
-    _check(load().dkv_select_positions(ctx, layer, n_sink, n_recent, _stream(stream)), "dkv_select_positions")
+    _check(_native().select_positions(ctx, layer, n_sink, n_recent, stream), "dkv_select_positions")
 
 
 def dkv_decode_attend(ctx: int, layer0: int, n_layers: int, nq: int, q_dec: Sequence, kb: Sequence, vb: Sequence,
                       out: Sequence, stream=None) -> None:
     """Attention of nq new queries per sample over the compressed buffers of layers [layer0, layer0 + n_layers)."""
-    _check(load().dkv_decode_attend(ctx, layer0, n_layers, nq, _ptr_array(q_dec), _ptr_array(kb), _ptr_array(vb),
-                                    _ptr_array(out), _stream(stream)), "dkv_decode_attend")
+    _check(_native().decode_attend(ctx, layer0, n_layers, nq, q_dec, kb, vb, out, stream), "dkv_decode_attend")
 
 
 def dkv_get_counts(ctx: int, host_counts, stream=None) -> None:
-    _check(load().dkv_get_counts(ctx, _ptr(host_counts), _stream(stream)), "dkv_get_counts")
+    _check(_native().get_counts(ctx, host_counts, stream), "dkv_get_counts")
 
 
 def dkv_layer_views(ctx: int, layer: int):
@@ -262,7 +250,7 @@ def dkv_layer_views(ctx: int, layer: int):
 
 
 def dkv_kept_sorted(ctx: int, layer: int, sorted_out, stream=None) -> None:
-    _check(load().dkv_kept_sorted(ctx, layer, _ptr(sorted_out), _stream(stream)), "dkv_kept_sorted")
+    _check(_native().kept_sorted(ctx, layer, sorted_out, stream), "dkv_kept_sorted")
 
 
 def dkv_budget_views(ctx: int):
@@ -273,7 +261,7 @@ def dkv_budget_views(ctx: int):
 
 
 def dkv_memcpy_to_host(ctx: int, host_dst, dev_src: int, nbytes: int, stream=None) -> None:
-    _check(load().dkv_memcpy_to_host(ctx, _ptr(host_dst), dev_src, nbytes, _stream(stream)), "dkv_memcpy_to_host")
+    _check(_native().memcpy_to_host(ctx, host_dst, dev_src, nbytes, stream), "dkv_memcpy_to_host")
 
 
 def read_device_i32(ctx: int, dev_src: int, shape):

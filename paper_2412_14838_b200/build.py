@@ -1,4 +1,5 @@
-"""Build libdkv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
+"""Build libdkv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _dkv_pycall.so (the native half of
+binding.py: argument conversion) with the host compiler.
 
 ``python -m paper_2412_14838_b200.build`` or ``build()``; nvcc cross-compiles without a GPU.
 """
@@ -13,6 +14,9 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdkv.so")
 SOURCES = ["dkv.cu"]
+PYCALL = os.path.join(HERE, "_dkv_pycall.so")
+PYCALL_SOURCE = os.path.join(CSRC, "pycall.cpp")
+HEADER = os.path.join(os.path.dirname(HERE), "include", "dkv.h")
 
 
 def _nvcc() -> str:
@@ -22,27 +26,39 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found: libdkv.so cannot be built")
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
-    deps.append(os.path.join(os.path.dirname(HERE), "include", "dkv.h"))
-    return any(os.path.getmtime(d) > t for d in deps)
+def _stale(lib: str, deps) -> bool:
+    return not os.path.exists(lib) or any(os.path.getmtime(d) > os.path.getmtime(lib) for d in deps)
+
+
+def _run(cmd, verbose: bool) -> None:
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"{os.path.basename(cmd[0])} failed:\n" + res.stdout + res.stderr)
+    if verbose:
+        print(res.stdout + res.stderr)
+
+
+def _build_pycall(verbose: bool) -> None:
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    inc = [os.path.join(root, "include"), sysconfig.get_paths()["include"], "/usr/local/cuda/include"]
+    _run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+          f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(f"-I{d}" for d in inc), PYCALL_SOURCE,
+          "-o", PYCALL, f"-L{HERE}", "-l:libdkv.so", f"-L{root}/lib", "-ltorch_python", "-lc10", "-lc10_cuda",
+          "-Wl,-rpath,$ORIGIN", f"-Wl,-rpath,{root}/lib"], verbose)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile the library if a source is newer than it; return its path."""
-    if not force and not _stale():
-        return LIB
-    cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-           "-shared", "-Xcompiler", "-fPIC", "-Xptxas", "-v" if verbose else "-O3",
-           "-o", LIB] + [os.path.join(CSRC, s) for s in SOURCES]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
-    if verbose:
-        print(res.stdout + res.stderr)
+    """Compile what is older than its sources; return the library's path."""
+    kernels = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != os.path.basename(PYCALL_SOURCE)]
+    if force or _stale(LIB, kernels + [HEADER]):
+        _run([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
+              "-shared", "-Xcompiler", "-fPIC", "-Xptxas", "-v" if verbose else "-O3",
+              "-o", LIB] + [os.path.join(CSRC, s) for s in SOURCES], verbose)
+    if force or _stale(PYCALL, [PYCALL_SOURCE, HEADER]):
+        _build_pycall(verbose)
     return LIB
 
 
