@@ -67,7 +67,7 @@ struct dkv_ctx {
   uint8_t selected[DKV_MAX_LAYERS];     // 1: by scores (dkv_select_topk), 2: by position (dkv_select_positions)
   int sel_n[DKV_MAX_LAYERS];            // positions selected per head: Blc, or what dkv_select_positions kept
   // decoding over the compressed cache (allocated on first use, grown on demand)
-  float* d_dec_scratch;
+  float* d_dec_scratch;                 // parts of heads that lie in more than one block's slice
   size_t dec_scratch_floats;
   unsigned int* d_dec_tickets;          // [L][Bt*Hkv], zero between launches
   long long launches;
@@ -384,6 +384,73 @@ int do_gather(dkv_ctx* c, int layer, const void* k_src, const void* v_src, void*
     c->stale[layer] = 0;
     return do_shrink(c, layer, 1, &kb, &vb, st);
   }
+  return DKV_OK;
+}
+
+// ---- decoding ------------------------------------------------------------------------------------
+// Launch with programmatic stream serialisation (the kernel waits for its predecessor itself, so that its scheduling
+// overlaps the predecessor's end) and, if cluster > 1, clusters of that many blocks along x.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t st, const Args&... args) {
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = at; cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// QB = 8: up to 8 queries a head group; 16: more than 8, 16 at a time.
+template <int D, int QB>
+cudaError_t launch_decode(const DecodePtrs& ptrs, const DecodeArgs& a, int cluster, int split_grid, cudaStream_t st) {
+  constexpr int NW = QB == 8 ? 8 : 4;
+  if (split_grid > 0)
+    return launch_pdl(decode_split_kernel<D, QB, 4>, dim3(split_grid), 128, (size_t)(a.nl * a.Bt + 1) * 4, 1, st, ptrs, a);
+  return launch_pdl(decode_cluster_kernel<D, QB, NW>, dim3(cluster, a.Bt * a.Hkv, a.nl), NW * 32, 0, cluster, st, ptrs, a);
+}
+
+int do_decode(dkv_ctx* c, int layer0, int nl, int nq, const void* const* q, const void* const* kb, const void* const* vb,
+              float* const* out, cudaStream_t st) {
+  const Shape& s = c->s;
+  const int BH = s.Bt * s.Hkv, heads = BH * nl, GQ = s.G * nq;
+  DecodeArgs a;
+  a.layer0 = layer0; a.nl = nl; a.Bt = s.Bt; a.Hkv = s.Hkv; a.GQ = GQ; a.L = s.L; a.ws = s.ws; a.row_stride = s.rows;
+  a.scale2 = kLog2e / sqrtf((float)s.D);
+  a.held = c->d_held; a.scratch = nullptr; a.tickets = nullptr;
+  // A cluster per head while the heads alone leave SMs idle (as many blocks a head as fit one wave, at most the
+  // portable 8, and one row block a warp at least); equal slices of all rows once there is a head per SM or so.
+  int cluster = 1, split_grid = 0;
+  const int warps = GQ <= 8 ? 8 : 4;
+  while (cluster < 8 && heads * cluster * 2 <= c->n_sms && cluster * warps * kDecRowBlock < s.rows) cluster *= 2;
+  if (heads * 4 > c->n_sms && nl * s.Bt <= kDecMaxPairs) {
+    // as many blocks of four warps as are resident at once, but no more warps than there can be row blocks
+    const long long most = ((long long)heads * ((s.rows + kDecRowBlock - 1) / kDecRowBlock) + 3) / 4;
+    split_grid = c->n_sms * 2;
+    if (split_grid > most) split_grid = (int)most;
+    const int qb = GQ <= 8 ? 8 : 16;
+    const size_t need = (size_t)split_grid * 4 * 2 * ((GQ + qb - 1) / qb) * (qb * s.D + qb * 2);
+    if (!c->d_dec_tickets) {
+      DKV_CUDA(c, cudaMalloc(&c->d_dec_tickets, sizeof(unsigned int) * s.L * BH));
+      DKV_CUDA(c, cudaMemset(c->d_dec_tickets, 0, sizeof(unsigned int) * s.L * BH));
+    }
+    if (need > c->dec_scratch_floats) {
+      if (c->d_dec_scratch) { DKV_CUDA(c, cudaDeviceSynchronize()); cudaFree(c->d_dec_scratch); c->d_dec_scratch = nullptr; c->dec_scratch_floats = 0; }
+      DKV_CUDA(c, cudaMalloc(&c->d_dec_scratch, need * sizeof(float)));
+      c->dec_scratch_floats = need;
+    }
+    a.scratch = c->d_dec_scratch; a.tickets = c->d_dec_tickets + (size_t)layer0 * BH;
+  }
+  DecodePtrs ptrs;
+  for (int i = 0; i < nl; ++i) { ptrs.q[i] = q[i]; ptrs.kb[i] = kb[i]; ptrs.vb[i] = vb[i]; ptrs.out[i] = out[i]; }
+  ProfScope ps(c, DKV_STEP_DECODE, 1, st);
+  cudaError_t e;
+  if (s.D == 128) e = GQ <= 8 ? launch_decode<128, 8>(ptrs, a, cluster, split_grid, st) : launch_decode<128, 16>(ptrs, a, cluster, split_grid, st);
+  else e = GQ <= 8 ? launch_decode<64, 8>(ptrs, a, cluster, split_grid, st) : launch_decode<64, 16>(ptrs, a, cluster, split_grid, st);
+  if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(c, e); }
+  c->launches++;
   return DKV_OK;
 }
 
@@ -943,40 +1010,10 @@ int dkv_decode_attend(dkv_ctx* c, int32_t layer0, int32_t n_layers, int32_t nq, 
     if (!c->gathered[layer0 + i]) return DKV_ERR_STATE;
   }
   cudaStream_t st = as_stream(stream);
-  const int BH = s.Bt * s.Hkv, GQ = s.G * nq;
-  if (!c->d_dec_tickets) {
-    DKV_CUDA(c, cudaMalloc(&c->d_dec_tickets, sizeof(unsigned int) * s.L * BH));
-    DKV_CUDA(c, cudaMemset(c->d_dec_tickets, 0, sizeof(unsigned int) * s.L * BH));
-  }
   for (int l0 = 0; l0 < n_layers; l0 += kDecMaxLayers) {
     const int nl = n_layers - l0 < kDecMaxLayers ? n_layers - l0 : kDecMaxLayers;
-    // a launch over few heads is latency-bound: one resident wave of thread blocks (two fit an SM); one over many
-    // heads is bandwidth-bound: a few waves, for more loads in flight; every block gets at least a few dozen rows
-    const int waves = BH * nl >= c->n_sms ? 4 : 2;
-    int splits = (waves * c->n_sms + BH * nl - 1) / (BH * nl);
-    const int most = (s.rows + 31) / 32;
-    if (splits > most) splits = most;
-    if (splits > 64) splits = 64;
-    if (splits < 1) splits = 1;
-    const size_t need = (size_t)nl * BH * splits * GQ * (s.D + 2);
-    if (need > c->dec_scratch_floats) {
-      if (c->d_dec_scratch) { DKV_CUDA(c, cudaDeviceSynchronize()); cudaFree(c->d_dec_scratch); c->d_dec_scratch = nullptr; c->dec_scratch_floats = 0; }
-      DKV_CUDA(c, cudaMalloc(&c->d_dec_scratch, need * sizeof(float)));
-      c->dec_scratch_floats = need;
-    }
-    DecodePtrs ptrs;
-    memset(&ptrs, 0, sizeof ptrs);
-    for (int i = 0; i < nl; ++i) { ptrs.q[i] = q_dec[l0 + i]; ptrs.kb[i] = kb[l0 + i]; ptrs.vb[i] = vb[l0 + i]; ptrs.out[i] = out[l0 + i]; }
-    const dim3 grid(splits, BH, nl);
-    const float scale2 = kLog2e / sqrtf((float)s.D);
-    ProfScope ps(c, DKV_STEP_DECODE, 1, st);
-    if (s.D == 128)
-      decode_attend_kernel<128><<<grid, kDecThreads, 0, st>>>(ptrs, layer0 + l0, c->d_held, s.Hkv, s.G, nq, s.L, s.ws, s.rows, scale2,
-                                                             c->d_dec_scratch, c->d_dec_tickets + (size_t)(layer0 + l0) * BH);
-    else
-      decode_attend_kernel<64><<<grid, kDecThreads, 0, st>>>(ptrs, layer0 + l0, c->d_held, s.Hkv, s.G, nq, s.L, s.ws, s.rows, scale2,
-                                                            c->d_dec_scratch, c->d_dec_tickets + (size_t)(layer0 + l0) * BH);
-    DKV_LAUNCHED(c);
+    const int rc = do_decode(c, layer0 + l0, nl, nq, q_dec + l0, kb + l0, vb + l0, out + l0, st);
+    if (rc) return rc;
   }
   return DKV_OK;
 }
