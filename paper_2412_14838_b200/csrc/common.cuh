@@ -26,6 +26,11 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
+// Programmatic dependent launch: the kernel may have been scheduled while its predecessor on the stream still ran;
+// nothing that a predecessor may have written is touched before pdl_wait.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Per-layer device pointers passed by value to kernels that work on several layers at once.
 struct LayerPtrs {
   void* kb[128];

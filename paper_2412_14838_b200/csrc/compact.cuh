@@ -8,35 +8,47 @@ namespace dkv {
 
 constexpr int kGatherRows = 4;      // rows per thread, all loads issued before the stores
 
-// Gather: dst[b,h,i] = src[b,h, i < n ? idx[i] : P + (i - n)], i < n + ws.  16 bytes per thread per row.
-// grid (row blocks, Bt*Hkv, 2 tensors).  n = kept positions per head (same for all heads), idx_stride = entries
-// per head in idx; also records held[b][layer] = n.
-__global__ void __launch_bounds__(256)
-gather_rows_kernel(const uint4* __restrict__ k_src, const uint4* __restrict__ v_src, uint4* __restrict__ kb,
-                   uint4* __restrict__ vb, const int* __restrict__ idx, int n, int idx_stride, int S, int P, int ws,
-                   int row_stride /* rows per head in kb/vb */, int vec_per_row /* D*2/16 */,
-                   int* __restrict__ held, int Hkv, int L, int layer) {
-  const int bh = blockIdx.y;
-  const uint4* src = (blockIdx.z == 0 ? k_src : v_src) + (size_t)bh * S * vec_per_row;
-  uint4* dst = (blockIdx.z == 0 ? kb : vb) + (size_t)bh * row_stride * vec_per_row;
-  if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.z == 0 && bh % Hkv == 0) held[(bh / Hkv) * L + layer] = n;
-  const int rows_per_pass = 256 / vec_per_row;
-  const int row0 = blockIdx.x * rows_per_pass * kGatherRows + threadIdx.x / vec_per_row;
-  const int c = threadIdx.x % vec_per_row;
-  uint4 val[kGatherRows];
+// One head's buffer rows: row r < n is source row sel[r] (shared or global memory), the ws window rows P .. S-1 follow.
+// 16 bytes of K and of V per thread and row, `threads` threads (a multiple of vec = 16-byte pieces per row); `part` of
+// `parts` sets of threads share the head.
+__device__ __forceinline__ void gather_rows(const uint4* __restrict__ k_src, const uint4* __restrict__ v_src, uint4* __restrict__ kb,
+                                            uint4* __restrict__ vb, const int* sel, int n, int bh, int S, int P, int ws,
+                                            int row_stride /* rows per head in kb/vb */, int vec, int tid, int threads, int part, int parts) {
+  const int per_pass = threads / vec, c = tid % vec, rows = n + ws;
+  const size_t src0 = (size_t)bh * S * vec + c, dst0 = (size_t)bh * row_stride * vec + c;
+  for (int row0 = part * per_pass * kGatherRows + tid / vec; row0 < rows; row0 += parts * per_pass * kGatherRows) {
+    uint4 kv[kGatherRows], vv[kGatherRows];
 #pragma unroll
-  for (int j = 0; j < kGatherRows; ++j) {
-    const int row = row0 + j * rows_per_pass;
-    if (row < n + ws) {
-      const int from = row < n ? idx[(size_t)bh * idx_stride + row] : P + (row - n);
-      val[j] = __ldcs(&src[(size_t)from * vec_per_row + c]);      // read once: first in line for eviction from L2
+    for (int j = 0; j < kGatherRows; ++j) {
+      const int row = row0 + j * per_pass;
+      if (row < rows) {
+        const size_t from = src0 + (size_t)(row < n ? sel[row] : P + (row - n)) * vec;
+        kv[j] = __ldcs(&k_src[from]);                             // read once: first in line for eviction from L2
+        vv[j] = __ldcs(&v_src[from]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kGatherRows; ++j) {
+      const int row = row0 + j * per_pass;
+      if (row < rows) { kb[dst0 + (size_t)row * vec] = kv[j]; vb[dst0 + (size_t)row * vec] = vv[j]; }
     }
   }
-#pragma unroll
-  for (int j = 0; j < kGatherRows; ++j) {
-    const int row = row0 + j * rows_per_pass;
-    if (row < n + ws) __stcs(&dst[(size_t)row * vec_per_row + c], val[j]);
-  }
+}
+
+// Gather of one layer with its current count: n = min(count[b][layer], sel_n) rows per head of idx, idx_stride apart;
+// records held[b][layer] = n.  grid (row blocks, Bt*Hkv).
+constexpr int kGatherThreads = 256;
+__global__ void __launch_bounds__(kGatherThreads)
+gather_rows_kernel(const uint4* __restrict__ k_src, const uint4* __restrict__ v_src, uint4* __restrict__ kb,
+                   uint4* __restrict__ vb, const int* __restrict__ idx, const int* __restrict__ count, int sel_n, int idx_stride,
+                   int S, int P, int ws, int row_stride, int vec, int* __restrict__ held, int Hkv, int L, int layer) {
+  const int bh = blockIdx.y, b = bh / Hkv;
+  pdl_launch();
+  pdl_wait();
+  const int n = min(count[b * L + layer], sel_n);
+  if (threadIdx.x == 0 && blockIdx.x == 0 && bh % Hkv == 0) held[b * L + layer] = n;
+  gather_rows(k_src, v_src, kb, vb, idx + (size_t)bh * idx_stride, n, bh, S, P, ws, row_stride, vec, threadIdx.x, kGatherThreads,
+              blockIdx.x, gridDim.x);
 }
 
 constexpr int kShrinkThreads = 256;
@@ -45,15 +57,18 @@ constexpr int kShrinkThreads = 256;
 // The buffers are in Algorithm 1's own order (score descending), so cutting a layer from `have` to
 // `want` kept rows keeps the first `want` rows where they are; only the ws window rows move, from
 // [have, have+ws) to [want, want+ws).  The two ranges may overlap (dst < src): rows are moved in
-// blocks, each block read completely before it is written.
+// blocks, each block read completely before it is written.  The last block of a (layer, sample) to arrive (a ticket
+// each, zero between launches) records held[b][layer] = want: everyone has read the old value by then.
 __global__ void __launch_bounds__(kShrinkThreads)
-shrink_kernel(LayerPtrs ptrs, int layer0, const int* __restrict__ count, const int* __restrict__ held, int Hkv, int L,
-              int ws, int row_stride, int vec_per_row) {
+shrink_kernel(LayerPtrs ptrs, int layer0, const int* __restrict__ count, int* __restrict__ held, unsigned int* __restrict__ tickets,
+              int Hkv, int L, int ws, int row_stride, int vec_per_row) {
   const int layer = layer0 + blockIdx.y;
   const int bh = blockIdx.x, b = bh / Hkv;
+  pdl_launch();
+  pdl_wait();
   const int have = held[b * L + layer];
   const int want = min(count[b * L + layer], have);
-  if (want == have) return;                                  // uniform across the block
+  if (want == have) return;                                  // the same for every block of the (layer, sample)
   uint4* buf = reinterpret_cast<uint4*>(blockIdx.z == 0 ? ptrs.kb[layer] : ptrs.vb[layer]) + (size_t)bh * row_stride * vec_per_row;
   const uint4* src = buf + (size_t)have * vec_per_row;
   uint4* dst = buf + (size_t)want * vec_per_row;
@@ -66,15 +81,13 @@ shrink_kernel(LayerPtrs ptrs, int layer0, const int* __restrict__ count, const i
     if (e < n) dst[e] = val;
     __syncthreads();
   }
-}
-
-// After a shrink: the buffers of layers [layer0, layer0 + n) now hold min(held, count) rows.
-__global__ void commit_held_kernel(int* __restrict__ held, const int* __restrict__ count, int Bt, int L, int layer0, int n) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= Bt * n) return;
-  const int b = e / n, layer = layer0 + e % n;
-  const int h = held[b * L + layer], c = count[b * L + layer];
-  held[b * L + layer] = c < h ? c : h;
+  if (threadIdx.x == 0) {                                    // the barriers above: the whole block has read `held`
+    __threadfence();
+    if (atomicAdd(&tickets[b * L + layer], 1u) == (unsigned int)(2 * Hkv - 1)) {
+      tickets[b * L + layer] = 0;
+      held[b * L + layer] = want;
+    }
+  }
 }
 
 // len_out[b][h] = held[b][layer] + ws

@@ -247,11 +247,6 @@ struct DecodeWarp {
   }
 };
 
-// Programmatic dependent launch: the kernel may have been scheduled while its predecessor on the stream still ran;
-// nothing that a predecessor may have written is touched before pdl_wait.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // One 4-value piece x (query qi = x / (D/4)) of the warps' parked results, merged in warp order: value sums, and the
 // query's (max, sum); max = -inf: no rows.
 template <int D, int QB, int NW>

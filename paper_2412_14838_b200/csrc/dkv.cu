@@ -20,9 +20,6 @@ using namespace dkv;
 
 struct ProfRec { cudaEvent_t a, b; int step; int launches; };
 
-constexpr int kSideStreams = 4;
-constexpr int kSelMaxSmem = DKV_MAX_LAYER_BUDGET * 8 + DKV_MAX_LAYER_BUDGET * 4;
-
 struct dkv_ctx {
   dkv_config cfg;
   Shape s;
@@ -33,21 +30,16 @@ struct dkv_ctx {
   int* d_count;         // [Bt][L] budget of each layer
   int* d_held;          // [Bt][L] rows the layer's buffers hold
   int* d_dbg;           // 3 x [Bt][L] : cnt, Z, Z' of the last update
-  unsigned int* d_layer_hist; // [L][Bt][2048] first-digit histogram of every layer's scores (all heads of a sample)
-  uint2* d_cand;              // [Bt][L*Hkv*P] (score bits, layer) of the scores in the global top-K's first bucket
+  unsigned int* d_layer_hist; // [L][Bt][2048] digit histogram of every layer's scores (all heads of a sample)
+  uint2* d_cand;              // [Bt][L*Hkv*P] (score bits, layer) of the scores with the digit of a global top-K's threshold
   unsigned int* d_cand_n;     // [Bt]
-  RbState* d_rb_state;        // [Bt]
-  unsigned int* d_rb_above;   // [Bt][L]
-  unsigned int* d_rb_hist1;   // [Bt][2048]
-  unsigned int* d_rb_above2;  // [Bt][L]
-  unsigned int* d_rb_hist2;   // [Bt][L][1024]
+  RbState* d_rb_state;        // [kRbUpdates][Bt]
+  unsigned int* d_rb_above;   // [kRbUpdates][Bt][L]
+  unsigned int* d_shrink_tickets;   // [Bt][L], zero between launches
   int* d_status;        // [8]
-  int sort_n;
-  bool sel_reg;         // a head's scores fit the select kernel's registers and shared memory
-  size_t sel_smem;
+  int sel_cap;          // entries of the select kernels' list
   // tensor-core scoring
-  int n_sms, tc_grid, tc_slots;
-  int pass_taper;       // group sizes halve towards the end of the pass
+  int n_sms, tc_slots;
   int pass_group;       // layers per scoring launch of dkv_run_prefill_pass (1..tc::kMaxGroup)
   bool emit_backward;   // sweep 2 walks every CTA's slice from the end to the start
   bool host_v_staged;   // dkv_run_prefill_pass_host copies V in full even where the gather could read its rows in place
@@ -56,14 +48,8 @@ struct dkv_ctx {
   long long wait_cycles;   // limit of the scoring kernel's mbarrier waits (dkv_set_wait_limit)
   int withhold_sweep, withhold_tile;   // test hook of dkv_debug_withhold_tile (-1: off)
   float2* d_tc_stats;   // [3][kMaxGroup*Bt*Hkv][tc_slots][256]: partial softmax statistics, three jobs in rotation
-  cudaStream_t hi;      // scoring launches of dkv_run_prefill_pass: highest priority, so that a freed SM goes to a
-                        // waiting scoring CTA before the side streams' many short CTAs
-  cudaStream_t upd;     // budget updates (rebudget + shrink) of dkv_run_prefill_pass, off the select streams
-  cudaStream_t side[kSideStreams]; // side streams of dkv_run_prefill_pass (select / gather), layers in rotation
-  int n_side;           // how many of them the pass uses
-  cudaEvent_t ev_fork, ev_join[kSideStreams + 1], ev_update, ev_scored[DKV_MAX_LAYERS], ev_picked[DKV_MAX_LAYERS], ev_selected[DKV_MAX_LAYERS];
   // host state
-  uint8_t scored[DKV_MAX_LAYERS], gathered[DKV_MAX_LAYERS], stale[DKV_MAX_LAYERS];
+  uint8_t scored[DKV_MAX_LAYERS], gathered[DKV_MAX_LAYERS];
   uint8_t selected[DKV_MAX_LAYERS];     // 1: by scores (dkv_select_topk), 2: by position (dkv_select_positions)
   int sel_n[DKV_MAX_LAYERS];            // positions selected per head: Blc, or what dkv_select_positions kept
   // decoding over the compressed cache (allocated on first use, grown on demand)
@@ -73,8 +59,7 @@ struct dkv_ctx {
   long long launches;
   // dkv_run_prefill_pass as a CUDA graph: captured on the first call with a set of pointers, replayed afterwards
   bool use_graph;
-  cudaStream_t gstream;        // the graph is captured and replayed here, forked from / joined to the caller's stream
-  cudaEvent_t ev_gfork, ev_gjoin;
+  cudaStream_t gstream;        // the graph is captured here
   cudaGraphExec_t pass_exec;
   std::vector<const void*>* pass_key;
   long long pass_launches;
@@ -109,6 +94,12 @@ int cuda_fail(dkv_ctx* c, cudaError_t e) {
   } while (0)
 // After a launch: a launch error is reported once and cleared (cudaGetLastError), so that a refused launch
 // does not make every later call of every context fail.
+#define DKV_LAUNCH(ctx, call)                                 \
+  do {                                                        \
+    cudaError_t e__ = (call);                                 \
+    if (e__ != cudaSuccess) { cudaGetLastError(); return cuda_fail((ctx), e__); } \
+    (ctx)->launches++;                                        \
+  } while (0)
 #define DKV_LAUNCHED(ctx)                                     \
   do {                                                        \
     (ctx)->launches++;                                        \
@@ -132,6 +123,21 @@ struct ProfScope {
   }
   ~ProfScope() { if (r) cudaEventRecord(r->b, st); }
 };
+
+// Launch with programmatic stream serialisation (the kernel waits for its predecessor itself, so that its scheduling
+// overlaps the predecessor's end) and, if cluster > 1, clusters of that many blocks along x.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t st, const Args&... args) {
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = at; cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 size_t layer_scores(const Shape& s) { return (size_t)s.Bt * s.Hkv * s.P; }
 size_t layer_idx(const Shape& s) { return (size_t)s.Bt * s.Hkv * s.Blc; }
@@ -213,8 +219,9 @@ uint32_t make_idesc(int M, int N) {
 // pointers); `buf` picks the statistics scratch (jobs in flight rotate).  In sweep 2 every CTA walks its slice of the
 // key space from the end to the start: sweep 1 cut the same space into the same slices, so each CTA begins with
 // the keys that were streamed last and may still be in L2.
+// `grid`: thread blocks of the launch; `stats_grid`: of the launch that ran sweep 1 for these layers (sweep 2).
 bool make_job(dkv_ctx* c, int mode, int layer, int nl, const void* const* q, const void* const* k, float* scores_out,
-              int buf, tc::Maps* maps, tc::Params* p, const float* const* lse = nullptr) {
+              int buf, int grid, int stats_grid, bool hist, tc::Maps* maps, tc::Params* p, const float* const* lse = nullptr) {
   const Shape& s = c->s;
   const int heads = s.Bt * s.Hkv;
   memset(maps, 0, sizeof *maps);                           // entries past nl are never read
@@ -224,7 +231,7 @@ bool make_job(dkv_ctx* c, int mode, int layer, int nl, const void* const* q, con
   p->S = s.S; p->P = s.P; p->ws = s.ws; p->M = s.M; p->D = s.D; p->heads = nl * heads; p->half = s.pool / 2;
   p->nl = nl; p->hpl = heads;
   p->back = (mode == tc::kEmit && c->emit_backward) ? 1 : 0;
-  p->retain_tiles = (int)((long long)c->retain_mb * (1 << 20) / ((long long)(c->tc_grid > 0 ? c->tc_grid : 1) * tc::kTileKeys * s.D * 2));
+  p->retain_tiles = (int)((long long)c->retain_mb * (1 << 20) / ((long long)grid * tc::kTileKeys * s.D * 2));
   p->wait_cycles = c->wait_cycles;
   p->withhold_tile = c->withhold_sweep == mode ? c->withhold_tile : -1;
   p->tph = (s.S + tc::kTileKeys - 1) / tc::kTileKeys;
@@ -236,7 +243,9 @@ bool make_job(dkv_ctx* c, int mode, int layer, int nl, const void* const* q, con
   p->scores = c->d_scores + (size_t)layer * layer_scores(s);
   p->copy_out = scores_out;
   p->status = c->d_status;
-  p->stats_grid = c->tc_grid;
+  p->stats_grid = stats_grid;
+  p->layer_hist = hist ? c->d_layer_hist + (size_t)layer * s.Bt * kBins : nullptr;
+  p->hkv = s.Hkv;
   p->mode = mode;
   p->out_scale = (c->cfg.flags & DKV_F_WINDOW_MEAN) ? 1.0f / (float)s.M : 1.0f;
   p->pool_avg = c->cfg.pool_kind == 1;
@@ -246,110 +255,108 @@ bool make_job(dkv_ctx* c, int mode, int layer, int nl, const void* const* q, con
 
 // The scoring kernel for two jobs (either may be kNone): the specialised build when every job has exactly 128 window
 // rows of 128 dims, the general one otherwise.
-void launch_tc(int grid, cudaStream_t st, const tc::Maps& m0, const tc::Maps& m1, const tc::Params& j0, const tc::Params& j1) {
+cudaError_t launch_tc(int grid, cudaStream_t st, const tc::Maps& m0, const tc::Maps& m1, const tc::Params& j0, const tc::Params& j1) {
   auto fast = [](const tc::Params& p) { return p.mode == tc::kNone || (p.M == 128 && p.D == 128); };
-  if (fast(j0) && fast(j1)) tc::score_tc_kernel<true><<<grid, tc::kThreads, tc::kSmemBytes, st>>>(m0, m1, j0, j1);
-  else tc::score_tc_kernel<false><<<grid, tc::kThreads, tc::kSmemBytes, st>>>(m0, m1, j0, j1);
+  return launch_pdl(fast(j0) && fast(j1) ? tc::score_tc_kernel<true> : tc::score_tc_kernel<false>, dim3(grid), tc::kThreads,
+                    (size_t)tc::kSmemBytes, 1, st, m0, m1, j0, j1);
 }
 
-// One launch: sweep 2 of the `en` layers from `emit_layer` (if >= 0), then sweep 1 of the `sn` layers from
-// `stats_layer` (if >= 0).  In the pass the emit layers are the ones the previous launch streamed.  `sbuf`, `ebuf`: statistics scratch of either job.
-int launch_score(dkv_ctx* c, int stats_layer, int sn, const void* const* sq, const void* const* sk, int sbuf,
-                 int emit_layer, int en, const void* const* eq, const void* const* ek, int ebuf, float* scores_out,
-                 cudaStream_t st, const float* const* emit_lse = nullptr) {
+// Thread blocks of a scoring launch over `nl` layers: one an SM, fewer if there are fewer key tiles.
+int score_grid(const dkv_ctx* c, int nl) {
+  const long long tiles = (long long)nl * c->s.Bt * c->s.Hkv * ((c->s.S + tc::kTileKeys - 1) / tc::kTileKeys);
+  return (int)(tiles < c->n_sms ? tiles : c->n_sms);
+}
+
+// A group of consecutive layers that is scored together: its first layer, how many, the statistics scratch its sweep 1
+// writes and the grid it ran on.
+struct ScoreGroup { int first, n, buf, grid; };
+
+// One launch: sweep 2 of group `e` (if not null), then sweep 1 of group `s` (if not null), whose grid it sets.  `q`, `k`,
+// `lse`: all layers' pointers, indexed by layer (lse: null, or the caller's normalisers instead of sweep 1).
+int launch_score(dkv_ctx* c, const ScoreGroup* e, ScoreGroup* s, const void* const* q, const void* const* k, const float* const* lse,
+                 float* scores_out, bool hist, cudaStream_t st) {
   tc::Maps m0, m1;
   tc::Params j0, j1;
   memset(&j0, 0, sizeof j0); memset(&j1, 0, sizeof j1);
-  memset(&m0, 0, sizeof m0); memset(&m1, 0, sizeof m1);
   j0.mode = j1.mode = tc::kNone;
-  if (emit_layer >= 0 && !make_job(c, tc::kEmit, emit_layer, en, eq, ek, scores_out, ebuf, &m0, &j0, emit_lse)) return DKV_ERR_CUDA;
-  if (stats_layer >= 0 && !make_job(c, tc::kStats, stats_layer, sn, sq, sk, nullptr, sbuf, &m1, &j1)) return DKV_ERR_CUDA;
-  ProfScope ps(c, stats_layer >= 0 ? DKV_STEP_SCORE_STATS : DKV_STEP_SCORE_EMIT, 1, st);
-  launch_tc(c->tc_grid, st, m0, m1, j0, j1);
-  DKV_LAUNCHED(c);
+  const int most = e && (!s || e->n > s->n) ? e->n : s->n, grid = score_grid(c, most);
+  if (s) s->grid = grid;
+  if (e && !make_job(c, tc::kEmit, e->first, e->n, q + e->first, k + e->first, scores_out, e->buf, grid, e->grid, hist, &m0, &j0, lse ? lse + e->first : nullptr)) return DKV_ERR_CUDA;
+  if (s && !make_job(c, tc::kStats, s->first, s->n, q + s->first, k + s->first, nullptr, s->buf, grid, grid, hist, &m1, &j1)) return DKV_ERR_CUDA;
+  ProfScope ps(c, s ? DKV_STEP_SCORE_STATS : DKV_STEP_SCORE_EMIT, 1, st);
+  DKV_LAUNCH(c, launch_tc(grid, st, e ? m0 : m1, s ? m1 : m0, j0, j1));
   return DKV_OK;
 }
 
-// Sweep 2 alone, with the window rows' normalisers supplied by the caller instead of sweep 1.
-int do_score_lse(dkv_ctx* c, int layer, const void* q, const void* k, const float* lse, float* scores_out,
-                 cudaStream_t st) {
-  tc::Maps maps;
-  tc::Params job, none;
-  memset(&job, 0, sizeof job); memset(&none, 0, sizeof none);
-  none.mode = tc::kNone;
-  if (!make_job(c, tc::kEmit, layer, 1, &q, &k, scores_out, layer % 3, &maps, &job, &lse)) return DKV_ERR_CUDA;
-  ProfScope ps(c, DKV_STEP_SCORE_EMIT, 1, st);
-  launch_tc(c->tc_grid, st, maps, maps, job, none);
-  DKV_LAUNCHED(c);
+// One layer on its own; lse: as for dkv_score_lse, or null.
+int do_score(dkv_ctx* c, int layer, const void* q, const void* k, const float* lse, float* scores_out, cudaStream_t st) {
+  ScoreGroup g = {layer, 1, layer % 3, 0};
+  const void *qs[DKV_MAX_LAYERS], *ks[DKV_MAX_LAYERS];      // indexed by layer
+  const float* ls[DKV_MAX_LAYERS];
+  qs[layer] = q; ks[layer] = k; ls[layer] = lse;
+  int rc;
+  if (!lse && (rc = launch_score(c, nullptr, &g, qs, ks, nullptr, nullptr, false, st))) return rc;
+  if ((rc = launch_score(c, &g, nullptr, qs, ks, lse ? ls : nullptr, scores_out, false, st))) return rc;
   c->scored[layer] = 1;
-  c->selected[layer] = c->gathered[layer] = c->stale[layer] = 0;
-  return DKV_OK;
-}
-
-int do_score(dkv_ctx* c, int layer, const void* q, const void* k, float* scores_out, cudaStream_t st) {
-  int rc = launch_score(c, layer, 1, &q, &k, layer % 3, -1, 0, nullptr, nullptr, 0, nullptr, st);
-  if (rc) return rc;
-  if ((rc = launch_score(c, -1, 0, nullptr, nullptr, 0, layer, 1, &q, &k, layer % 3, scores_out, st))) return rc;
-  c->scored[layer] = 1;
-  c->selected[layer] = c->gathered[layer] = c->stale[layer] = 0;
+  c->selected[layer] = c->gathered[layer] = 0;
   return DKV_OK;
 }
 
 // ---- step (2): per-head top-Bl' ----------------------------------------------------------------
-int do_kept_sorted(dkv_ctx* c, int layer, int* sorted_out, cudaStream_t st) {
+// Positions of a layer's idx in ascending order and their places, see sort_positions_kernel.
+int do_sort_positions(dkv_ctx* c, int layer, const int* held, int keep, int* sorted_out, int* rank_out, cudaStream_t st) {
   const Shape& s = c->s;
-  kept_sorted_kernel<<<s.Bt * s.Hkv, kSelThreads, (size_t)((s.P + 31) / 32) * 4, st>>>(
-      c->d_idx + (size_t)layer * layer_idx(s), c->d_held, sorted_out, s.P, s.Blc, s.Hkv, s.L, layer);
+  size_t smem = 16;
+  while (smem < (size_t)keep * 8) smem <<= 1;
+  sort_positions_kernel<<<s.Bt * s.Hkv, kSelThreads, smem, st>>>(c->d_idx + (size_t)layer * layer_idx(s), held, keep, sorted_out, rank_out,
+                                                                 s.Blc, s.Hkv, s.L, layer);
   DKV_LAUNCHED(c);
   return DKV_OK;
 }
 
 int do_select(dkv_ctx* c, int layer, int* sorted_out, int* rank_out, cudaStream_t st) {
   const Shape& s = c->s;
-  const size_t heads = (size_t)s.Bt * s.Hkv;
-  ProfScope ps(c, DKV_STEP_SELECT, 1, st);
-  const float* sc = c->d_scores + (size_t)layer * layer_scores(s);
-  int* idx = c->d_idx + (size_t)layer * layer_idx(s);
-  unsigned int* lh = c->d_layer_hist + (size_t)layer * s.Bt * kBins;
-  DKV_CUDA(c, cudaMemsetAsync(lh, 0, sizeof(unsigned int) * s.Bt * kBins, st));
-  if (c->sel_reg)
-    select_topk_kernel<true><<<(unsigned)heads, kSelThreads, c->sel_smem, st>>>(
-        sc, idx, sorted_out, rank_out, lh, s.P, s.Blc, c->sort_n, c->d_count, s.Hkv, s.L, layer);
-  else
-    select_topk_kernel<false><<<(unsigned)heads, kSelThreads, c->sel_smem, st>>>(
-        sc, idx, sorted_out, rank_out, lh, s.P, s.Blc, c->sort_n, c->d_count, s.Hkv, s.L, layer);
-  DKV_LAUNCHED(c);
+  {
+    ProfScope ps(c, DKV_STEP_SELECT, 1, st);
+    unsigned int* lh = c->d_layer_hist + (size_t)layer * s.Bt * kBins;
+    DKV_CUDA(c, cudaMemsetAsync(lh, 0, sizeof(unsigned int) * s.Bt * kBins, st));
+    DKV_LAUNCH(c, launch_pdl(select_topk_kernel, dim3(s.Bt * s.Hkv), kSelThreads, select_smem(c->sel_cap), 1, st,
+                             (const float*)(c->d_scores + (size_t)layer * layer_scores(s)), c->d_idx + (size_t)layer * layer_idx(s), lh, s.P, s.Blc,
+                             c->sel_cap, c->d_count, s.Hkv, s.L, layer));
+  }
   c->selected[layer] = 1;
   c->sel_n[layer] = s.Blc;
-  c->gathered[layer] = c->stale[layer] = 0;
-  return DKV_OK;
+  c->gathered[layer] = 0;
+  return sorted_out || rank_out ? do_sort_positions(c, layer, nullptr, s.Blc, sorted_out, rank_out, st) : DKV_OK;
 }
 
 // ---- step (3): Update_Buffer_Length ------------------------------------------------------------
-int do_rebudget(dkv_ctx* c, int l, int* counts_out, cudaStream_t st) {
+// The updates after l[0] < l[1] < ... layers.  fill > 0: the counts of all layers start at `fill` (else they are what
+// the selections and earlier updates left).  The last update's integers are left in d_dbg.
+int do_rebudget(dkv_ctx* c, const int* l, int n, int fill, int* counts_out, cudaStream_t st) {
   const Shape& s = c->s;
-  long long k = (long long)s.N * s.Hkv * l;
-  const long long pop = (long long)l * s.Hkv * s.P;
-  if (k > pop) k = pop;
-  ProfScope ps(c, DKV_STEP_REBUDGET, 4, st);
-  const size_t per_layer = (size_t)s.Hkv * s.P, cand_stride = (size_t)s.L * per_layer;
-  rb_locate_kernel<<<s.Bt, 1024, 0, st>>>(c->d_layer_hist, c->d_rb_state, c->d_rb_above, c->d_rb_hist1,
-                                         c->d_rb_above2, c->d_rb_hist2, c->d_cand_n, s.Bt, s.Hkv, s.L, l, s.P, k);
-  DKV_LAUNCHED(c);
-  int slices = (int)((per_layer + (size_t)kRbThreads * 16 - 1) / ((size_t)kRbThreads * 16));
+  ProfScope ps(c, DKV_STEP_REBUDGET, 3 * ((n + kRbUpdates - 1) / kRbUpdates), st);
+  const size_t per_layer = (size_t)s.Hkv * s.P, cand_stride = (size_t)s.L * per_layer, bl = (size_t)s.Bt * s.L;
+  int slices = (int)((per_layer + kRbChunk - 1) / kRbChunk);
   if (slices > 64) slices = 64;
-  rb_refine1_kernel<<<dim3(slices, l, s.Bt), kRbThreads, 0, st>>>(c->d_scores, c->d_rb_state, c->d_rb_hist1, c->d_cand,
-                                                                 c->d_cand_n, s.Bt, per_layer, cand_stride);
-  DKV_LAUNCHED(c);
-  rb_refine2_kernel<<<dim3(256, s.Bt), kRbThreads, 0, st>>>(c->d_cand, c->d_cand_n, c->d_rb_state, c->d_rb_hist1,
-                                                          c->d_rb_above2, c->d_rb_hist2, s.L, cand_stride);
-  DKV_LAUNCHED(c);
-  const size_t bl = (size_t)s.Bt * s.L;
-  rb_budget_kernel<<<s.Bt, 1024, 0, st>>>(c->d_rb_state, c->d_rb_hist1, c->d_rb_above, c->d_rb_above2, c->d_rb_hist2,
-                                         c->d_count, c->d_dbg, c->d_dbg + bl, c->d_dbg + 2 * bl, counts_out, s.Bt, s.L, l,
-                                         s.Bl, s.N, (c->cfg.flags & DKV_F_PRORATA) != 0, (c->cfg.flags & DKV_F_NORM_MINMAX) != 0);
-  DKV_LAUNCHED(c);
-  for (int i = 0; i < l; ++i) if (!c->gathered[i]) c->stale[i] = 1;
+  for (int u0 = 0; u0 < n; u0 += kRbUpdates) {
+    RbBatch batch = {};
+    batch.n = n - u0 < kRbUpdates ? n - u0 : kRbUpdates;
+    for (int u = 0; u < batch.n; ++u) {
+      batch.l[u] = l[u0 + u];
+      batch.k[u] = (long long)s.N * s.Hkv * batch.l[u];
+      const long long pop = (long long)batch.l[u] * s.Hkv * s.P;
+      if (batch.k[u] > pop) batch.k[u] = pop;
+    }
+    DKV_LAUNCH(c, launch_pdl(rb_locate_kernel, dim3(batch.n, s.Bt), 1024, 0, 1, st, batch, (const unsigned int*)c->d_layer_hist, c->d_rb_state,
+                             c->d_rb_above, c->d_cand_n, c->d_count, u0 == 0 ? fill : 0, s.Bt, s.Hkv, s.L, s.P));
+    DKV_LAUNCH(c, launch_pdl(rb_collect_kernel, dim3(slices, batch.l[batch.n - 1], s.Bt), kRbThreads, 0, 1, st, batch, (const float*)c->d_scores,
+                             (const RbState*)c->d_rb_state, c->d_cand, c->d_cand_n, s.Bt, per_layer, cand_stride));
+    DKV_LAUNCH(c, launch_pdl(rb_finish_kernel, dim3(kRbCluster, batch.n, s.Bt), 1024, 0, kRbCluster, st, batch, (const RbState*)c->d_rb_state,
+                             (const unsigned int*)c->d_rb_above, (const uint2*)c->d_cand, (const unsigned int*)c->d_cand_n, cand_stride, c->d_count,
+                             c->d_dbg, c->d_dbg + bl, c->d_dbg + 2 * bl, u0 + batch.n == n ? batch.n - 1 : -1, counts_out, s.Bt, s.L, s.Bl, s.N,
+                             (int)((c->cfg.flags & DKV_F_PRORATA) != 0), (int)((c->cfg.flags & DKV_F_NORM_MINMAX) != 0)));
+  }
   return DKV_OK;
 }
 
@@ -358,51 +365,52 @@ int do_shrink(dkv_ctx* c, int layer0, int n, void* const* kb, void* const* vb, c
   const Shape& s = c->s;
   LayerPtrs ptrs;
   for (int i = 0; i < n; ++i) { ptrs.kb[layer0 + i] = kb[i]; ptrs.vb[layer0 + i] = vb[i]; }
-  ProfScope ps(c, DKV_STEP_SHRINK, 2, st);
-  shrink_kernel<<<dim3(s.Bt * s.Hkv, n, 2), kShrinkThreads, 0, st>>>(ptrs, layer0, c->d_count, c->d_held, s.Hkv, s.L, s.ws,
-                                                                      s.rows, s.D * 2 / 16);
-  DKV_LAUNCHED(c);
-  commit_held_kernel<<<(s.Bt * n + 127) / 128, 128, 0, st>>>(c->d_held, c->d_count, s.Bt, s.L, layer0, n);
-  DKV_LAUNCHED(c);
+  ProfScope ps(c, DKV_STEP_SHRINK, 1, st);
+  DKV_LAUNCH(c, launch_pdl(shrink_kernel, dim3(s.Bt * s.Hkv, n, 2), kShrinkThreads, 0, 1, st, ptrs, layer0, (const int*)c->d_count, c->d_held,
+                           c->d_shrink_tickets, s.Hkv, s.L, s.ws, s.rows, s.D * 2 / 16));
   return DKV_OK;
 }
 
 int do_gather(dkv_ctx* c, int layer, const void* k_src, const void* v_src, void* kb, void* vb, cudaStream_t st) {
   const Shape& s = c->s;
-  const int vec = s.D * 2 / 16, rpb = 256 / vec * kGatherRows;
-  const dim3 grid((s.rows + rpb - 1) / rpb, s.Bt * s.Hkv, 2);
-  {
+  const int vec = s.D * 2 / 16, rpb = kGatherThreads / vec * kGatherRows;
+  const dim3 grid((s.rows + rpb - 1) / rpb, s.Bt * s.Hkv);
   ProfScope ps(c, DKV_STEP_GATHER, 1, st);
-  gather_rows_kernel<<<grid, 256, 0, st>>>(static_cast<const uint4*>(k_src), static_cast<const uint4*>(v_src),
-                                           static_cast<uint4*>(kb), static_cast<uint4*>(vb),
-                                           c->d_idx + (size_t)layer * layer_idx(s), c->sel_n[layer], s.Blc, s.S, s.P, s.ws, s.rows, vec,
-                                           c->d_held, s.Hkv, s.L, layer);
-  DKV_LAUNCHED(c);
-  }
+  DKV_LAUNCH(c, launch_pdl(gather_rows_kernel, grid, kGatherThreads, 0, 1, st, static_cast<const uint4*>(k_src), static_cast<const uint4*>(v_src),
+                           static_cast<uint4*>(kb), static_cast<uint4*>(vb), (const int*)(c->d_idx + (size_t)layer * layer_idx(s)),
+                           (const int*)c->d_count, c->sel_n[layer], s.Blc, s.S, s.P, s.ws, s.rows, vec, c->d_held, s.Hkv, s.L, layer));
   c->gathered[layer] = 1;
-  if (c->stale[layer]) {           // an update ran between select and gather: apply it now
-    c->stale[layer] = 0;
-    return do_shrink(c, layer, 1, &kb, &vb, st);
-  }
   return DKV_OK;
 }
 
-// ---- decoding ------------------------------------------------------------------------------------
-// Launch with programmatic stream serialisation (the kernel waits for its predecessor itself, so that its scheduling
-// overlaps the predecessor's end) and, if cluster > 1, clusters of that many blocks along x.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t st, const Args&... args) {
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cfg.attrs = at; cfg.numAttrs = cluster > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+// The end of a pass: select and gather every layer with its final count.
+int do_select_gather(dkv_ctx* c, const void* const* k, const void* const* v, void* const* kb, void* const* vb, cudaStream_t st) {
+  const Shape& s = c->s;
+  PassPtrs ptrs;
+  for (int l = 0; l < s.L; ++l) { ptrs.k[l] = k[l]; ptrs.v[l] = v[l]; ptrs.kb[l] = kb[l]; ptrs.vb[l] = vb[l]; }
+  ProfScope ps(c, DKV_STEP_SELECT, 1, st);
+  DKV_LAUNCH(c, launch_pdl(select_gather_kernel, dim3(s.Bt * s.Hkv, s.L), kSelThreads, select_smem(c->sel_cap), 1, st, ptrs, (const float*)c->d_scores,
+                           c->d_idx, (const int*)c->d_count, c->d_held, s.P, s.ws, s.Blc, c->sel_cap, s.S, s.D * 2 / 16, s.Hkv, s.L));
+  return DKV_OK;
 }
 
+int do_reset(dkv_ctx* c, cudaStream_t st) {
+  const Shape& s = c->s;
+  DKV_CUDA(c, cudaMemsetAsync(c->d_count, 0, sizeof(int) * s.Bt * s.L, st));
+  DKV_CUDA(c, cudaMemsetAsync(c->d_held, 0, sizeof(int) * s.Bt * s.L, st));
+  DKV_CUDA(c, cudaMemsetAsync(c->d_dbg, 0, sizeof(int) * 3 * s.Bt * s.L, st));
+  memset(c->scored, 0, sizeof c->scored);
+  memset(c->selected, 0, sizeof c->selected);
+  memset(c->gathered, 0, sizeof c->gathered);
+  return DKV_OK;
+}
+
+// What the host knows after a pass.
+void mark_pass_done(dkv_ctx* c) {
+  for (int l = 0; l < c->s.L; ++l) { c->scored[l] = c->selected[l] = c->gathered[l] = 1; c->sel_n[l] = c->s.Blc; }
+}
+
+// ---- decoding ------------------------------------------------------------------------------------
 // QB = 8: up to 8 queries a head group; 16: more than 8, 16 at a time.
 template <int D, int QB>
 cudaError_t launch_decode(const DecodePtrs& ptrs, const DecodeArgs& a, int cluster, int split_grid, cudaStream_t st) {
@@ -449,114 +457,54 @@ int do_decode(dkv_ctx* c, int layer0, int nl, int nq, const void* const* q, cons
   cudaError_t e;
   if (s.D == 128) e = GQ <= 8 ? launch_decode<128, 8>(ptrs, a, cluster, split_grid, st) : launch_decode<128, 16>(ptrs, a, cluster, split_grid, st);
   else e = GQ <= 8 ? launch_decode<64, 8>(ptrs, a, cluster, split_grid, st) : launch_decode<64, 16>(ptrs, a, cluster, split_grid, st);
-  if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(c, e); }
-  c->launches++;
+  DKV_LAUNCH(c, e);
   return DKV_OK;
 }
 
-int do_reset(dkv_ctx* c, cudaStream_t st) {
-  const Shape& s = c->s;
-  DKV_CUDA(c, cudaMemsetAsync(c->d_count, 0, sizeof(int) * s.Bt * s.L, st));
-  DKV_CUDA(c, cudaMemsetAsync(c->d_held, 0, sizeof(int) * s.Bt * s.L, st));
-  DKV_CUDA(c, cudaMemsetAsync(c->d_dbg, 0, sizeof(int) * 3 * s.Bt * s.L, st));
-  memset(c->scored, 0, sizeof c->scored);
-  memset(c->selected, 0, sizeof c->selected);
-  memset(c->gathered, 0, sizeof c->gathered);
-  memset(c->stale, 0, sizeof c->stale);
-  return DKV_OK;
-}
-
-// Algorithm 1's loop.  The scoring launches run back to back on a stream of their own; launch g runs sweep 2
-// of layer group g-1 and then sweep 1 of group g (a group = up to `pass_group` consecutive layers, so that the
-// fixed cost of a launch and of a job is paid once per group).  Everything that consumes a layer's scores (select,
-// gather, and every m layers rebudget + shrink) runs on side streams behind events, layers alternating between
-// two of them, so that it overlaps the scoring of the following groups.  `st` rejoins all of them at the end.
-// With `lse` (the window rows' log-denominators of every layer) sweep 1 is not needed: launch g runs sweep 2 of group g.
+// Algorithm 1's loop, one chain of launches on `st`.
+//   scoring   launch g runs sweep 2 of layer group g-1 and then sweep 1 of group g (a group = up to `pass_group` layers, so
+//             that the fixed cost of a launch is paid once per group) on all SMs; sweep 2 also counts the scores' digits.
+//             With `lse` (the window rows' log-denominators of every layer) launch g runs sweep 2 of group g only.
+//   updates   all of Eq. 4-6's updates together: their order does not matter, a layer's count is the minimum over them
+//             and nothing reads an intermediate one.
+//   select, gather   with the final counts.
+// (Selecting and gathering B^l rows of each layer and truncating them at every update, on side streams beside the
+// scoring, took 32 of the 148 SMs from the scoring kernel and still left a tail of 0.1 ms after the last layer.)
 int do_pass(dkv_ctx* c, const void* const* q, const void* const* k, const void* const* v, const float* const* lse,
             void* const* kb, void* const* vb, cudaStream_t st) {
   const Shape& s = c->s;
-  int rc = do_reset(c, st);
-  if (rc) return rc;
-  DKV_CUDA(c, cudaEventRecord(c->ev_fork, st));
-  for (int i = 0; i < c->n_side; ++i) DKV_CUDA(c, cudaStreamWaitEvent(c->side[i], c->ev_fork, 0));
-  DKV_CUDA(c, cudaStreamWaitEvent(c->hi, c->ev_fork, 0));
-  DKV_CUDA(c, cudaStreamWaitEvent(c->upd, c->ev_fork, 0));
-  cudaStream_t caller = st;
-  st = c->hi;
-  // Group sizes: `pass_group` layers each.  (With DKV_PASS_TAPER=1 they halve towards the end, so that less work
-  // is left for after the last launch; with four select streams that tail is as short either way.)
-  int first[DKV_MAX_LAYERS + 2], groups = 0;
-  for (int done = 0; done < s.L;) {
-    int n = c->pass_taper ? (s.L - done) / 2 : c->pass_group;
-    if (n > c->pass_group) n = c->pass_group;
-    if (n > s.L - done) n = s.L - done;
-    if (n < 1) n = 1;
-    first[groups++] = done;
-    done += n;
-  }
-  first[groups] = s.L;
-  for (int g = lse ? 1 : 0; g <= groups; ++g) {
-    const int sl = g < groups && !lse ? first[g] : -1, sn = sl >= 0 ? first[g + 1] - first[g] : 0;
-    const int e0 = g > 0 ? first[g - 1] : -1, en = g > 0 ? first[g] - first[g - 1] : 0;
-    if ((rc = launch_score(c, sl, sn, sl >= 0 ? q + sl : nullptr, sl >= 0 ? k + sl : nullptr, g % 3, e0, en,
-                           e0 >= 0 ? q + e0 : nullptr, e0 >= 0 ? k + e0 : nullptr, (g + 2) % 3, nullptr, st,
-                           lse && e0 >= 0 ? lse + e0 : nullptr)))
-      return rc;
-    if (e0 < 0) continue;
-    DKV_CUDA(c, cudaEventRecord(c->ev_scored[e0], st));
-    for (int el = e0; el < e0 + en; ++el) {
-      c->scored[el] = 1;
-      cudaStream_t sd = c->side[el % c->n_side];
-      DKV_CUDA(c, cudaStreamWaitEvent(sd, c->ev_scored[e0], 0));
-      if ((rc = do_select(c, el, nullptr, nullptr, sd))) return rc;
-      DKV_CUDA(c, cudaEventRecord(c->ev_picked[el], sd));
-      if ((rc = do_gather(c, el, k[el], v[el], kb[el], vb[el], sd))) return rc;
-      DKV_CUDA(c, cudaEventRecord(c->ev_selected[el], sd));
-      const bool update = ((el + 1) % s.m == 0) || (el + 1 == s.L && s.L % s.m != 0);
-      if (update) {
-        // The rebudget needs every earlier layer selected (every select stream, each in layer order), the shrink
-        // also gathered; the previous update precedes it on the same stream.  Later layers' select and gather
-        // do not wait for it: an update changes the counts and buffers of the layers before it only.
-        for (int b = 0; b < c->n_side && b <= el; ++b) DKV_CUDA(c, cudaStreamWaitEvent(c->upd, c->ev_picked[el - b], 0));
-        if ((rc = do_rebudget(c, el + 1, nullptr, c->upd))) return rc;
-        for (int b = 0; b < c->n_side && b <= el; ++b) DKV_CUDA(c, cudaStreamWaitEvent(c->upd, c->ev_selected[el - b], 0));
-        if ((rc = do_shrink(c, 0, el + 1, kb, vb, c->upd))) return rc;
-      }
+  int rc;
+  if (lse) DKV_CUDA(c, cudaMemsetAsync(c->d_layer_hist, 0, sizeof(unsigned int) * s.L * s.Bt * kBins, st));   // else sweep 1 does it
+  ScoreGroup prev = {}, cur = {};
+  for (int g = 0, done = 0; done < s.L || prev.n; ++g) {
+    cur.first = done; cur.n = s.L - done < c->pass_group ? s.L - done : c->pass_group; cur.buf = g % 3;
+    done += cur.n;
+    if (lse) {
+      if (!cur.n) break;
+      rc = launch_score(c, &cur, nullptr, q, k, lse, nullptr, true, st);
+    } else {
+      rc = launch_score(c, prev.n ? &prev : nullptr, cur.n ? &cur : nullptr, q, k, nullptr, nullptr, true, st);
+      prev = cur;
     }
+    if (rc) return rc;
   }
-  for (int i = 0; i < c->n_side; ++i) {
-    DKV_CUDA(c, cudaEventRecord(c->ev_join[i], c->side[i]));
-    DKV_CUDA(c, cudaStreamWaitEvent(caller, c->ev_join[i], 0));
-  }
-  DKV_CUDA(c, cudaEventRecord(c->ev_join[kSideStreams], c->hi));
-  DKV_CUDA(c, cudaStreamWaitEvent(caller, c->ev_join[kSideStreams], 0));
-  DKV_CUDA(c, cudaEventRecord(c->ev_update, c->upd));
-  DKV_CUDA(c, cudaStreamWaitEvent(caller, c->ev_update, 0));
+  int l[DKV_MAX_LAYERS], n = 0;
+  for (int u = s.m; u < s.L; u += s.m) l[n++] = u;
+  l[n++] = s.L;                                              // after the last layer whether or not m divides L
+  if ((rc = do_rebudget(c, l, n, s.Blc, nullptr, st))) return rc;
+  if ((rc = do_select_gather(c, k, v, kb, vb, st))) return rc;
+  mark_pass_done(c);
   return DKV_OK;
 }
 
 void free_all(dkv_ctx* c) {
-  cudaFree(c->d_scores); cudaFree(c->d_idx); cudaFree(c->d_count);
-  cudaFree(c->d_held); cudaFree(c->d_dbg); cudaFree(c->d_rb_state); cudaFree(c->d_rb_above); cudaFree(c->d_rb_hist1);
-  cudaFree(c->d_rb_above2); cudaFree(c->d_rb_hist2); cudaFree(c->d_layer_hist);
+  cudaFree(c->d_scores); cudaFree(c->d_idx); cudaFree(c->d_count); cudaFree(c->d_held); cudaFree(c->d_dbg);
+  cudaFree(c->d_rb_state); cudaFree(c->d_rb_above); cudaFree(c->d_layer_hist); cudaFree(c->d_shrink_tickets);
   cudaFree(c->d_cand); cudaFree(c->d_cand_n); cudaFree(c->d_status); cudaFree(c->d_tc_stats);
   cudaFree(c->d_dec_scratch); cudaFree(c->d_dec_tickets);
-  for (int i = 0; i < kSideStreams; ++i) if (c->side[i]) cudaStreamDestroy(c->side[i]);
-  if (c->hi) cudaStreamDestroy(c->hi);
   if (c->pass_exec) cudaGraphExecDestroy(c->pass_exec);
   delete c->pass_key;
   if (c->gstream) cudaStreamDestroy(c->gstream);
-  if (c->ev_gfork) cudaEventDestroy(c->ev_gfork);
-  if (c->ev_gjoin) cudaEventDestroy(c->ev_gjoin);
-  if (c->upd) cudaStreamDestroy(c->upd);
-  for (int i = 0; i <= kSideStreams; ++i) if (c->ev_join[i]) cudaEventDestroy(c->ev_join[i]);
-  if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-  if (c->ev_update) cudaEventDestroy(c->ev_update);
-  for (int l = 0; l < DKV_MAX_LAYERS; ++l) {
-    if (c->ev_scored[l]) cudaEventDestroy(c->ev_scored[l]);
-    if (c->ev_selected[l]) cudaEventDestroy(c->ev_selected[l]);
-    if (c->ev_picked[l]) cudaEventDestroy(c->ev_picked[l]);
-  }
   if (c->prof_recs) {
     for (ProfRec& r : *c->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     delete c->prof_recs;
@@ -628,35 +576,20 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   s.m = cfg->update_interval;
   s.G = s.Hq / s.Hkv; s.P = s.S - s.ws; s.M = s.ws * s.G; s.Blc = s.Bl < s.P ? s.Bl : s.P; s.rows = s.Blc + s.ws;
   const int heads = s.Bt * s.Hkv;
-  c->sort_n = 2;
-  while (c->sort_n < s.Blc) c->sort_n <<= 1;
+  c->sel_cap = 1024;                                       // a quarter more than B^l for the rest of the threshold's digit
+  while (c->sel_cap < s.Blc + s.Blc / 4 && c->sel_cap < DKV_MAX_LAYER_BUDGET) c->sel_cap <<= 1;
 
   cudaError_t e = cudaGetDevice(&c->device);
   {
     int sms = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     c->n_sms = sms > 0 ? sms : 1;
+    // thread blocks that share a head in sweep 1: its share of the grid, one cut at either end
+    c->tc_slots = c->n_sms / heads + 2;
     const int tph = (s.S + tc::kTileKeys - 1) / tc::kTileKeys;
-    const long long total_tiles = (long long)heads * tph;
-    // leave some SMs to the select / gather / update kernels that dkv_run_prefill_pass runs beside the scoring:
-    // with grouped launches up to four layers' selects (one CTA per head) are in flight at once
-    int side = 4 * heads < c->n_sms * 2 / 9 ? 4 * heads : c->n_sms * 2 / 9;
-    side = env_int("DKV_SIDE_SMS", side, 0, c->n_sms - 1);
-    int score_sms = c->n_sms - side;
-    if (score_sms < 1) score_sms = 1;
-    c->tc_grid = (int)(total_tiles < score_sms ? total_tiles : score_sms);
-    int slots = 1;
-    for (int nl = 1; nl <= tc::kMaxGroup; ++nl)           // a job may cover up to kMaxGroup layers (the pass groups them)
-      for (int bh = 0; bh < nl * heads; ++bh) {
-        const int lo = tc::tile_owner((long long)bh * tph, nl * total_tiles, c->tc_grid);
-        const int hi = tc::tile_owner((long long)(bh + 1) * tph - 1, nl * total_tiles, c->tc_grid);
-        if (hi - lo + 1 > slots) slots = hi - lo + 1;
-      }
-    c->tc_slots = slots;
+    const long long per_cta = (long long)heads * tph / c->n_sms;
     // layers per scoring launch of the pass: enough that a CTA's share of a job is some tens of tiles
-    c->pass_group = env_int("DKV_PASS_GROUP", total_tiles / c->tc_grid < 8 ? tc::kMaxGroup : 4, 1, tc::kMaxGroup);
-    c->pass_taper = env_int("DKV_PASS_TAPER", 0, 0, 1);
-    c->n_side = env_int("DKV_SIDE_STREAMS", kSideStreams, 1, kSideStreams);
+    c->pass_group = env_int("DKV_PASS_GROUP", per_cta < 8 ? tc::kMaxGroup : 4, 1, tc::kMaxGroup);
     c->emit_backward = env_int("DKV_EMIT_FORWARD", 0, 0, 1) == 0;
     // Sweep 2 starts on the keys sweep 1 streamed last: that much of a job (4/7 of L2, 72 of 126 MB) is loaded with
     // an evict-last policy, every other key tile and the gather's rows evict-first, so that neither the rest of the
@@ -676,51 +609,33 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   TRY(cudaMalloc(&c->d_count, sizeof(int) * bl));
   TRY(cudaMalloc(&c->d_held, sizeof(int) * bl));
   TRY(cudaMalloc(&c->d_dbg, sizeof(int) * 3 * bl));
-  TRY(cudaMalloc(&c->d_rb_state, sizeof(RbState) * s.Bt));
-  TRY(cudaMalloc(&c->d_rb_above, sizeof(unsigned int) * bl));
-  TRY(cudaMalloc(&c->d_rb_above2, sizeof(unsigned int) * bl));
-  TRY(cudaMalloc(&c->d_rb_hist1, sizeof(unsigned int) * s.Bt * kBins));
-  TRY(cudaMalloc(&c->d_rb_hist2, sizeof(unsigned int) * bl * 1024));
+  TRY(cudaMalloc(&c->d_rb_state, sizeof(RbState) * kRbUpdates * s.Bt));
+  TRY(cudaMalloc(&c->d_rb_above, sizeof(unsigned int) * kRbUpdates * bl));
+  TRY(cudaMalloc(&c->d_shrink_tickets, sizeof(unsigned int) * bl));
+  TRY(cudaMemset(c->d_shrink_tickets, 0, sizeof(unsigned int) * bl));
   TRY(cudaMalloc(&c->d_layer_hist, sizeof(unsigned int) * s.L * s.Bt * kBins));
   TRY(cudaMalloc(&c->d_cand, sizeof(uint2) * s.L * layer_scores(s)));
   TRY(cudaMalloc(&c->d_cand_n, sizeof(unsigned int) * s.Bt));
   TRY(cudaMalloc(&c->d_tc_stats, sizeof(float2) * 3 * tc::kMaxGroup * heads * c->tc_slots * 256));
   TRY(cudaFuncSetAttribute(tc::score_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes));
   TRY(cudaFuncSetAttribute(tc::score_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes));
-  for (int i = 0; i < kSideStreams; ++i) TRY(cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking));
   TRY(cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking));
-  TRY(cudaEventCreateWithFlags(&c->ev_gfork, cudaEventDisableTiming));
-  TRY(cudaEventCreateWithFlags(&c->ev_gjoin, cudaEventDisableTiming));
   c->pass_key = new (std::nothrow) std::vector<const void*>();
   if (!c->pass_key) { free_all(c); delete c; return DKV_ERR_NOMEM; }
   c->use_graph = env_int("DKV_NO_GRAPH", 0, 0, 1) == 0;
-  TRY(cudaStreamCreateWithFlags(&c->upd, cudaStreamNonBlocking));
-  {
-    int least = 0, greatest = 0;
-    TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-    TRY(cudaStreamCreateWithPriority(&c->hi, cudaStreamNonBlocking, greatest));
-  }
-  for (int i = 0; i <= kSideStreams; ++i) TRY(cudaEventCreateWithFlags(&c->ev_join[i], cudaEventDisableTiming));
-  TRY(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
-  TRY(cudaEventCreateWithFlags(&c->ev_update, cudaEventDisableTiming));
-  for (int l = 0; l < s.L; ++l) {
-    TRY(cudaEventCreateWithFlags(&c->ev_scored[l], cudaEventDisableTiming));
-    TRY(cudaEventCreateWithFlags(&c->ev_selected[l], cudaEventDisableTiming));
-    TRY(cudaEventCreateWithFlags(&c->ev_picked[l], cudaEventDisableTiming));
-  }
   TRY(cudaMalloc(&c->d_status, sizeof(int) * 8));
   TRY(cudaMemset(c->d_status, 0, sizeof(int) * 8));
   TRY(cudaMemset(c->d_count, 0, sizeof(int) * bl));
   TRY(cudaMemset(c->d_held, 0, sizeof(int) * bl));
   TRY(cudaMemset(c->d_dbg, 0, sizeof(int) * 3 * bl));
+  // The attributes belong to the functions, not to this context: always the most any valid configuration needs, so that
+  // contexts do not undo each other.
   {
-    c->sel_reg = (s.P + kSelThreads - 1) / kSelThreads <= kRegChunk;
-    c->sel_smem = (size_t)c->sort_n * 8 + (size_t)s.Blc * 4;
+    const int most = (int)(select_smem(kMaxCountingList) > select_smem(DKV_MAX_LAYER_BUDGET) ? select_smem(kMaxCountingList) : select_smem(DKV_MAX_LAYER_BUDGET));
+    TRY(cudaFuncSetAttribute(select_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRY(cudaFuncSetAttribute(select_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRY(cudaFuncSetAttribute(sort_positions_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DKV_MAX_LAYER_BUDGET * 8));
   }
-  // The attribute belongs to the function, not to this context: always the most any valid configuration needs
-  // (sort keys 8 B and positions 4 B for DKV_MAX_LAYER_BUDGET entries), so that contexts do not undo each other.
-  TRY(cudaFuncSetAttribute(select_topk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelMaxSmem));
-  TRY(cudaFuncSetAttribute(select_topk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelMaxSmem));
 #undef TRY
   if (e != cudaSuccess) {
     rc = e == cudaErrorMemoryAllocation ? DKV_ERR_NOMEM : DKV_ERR_CUDA;
@@ -750,7 +665,7 @@ int dkv_score(dkv_ctx* c, int32_t layer, const void* q_win, const void* k, float
   int rc = check_layer(c, layer);
   if (rc) return rc;
   if (!q_win || !k || !aligned16(q_win) || !aligned16(k) || !aligned16(scores_out)) return DKV_ERR_INVALID_ARG;
-  return do_score(c, layer, q_win, k, scores_out, as_stream(stream));
+  return do_score(c, layer, q_win, k, nullptr, scores_out, as_stream(stream));
 }
 
 int dkv_score_lse(dkv_ctx* c, int32_t layer, const void* q_win, const void* k, const float* lse, float* scores_out,
@@ -759,7 +674,7 @@ int dkv_score_lse(dkv_ctx* c, int32_t layer, const void* q_win, const void* k, c
   if (rc) return rc;
   if (!q_win || !k || !lse || !aligned16(q_win) || !aligned16(k) || !aligned16(scores_out) || ((uintptr_t)lse & 3))
     return DKV_ERR_INVALID_ARG;
-  return do_score_lse(c, layer, q_win, k, lse, scores_out, as_stream(stream));
+  return do_score(c, layer, q_win, k, lse, scores_out, as_stream(stream));
 }
 
 int dkv_set_scores(dkv_ctx* c, int32_t layer, const float* scores, void* stream) {
@@ -770,7 +685,7 @@ int dkv_set_scores(dkv_ctx* c, int32_t layer, const float* scores, void* stream)
   DKV_CUDA(c, cudaMemcpyAsync(c->d_scores + (size_t)layer * n, scores, n * sizeof(float), cudaMemcpyDeviceToDevice,
                               as_stream(stream)));
   c->scored[layer] = 1;
-  c->selected[layer] = c->gathered[layer] = c->stale[layer] = 0;
+  c->selected[layer] = c->gathered[layer] = 0;
   return DKV_OK;
 }
 
@@ -784,7 +699,7 @@ int dkv_select_topk(dkv_ctx* c, int32_t layer, int32_t* idx_out, int32_t* rank_o
 int dkv_rebudget(dkv_ctx* c, int32_t upto_layer, int32_t* counts_out, void* stream) {
   if (!c || upto_layer < 1 || upto_layer > c->s.L) return DKV_ERR_INVALID_ARG;
   for (int i = 0; i < upto_layer; ++i) if (!c->scored[i] || c->selected[i] != 1) return DKV_ERR_STATE;
-  return do_rebudget(c, upto_layer, counts_out, as_stream(stream));
+  return do_rebudget(c, &upto_layer, 1, 0, counts_out, as_stream(stream));
 }
 
 int dkv_compact(dkv_ctx* c, int32_t layer, const void* k_src, const void* v_src, void* kb, void* vb, int32_t* len_out,
@@ -842,7 +757,7 @@ static int run_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, 
     key.push_back(lse ? lse[l] : nullptr);
   }
   if (!c->pass_exec || *c->pass_key != key) {
-    // first call with these buffers: record the whole pass (all streams of do_pass fork from and rejoin gstream)
+    // first call with these buffers: record the whole pass
     if (c->pass_exec) { cudaGraphExecDestroy(c->pass_exec); c->pass_exec = nullptr; }
     const long long before = c->launches;
     cudaGraph_t graph = nullptr;
@@ -867,13 +782,9 @@ static int run_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, 
     }
     *c->pass_key = key;
   }
-  DKV_CUDA(c, cudaEventRecord(c->ev_gfork, st));
-  DKV_CUDA(c, cudaStreamWaitEvent(c->gstream, c->ev_gfork, 0));
-  DKV_CUDA(c, cudaGraphLaunch(c->pass_exec, c->gstream));
-  DKV_CUDA(c, cudaEventRecord(c->ev_gjoin, c->gstream));
-  DKV_CUDA(c, cudaStreamWaitEvent(st, c->ev_gjoin, 0));
+  DKV_CUDA(c, cudaGraphLaunch(c->pass_exec, st));
   c->launches += c->pass_launches;
-  for (int l = 0; l < c->s.L; ++l) { c->scored[l] = c->selected[l] = c->gathered[l] = 1; c->stale[l] = 0; c->sel_n[l] = c->s.Blc; }
+  mark_pass_done(c);
   return DKV_OK;
 }
 
@@ -925,14 +836,15 @@ int dkv_run_prefill_pass_host(dkv_ctx* c, const void* const* q_win, const void* 
     }
     DKV_CUDA(c, cudaEventRecord(c->ev_copied[slot], cp));
     DKV_CUDA(c, cudaStreamWaitEvent(st, c->ev_copied[slot], 0));
-    if ((rc = do_score(c, l, c->st_q[slot], c->st_k[slot], nullptr, st))) return rc;
+    if ((rc = do_score(c, l, c->st_q[slot], c->st_k[slot], nullptr, nullptr, st))) return rc;
     if ((rc = do_select(c, l, nullptr, nullptr, st))) return rc;
     if ((rc = do_gather(c, l, c->st_k[slot], v_dev[l] ? v_dev[l] : c->st_v[slot], c->st_kb[l], c->st_vb[l], st))) return rc;
     if (v_dev[l]) h2d += (long long)(c->sel_n[l] + s.ws) * s.Bt * s.Hkv * row_bytes;
     DKV_CUDA(c, cudaEventRecord(c->ev_consumed[slot], st));
     const bool update = ((l + 1) % s.m == 0) || (l + 1 == s.L && s.L % s.m != 0);
     if (update) {
-      if ((rc = do_rebudget(c, l + 1, nullptr, st))) return rc;
+      const int upto = l + 1;
+      if ((rc = do_rebudget(c, &upto, 1, 0, nullptr, st))) return rc;
       if ((rc = do_shrink(c, 0, l + 1, c->st_kb, c->st_vb, st))) return rc;
     }
   }
@@ -973,7 +885,6 @@ int dkv_apply_policy(dkv_ctx* c, int32_t policy, int32_t* counts_out, void* stre
   for (int i = 0; i < s.L; ++i) if (!c->selected[i]) return DKV_ERR_STATE;
   policy_counts_kernel<<<(s.Bt * s.L + 127) / 128, 128, 0, as_stream(stream)>>>(c->d_count, counts_out, s.Bt, s.L, s.N, policy);
   DKV_LAUNCHED(c);
-  for (int i = 0; i < s.L; ++i) if (!c->gathered[i]) c->stale[i] = 1;
   return DKV_OK;
 }
 
@@ -995,7 +906,7 @@ int dkv_select_positions(dkv_ctx* c, int32_t layer, int32_t n_sink, int32_t n_re
   }
   c->selected[layer] = 2;
   c->sel_n[layer] = n;
-  c->gathered[layer] = c->stale[layer] = 0;
+  c->gathered[layer] = 0;
   return DKV_OK;
 }
 
@@ -1039,7 +950,7 @@ int dkv_kept_sorted(dkv_ctx* c, int32_t layer, int32_t* sorted_out, void* stream
   if (rc) return rc;
   if (!sorted_out) return DKV_ERR_INVALID_ARG;
   if (!c->gathered[layer]) return DKV_ERR_STATE;
-  return do_kept_sorted(c, layer, sorted_out, as_stream(stream));
+  return do_sort_positions(c, layer, c->d_held, c->sel_n[layer], sorted_out, nullptr, as_stream(stream));
 }
 
 int dkv_budget_views(dkv_ctx* c, const int32_t** cnt, const int32_t** z, const int32_t** zp, const int32_t** held) {
@@ -1129,12 +1040,10 @@ int dkv_score_static(const dkv_config* cfg, const void* q_win, const void* k, fl
   p.stats_grid = grid;
   p.mode = tc::kStats;
   p.idesc = make_idesc(128, 128);
-  launch_tc(grid, st, maps, maps, p, none);
-  if (cudaGetLastError() != cudaSuccess) return DKV_ERR_CUDA;
+  if (launch_tc(grid, st, maps, maps, p, none) != cudaSuccess) { cudaGetLastError(); return DKV_ERR_CUDA; }
   p.mode = tc::kEmit;
   p.idesc = make_idesc(128, p.nq16);
-  launch_tc(grid, st, maps, maps, none, p);
-  if (cudaGetLastError() != cudaSuccess) return DKV_ERR_CUDA;
+  if (launch_tc(grid, st, maps, maps, none, p) != cudaSuccess) { cudaGetLastError(); return DKV_ERR_CUDA; }
   return DKV_OK;
 }
 

@@ -1,109 +1,120 @@
 // Update_Buffer_Length (Eq. 4-6) on the device: the K-th largest of all scores of the layers processed
 // so far, the number of top-K hits per layer, then the integer budget arithmetic.
 //
-// Only per-layer counts leave the selection.  Every layer's scores were histogrammed by their first
-// 11-bit digit when the layer was selected (select.cuh), so:
-//   rb_locate   adds up the histograms of layers [0, l), finds the digit b* that holds the K-th
-//               largest score, and counts each layer's scores above b* from its histogram;
-//   rb_refine1  streams the history once, copies the scores whose first digit is b* (with their layer)
-//               into a candidate list and histograms their next 11 bits;
-//   rb_refine2  counts, per layer, the candidates above the second digit and histograms the last
-//               10 bits of those that match it;
-//   rb_budget   fixes the exact threshold T, gives the entries equal to T to the lowest layers first
+// Only per-layer counts leave the selection.  Every layer's scores were histogrammed by their digit (select.cuh) when
+// they were computed or selected, so:
+//   rb_locate   adds up the histograms of layers [0, l), finds the digit that holds the K-th largest score and
+//               counts each layer's scores above it (no score is read);
+//   rb_collect  streams the history once and lists the scores with that digit (1 or 2 % of it) with their layers;
+//   rb_finish   fixes the exact threshold T from the list, gives the entries equal to T to the lowest layers first
 //               (flat-index tie rule), and evaluates Eq. 5-6 in exact integers.
+// Counts only ever shrink (count_i = min over the updates that include layer i), so a pass runs all its updates
+// together when every layer has been scored: one launch of each kernel for up to kRbUpdates updates, one read of the
+// history instead of one per update.
 #pragma once
+#include <cooperative_groups.h>
 #include "common.cuh"
 #include "select.cuh"
 
 namespace dkv {
 
+constexpr int kRbUpdates = 8;      // updates worked on together
 constexpr int kRbThreads = 256;
+constexpr int kRbChunk = 4096;     // scores of a block's slice read at a time
+constexpr int kRbCluster = 8;      // blocks that share a long candidate list
+constexpr unsigned int kRbSolo = 32768;   // candidates one block works through by itself (32 per thread)
 
-struct RbState {          // per sample
-  int bstar;              // first digit of T
-  int need1;              // entries still to take inside bucket b*
-  int cand;               // entries in bucket b* over all layers and heads
+struct RbBatch {                   // updates u = 0 .. n-1, l ascending
+  int n;
+  int l[kRbUpdates];               // layers [0, l) take part
+  long long k[kRbUpdates];         // the K of the global top-K
+};
+
+struct RbState {                   // per update and sample
+  int digit;                       // digit of T
+  int need;                        // entries still to take inside it
+  int inside;                      // entries with that digit over all layers and heads
   int pad;
 };
 
-// One CTA of 1024 threads per sample.
-// layer_hist: [L][Bt][2048].  above: [Bt][L] scores above bucket b* per layer.
-// hist1: [Bt][2048], above2: [Bt][L], hist2: [Bt][L][1024], cand_n: [Bt] are cleared here for the refine kernels.
+// grid (updates, Bt).  layer_hist: [L][Bt][2048].  state: [updates][Bt].  above: [updates][Bt][L] scores above the digit
+// per layer.  Clears cand_n [Bt]; fill > 0: count[b][.] starts at `fill` (a pass selects after the updates).
 __global__ void __launch_bounds__(1024)
-rb_locate_kernel(const unsigned int* __restrict__ layer_hist, RbState* __restrict__ state,
-                 unsigned int* __restrict__ above, unsigned int* __restrict__ hist1, unsigned int* __restrict__ above2,
-                 unsigned int* __restrict__ hist2, unsigned int* __restrict__ cand_n, int Bt, int Hkv, int L, int l, int P,
-                 long long k) {
+rb_locate_kernel(const __grid_constant__ RbBatch batch, const unsigned int* __restrict__ layer_hist, RbState* __restrict__ state,
+                 unsigned int* __restrict__ above, unsigned int* __restrict__ cand_n, int* __restrict__ count, int fill, int Bt,
+                 int Hkv, int L, int P) {
   __shared__ unsigned int hist[kBins];
   __shared__ int sm_scan[33];
   __shared__ int found[2];
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int u = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, l = batch.l[u];
+  pdl_launch();
+  pdl_wait();
   {
     // two digits per thread, summed over the layers (consecutive threads read consecutive words)
     uint2 a = make_uint2(0, 0);
+#pragma unroll 8
     for (int i = 0; i < l; ++i) {
       const uint2 x = reinterpret_cast<const uint2*>(layer_hist + ((size_t)i * Bt + b) * kBins)[tid];
       a.x += x.x; a.y += x.y;
     }
     hist[2 * tid] = a.x; hist[2 * tid + 1] = a.y;
-    hist1[(size_t)b * kBins + 2 * tid] = 0; hist1[(size_t)b * kBins + 2 * tid + 1] = 0;
   }
-  if (tid == 0) cand_n[b] = 0;
-  for (int e = tid; e < L; e += 1024) above2[b * L + e] = 0;
-  for (int e = tid; e < l * 1024; e += 1024) hist2[(size_t)b * L * 1024 + e] = 0;
+  if (u == 0) {
+    if (tid == 0) cand_n[b] = 0;
+    if (fill > 0) for (int e = tid; e < L; e += 1024) count[b * L + e] = fill;
+  }
   __syncthreads();
-  const long long total = (long long)l * Hkv * P;
-  find_digit(hist, kBins, (int)total, (int)k, sm_scan, found, nullptr);
+  find_digit(hist, kBins, (int)((long long)l * Hkv * P), (int)batch.k[u], sm_scan, found);
   const int d = found[0];
-  if (tid == 0) { RbState st; st.bstar = d; st.need1 = found[1]; st.cand = (int)hist[d]; st.pad = 0; state[b] = st; }
-  // one warp per layer: the layer's scores in the digits above b*
+  if (tid == 0) { RbState st; st.digit = d; st.need = found[1]; st.inside = (int)hist[d]; st.pad = 0; state[u * Bt + b] = st; }
+  // one warp per layer: the layer's scores in the digits above
   for (int i = warp; i < l; i += 32) {
     const unsigned int* lh = layer_hist + ((size_t)i * Bt + b) * kBins;
     unsigned int a = 0;
+#pragma unroll 8
     for (int bin = d + 1 + lane; bin < kBins; bin += 32) a += lh[bin];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-    if (lane == 0) above[b * L + i] = a;
+    a = __reduce_add_sync(0xFFFFFFFFu, a);
+    if (lane == 0) above[((size_t)u * Bt + b) * L + i] = a;
   }
 }
 
-// grid (slices, l, Bt): one pass over the scores of layers [0, l).  Scores whose first digit is b* go to the
-// sample's candidate list (value, layer) and into the second-digit histogram.  The list has room for every
-// score (cand[b] holds l*Hkv*P pairs at most); its order is arbitrary, only counts are taken from it.
-// A block reads its slice once, in chunks of kRbChunk scores: matches are parked in shared memory, then the
-// block reserves a range of the list with one atomic and copies them out.
-constexpr int kRbChunk = 4096;
+// grid (slices, layers, Bt): one pass over the scores of the batch's layers.  A score whose digit is that of an update
+// that includes its layer goes to the sample's candidate list as (pattern, layer).  The list has room for every score
+// (cand_stride pairs per sample); its order is arbitrary, only counts are taken from it.  Matches are parked in shared
+// memory, then the block reserves a range of the list with one atomic and copies them out.
 __global__ void __launch_bounds__(kRbThreads)
-rb_refine1_kernel(const float* __restrict__ scores, const RbState* __restrict__ state, unsigned int* __restrict__ hist1,
-                  uint2* __restrict__ cand, unsigned int* __restrict__ cand_n, int Bt, size_t per_layer /* Hkv*P */,
-                  size_t cand_stride) {
-  __shared__ unsigned int sh[kBins];
+rb_collect_kernel(const __grid_constant__ RbBatch batch, const float* __restrict__ scores, const RbState* __restrict__ state,
+                  uint2* __restrict__ cand, unsigned int* __restrict__ cand_n, int Bt, size_t per_layer /* Hkv*P */, size_t cand_stride) {
   __shared__ uint32_t parked[kRbChunk];
+  __shared__ unsigned int wanted[kBins / 32];
   __shared__ unsigned int s_cnt, s_base;
   const int b = blockIdx.z, i = blockIdx.y;
-  const uint32_t d = (uint32_t)state[b].bstar;
   const uint32_t* v = reinterpret_cast<const uint32_t*>(scores) + ((size_t)i * Bt + b) * per_layer;
-  for (int j = threadIdx.x; j < kBins; j += kRbThreads) sh[j] = 0;
   const size_t per_block = (per_layer + gridDim.x - 1) / gridDim.x;
   const size_t e0 = (size_t)blockIdx.x * per_block, e1 = e0 + per_block < per_layer ? e0 + per_block : per_layer;
   uint2* list = cand + (size_t)b * cand_stride;
+  if (threadIdx.x < kBins / 32) wanted[threadIdx.x] = 0;
+  pdl_launch();
+  pdl_wait();
+  __syncthreads();
+  if (threadIdx.x < batch.n && batch.l[threadIdx.x] > i) {
+    const int d = state[threadIdx.x * Bt + b].digit;
+    atomicOr(&wanted[d >> 5], 1u << (d & 31));
+  }
   for (size_t c0 = e0; c0 < e1; c0 += kRbChunk) {
     if (threadIdx.x == 0) s_cnt = 0;
     __syncthreads();
-    const size_t c1 = c0 + kRbChunk < e1 ? c0 + kRbChunk : e1;
     uint32_t u[kRbChunk / kRbThreads];
 #pragma unroll
     for (int j = 0; j < kRbChunk / kRbThreads; ++j) {          // all loads of the chunk in flight together
       const size_t e = c0 + threadIdx.x + (size_t)j * kRbThreads;
-      u[j] = e < c1 ? v[e] : 0xFFFFFFFFu;                      // (a NaN pattern: its first digit 2047 never is b*)
+      u[j] = e < e1 ? v[e] : 0u;
     }
 #pragma unroll
     for (int j = 0; j < kRbChunk / kRbThreads; ++j) {
       const size_t e = c0 + threadIdx.x + (size_t)j * kRbThreads;
-      if (e < c1 && (u[j] >> 21) == d) {
-        parked[atomicAdd(&s_cnt, 1u)] = u[j];
-        atomicAdd(&sh[(u[j] >> 10) & 2047u], 1u);
-      }
+      const int d = digit_of(u[j]);
+      if (e < e1 && (wanted[d >> 5] >> (d & 31) & 1u)) parked[atomicAdd(&s_cnt, 1u)] = u[j];
     }
     __syncthreads();
     const unsigned int n = s_cnt;
@@ -114,134 +125,127 @@ rb_refine1_kernel(const float* __restrict__ scores, const RbState* __restrict__ 
     }
     __syncthreads();
   }
-  for (int j = threadIdx.x; j < kBins; j += kRbThreads) { const unsigned int c = sh[j]; if (c) atomicAdd(&hist1[(size_t)b * kBins + j], c); }
 }
 
-// grid (slices, Bt) over the candidate list.  Every block re-derives the second digit s* from hist1; then per
-// layer: candidates with a larger second digit (above2) and the last-10-bit histogram of those with second
-// digit s* (hist2).
-__global__ void __launch_bounds__(kRbThreads)
-rb_refine2_kernel(const uint2* __restrict__ cand, const unsigned int* __restrict__ cand_n, const RbState* __restrict__ state,
-                  const unsigned int* __restrict__ hist1, unsigned int* __restrict__ above2,
-                  unsigned int* __restrict__ hist2, int L, size_t cand_stride) {
-  __shared__ unsigned int sh[kBins];
-  __shared__ int sm_scan[33];
-  __shared__ int found[2];
-  const int b = blockIdx.y;
-  const RbState st = state[b];
-  const unsigned int n = cand_n[b];
-  if (blockIdx.x * kRbThreads >= n) return;
-  for (int j = threadIdx.x; j < kBins; j += kRbThreads) sh[j] = hist1[(size_t)b * kBins + j];
-  __syncthreads();
-  find_digit(sh, kBins, st.cand, st.need1, sm_scan, found, nullptr);
-  const uint32_t s2 = (uint32_t)found[0];
-  const uint2* list = cand + (size_t)b * cand_stride;
-  // the per-layer counters are few and hot: count in shared memory (sh is free again), one global add per layer
-  __syncthreads();
-  for (int j = threadIdx.x; j < L; j += kRbThreads) sh[j] = 0;
-  __syncthreads();
-  for (unsigned int e = blockIdx.x * kRbThreads + threadIdx.x; e < n; e += gridDim.x * kRbThreads) {
-    const uint2 c = list[e];
-    const uint32_t dd = (c.x >> 10) & 2047u;
-    if (dd > s2) atomicAdd(&sh[c.y], 1u);
-    else if (dd == s2) atomicAdd(&hist2[((size_t)b * L + c.y) * 1024 + (c.x & 1023u)], 1u);
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < L; j += kRbThreads) { const unsigned int v = sh[j]; if (v) atomicAdd(&above2[b * L + j], v); }
-}
-
-// One CTA of 1024 threads per sample: exact T, per-layer hits, Eq. 5-6.
+// One cluster of kRbCluster blocks of 1024 threads per update and sample: exact T, per-layer hits, Eq. 5-6.  A list of
+// up to kRbSolo candidates is left to the cluster's first block, a longer one (flat scores, many ties) is shared.
 // cnt_i = hits of layer i among the K largest (ties at T to the lowest layers first);
 // Z_i = floor(Bl*cnt_i/max cnt); Z'_i = floor(Z_i*N*L/sum Z); count_i = min(count_i, Z'_i).
+// grid (kRbCluster, updates, Bt).  dbg_*: [Bt][L], of update `shown` (-1: none).  counts_out (single updates only): a copy.
 __global__ void __launch_bounds__(1024)
-rb_budget_kernel(const RbState* __restrict__ state, const unsigned int* __restrict__ hist1,
-                 const unsigned int* __restrict__ above, const unsigned int* __restrict__ above2,
-                 const unsigned int* __restrict__ hist2, int* __restrict__ count, int* __restrict__ dbg_cnt,
-                 int* __restrict__ dbg_z, int* __restrict__ dbg_zp, int* __restrict__ counts_out,
-                 int Bt, int L, int l, int Bl, int N, int prorata, int minmax) {
-  __shared__ unsigned int sh[kBins];
+rb_finish_kernel(const __grid_constant__ RbBatch batch, const RbState* __restrict__ state, const unsigned int* __restrict__ above,
+                 const uint2* __restrict__ cand, const unsigned int* __restrict__ cand_n, size_t cand_stride, int* __restrict__ count,
+                 int* __restrict__ dbg_cnt, int* __restrict__ dbg_z, int* __restrict__ dbg_zp, int shown, int* __restrict__ counts_out,
+                 int Bt, int L, int Bl, int N, int prorata, int minmax) {
+  namespace cg = cooperative_groups;
+  __shared__ unsigned int hist[kBins], total_hist[kBins];
   __shared__ int sm_scan[33];
   __shared__ int found[2];
   __shared__ long long s_gt[128], s_eq[128];
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const RbState st = state[b];
-  for (int j = tid; j < kBins; j += 1024) sh[j] = hist1[(size_t)b * kBins + j];
-  __syncthreads();
-  find_digit(sh, kBins, st.cand, st.need1, sm_scan, found, nullptr);
-  const int need2 = found[1];
-  const int cand2 = (int)sh[found[0]];
-  __syncthreads();
-  // last digit: total histogram over layers
-  for (int j = tid; j < kBins; j += 1024) {
-    unsigned int s = 0;
-    if (j < 1024) for (int i = 0; i < l; ++i) s += hist2[((size_t)b * L + i) * 1024 + j];
-    sh[j] = s;
+  const int u = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, l = batch.l[u];
+  const int rank = blockIdx.x;
+  pdl_launch();
+  pdl_wait();
+  const RbState st = state[u * Bt + b];
+  const unsigned int n = cand_n[b];
+  const bool shared = n > kRbSolo;                           // the same for the whole cluster
+  if (!shared && rank > 0) return;
+  const unsigned int first = (shared ? rank * 1024 : 0) + tid, step = shared ? kRbCluster * 1024 : 1024;
+  const uint2* list = cand + (size_t)b * cand_stride;
+  // a counter array of every block in the cluster, added up in each block
+  auto add_up = [&](const unsigned int* mine, unsigned int* sum, int len) {
+    if (shared) cg::this_cluster().sync(); else __syncthreads();
+    for (int j = tid; j < len; j += 1024) {
+      unsigned int s = 0;
+      if (shared) { for (int r = 0; r < kRbCluster; ++r) s += cg::this_cluster().map_shared_rank(const_cast<unsigned int*>(mine), r)[j]; }
+      else s = mine[j];
+      sum[j] = s;
+    }
+    if (shared) cg::this_cluster().sync(); else __syncthreads();
+  };
+  const uint32_t low0 = digit_low(st.digit), last0 = digit_last(st.digit);
+  uint32_t low = low0, last = last0;
+  int need = st.need, inside = st.inside;
+  while (last > low) {
+    const int shift = range_shift(low, last);
+    hist[tid] = 0; hist[tid + 1024] = 0;
+    __syncthreads();
+#pragma unroll 4
+    for (unsigned int e = first; e < n; e += step) {
+      const uint2 c = list[e];
+      if (c.x >= low && c.x <= last && (int)c.y < l) atomicAdd(&hist[(c.x - low) >> shift], 1u);
+    }
+    add_up(hist, total_hist, kBins);
+    find_digit(total_hist, kBins, inside, need, sm_scan, found);
+    inside = (int)total_hist[found[0]]; need = found[1];
+    range_part(low, last, found[0], shift);
+    __syncthreads();
   }
+  const uint32_t T = low;
+  long long ties = need;                                     // entries equal to T that are taken, lowest layers first
+  for (int j = tid; j < 256; j += 1024) hist[j] = 0;         // [0, 128): above T inside the digit, [128, 256): equal to T
   __syncthreads();
-  find_digit(sh, kBins, cand2, need2, sm_scan, found, nullptr);
-  const int t_low = found[0];
-  long long ties = found[1];                  // entries equal to T that are taken, lowest layers first
-  // per layer: entries above T and equal to T (one warp per layer)
-  for (int i = warp; i < l; i += 32) {
-    unsigned int g = 0;
-    for (int j = t_low + 1 + lane; j < 1024; j += 32) g += hist2[((size_t)b * L + i) * 1024 + j];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xFFFFFFFFu, g, o);
-    if (lane == 0) {
-      s_gt[i] = (long long)above[b * L + i] + above2[b * L + i] + g;
-      s_eq[i] = hist2[((size_t)b * L + i) * 1024 + t_low];
-    }
+#pragma unroll 4
+  for (unsigned int e = first; e < n; e += step) {
+    const uint2 c = list[e];
+    if (c.x >= T && c.x <= last0 && (int)c.y < l) atomicAdd(&hist[c.y + (c.x == T ? 128 : 0)], 1u);
   }
-  __syncthreads();
-  // Eq. 5-6 with one thread per layer (warp 0; layers lane, lane + 32, ...): the ties go to the lowest layers
-  // first, i.e. layer i takes min(eq_i, ties - sum of eq below i).
-  if (warp == 0) {
-    long long carry = 0, cmax = 0, cmin = 0x7FFFFFFFFFFFFFFFll;
-    for (int i0 = 0; i0 < l; i0 += 32) {
-      const int i = i0 + lane;
-      const long long eq = i < l ? s_eq[i] : 0;
-      long long incl = eq;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) { const long long y = __shfl_up_sync(0xFFFFFFFFu, incl, o); if (lane >= o) incl += y; }
-      const long long before = carry + incl - eq;
-      long long take = ties - before;
-      take = take < 0 ? 0 : (take < eq ? take : eq);
-      if (i < l) {
-        s_gt[i] += take;                      // = cnt_i
-        dbg_cnt[b * L + i] = (int)s_gt[i];
-        cmax = s_gt[i] > cmax ? s_gt[i] : cmax;
-        cmin = s_gt[i] < cmin ? s_gt[i] : cmin;
-      }
-      carry += __shfl_sync(0xFFFFFFFFu, incl, 31);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) { const long long y = __shfl_xor_sync(0xFFFFFFFFu, cmax, o); cmax = y > cmax ? y : cmax; }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) { const long long y = __shfl_xor_sync(0xFFFFFFFFu, cmin, o); cmin = y < cmin ? y : cmin; }
-    if (cmax <= 0) cmax = 1;
-    long long sumz = 0;
-    for (int i = lane; i < l; i += 32) {
-      // Z_i: counts scaled by their maximum, or (variant) min-max scaled; all layers equal under min-max -> Bl each
-      if (minmax) s_eq[i] = cmax == cmin ? (long long)Bl : ((long long)Bl * (s_gt[i] - cmin)) / (cmax - cmin);
-      else s_eq[i] = ((long long)Bl * s_gt[i]) / cmax;
-      dbg_z[b * L + i] = (int)s_eq[i];
-      sumz += s_eq[i];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sumz += __shfl_xor_sync(0xFFFFFFFFu, sumz, o);
-    if (sumz <= 0) sumz = 1;
-    const long long B = (long long)N * (prorata ? l : L);      // Eq. 6's budget (variant: of the layers seen so far)
-    for (int i = lane; i < l; i += 32) {
-      const long long zp = (s_eq[i] * B) / sumz;              // Z'_i
-      const int zpi = zp > 0x7FFFFFFF ? 0x7FFFFFFF : (int)zp;
-      dbg_zp[b * L + i] = zpi;
-      const int c = count[b * L + i];
-      count[b * L + i] = c < zpi ? c : zpi;
-    }
-    for (int i = l + lane; i < L; i += 32) { dbg_cnt[b * L + i] = 0; dbg_z[b * L + i] = 0; dbg_zp[b * L + i] = 0; }
+  add_up(hist, total_hist, 256);
+  if (rank > 0 || warp != 0) return;
+  for (int i = lane; i < l; i += 32) {
+    s_gt[i] = (long long)above[((size_t)u * Bt + b) * L + i] + total_hist[i];
+    s_eq[i] = total_hist[128 + i];
   }
-  __syncthreads();
-  if (counts_out) for (int i = tid; i < L; i += 1024) counts_out[b * L + i] = count[b * L + i];
+  __syncwarp();
+  // Eq. 5-6 with one lane per layer (layers lane, lane + 32, ...): the ties go to the lowest layers first, i.e. layer i
+  // takes min(eq_i, ties - sum of eq below i).
+  const bool show = u == shown;
+  long long carry = 0, cmax = 0, cmin = 0x7FFFFFFFFFFFFFFFll;
+  for (int i0 = 0; i0 < l; i0 += 32) {
+    const int i = i0 + lane;
+    const long long eq = i < l ? s_eq[i] : 0;
+    long long incl = eq;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const long long y = __shfl_up_sync(0xFFFFFFFFu, incl, o); if (lane >= o) incl += y; }
+    const long long before = carry + incl - eq;
+    long long take = ties - before;
+    take = take < 0 ? 0 : (take < eq ? take : eq);
+    if (i < l) {
+      s_gt[i] += take;                      // = cnt_i
+      if (show) dbg_cnt[b * L + i] = (int)s_gt[i];
+      cmax = s_gt[i] > cmax ? s_gt[i] : cmax;
+      cmin = s_gt[i] < cmin ? s_gt[i] : cmin;
+    }
+    carry += __shfl_sync(0xFFFFFFFFu, incl, 31);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) { const long long y = __shfl_xor_sync(0xFFFFFFFFu, cmax, o); cmax = y > cmax ? y : cmax; }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) { const long long y = __shfl_xor_sync(0xFFFFFFFFu, cmin, o); cmin = y < cmin ? y : cmin; }
+  if (cmax <= 0) cmax = 1;
+  long long sumz = 0;
+  for (int i = lane; i < l; i += 32) {
+    // Z_i: counts scaled by their maximum, or (variant) min-max scaled; all layers equal under min-max -> Bl each
+    if (minmax) s_eq[i] = cmax == cmin ? (long long)Bl : ((long long)Bl * (s_gt[i] - cmin)) / (cmax - cmin);
+    else s_eq[i] = ((long long)Bl * s_gt[i]) / cmax;
+    if (show) dbg_z[b * L + i] = (int)s_eq[i];
+    sumz += s_eq[i];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sumz += __shfl_xor_sync(0xFFFFFFFFu, sumz, o);
+  if (sumz <= 0) sumz = 1;
+  const long long B = (long long)N * (prorata ? l : L);      // Eq. 6's budget (variant: of the layers seen so far)
+  for (int i = lane; i < l; i += 32) {
+    const long long zp = (s_eq[i] * B) / sumz;              // Z'_i
+    const int zpi = zp > 0x7FFFFFFF ? 0x7FFFFFFF : (int)zp;
+    if (show) dbg_zp[b * L + i] = zpi;
+    atomicMin(&count[b * L + i], zpi);                       // other updates of the batch do the same
+  }
+  if (show) for (int i = l + lane; i < L; i += 32) { dbg_cnt[b * L + i] = 0; dbg_z[b * L + i] = 0; dbg_zp[b * L + i] = 0; }
+  if (counts_out) {
+    __threadfence();
+    for (int i = lane; i < L; i += 32) counts_out[b * L + i] = *(volatile int*)&count[b * L + i];   // lanes read what they wrote
+  }
 }
 
 }  // namespace dkv

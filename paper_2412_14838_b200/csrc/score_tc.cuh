@@ -18,6 +18,7 @@
 #pragma once
 #include <cuda.h>
 #include "common.cuh"
+#include "select.cuh"
 
 namespace dkv {
 namespace tc {
@@ -36,7 +37,7 @@ constexpr int kQRegion = 2 * 2 * kHalfBytes;          // up to 256 rows x 128 co
 constexpr int kKRegion = kStages * 2 * kHalfBytes;    // ring of 128 x 128 tiles
 constexpr int kMiscBytes = 1024 /*lse*/ + 3 * 256 * 8 /*merge*/;
 constexpr int kRawBytes = 2 * kMaxSegTiles * kTileKeys * 4;   // sweep 2: one partial-sum array per column half
-constexpr int kSmemBytes = 1024 /*align*/ + kQRegion + kKRegion + kMiscBytes + kRawBytes + 256 /*barriers*/;
+constexpr int kSmemBytes = 1024 /*align*/ + kQRegion + kKRegion + kMiscBytes + kRawBytes + 256 /*barriers*/ + kBins * 4 /*digit counts*/;
 constexpr long long kDefaultWaitCycles = 4000000000ll;  // ~2 s: a wait that long is reported, not spun on
 constexpr uint32_t kSuspendNs = 4000;                   // a waiting thread sleeps in the barrier unit, not in a polling loop
 constexpr long long kDrainCycles = 2000000ll;           // ~1 ms: wait for own copies / MMAs in flight after an abort
@@ -55,6 +56,8 @@ struct Params {
   float2* stats;
   float* scores;           // [heads][P] pooled scores (sweep 2)
   float* copy_out;         // optional second copy
+  unsigned int* layer_hist;   // null, or [layers][samples][kBins] counters: sweep 1 clears them, sweep 2 counts the digits of its scores
+  int hkv;                 // KV heads per sample
   int* status;             // device status words; [0] = first error
   int stats_grid;          // CTAs of the launch that ran sweep 1 for this layer
   int mode;                // kNone: nothing to do
@@ -348,6 +351,7 @@ score_tc_kernel(const __grid_constant__ Maps maps0, const __grid_constant__ Maps
   float2* merge_s = reinterpret_cast<float2*>(nlse_s + 256);            // [3][256] partials of column parts 1..3 (sweep 1)
   float* raw_s = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(nlse_s) + kMiscBytes);   // [half][kMaxSegTiles * 128]
   uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(raw_s) + kRawBytes);
+  unsigned int* hist_s = reinterpret_cast<unsigned int*>(bars + 32);   // [kBins] digits of the scores of one layer and sample (sweep 2)
   // barriers: full[kStages], empty[kStages], tmem_full[4], tmem_empty[4], q_full, drain[2]
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
@@ -376,10 +380,13 @@ score_tc_kernel(const __grid_constant__ Maps maps0, const __grid_constant__ Maps
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::);
   }
+  for (int i = threadIdx.x; i < kBins; i += kThreads) hist_s[i] = 0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  pdl_launch();
+  pdl_wait();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -523,11 +530,24 @@ score_tc_kernel(const __grid_constant__ Maps maps0, const __grid_constant__ Maps
     const int sid = threadIdx.x - 64;          // 0..511 among the softmax threads
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
     int tile = 0;
+    int hist_of = -1;                          // whose digits hist_s holds: layer * samples + sample of the job
+    // adds hist_s to the counters of `hist_of` and clears it; followed by a barrier before anything is counted again
+    auto flush_hist = [&](const Params& p) {
+      unsigned int* to = p.layer_hist + (size_t)hist_of * kBins;
+      for (int i = sid; i < kBins; i += kSoftmaxThreads) {
+        const unsigned int n = hist_s[i];
+        if (n) { atomicAdd(&to[i], n); hist_s[i] = 0; }
+      }
+    };
     for (int jb = 0; jb < 2; ++jb) {
       const Params& p = jb ? job1 : job0;
       if (p.mode == kNone) continue;
       SegIter it(p, blockIdx.x, gridDim.x);
       Seg sg;
+      if (p.mode == kStats && p.layer_hist) {  // sweep 2 of these layers, which counts, is in a later launch
+        const int n = p.heads / p.hkv * kBins;
+        for (int i = blockIdx.x * kSoftmaxThreads + sid; i < n; i += gridDim.x * kSoftmaxThreads) p.layer_hist[i] = 0;
+      }
       const int tmask = NMBLK(p) == 1 ? 3 : 1, tshift = NMBLK(p) == 1 ? 2 : 1, scols = NMBLK(p) == 1 ? 128 : 256;
       const uint64_t scale22 = pack2(p.scale2, p.scale2);
       while (it.next(sg)) {
@@ -615,6 +635,10 @@ score_tc_kernel(const __grid_constant__ Maps maps0, const __grid_constant__ Maps
         } else {
           // ------------------------------------------------------------ sweep 2: one thread per key
           const int nb = sg.bh;
+          if (p.layer_hist && nb / p.hkv != hist_of) {
+            if (hist_of >= 0) flush_hist(p);
+            hist_of = nb / p.hkv;
+          }
           if (sg.new_head && sid < 256) {
             // lse2 of every window row from the partial statistics of sweep 1
             const long long total = (long long)p.heads * p.tph;
@@ -692,28 +716,37 @@ score_tc_kernel(const __grid_constant__ Maps maps0, const __grid_constant__ Maps
             raw_s[x] = (raw_s[x] + raw_s[kMaxSegTiles * kTileKeys + x]) * p.out_scale;
           asm volatile("bar.sync 1, 512;" ::: "memory");
           // Eq. 2's pooling over this segment
-          for (int o = sg.out0 + sid; o < sg.out1; o += kSoftmaxThreads) {
-            const int x = o - sg.key0;
-            float v = raw_s[x];
-            if (p.pool_avg) {
-              int cnt = 1;
-              for (int d = 1; d <= p.half; ++d) {
-                if (o - d >= 0) { v += raw_s[x - d]; ++cnt; }
-                if (o + d < p.P) { v += raw_s[x + d]; ++cnt; }
+          for (int o0 = sg.out0 + (sid & ~31); o0 < sg.out1; o0 += kSoftmaxThreads) {
+            const int o = o0 + lane, x = o - sg.key0;
+            const bool ok = o < sg.out1;
+            float v = 0.f;
+            if (ok) {
+              v = raw_s[x];
+              if (p.pool_avg) {
+                int cnt = 1;
+                for (int d = 1; d <= p.half; ++d) {
+                  if (o - d >= 0) { v += raw_s[x - d]; ++cnt; }
+                  if (o + d < p.P) { v += raw_s[x + d]; ++cnt; }
+                }
+                v = v / (float)cnt;
+              } else {
+                for (int d = 1; d <= p.half; ++d) {
+                  if (o - d >= 0) v = fmaxf(v, raw_s[x - d]);
+                  if (o + d < p.P) v = fmaxf(v, raw_s[x + d]);
+                }
               }
-              v = v / (float)cnt;
-            } else {
-              for (int d = 1; d <= p.half; ++d) {
-                if (o - d >= 0) v = fmaxf(v, raw_s[x - d]);
-                if (o + d < p.P) v = fmaxf(v, raw_s[x + d]);
-              }
+              const size_t at = (size_t)nb * p.P + o;
+              p.scores[at] = v;
+              if (p.copy_out) p.copy_out[at] = v;
             }
-            const size_t at = (size_t)nb * p.P + o;
-            p.scores[at] = v;
-            if (p.copy_out) p.copy_out[at] = v;
+            if (p.layer_hist) run_bump(hist_s, digit_of(__float_as_uint(v)), ok);
           }
           asm volatile("bar.sync 1, 512;" ::: "memory");
         }
+      }
+      if (hist_of >= 0) {
+        flush_hist(p);
+        hist_of = -1;
       }
     }
   }

@@ -1,27 +1,43 @@
-// Per-head top-B^l (Eq. 3; Algorithm 1's "topk(B^l)") under the total order
-// (score descending, position ascending), plus what the later global top-K (Eq. 4) needs from
-// this layer.  One CTA per (sample, KV head).
+// Per-head top-n (Eq. 3; Algorithm 1's "topk(B^l)") under the total order (score descending, position
+// ascending), and the digits that it shares with the global top-K of Eq. 4.  One thread block per (sample, KV head).
 //
-// Scores are non-negative floats, so their bit patterns order like unsigned integers.  The
-// threshold T (bit pattern of the B^l-th largest score) is found by a 3-pass radix select,
-// most significant digit first (11 + 11 + 10 bits), with a shared-memory histogram per pass.
-// The kept positions are then compacted in position order and sorted by (score descending,
-// position ascending): that is the order Algorithm 1's topk() returns and stores them in, and a
-// later truncation to a smaller budget is a prefix of it.
-// The first pass's histogram (top 11 bits: sign, exponent, 2 mantissa bits) is also kept per head
-// in global memory with its prefix offsets, so that Update_Buffer_Length can locate the first digit
-// of the global K-th value, and each layer's count of scores above it, from histograms alone.
+// Scores are non-negative floats, so their bit patterns order like unsigned integers.  A score's DIGIT is its exponent
+// and six mantissa bits, clamped to 2048 values around the range scores live in (a score is a sum of at most 256
+// probabilities): neighbouring digits are 1.6 % apart, so the digit that holds the n-th largest score holds few others.
+//   1  histogram of the digits (shared memory) -> the digit d that holds the n-th largest score;
+//   2  the scores with digit >= d (n and a few percent more) are collected into a list; where that does not fit the
+//      list, digit d is divided further, down to single values and the lowest positions among equal ones;
+//   3  the list is put in order by a counting sort: 4096 bins of equal width over the list's own range of bit patterns
+//      (a bin then holds a run of equal pooled scores or little more), and every entry ranks itself within its bin.
+//      A list with a bin of more than kMaxBin entries (many equal scores) goes through a bitonic network instead.
+// The result is the order Algorithm 1's topk() returns and stores positions in; a later truncation to a smaller
+// budget is a prefix of it.
+//
+// Latency-bound: chains of block-wide steps over L2-resident scores.  Two blocks of 512 threads share an SM, so that
+// one's barriers overlap the other's work.
 #pragma once
 #include "common.cuh"
+#include "compact.cuh"
 
 namespace dkv {
 
-constexpr int kSelThreads = 1024;
-constexpr int kBins = 2048;               // 11-bit digits
-constexpr int kRegChunk = 32;             // scores per thread held in registers
+constexpr int kSelThreads = 512;
+constexpr int kBins = 2048;                  // digits
+constexpr int kDigitBase = (127 - 24) << 6;  // digit 0: everything below 2^-24; digit 2047: from 2^8 (63/64) up
+constexpr int kSortBins = 4096;
+constexpr int kMaxBin = 128;
+constexpr int kMaxCountingList = 8192;       // longest list that is sorted by counting (twice 8 bytes an entry)
 
-__device__ __forceinline__ int digit_shift(int pass) { return pass == 0 ? 21 : (pass == 1 ? 10 : 0); }
-__device__ __forceinline__ uint32_t digit_mask(int pass) { return pass == 2 ? 1023u : 2047u; }
+__device__ __forceinline__ int digit_of(uint32_t bits) { return min(max((int)(bits >> 17) - kDigitBase, 0), kBins - 1); }
+// The bit patterns of digit d are [digit_low(d), digit_last(d)].
+__device__ __forceinline__ uint32_t digit_low(int d) { return d == 0 ? 0u : (uint32_t)(kDigitBase + d) << 17; }
+__device__ __forceinline__ uint32_t digit_last(int d) { return d == kBins - 1 ? 0xFFFFFFFFu : ((uint32_t)(kDigitBase + d + 1) << 17) - 1u; }
+// A range of patterns longer than 2048 is divided by its leading 11 bits: how far to shift an offset into it.
+__device__ __forceinline__ int range_shift(uint32_t low, uint32_t last) { const int bits = 32 - __clz(last - low); return bits > 11 ? bits - 11 : 0; }
+__device__ __forceinline__ void range_part(uint32_t& low, uint32_t& last, int part, int shift) {
+  low += (uint32_t)part << shift;
+  last = min(last, low + (1u << shift) - 1u);
+}
 
 // Exclusive prefix sum of one int per thread over the block; *total gets the block sum.
 // sm must hold 33 ints.  Ends with a barrier.
@@ -51,10 +67,9 @@ __device__ __forceinline__ int block_excl_scan(int v, int* sm, int* total) {
 // Given hist[nbins] in shared memory (counts per digit, `total` entries in all), find the digit d
 // holding the need-th largest entry: (#entries with digit > d) < need <= that + hist[d].
 // Results go to out[0] = d, out[1] = need - (#entries with digit > d).  Every thread owns
-// nbins / blockDim.x consecutive digits.  If offs != nullptr, the ascending exclusive offsets of all
-// digits are written there (global).  Ends with a barrier; hist is unchanged.
+// nbins / blockDim.x consecutive digits.  Ends with a barrier; hist is unchanged.
 __device__ __forceinline__ void find_digit(const unsigned int* hist, int nbins, int total, int need, int* sm_scan,
-                                           volatile int* out, unsigned int* offs) {
+                                           volatile int* out) {
   const int per = nbins / (int)blockDim.x;
   const int b0 = threadIdx.x * per;
   int mine = 0;
@@ -63,7 +78,6 @@ __device__ __forceinline__ void find_digit(const unsigned int* hist, int nbins, 
   int off = block_excl_scan(mine, sm_scan, &tot);
   for (int j = 0; j < per; ++j) {
     const int c = (int)hist[b0 + j];
-    if (offs) offs[b0 + j] = (unsigned int)off;
     const int above = total - off - c;
     if (c > 0 && above < need && need <= above + c) { out[0] = b0 + j; out[1] = need - above; }
     off += c;
@@ -153,150 +167,218 @@ __device__ __forceinline__ void bitonic_sort(unsigned long long* keys, int sort_
   }
 }
 
-// scores: [Bt*Hkv][P] of one layer.
-// idx: [Bt*Hkv][keep] kept positions in buffer order = (score descending, position ascending).
-// sorted_out (optional): the same positions ascending; rank_out (optional): rank of each of those.
-// layer_hist: [Bt][2048] first-digit counts of the layer's scores, all heads of a sample added up (zeroed by
-// the host before the launch); the rebudget works from these.
-// Also records count[b][layer] = keep.
-// Every warp owns a run of 32*chunk consecutive positions; lane j holds positions run + 32*e + j.
-// Dynamic shared memory: 8*sort_n bytes, then 4*keep bytes.
-template <bool REG>
-__global__ void __launch_bounds__(kSelThreads)
-select_topk_kernel(const float* __restrict__ scores, int* __restrict__ idx, int* __restrict__ sorted_out,
-                   int* __restrict__ rank_out, unsigned int* __restrict__ layer_hist,
-                   int P, int keep, int sort_n, int* __restrict__ count, int Hkv, int L, int layer) {
-  extern __shared__ __align__(16) unsigned char dyn[];
-  __shared__ unsigned int hist[kBins];
-  __shared__ int sm_scan[33], sm_scan2[33];
+// The `n` best positions of one head (1 <= n <= P), in order, in sel[0 .. n) (shared memory, returned).
+// v: the head's scores.  gh: if not null, the head's digit counts are added to these 2048 counters (global).
+// `cap`: entries of the list, a power of two; at least n.  Dynamic shared memory `dyn`: select_smem(cap) bytes.
+// Ends with a barrier.
+__host__ __device__ inline size_t select_smem(int cap) {
+  return (size_t)cap * 8 * (cap <= kMaxCountingList ? 2 : 1) + sizeof(unsigned int) * kSortBins;
+}
+__device__ __forceinline__ int* select_head(const uint32_t* __restrict__ v, int P, int n, int cap, unsigned char* dyn, unsigned int* gh) {
+  __shared__ int sm_scan[33];
   __shared__ int found[2];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t* v = reinterpret_cast<const uint32_t*>(scores) + (size_t)blockIdx.x * P;
-  if (tid == 0 && blockIdx.x % Hkv == 0) count[(blockIdx.x / Hkv) * L + layer] = keep;
-
+  __shared__ unsigned int s_n, s_max, s_full;
+  const int tid = threadIdx.x, lane = tid & 31;
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(dyn);
-  int* sel_pos = reinterpret_cast<int*>(dyn + (size_t)sort_n * 8);
+  unsigned long long* sorted = keys + (cap <= kMaxCountingList ? cap : 0);
+  unsigned int* bins = reinterpret_cast<unsigned int*>(sorted + cap);
+  constexpr int kUnroll = 8;                               // scores a thread has in flight
+  const int P32 = (P + 31) & ~31;
 
-  const int chunk = (P + kSelThreads - 1) / kSelThreads;       // REG: chunk <= kRegChunk
-  const int run0 = warp * chunk * 32;
-  const int n_e = REG ? kRegChunk : chunk;
-  // which of this lane's slots hold a position: slots [0, n_ok)
-  const int n_ok = min(chunk, max(0, (P - run0 - lane + 31) / 32));
-  uint32_t r[REG ? kRegChunk : 1];
-  if constexpr (REG) {
+  // 1: the digit of the n-th largest score
+  for (int i = tid; i < kBins; i += kSelThreads) bins[i] = 0;
+  if (tid == 0) { s_n = 0; s_max = 0; s_full = 0; }
+  __syncthreads();
+  for (int p0 = tid; p0 < P32; p0 += kSelThreads * kUnroll) {
+    uint32_t u[kUnroll];
 #pragma unroll
-    for (int e = 0; e < kRegChunk; ++e) r[e] = e < n_ok ? v[run0 + e * 32 + lane] : 0u;
+    for (int j = 0; j < kUnroll; ++j) { const int p = p0 + j * kSelThreads; u[j] = p < P ? v[p] : 0u; }
+#pragma unroll
+    for (int j = 0; j < kUnroll; ++j) {
+      const int p = p0 + j * kSelThreads;
+      if (p < P32) run_bump(bins, digit_of(u[j]), p < P);   // warp-uniform: neighbours share digits after pooling
+    }
   }
-#define DKV_SEL_FOR(e) _Pragma("unroll") for (int e = 0; e < n_e; ++e)
-#define DKV_SEL_POS(e) (run0 + (e) * 32 + lane)
-#define DKV_SEL_OK(e) ((e) < n_ok)
-  auto val = [&](int e) -> uint32_t {
-    if constexpr (REG) return r[e]; else return DKV_SEL_OK(e) ? v[DKV_SEL_POS(e)] : 0u;
-  };
-
-  // pass 0: first digit of every score; neighbours share digits after pooling, so lanes combine their bumps
-  for (int i = tid; i < kBins; i += kSelThreads) hist[i] = 0;
   __syncthreads();
-  DKV_SEL_FOR(e) run_bump(hist, val(e) >> 21, DKV_SEL_OK(e));
-  __syncthreads();
-  {
-    unsigned int* gh = layer_hist + (size_t)(blockIdx.x / Hkv) * kBins;
-    for (int i = tid; i < kBins; i += kSelThreads) { const unsigned int c = hist[i]; if (c) atomicAdd(&gh[i], c); }
-  }
-  find_digit(hist, kBins, P, keep, sm_scan, found, nullptr);
-  uint32_t prefix = ((uint32_t)found[0]) << 21, mask = 2047u << 21;
-  int need = found[1], total = (int)hist[found[0]];
-  __syncthreads();
-  // passes 1, 2: only the scores inside the first digit's bucket take part
-  for (int pass = 1; pass < 3; ++pass) {
-    const int shift = digit_shift(pass);
-    const uint32_t dm = digit_mask(pass);
-    for (int i = tid; i < kBins; i += kSelThreads) hist[i] = 0;
+  if (gh) for (int i = tid; i < kBins; i += kSelThreads) { const unsigned int c = bins[i]; if (c) atomicAdd(&gh[i], c); }
+  find_digit(bins, kBins, P, n, sm_scan, found);
+  uint32_t low = digit_low(found[0]), last = digit_last(found[0]);
+  int need = found[1], inside = (int)bins[found[0]];       // `need` of the `inside` scores in the range are kept
+  while (n - need + inside > cap && last > low) {          // too many for the list: divide the range
+    const int shift = range_shift(low, last);
     __syncthreads();
-    DKV_SEL_FOR(e) {
-      const uint32_t u = val(e);
-      if (DKV_SEL_OK(e) && (u & mask) == prefix) atomicAdd(&hist[(u >> shift) & dm], 1u);
+    for (int i = tid; i < kBins; i += kSelThreads) bins[i] = 0;
+    __syncthreads();
+    for (int p = tid; p < P; p += kSelThreads) {
+      const uint32_t u = v[p];
+      if (u >= low && u <= last) atomicAdd(&bins[(u - low) >> shift], 1u);
     }
     __syncthreads();
-    find_digit(hist, kBins, total, need, sm_scan, found, nullptr);
-    const int d = found[0];
-    total = (int)hist[d];
-    need = found[1];
-    prefix |= ((uint32_t)d) << shift;
-    mask |= dm << shift;
-    __syncthreads();
+    find_digit(bins, kBins, inside, need, sm_scan, found);
+    inside = (int)bins[found[0]]; need = found[1];
+    range_part(low, last, found[0], shift);
   }
-  const uint32_t T = prefix;
-  const int need_eq = need;                 // how many of the entries equal to T are kept (lowest positions)
+  __syncthreads();
 
-  // Ordered compaction.  Position order inside a warp's run is (e, lane), so ballots give the order.
-  int gt = 0, eq = 0;
-  DKV_SEL_FOR(e) { const uint32_t u = val(e); if (DKV_SEL_OK(e)) { gt += (u > T); eq += (u == T); } }
+  // 2: everything in or above the range; if equal scores alone overflow the list (one pattern), the first `need` of them
+  const bool some_equal = n - need + inside > cap;
+  const uint32_t from = low + (some_equal ? 1u : 0u);
+  for (int p0 = tid; p0 < P32; p0 += kSelThreads * kUnroll) {
+    uint32_t u[kUnroll];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) { gt += __shfl_xor_sync(0xFFFFFFFFu, gt, o); eq += __shfl_xor_sync(0xFFFFFFFFu, eq, o); }
-  int tot_gt, tot_eq;
-  int g_run = block_excl_scan(lane == 0 ? gt : 0, sm_scan, &tot_gt);       // one value per warp, carried by lane 0
-  int q_run = block_excl_scan(lane == 0 ? eq : 0, sm_scan2, &tot_eq);
-  g_run = __shfl_sync(0xFFFFFFFFu, g_run, 0);
-  q_run = __shfl_sync(0xFFFFFFFFu, q_run, 0);
-  const unsigned int lt = (1u << lane) - 1u;
-  int* my_sorted = sorted_out ? sorted_out + (size_t)blockIdx.x * keep : nullptr;
-  DKV_SEL_FOR(e) {
-    const uint32_t u = val(e);
-    const bool ok = DKV_SEL_OK(e);
-    const bool is_gt = ok && u > T, is_eq = ok && u == T;
-    const unsigned int bg = __ballot_sync(0xFFFFFFFFu, is_gt), be = __ballot_sync(0xFFFFFFFFu, is_eq);
-    if (bg | be) {                           // warp-uniform: most rows of 32 positions keep nothing
-      const int g = g_run + __popc(bg & lt), q = q_run + __popc(be & lt);
-      if (is_gt || (is_eq && q < need_eq)) {
-        const int out = g + min(q, need_eq);
-        const int p = DKV_SEL_POS(e);
-        sel_pos[out] = p;
-        if (my_sorted) my_sorted[out] = p;
-        keys[out] = ((unsigned long long)(~u) << 32) | (unsigned int)out;
+    for (int j = 0; j < kUnroll; ++j) { const int p = p0 + j * kSelThreads; u[j] = p < P ? v[p] : 0u; }
+#pragma unroll
+    for (int j = 0; j < kUnroll; ++j) {
+      const int p = p0 + j * kSelThreads;
+      const bool take = p < P && u[j] >= from;
+      const unsigned int m = __ballot_sync(0xFFFFFFFFu, take);
+      if (m) {                                             // warp-uniform: most rows of 32 positions keep nothing
+        unsigned int base = 0;
+        if (lane == 0) base = atomicAdd(&s_n, (unsigned int)__popc(m));
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        if (take) keys[base + __popc(m & ((1u << lane) - 1u))] = ((unsigned long long)(~u[j]) << 32) | (unsigned int)p;
+        const unsigned int mx = __reduce_max_sync(0xFFFFFFFFu, take ? u[j] : 0u);
+        if (lane == 0) atomicMax(&s_max, mx);
       }
-      g_run += __popc(bg); q_run += __popc(be);
     }
   }
-  for (int i = tid + keep; i < sort_n; i += kSelThreads) keys[i] = ~0ull;
+  __syncthreads();
+  int list = (int)s_n;
+  if (some_equal) {
+    int have = 0;                                          // equal scores taken so far, in position order
+    for (int p0 = 0; p0 < P && have < need; p0 += kSelThreads) {
+      const bool eq = p0 + tid < P && v[p0 + tid] == low;
+      int tot;
+      const int at = have + block_excl_scan(eq ? 1 : 0, sm_scan, &tot);
+      if (eq && at < need) keys[list + at] = ((unsigned long long)(~low) << 32) | (unsigned int)(p0 + tid);
+      have += tot;
+    }
+    list += need;
+    if (list == need && tid == 0) s_max = low;
+    __syncthreads();
+  }
+
+  // 3: order
+  bool counting = cap <= kMaxCountingList;
+  if (counting) {
+    const uint32_t top = s_max, range = top - low;
+    const int shift = range < kSortBins ? 0 : 32 - __clz(range) - 12;
+    for (int i = tid; i < kSortBins; i += kSelThreads) bins[i] = 0;
+    __syncthreads();
+    for (int i = tid; i < list; i += kSelThreads) atomicAdd(&bins[(top - ~(uint32_t)(keys[i] >> 32)) >> shift], 1u);
+    __syncthreads();
+    constexpr int kPer = kSortBins / kSelThreads;
+    unsigned int c[kPer], mine = 0, most = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) { c[j] = bins[tid * kPer + j]; mine += c[j]; most = max(most, c[j]); }
+    if (most > kMaxBin) s_full = 1;                           // any writer will do
+    int tot;
+    unsigned int off = (unsigned int)block_excl_scan((int)mine, sm_scan, &tot);
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) { bins[tid * kPer + j] = off; off += c[j]; }
+    __syncthreads();
+    counting = s_full == 0;
+    if (counting) {
+      for (int i = tid; i < list; i += kSelThreads) {
+        const unsigned long long k = keys[i];
+        sorted[atomicAdd(&bins[(top - ~(uint32_t)(k >> 32)) >> shift], 1u)] = k;      // bins: from starts to ends
+      }
+      __syncthreads();
+      int* sel = reinterpret_cast<int*>(keys);             // the unsorted list is done with
+      for (int i = tid; i < list; i += kSelThreads) {
+        const unsigned long long k = sorted[i];
+        const unsigned int b = (top - ~(uint32_t)(k >> 32)) >> shift, b0 = b ? bins[b - 1] : 0, b1 = bins[b];
+        if ((int)b0 >= n) continue;
+        int r = (int)b0;
+        for (unsigned int j = b0; j < b1; ++j) r += sorted[j] < k;
+        if (r < n) sel[r] = (int)(uint32_t)k;
+      }
+      __syncthreads();
+      return sel;
+    }
+  }
+  int sort_n = 2;
+  while (sort_n < list) sort_n <<= 1;
+  for (int i = list + tid; i < sort_n; i += kSelThreads) keys[i] = ~0ull;
   __syncthreads();
   bitonic_sort(keys, sort_n);
-  int* my_idx = idx + (size_t)blockIdx.x * keep;
-  for (int i = tid; i < keep; i += kSelThreads) {
-    const int slot = (int)(keys[i] & 0xFFFFFFFFull);
-    my_idx[i] = sel_pos[slot];
-    if (rank_out) rank_out[(size_t)blockIdx.x * keep + slot] = i;
+  int* sel = reinterpret_cast<int*>(keys);
+  for (int i0 = 0; i0 < n; i0 += kSelThreads) {            // in place: entry i moves to the front half, read before it is overwritten
+    const int i = i0 + tid;
+    const int p = i < n ? (int)(uint32_t)keys[i] : 0;
+    __syncthreads();
+    if (i < n) sel[i] = p;
+    __syncthreads();
   }
-#undef DKV_SEL_FOR
-#undef DKV_SEL_POS
-#undef DKV_SEL_OK
+  return sel;
 }
 
-// Ascending list of the positions a head currently holds: sorted_out[b,h,0:held] (one CTA per head).
-// Dynamic shared memory: ceil(P / 32) words (one bit per position).
+// dkv_select_topk: the `keep` best of every head of one layer.  idx: [Bt*Hkv][keep], in order.  Adds the heads' digit
+// counts to layer_hist [Bt][2048] and records count[b][layer] = keep.  grid Bt*Hkv.
+__global__ void __launch_bounds__(kSelThreads, 2)
+select_topk_kernel(const float* __restrict__ scores, int* __restrict__ idx, unsigned int* __restrict__ layer_hist, int P,
+                   int keep, int cap, int* __restrict__ count, int Hkv, int L, int layer) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  const int b = blockIdx.x / Hkv;
+  pdl_launch();
+  pdl_wait();
+  if (threadIdx.x == 0 && blockIdx.x % Hkv == 0) count[b * L + layer] = keep;
+  const int* sel = select_head(reinterpret_cast<const uint32_t*>(scores) + (size_t)blockIdx.x * P, P, keep, cap, dyn,
+                               layer_hist + (size_t)b * kBins);
+  for (int i = threadIdx.x; i < keep; i += kSelThreads) idx[(size_t)blockIdx.x * keep + i] = sel[i];
+}
+
+// Per-layer device pointers of a pass.
+struct PassPtrs {
+  const void* k[128];
+  const void* v[128];
+  void* kb[128];
+  void* vb[128];
+};
+
+// The end of a pass, for every layer and head at once: with the final counts known (count[b][layer], at most B^l), a
+// block selects its head's best `count` positions, writes them to idx [layer][Bt*Hkv][stride] and copies those rows and
+// the ws window rows of K and V into the layer's buffers.  Selecting and copying the final rows once replaces a
+// selection and copy of B^l rows per layer and a truncation per update: 32K prompt with B^l = 4 N: 71 MB of rows read
+// instead of 272, and no block of the scoring kernel gives way to it while keys are streamed.
+// grid (Bt*Hkv, layers).
+__global__ void __launch_bounds__(kSelThreads, 2)
+select_gather_kernel(const __grid_constant__ PassPtrs ptrs, const float* __restrict__ scores, int* __restrict__ idx,
+                     const int* __restrict__ count, int* __restrict__ held, int P, int ws, int stride, int cap, int S, int vec, int Hkv, int L) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  const int bh = blockIdx.x, b = bh / Hkv, layer = blockIdx.y, tid = threadIdx.x;
+  const size_t head = (size_t)layer * gridDim.x + bh;
+  pdl_launch();
+  pdl_wait();
+  const int n = count[b * L + layer];
+  if (tid == 0 && bh % Hkv == 0) held[b * L + layer] = n;
+  const int* sel = nullptr;
+  if (n > 0) {
+    sel = select_head(reinterpret_cast<const uint32_t*>(scores) + head * P, P, n, cap, dyn, nullptr);
+    for (int i = tid; i < n; i += kSelThreads) idx[head * stride + i] = sel[i];
+  }
+  gather_rows(static_cast<const uint4*>(ptrs.k[layer]), static_cast<const uint4*>(ptrs.v[layer]), static_cast<uint4*>(ptrs.kb[layer]),
+              static_cast<uint4*>(ptrs.vb[layer]), sel, n, bh, S, P, ws, stride + ws, vec, tid, kSelThreads, 0, 1);
+}
+
+// The positions idx[b,h,0..n) of one layer ascending (sorted_out) and the place each had in idx (rank_out), either
+// may be null.  n = held[b][layer], or `keep` where held is null.  Output rows are idx_stride apart, like idx's.
+// One thread block per head; dynamic shared memory: 8 bytes for each of the power of two >= n entries.
 __global__ void __launch_bounds__(kSelThreads)
-kept_sorted_kernel(const int* __restrict__ idx, const int* __restrict__ held, int* __restrict__ sorted_out, int P,
-                   int idx_stride, int Hkv, int L, int layer) {
-  extern __shared__ unsigned int bits[];
-  __shared__ int sm_scan[33];
-  const int tid = threadIdx.x;
-  const int n = held[(blockIdx.x / Hkv) * L + layer];
-  const int words = (P + 31) / 32;
-  for (int i = tid; i < words; i += kSelThreads) bits[i] = 0;
+sort_positions_kernel(const int* __restrict__ idx, const int* __restrict__ held, int keep, int* __restrict__ sorted_out,
+                      int* __restrict__ rank_out, int idx_stride, int Hkv, int L, int layer) {
+  extern __shared__ __align__(16) unsigned long long pos_keys[];
+  const int tid = threadIdx.x, n = held ? held[(blockIdx.x / Hkv) * L + layer] : keep;
+  int sort_n = 2;
+  while (sort_n < n) sort_n <<= 1;
+  const size_t row = (size_t)blockIdx.x * idx_stride;
+  for (int i = tid; i < sort_n; i += kSelThreads)
+    pos_keys[i] = i < n ? ((unsigned long long)(uint32_t)idx[row + i] << 32) | (unsigned int)i : ~0ull;
   __syncthreads();
-  const int* my = idx + (size_t)blockIdx.x * idx_stride;
-  for (int i = tid; i < n; i += kSelThreads) { const int p = my[i]; atomicOr(&bits[p >> 5], 1u << (p & 31)); }
-  __syncthreads();
-  const int per = (words + kSelThreads - 1) / kSelThreads;
-  const int w0 = min(words, tid * per), w1 = min(words, w0 + per);
-  int mine = 0;
-  for (int w = w0; w < w1; ++w) mine += __popc(bits[w]);
-  int tot;
-  int out = block_excl_scan(mine, sm_scan, &tot);
-  int* dst = sorted_out + (size_t)blockIdx.x * idx_stride;
-  for (int w = w0; w < w1; ++w) {
-    unsigned int m = bits[w];
-    while (m) { const int b = __ffs(m) - 1; dst[out++] = w * 32 + b; m &= m - 1; }
+  bitonic_sort(pos_keys, sort_n);
+  for (int i = tid; i < n; i += kSelThreads) {
+    if (sorted_out) sorted_out[row + i] = (int)(pos_keys[i] >> 32);
+    if (rank_out) rank_out[row + i] = (int)(uint32_t)pos_keys[i];
   }
 }
 
