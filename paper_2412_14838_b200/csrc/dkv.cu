@@ -39,7 +39,8 @@ struct dkv_ctx {
   int* d_status;        // [8]
   int sel_cap;          // entries of the select kernels' list
   // tensor-core scoring
-  int n_sms, tc_slots;
+  int n_sms;
+  size_t stats_rows;    // (head, slot) pairs of a job, at most
   int pass_group;       // layers per scoring launch of dkv_run_prefill_pass (1..tc::kMaxGroup)
   bool emit_backward;   // sweep 2 walks every CTA's slice from the end to the start
   bool host_v_staged;   // dkv_run_prefill_pass_host copies V in full even where the gather could read its rows in place
@@ -47,7 +48,7 @@ struct dkv_ctx {
   int retain_mb;        // MB of a sweep-1 job's keys (the end of every CTA's slice) marked to stay in L2 for sweep 2
   long long wait_cycles;   // limit of the scoring kernel's mbarrier waits (dkv_set_wait_limit)
   int withhold_sweep, withhold_tile;   // test hook of dkv_debug_withhold_tile (-1: off)
-  float2* d_tc_stats;   // [3][kMaxGroup*Bt*Hkv][tc_slots][256]: partial softmax statistics, three jobs in rotation
+  float2* d_tc_stats;   // [3][stats_rows][256]: partial softmax statistics, three jobs in rotation, each [heads][slots][256]
   // host state
   uint8_t scored[DKV_MAX_LAYERS], gathered[DKV_MAX_LAYERS];
   uint8_t selected[DKV_MAX_LAYERS];     // 1: by scores (dkv_select_topk), 2: by position (dkv_select_positions)
@@ -215,19 +216,22 @@ uint32_t make_idesc(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// Statistics slots a head of a job needs: thread blocks that can share it (its share of the grid, one cut at either end).
+int stats_slots(int n_sms, int job_heads) { return n_sms / job_heads + 2; }
+
 // Parameters of one sweep over the `nl` consecutive layers that start at `layer` (q, k: their nl device
 // pointers); `buf` picks the statistics scratch (jobs in flight rotate).  In sweep 2 every CTA walks its slice of the
 // key space from the end to the start: sweep 1 cut the same space into the same slices, so each CTA begins with
 // the keys that were streamed last and may still be in L2.
 // `grid`: thread blocks of the launch; `stats_grid`: of the launch that ran sweep 1 for these layers (sweep 2).
+template <int NL>
 bool make_job(dkv_ctx* c, int mode, int layer, int nl, const void* const* q, const void* const* k, float* scores_out,
-              int buf, int grid, int stats_grid, bool hist, tc::Maps* maps, tc::Params* p, const float* const* lse = nullptr) {
+              int buf, int grid, int stats_grid, bool hist, tc::Maps<NL>* maps, tc::Params* p, const float* const* lse = nullptr) {
   const Shape& s = c->s;
   const int heads = s.Bt * s.Hkv;
-  memset(maps, 0, sizeof *maps);                           // entries past nl are never read
   for (int i = 0; i < nl; ++i)
     if (!make_map(&maps->q[i], q[i], s.D, s.M, heads) || !make_map(&maps->k[i], k[i], s.D, s.S, heads)) return false;
-  if (lse) for (int i = 0; i < nl; ++i) maps->lse[i] = lse[i];
+  for (int i = 0; i < nl; ++i) maps->lse[i] = lse ? lse[i] : nullptr;      // (entries past nl are never read)
   p->S = s.S; p->P = s.P; p->ws = s.ws; p->M = s.M; p->D = s.D; p->heads = nl * heads; p->half = s.pool / 2;
   p->nl = nl; p->hpl = heads;
   p->back = (mode == tc::kEmit && c->emit_backward) ? 1 : 0;
@@ -237,9 +241,9 @@ bool make_job(dkv_ctx* c, int mode, int layer, int nl, const void* const* q, con
   p->tph = (s.S + tc::kTileKeys - 1) / tc::kTileKeys;
   p->nq16 = (s.M + 15) / 16 * 16;
   p->nmblk = (s.M + 127) / 128;
-  p->slots = c->tc_slots; p->m_stride = 256;
+  p->slots = stats_slots(c->n_sms, nl * heads); p->m_stride = 256;
   p->scale2 = kLog2e / sqrtf((float)s.D);
-  p->stats = c->d_tc_stats + (size_t)buf * tc::kMaxGroup * heads * c->tc_slots * 256;
+  p->stats = c->d_tc_stats + (size_t)buf * c->stats_rows * 256;
   p->scores = c->d_scores + (size_t)layer * layer_scores(s);
   p->copy_out = scores_out;
   p->status = c->d_status;
@@ -253,11 +257,21 @@ bool make_job(dkv_ctx* c, int mode, int layer, int nl, const void* const* q, con
   return true;
 }
 
+cudaError_t set_score_attributes() {
+  for (const void* f : {(const void*)tc::score_tc_kernel<1, true>, (const void*)tc::score_tc_kernel<1, false>,
+                        (const void*)tc::score_tc_kernel<tc::kMaxGroup, true>, (const void*)tc::score_tc_kernel<tc::kMaxGroup, false>}) {
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 // The scoring kernel for two jobs (either may be kNone): the specialised build when every job has exactly 128 window
 // rows of 128 dims, the general one otherwise.
-cudaError_t launch_tc(int grid, cudaStream_t st, const tc::Maps& m0, const tc::Maps& m1, const tc::Params& j0, const tc::Params& j1) {
+template <int NL>
+cudaError_t launch_tc(int grid, cudaStream_t st, const tc::Maps<NL>& m0, const tc::Maps<NL>& m1, const tc::Params& j0, const tc::Params& j1) {
   auto fast = [](const tc::Params& p) { return p.mode == tc::kNone || (p.M == 128 && p.D == 128); };
-  return launch_pdl(fast(j0) && fast(j1) ? tc::score_tc_kernel<true> : tc::score_tc_kernel<false>, dim3(grid), tc::kThreads,
+  return launch_pdl(fast(j0) && fast(j1) ? tc::score_tc_kernel<NL, true> : tc::score_tc_kernel<NL, false>, dim3(grid), tc::kThreads,
                     (size_t)tc::kSmemBytes, 1, st, m0, m1, j0, j1);
 }
 
@@ -273,9 +287,10 @@ struct ScoreGroup { int first, n, buf, grid; };
 
 // One launch: sweep 2 of group `e` (if not null), then sweep 1 of group `s` (if not null), whose grid it sets.  `q`, `k`,
 // `lse`: all layers' pointers, indexed by layer (lse: null, or the caller's normalisers instead of sweep 1).
+template <int NL>
 int launch_score(dkv_ctx* c, const ScoreGroup* e, ScoreGroup* s, const void* const* q, const void* const* k, const float* const* lse,
                  float* scores_out, bool hist, cudaStream_t st) {
-  tc::Maps m0, m1;
+  tc::Maps<NL> m0, m1;                       // only the layers of the jobs are filled in and read
   tc::Params j0, j1;
   memset(&j0, 0, sizeof j0); memset(&j1, 0, sizeof j1);
   j0.mode = j1.mode = tc::kNone;
@@ -295,8 +310,8 @@ int do_score(dkv_ctx* c, int layer, const void* q, const void* k, const float* l
   const float* ls[DKV_MAX_LAYERS];
   qs[layer] = q; ks[layer] = k; ls[layer] = lse;
   int rc;
-  if (!lse && (rc = launch_score(c, nullptr, &g, qs, ks, nullptr, nullptr, false, st))) return rc;
-  if ((rc = launch_score(c, &g, nullptr, qs, ks, lse ? ls : nullptr, scores_out, false, st))) return rc;
+  if (!lse && (rc = launch_score<1>(c, nullptr, &g, qs, ks, nullptr, nullptr, false, st))) return rc;
+  if ((rc = launch_score<1>(c, &g, nullptr, qs, ks, lse ? ls : nullptr, scores_out, false, st))) return rc;
   c->scored[layer] = 1;
   c->selected[layer] = c->gathered[layer] = 0;
   return DKV_OK;
@@ -481,9 +496,9 @@ int do_pass(dkv_ctx* c, const void* const* q, const void* const* k, const void* 
     done += cur.n;
     if (lse) {
       if (!cur.n) break;
-      rc = launch_score(c, &cur, nullptr, q, k, lse, nullptr, true, st);
+      rc = launch_score<tc::kMaxGroup>(c, &cur, nullptr, q, k, lse, nullptr, true, st);
     } else {
-      rc = launch_score(c, prev.n ? &prev : nullptr, cur.n ? &cur : nullptr, q, k, nullptr, nullptr, true, st);
+      rc = launch_score<tc::kMaxGroup>(c, prev.n ? &prev : nullptr, cur.n ? &cur : nullptr, q, k, nullptr, nullptr, true, st);
       prev = cur;
     }
     if (rc) return rc;
@@ -584,12 +599,15 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
     int sms = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     c->n_sms = sms > 0 ? sms : 1;
-    // thread blocks that share a head in sweep 1: its share of the grid, one cut at either end
-    c->tc_slots = c->n_sms / heads + 2;
-    const int tph = (s.S + tc::kTileKeys - 1) / tc::kTileKeys;
-    const long long per_cta = (long long)heads * tph / c->n_sms;
-    // layers per scoring launch of the pass: enough that a CTA's share of a job is some tens of tiles
-    c->pass_group = env_int("DKV_PASS_GROUP", per_cta < 8 ? tc::kMaxGroup : 4, 1, tc::kMaxGroup);
+    c->stats_rows = (size_t)c->n_sms + 2 * tc::kMaxGroup * heads;
+    // Layers per scoring launch of the pass: enough that a thread block has about 110 tiles a sweep.  A launch costs some 8 us
+    // (fill, drain, statistics) whatever it does: 32 layers of 8K in launches of 8 / 16 / 32 layers take 299 / 290 / 286 us,
+    // 28 layers of 16K with 224 window rows 449 / 414 / 406; at 32K eight layers are as good as more.
+    const long long tiles = (long long)heads * ((s.S + tc::kTileKeys - 1) / tc::kTileKeys), want = (110ll * c->n_sms + tiles - 1) / tiles;
+    int g = want < s.L ? (int)want : s.L;
+    if (g > tc::kMaxGroup) g = tc::kMaxGroup;
+    const int launches = (s.L + g - 1) / g;
+    c->pass_group = env_int("DKV_PASS_GROUP", (s.L + launches - 1) / launches, 1, tc::kMaxGroup);
     c->emit_backward = env_int("DKV_EMIT_FORWARD", 0, 0, 1) == 0;
     // Sweep 2 starts on the keys sweep 1 streamed last: that much of a job (4/7 of L2, 72 of 126 MB) is loaded with
     // an evict-last policy, every other key tile and the gather's rows evict-first, so that neither the rest of the
@@ -616,9 +634,8 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   TRY(cudaMalloc(&c->d_layer_hist, sizeof(unsigned int) * s.L * s.Bt * kBins));
   TRY(cudaMalloc(&c->d_cand, sizeof(uint2) * s.L * layer_scores(s)));
   TRY(cudaMalloc(&c->d_cand_n, sizeof(unsigned int) * s.Bt));
-  TRY(cudaMalloc(&c->d_tc_stats, sizeof(float2) * 3 * tc::kMaxGroup * heads * c->tc_slots * 256));
-  TRY(cudaFuncSetAttribute(tc::score_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes));
-  TRY(cudaFuncSetAttribute(tc::score_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes));
+  TRY(cudaMalloc(&c->d_tc_stats, sizeof(float2) * 3 * c->stats_rows * 256));
+  TRY(set_score_attributes());
   TRY(cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking));
   c->pass_key = new (std::nothrow) std::vector<const void*>();
   if (!c->pass_key) { free_all(c); delete c; return DKV_ERR_NOMEM; }
@@ -991,11 +1008,7 @@ int dkv_score_static(const dkv_config* cfg, const void* q_win, const void* k, fl
       if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess || !ptr) return DKV_ERR_CUDA;
       int sms = 0;
       if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return DKV_ERR_CUDA;
-      if (cudaFuncSetAttribute(tc::score_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes) !=
-              cudaSuccess ||
-          cudaFuncSetAttribute(tc::score_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes) !=
-              cudaSuccess)
-        return DKV_ERR_CUDA;
+      if (set_score_attributes() != cudaSuccess) return DKV_ERR_CUDA;
       g.ptr = static_cast<unsigned char*>(ptr);
       g.sms = sms;
       g.done = true;
@@ -1016,8 +1029,8 @@ int dkv_score_static(const dkv_config* cfg, const void* q_win, const void* k, fl
   const unsigned long long need = 256ull + (unsigned long long)heads * slots * 256ull * sizeof(float2);
   if (need > DKV_STATIC_SCRATCH_BYTES) return DKV_ERR_TOO_LARGE;
   cudaStream_t st = as_stream(stream);
-  tc::Maps maps;
-  memset(&maps, 0, sizeof maps);
+  tc::Maps<1> maps;
+  maps.lse[0] = nullptr;
   if (!make_map(&maps.q[0], q_win, D, M, heads) || !make_map(&maps.k[0], k, D, S, heads)) return DKV_ERR_CUDA;
   if (cudaMemsetAsync(su.ptr, 0, 256, st) != cudaSuccess) return DKV_ERR_CUDA;   // status words start at zero
   tc::Params p, none;

@@ -74,10 +74,11 @@ struct Params {
                            // so that the wait for it runs out and the timeout path can be exercised
 };
 
-constexpr int kMaxGroup = 8;               // layers one job may cover
+constexpr int kMaxGroup = 32;              // layers one job may cover
+template <int NL>                          // 1 or kMaxGroup: a launch carries its jobs' maps as arguments
 struct Maps {                              // tensor maps of a job's layers, in storage order
-  CUtensorMap q[kMaxGroup], k[kMaxGroup];
-  const float* lse[kMaxGroup];             // sweep 2: the caller's natural-log normalisers [heads per layer][M] of each
+  CUtensorMap q[NL], k[NL];
+  const float* lse[NL];             // sweep 2: the caller's natural-log normalisers [heads per layer][M] of each
                                            // layer (then sweep 1 never ran for the job), or null
 };
 
@@ -339,9 +340,9 @@ __host__ __device__ __forceinline__ int tile_owner(long long x, long long total,
 // job0 uses maps0, job1 uses maps1; a job with mode kNone is skipped.
 // kFast: both jobs have exactly 128 window rows of 128 dims (ws*G = 128, D = 128, the shape of the 32/8-head models):
 // the row-block count, the chunk count and the k-step count are then compile-time constants.
-template <bool kFast>
+template <int NL, bool kFast>
 __global__ void __launch_bounds__(kThreads, 1)
-score_tc_kernel(const __grid_constant__ Maps maps0, const __grid_constant__ Maps maps1,
+score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ Maps<NL> maps1,
                 const __grid_constant__ Params job0, const __grid_constant__ Params job1) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -397,7 +398,7 @@ score_tc_kernel(const __grid_constant__ Maps maps0, const __grid_constant__ Maps
       for (int jb = 0; jb < 2 && ok; ++jb) {
         const Params& p = jb ? job1 : job0;
         if (p.mode == kNone) continue;
-        const Maps& maps = jb ? maps1 : maps0;
+        const Maps<NL>& maps = jb ? maps1 : maps0;
         const int halves = DIMS(p) / 64;
         const uint32_t tile_bytes = (uint32_t)halves * kHalfBytes;
         const int withhold = blockIdx.x == 0 ? p.withhold_tile : -1;
@@ -639,26 +640,47 @@ score_tc_kernel(const __grid_constant__ Maps maps0, const __grid_constant__ Maps
             if (hist_of >= 0) flush_hist(p);
             hist_of = nb / p.hkv;
           }
-          if (sg.new_head && sid < 256) {
-            // lse2 of every window row from the partial statistics of sweep 1
-            const long long total = (long long)p.heads * p.tph;
-            const int c_lo = tile_owner((long long)nb * p.tph, total, p.stats_grid);
-            const int c_hi = tile_owner((long long)(nb + 1) * p.tph - 1, total, p.stats_grid);
-            float lse = INFINITY;
+          if (sg.new_head) {
+            // lse2 of every window row from the partial statistics of sweep 1, 512 / 128 (or 256) threads a row and four
+            // loads in flight each: a head of a one-layer job has some twenty parts, and read one after the other by one
+            // thread they delayed the start of the job by 13 us
+            const int rows = NMBLK(p) * 128, parts = kSoftmaxThreads / rows, r = sid & (rows - 1), part_ = sid / rows;
             const float* lse_in = (jb ? maps1 : maps0).lse[nb / p.hpl];
-            if (lse_in) {
-              if (sid < p.M) lse = lse_in[(size_t)(nb % p.hpl) * p.M + sid] * kLog2e;
-            } else if (sid < p.M) {
-              float m = -INFINITY;
-              for (int c = 0; c <= c_hi - c_lo; ++c) m = fmaxf(m, p.stats[((size_t)nb * p.slots + c) * p.m_stride + sid].x);
-              float l = 0.f;
-              for (int c = 0; c <= c_hi - c_lo; ++c) {
-                const float2 st = p.stats[((size_t)nb * p.slots + c) * p.m_stride + sid];
-                l += st.y * fast_exp2(st.x - m);
+            float m = -INFINITY, l = 0.f;
+            if (!lse_in && r < p.M) {
+              const long long total = (long long)p.heads * p.tph;
+              const int c_lo = tile_owner((long long)nb * p.tph, total, p.stats_grid);
+              const int n = tile_owner((long long)(nb + 1) * p.tph - 1, total, p.stats_grid) - c_lo + 1;
+              const float2* st = p.stats + (size_t)nb * p.slots * p.m_stride + r;
+              for (int c = part_; c < n; c += 4 * parts) {
+                float2 x[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) x[j] = c + j * parts < n ? st[(size_t)(c + j * parts) * p.m_stride] : make_float2(-INFINITY, 0.f);
+                const float mn = fmaxf(fmaxf(m, fmaxf(x[0].x, x[1].x)), fmaxf(x[2].x, x[3].x));
+                if (mn > -INFINITY) {
+                  l *= fast_exp2(m - mn);
+#pragma unroll
+                  for (int j = 0; j < 4; ++j) l += x[j].y * fast_exp2(x[j].x - mn);
+                  m = mn;
+                }
               }
-              lse = m + log2f(l);
             }
-            nlse_s[sid] = -lse;
+            if (part_ > 0) merge_s[(part_ - 1) * rows + r] = make_float2(m, l);
+            asm volatile("bar.sync 1, 512;" ::: "memory");
+            if (part_ == 0) {
+              float lse = INFINITY;
+              if (r < p.M) {
+                if (lse_in) lse = lse_in[(size_t)(nb % p.hpl) * p.M + r] * kLog2e;
+                else {
+                  float mn = m;
+                  for (int q = 0; q < parts - 1; ++q) mn = fmaxf(mn, merge_s[q * rows + r].x);
+                  l *= fast_exp2(m - mn);
+                  for (int q = 0; q < parts - 1; ++q) { const float2 o = merge_s[q * rows + r]; l += o.y * fast_exp2(o.x - mn); }
+                  lse = mn + log2f(l);
+                }
+              }
+              nlse_s[r] = -lse;
+            }
           }
           asm volatile("bar.sync 1, 512;" ::: "memory");
           const int nchunk = kFast ? 8 : p.nq16 >> 4;               // 16-column chunks; this warp takes half, half+2, ...
