@@ -335,9 +335,13 @@ int do_select(dkv_ctx* c, int layer, int* sorted_out, int* rank_out, cudaStream_
     ProfScope ps(c, DKV_STEP_SELECT, 1, st);
     unsigned int* lh = c->d_layer_hist + (size_t)layer * s.Bt * kBins;
     DKV_CUDA(c, cudaMemsetAsync(lh, 0, sizeof(unsigned int) * s.Bt * kBins, st));
-    DKV_LAUNCH(c, launch_pdl(select_topk_kernel, dim3(s.Bt * s.Hkv), kSelThreads, select_smem(c->sel_cap), 1, st,
-                             (const float*)(c->d_scores + (size_t)layer * layer_scores(s)), c->d_idx + (size_t)layer * layer_idx(s), lh, s.P, s.Blc,
-                             c->sel_cap, c->d_count, s.Hkv, s.L, layer));
+    // a cluster a head while the heads leave SMs idle and a block's share is a few thousand positions at least
+    const int heads = s.Bt * s.Hkv;
+    int parts = 1;
+    while (parts < 8 && heads * parts * 2 <= c->n_sms && s.P > parts * 2 * kSelThreads) parts *= 2;
+    DKV_LAUNCH(c, launch_pdl(parts > 1 ? select_topk_kernel<true> : select_topk_kernel<false>, dim3(heads * parts), kSelThreads, select_smem(c->sel_cap),
+                             parts, st, (const float*)(c->d_scores + (size_t)layer * layer_scores(s)), c->d_idx + (size_t)layer * layer_idx(s), lh, s.P,
+                             s.Blc, c->sel_cap, c->d_count, s.Hkv, s.L, layer, parts));
   }
   c->selected[layer] = 1;
   c->sel_n[layer] = s.Blc;
@@ -649,7 +653,8 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   // contexts do not undo each other.
   {
     const int most = (int)(select_smem(kMaxCountingList) > select_smem(DKV_MAX_LAYER_BUDGET) ? select_smem(kMaxCountingList) : select_smem(DKV_MAX_LAYER_BUDGET));
-    TRY(cudaFuncSetAttribute(select_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRY(cudaFuncSetAttribute(select_topk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRY(cudaFuncSetAttribute(select_topk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     TRY(cudaFuncSetAttribute(select_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     TRY(cudaFuncSetAttribute(sort_positions_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DKV_MAX_LAYER_BUDGET * 8));
   }
