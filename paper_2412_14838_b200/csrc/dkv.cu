@@ -413,6 +413,25 @@ int do_select_gather(dkv_ctx* c, const void* const* k, const void* const* v, voi
   return DKV_OK;
 }
 
+// The address under which kernels can use page-locked host memory, if `host` is that (and 16-byte aligned).
+bool host_view(const void* host, void** dev) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, host) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer && aligned16(at.devicePointer)) {
+    *dev = at.devicePointer;
+    return true;
+  }
+  cudaGetLastError();                          // an unregistered pointer is not an error here
+  return false;
+}
+
+// Layer counts after which Algorithm 1 updates the budgets: every m layers, and after the last.
+int update_points(const Shape& s, int* l) {
+  int n = 0;
+  for (int u = s.m; u < s.L; u += s.m) l[n++] = u;
+  l[n++] = s.L;
+  return n;
+}
+
 int do_reset(dkv_ctx* c, cudaStream_t st) {
   const Shape& s = c->s;
   DKV_CUDA(c, cudaMemsetAsync(c->d_count, 0, sizeof(int) * s.Bt * s.L, st));
@@ -507,10 +526,8 @@ int do_pass(dkv_ctx* c, const void* const* q, const void* const* k, const void* 
     }
     if (rc) return rc;
   }
-  int l[DKV_MAX_LAYERS], n = 0;
-  for (int u = s.m; u < s.L; u += s.m) l[n++] = u;
-  l[n++] = s.L;                                              // after the last layer whether or not m divides L
-  if ((rc = do_rebudget(c, l, n, s.Blc, nullptr, st))) return rc;
+  int l[DKV_MAX_LAYERS];
+  if ((rc = do_rebudget(c, l, update_points(s, l), s.Blc, nullptr, st))) return rc;
   if ((rc = do_select_gather(c, k, v, kb, vb, st))) return rc;
   mark_pass_done(c);
   return DKV_OK;
@@ -836,13 +853,15 @@ int dkv_run_prefill_pass_host(dkv_ctx* c, const void* const* q_win, const void* 
   // V being copied in full first; pageable memory (or DKV_HOST_V_STAGED=1) takes the full copy.
   const void* v_dev[DKV_MAX_LAYERS];
   for (int l = 0; l < s.L; ++l) {
-    v_dev[l] = nullptr;
-    if (c->host_v_staged) continue;
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, v[l]) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer && aligned16(at.devicePointer))
-      v_dev[l] = at.devicePointer;
-    else
-      cudaGetLastError();                      // an unregistered pointer is not an error here
+    void* p = nullptr;
+    v_dev[l] = !c->host_v_staged && host_view(v[l], &p) ? p : nullptr;
+  }
+  // Page-locked output buffers are written by one kernel at the end.
+  PassPtrs out;
+  bool out_mapped = true;
+  for (int l = 0; l < s.L && out_mapped; ++l) {
+    out.k[l] = c->st_kb[l]; out.v[l] = c->st_vb[l];
+    out_mapped = host_view(kb[l], &out.kb[l]) && host_view(vb[l], &out.vb[l]);
   }
   const long long row_bytes = (long long)s.D * 2;
   long long h2d = 0;
@@ -863,35 +882,38 @@ int dkv_run_prefill_pass_host(dkv_ctx* c, const void* const* q_win, const void* 
     if ((rc = do_gather(c, l, c->st_k[slot], v_dev[l] ? v_dev[l] : c->st_v[slot], c->st_kb[l], c->st_vb[l], st))) return rc;
     if (v_dev[l]) h2d += (long long)(c->sel_n[l] + s.ws) * s.Bt * s.Hkv * row_bytes;
     DKV_CUDA(c, cudaEventRecord(c->ev_consumed[slot], st));
-    const bool update = ((l + 1) % s.m == 0) || (l + 1 == s.L && s.L % s.m != 0);
-    if (update) {
-      const int upto = l + 1;
-      if ((rc = do_rebudget(c, &upto, 1, 0, nullptr, st))) return rc;
-      if ((rc = do_shrink(c, 0, l + 1, c->st_kb, c->st_vb, st))) return rc;
-    }
   }
-  // The final counts come back first; then only the valid rows of every head (count + ws of the fixed stride)
-  // are copied out, one strided copy per (layer, sample, tensor).
+  // all updates together, as in do_pass
+  int upd[DKV_MAX_LAYERS];
+  if ((rc = do_rebudget(c, upd, update_points(s, upd), 0, nullptr, st))) return rc;
+  if ((rc = do_shrink(c, 0, s.L, c->st_kb, c->st_vb, st))) return rc;
+  if (out_mapped) {
+    const int per_block = kGatherThreads / (s.D * 2 / 16) * kGatherRows;
+    DKV_LAUNCH(c, launch_pdl(copy_valid_kernel, dim3((s.rows + per_block - 1) / per_block, s.Bt * s.Hkv, s.L), kGatherThreads, 0, 1, st, out,
+                             (const int*)c->d_held, s.ws, s.rows, s.D * 2 / 16, s.Hkv, s.L));
+  }
   std::vector<int> counts((size_t)s.Bt * s.L);
   DKV_CUDA(c, cudaMemcpyAsync(counts.data(), c->d_count, sizeof(int) * s.Bt * s.L, cudaMemcpyDeviceToHost, st));
   DKV_CUDA(c, cudaStreamSynchronize(st));
-  const size_t row = (size_t)s.D * 2, head_pitch = (size_t)s.rows * row, sample = (size_t)s.Hkv * head_pitch;
-  for (int l = 0; l < s.L; ++l)
-    for (int b = 0; b < s.Bt; ++b) {
-      const size_t valid = (size_t)(counts[(size_t)b * s.L + l] + s.ws) * row;
-      DKV_CUDA(c, cudaMemcpy2DAsync(static_cast<char*>(kb[l]) + b * sample, head_pitch,
-                                    static_cast<const char*>(c->st_kb[l]) + b * sample, head_pitch, valid, s.Hkv,
-                                    cudaMemcpyDeviceToHost, st));
-      DKV_CUDA(c, cudaMemcpy2DAsync(static_cast<char*>(vb[l]) + b * sample, head_pitch,
-                                    static_cast<const char*>(c->st_vb[l]) + b * sample, head_pitch, valid, s.Hkv,
-                                    cudaMemcpyDeviceToHost, st));
-    }
+  if (!out_mapped) {                           // one strided copy of the valid rows per (layer, sample, tensor)
+    const size_t row = (size_t)s.D * 2, head_pitch = (size_t)s.rows * row, sample = (size_t)s.Hkv * head_pitch;
+    for (int l = 0; l < s.L; ++l)
+      for (int b = 0; b < s.Bt; ++b) {
+        const size_t valid = (size_t)(counts[(size_t)b * s.L + l] + s.ws) * row;
+        DKV_CUDA(c, cudaMemcpy2DAsync(static_cast<char*>(kb[l]) + b * sample, head_pitch,
+                                      static_cast<const char*>(c->st_kb[l]) + b * sample, head_pitch, valid, s.Hkv,
+                                      cudaMemcpyDeviceToHost, st));
+        DKV_CUDA(c, cudaMemcpy2DAsync(static_cast<char*>(vb[l]) + b * sample, head_pitch,
+                                      static_cast<const char*>(c->st_vb[l]) + b * sample, head_pitch, valid, s.Hkv,
+                                      cudaMemcpyDeviceToHost, st));
+      }
+    DKV_CUDA(c, cudaStreamSynchronize(st));
+  }
   if (counts_out) memcpy(counts_out, counts.data(), sizeof(int) * s.Bt * s.L);
   long long d2h = (long long)sizeof(int) * s.Bt * s.L;
   for (size_t i = 0; i < counts.size(); ++i) d2h += 2ll * (counts[i] + s.ws) * s.Hkv * row_bytes;
   c->host_h2d = h2d; c->host_d2h = d2h;
   DKV_CUDA(c, cudaStreamSynchronize(cp));
-  DKV_CUDA(c, cudaStreamSynchronize(st));
   return DKV_OK;
 }
 

@@ -368,14 +368,6 @@ select_topk_kernel(const float* __restrict__ scores, int* __restrict__ idx, unsi
   if (sel) for (int i = threadIdx.x; i < keep; i += kSelThreads) idx[(size_t)head * keep + i] = sel[i];
 }
 
-// Per-layer device pointers of a pass.
-struct PassPtrs {
-  const void* k[128];
-  const void* v[128];
-  void* kb[128];
-  void* vb[128];
-};
-
 // The end of a pass, for every layer and head at once: with the final counts known (count[b][layer], at most B^l), a
 // block selects its head's best `count` positions, writes them to idx [layer][Bt*Hkv][stride] and copies those rows and
 // the ws window rows of K and V into the layer's buffers.  Selecting and copying the final rows once replaces a
