@@ -48,8 +48,7 @@ struct dkv_ctx {
   int retain_mb;        // MB of a sweep-1 job's keys (the end of every CTA's slice) marked to stay in L2 for sweep 2
   long long wait_cycles;   // limit of the scoring kernel's mbarrier waits (dkv_set_wait_limit)
   int withhold_sweep, withhold_tile;   // test hook of dkv_debug_withhold_tile (-1: off)
-  float2* d_tc_stats;   // [stats_rows][256]: partial softmax statistics, [heads of a launch][slots][256]
-  unsigned int* d_done; // [heads of a launch + 2] arrival counters of the scoring kernel, zero between launches
+  float2* d_tc_stats;   // [3][stats_rows][256]: partial softmax statistics, three jobs in rotation, each [heads][slots][256]
   // host state
   uint8_t scored[DKV_MAX_LAYERS], gathered[DKV_MAX_LAYERS];
   uint8_t selected[DKV_MAX_LAYERS];     // 1: by scores (dkv_select_topk), 2: by position (dkv_select_positions)
@@ -126,17 +125,6 @@ struct ProfScope {
   ~ProfScope() { if (r) cudaEventRecord(r->b, st); }
 };
 
-// Cooperative launch: all blocks resident at once (they wait for one another).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_coop(void (*kernel)(KArgs...), int grid, int threads, size_t smem, cudaStream_t st, const Args&... args) {
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeCooperative;
-  at[0].val.cooperative = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cfg.attrs = at; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
 // Launch with programmatic stream serialisation (the kernel waits for its predecessor itself, so that its scheduling
 // overlaps the predecessor's end) and, if cluster > 1, clusters of that many blocks along x.
 template <typename... KArgs, typename... Args>
@@ -231,13 +219,19 @@ uint32_t make_idesc(int M, int N) {
 // Statistics slots a head of a job needs: thread blocks that can share it (its share of the grid, one cut at either end).
 int stats_slots(int n_sms, int job_heads) { return n_sms / job_heads + 2; }
 
-// Parameters of one sweep over the `nl` consecutive layers that start at `layer`.  In sweep 2 every CTA walks its slice of the
-// key space from the end to the start: sweep 1 cut the same space into the same slices, so each CTA begins with the keys
-// that were streamed last and may still be in L2.  `done`: both sweeps are in this launch, whose `grid` blocks exchange
-// their statistics.
-void make_job(const dkv_ctx* c, int mode, int layer, int nl, float* scores_out, bool done, int grid, bool hist, tc::Params* p) {
+// Parameters of one sweep over the `nl` consecutive layers that start at `layer` (q, k: their nl device
+// pointers); `buf` picks the statistics scratch (jobs in flight rotate).  In sweep 2 every CTA walks its slice of the
+// key space from the end to the start: sweep 1 cut the same space into the same slices, so each CTA begins with
+// the keys that were streamed last and may still be in L2.
+// `grid`: thread blocks of the launch; `stats_grid`: of the launch that ran sweep 1 for these layers (sweep 2).
+template <int NL>
+bool make_job(dkv_ctx* c, int mode, int layer, int nl, const void* const* q, const void* const* k, float* scores_out,
+              int buf, int grid, int stats_grid, bool hist, tc::Maps<NL>* maps, tc::Params* p, const float* const* lse = nullptr) {
   const Shape& s = c->s;
   const int heads = s.Bt * s.Hkv;
+  for (int i = 0; i < nl; ++i)
+    if (!make_map(&maps->q[i], q[i], s.D, s.M, heads) || !make_map(&maps->k[i], k[i], s.D, s.S, heads)) return false;
+  for (int i = 0; i < nl; ++i) maps->lse[i] = lse ? lse[i] : nullptr;      // (entries past nl are never read)
   p->S = s.S; p->P = s.P; p->ws = s.ws; p->M = s.M; p->D = s.D; p->heads = nl * heads; p->half = s.pool / 2;
   p->nl = nl; p->hpl = heads;
   p->back = (mode == tc::kEmit && c->emit_backward) ? 1 : 0;
@@ -249,18 +243,18 @@ void make_job(const dkv_ctx* c, int mode, int layer, int nl, float* scores_out, 
   p->nmblk = (s.M + 127) / 128;
   p->slots = stats_slots(c->n_sms, nl * heads); p->m_stride = 256;
   p->scale2 = kLog2e / sqrtf((float)s.D);
-  p->stats = c->d_tc_stats;
-  p->done = done ? c->d_done : nullptr;
+  p->stats = c->d_tc_stats + (size_t)buf * c->stats_rows * 256;
   p->scores = c->d_scores + (size_t)layer * layer_scores(s);
   p->copy_out = scores_out;
   p->status = c->d_status;
-  p->stats_grid = grid;
+  p->stats_grid = stats_grid;
   p->layer_hist = hist ? c->d_layer_hist + (size_t)layer * s.Bt * kBins : nullptr;
   p->hkv = s.Hkv;
   p->mode = mode;
   p->out_scale = (c->cfg.flags & DKV_F_WINDOW_MEAN) ? 1.0f / (float)s.M : 1.0f;
   p->pool_avg = c->cfg.pool_kind == 1;
   p->idesc = mode == tc::kStats ? make_idesc(128, 128) : make_idesc(128, p->nq16);
+  return true;
 }
 
 cudaError_t set_score_attributes() {
@@ -275,11 +269,10 @@ cudaError_t set_score_attributes() {
 // The scoring kernel for two jobs (either may be kNone): the specialised build when every job has exactly 128 window
 // rows of 128 dims, the general one otherwise.
 template <int NL>
-cudaError_t launch_tc(int grid, cudaStream_t st, const tc::Maps<NL>& maps, const tc::Params& j0, const tc::Params& j1) {
+cudaError_t launch_tc(int grid, cudaStream_t st, const tc::Maps<NL>& m0, const tc::Maps<NL>& m1, const tc::Params& j0, const tc::Params& j1) {
   auto fast = [](const tc::Params& p) { return p.mode == tc::kNone || (p.M == 128 && p.D == 128); };
-  const auto kernel = fast(j0) && fast(j1) ? tc::score_tc_kernel<NL, true> : tc::score_tc_kernel<NL, false>;
-  if (j1.done) return launch_coop(kernel, grid, tc::kThreads, (size_t)tc::kSmemBytes, st, maps, j0, j1);
-  return launch_pdl(kernel, dim3(grid), tc::kThreads, (size_t)tc::kSmemBytes, 1, st, maps, j0, j1);
+  return launch_pdl(fast(j0) && fast(j1) ? tc::score_tc_kernel<NL, true> : tc::score_tc_kernel<NL, false>, dim3(grid), tc::kThreads,
+                    (size_t)tc::kSmemBytes, 1, st, m0, m1, j0, j1);
 }
 
 // Thread blocks of a scoring launch over `nl` layers: one an SM, fewer if there are fewer key tiles.
@@ -288,32 +281,37 @@ int score_grid(const dkv_ctx* c, int nl) {
   return (int)(tiles < c->n_sms ? tiles : c->n_sms);
 }
 
-// Scores of the `nl` consecutive layers from `layer` in one launch: both sweeps, or with `lse` (the caller's normalisers) sweep 2
-// alone.  q, k, lse: the layers' pointers.
+// A group of consecutive layers that is scored together: its first layer, how many, the statistics scratch its sweep 1
+// writes and the grid it ran on.
+struct ScoreGroup { int first, n, buf, grid; };
+
+// One launch: sweep 2 of group `e` (if not null), then sweep 1 of group `s` (if not null), whose grid it sets.  `q`, `k`,
+// `lse`: all layers' pointers, indexed by layer (lse: null, or the caller's normalisers instead of sweep 1).
 template <int NL>
-int launch_score(dkv_ctx* c, int layer, int nl, const void* const* q, const void* const* k, const float* const* lse, float* scores_out,
-                 bool hist, cudaStream_t st) {
-  const Shape& s = c->s;
-  const int heads = s.Bt * s.Hkv, grid = score_grid(c, nl);
-  tc::Maps<NL> maps;                         // only the layers of the jobs are filled in and read
+int launch_score(dkv_ctx* c, const ScoreGroup* e, ScoreGroup* s, const void* const* q, const void* const* k, const float* const* lse,
+                 float* scores_out, bool hist, cudaStream_t st) {
+  tc::Maps<NL> m0, m1;                       // only the layers of the jobs are filled in and read
   tc::Params j0, j1;
   memset(&j0, 0, sizeof j0); memset(&j1, 0, sizeof j1);
-  j0.mode = tc::kNone;
-  for (int i = 0; i < nl; ++i) {
-    if (!make_map(&maps.q[i], q[i], s.D, s.M, heads) || !make_map(&maps.k[i], k[i], s.D, s.S, heads)) return DKV_ERR_CUDA;
-    maps.lse[i] = lse ? lse[i] : nullptr;
-  }
-  if (!lse) make_job(c, tc::kStats, layer, nl, nullptr, true, grid, hist, &j0);
-  make_job(c, tc::kEmit, layer, nl, scores_out, !lse, grid, hist, &j1);
-  ProfScope ps(c, DKV_STEP_SCORE_EMIT, 1, st);
-  DKV_LAUNCH(c, launch_tc(grid, st, maps, j0, j1));
+  j0.mode = j1.mode = tc::kNone;
+  const int most = e && (!s || e->n > s->n) ? e->n : s->n, grid = score_grid(c, most);
+  if (s) s->grid = grid;
+  if (e && !make_job(c, tc::kEmit, e->first, e->n, q + e->first, k + e->first, scores_out, e->buf, grid, e->grid, hist, &m0, &j0, lse ? lse + e->first : nullptr)) return DKV_ERR_CUDA;
+  if (s && !make_job(c, tc::kStats, s->first, s->n, q + s->first, k + s->first, nullptr, s->buf, grid, grid, hist, &m1, &j1)) return DKV_ERR_CUDA;
+  ProfScope ps(c, s ? DKV_STEP_SCORE_STATS : DKV_STEP_SCORE_EMIT, 1, st);
+  DKV_LAUNCH(c, launch_tc(grid, st, e ? m0 : m1, s ? m1 : m0, j0, j1));
   return DKV_OK;
 }
 
-// Scores of one layer; lse: as for dkv_score_lse, or null.
+// One layer on its own; lse: as for dkv_score_lse, or null.
 int do_score(dkv_ctx* c, int layer, const void* q, const void* k, const float* lse, float* scores_out, cudaStream_t st) {
-  const int rc = launch_score<1>(c, layer, 1, &q, &k, lse ? &lse : nullptr, scores_out, false, st);
-  if (rc) return rc;
+  ScoreGroup g = {layer, 1, layer % 3, 0};
+  const void *qs[DKV_MAX_LAYERS], *ks[DKV_MAX_LAYERS];      // indexed by layer
+  const float* ls[DKV_MAX_LAYERS];
+  qs[layer] = q; ks[layer] = k; ls[layer] = lse;
+  int rc;
+  if (!lse && (rc = launch_score<1>(c, nullptr, &g, qs, ks, nullptr, nullptr, false, st))) return rc;
+  if ((rc = launch_score<1>(c, &g, nullptr, qs, ks, lse ? ls : nullptr, scores_out, false, st))) return rc;
   c->scored[layer] = 1;
   c->selected[layer] = c->gathered[layer] = 0;
   return DKV_OK;
@@ -502,8 +500,9 @@ int do_decode(dkv_ctx* c, int layer0, int nl, int nq, const void* const* q, cons
 }
 
 // Algorithm 1's loop, one chain of launches on `st`.
-//   scoring   in groups of up to `pass_group` layers a launch (the fixed cost of a launch is paid once per group), on all SMs,
-//             with the counts of the scores' digits.  With `lse` (the window rows' log-denominators) in one sweep.
+//   scoring   launch g runs sweep 2 of layer group g-1 and then sweep 1 of group g (a group = up to `pass_group` layers, so
+//             that the fixed cost of a launch is paid once per group) on all SMs; sweep 2 also counts the scores' digits.
+//             With `lse` (the window rows' log-denominators of every layer) launch g runs sweep 2 of group g only.
 //   updates   all of Eq. 4-6's updates together: their order does not matter, a layer's count is the minimum over them
 //             and nothing reads an intermediate one.
 //   select, gather   with the final counts.
@@ -513,10 +512,19 @@ int do_pass(dkv_ctx* c, const void* const* q, const void* const* k, const void* 
             void* const* kb, void* const* vb, cudaStream_t st) {
   const Shape& s = c->s;
   int rc;
-  if (lse) DKV_CUDA(c, cudaMemsetAsync(c->d_layer_hist, 0, sizeof(unsigned int) * s.L * s.Bt * kBins, st));   // (else sweep 1 clears the digit counters)
-  for (int l0 = 0; l0 < s.L; l0 += c->pass_group) {
-    const int n = s.L - l0 < c->pass_group ? s.L - l0 : c->pass_group;
-    if ((rc = launch_score<tc::kMaxGroup>(c, l0, n, q + l0, k + l0, lse ? lse + l0 : nullptr, nullptr, true, st))) return rc;
+  if (lse) DKV_CUDA(c, cudaMemsetAsync(c->d_layer_hist, 0, sizeof(unsigned int) * s.L * s.Bt * kBins, st));   // else sweep 1 does it
+  ScoreGroup prev = {}, cur = {};
+  for (int g = 0, done = 0; done < s.L || prev.n; ++g) {
+    cur.first = done; cur.n = s.L - done < c->pass_group ? s.L - done : c->pass_group; cur.buf = g % 3;
+    done += cur.n;
+    if (lse) {
+      if (!cur.n) break;
+      rc = launch_score<tc::kMaxGroup>(c, &cur, nullptr, q, k, lse, nullptr, true, st);
+    } else {
+      rc = launch_score<tc::kMaxGroup>(c, prev.n ? &prev : nullptr, cur.n ? &cur : nullptr, q, k, nullptr, nullptr, true, st);
+      prev = cur;
+    }
+    if (rc) return rc;
   }
   int l[DKV_MAX_LAYERS];
   if ((rc = do_rebudget(c, l, update_points(s, l), s.Blc, nullptr, st))) return rc;
@@ -528,7 +536,7 @@ int do_pass(dkv_ctx* c, const void* const* q, const void* const* k, const void* 
 void free_all(dkv_ctx* c) {
   cudaFree(c->d_scores); cudaFree(c->d_idx); cudaFree(c->d_count); cudaFree(c->d_held); cudaFree(c->d_dbg);
   cudaFree(c->d_rb_state); cudaFree(c->d_rb_above); cudaFree(c->d_layer_hist); cudaFree(c->d_shrink_tickets);
-  cudaFree(c->d_cand); cudaFree(c->d_cand_n); cudaFree(c->d_status); cudaFree(c->d_tc_stats); cudaFree(c->d_done);
+  cudaFree(c->d_cand); cudaFree(c->d_cand_n); cudaFree(c->d_status); cudaFree(c->d_tc_stats);
   cudaFree(c->d_dec_scratch); cudaFree(c->d_dec_tickets);
   if (c->pass_exec) cudaGraphExecDestroy(c->pass_exec);
   delete c->pass_key;
@@ -647,9 +655,7 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   TRY(cudaMalloc(&c->d_layer_hist, sizeof(unsigned int) * s.L * s.Bt * kBins));
   TRY(cudaMalloc(&c->d_cand, sizeof(uint2) * s.L * layer_scores(s)));
   TRY(cudaMalloc(&c->d_cand_n, sizeof(unsigned int) * s.Bt));
-  TRY(cudaMalloc(&c->d_tc_stats, sizeof(float2) * c->stats_rows * 256));
-  TRY(cudaMalloc(&c->d_done, sizeof(unsigned int) * ((size_t)tc::kMaxGroup * heads + 2)));
-  TRY(cudaMemset(c->d_done, 0, sizeof(unsigned int) * ((size_t)tc::kMaxGroup * heads + 2)));
+  TRY(cudaMalloc(&c->d_tc_stats, sizeof(float2) * 3 * c->stats_rows * 256));
   TRY(set_score_attributes());
   TRY(cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking));
   c->pass_key = new (std::nothrow) std::vector<const void*>();
@@ -1074,10 +1080,10 @@ int dkv_score_static(const dkv_config* cfg, const void* q_win, const void* k, fl
   p.stats_grid = grid;
   p.mode = tc::kStats;
   p.idesc = make_idesc(128, 128);
-  if (launch_tc(grid, st, maps, p, none) != cudaSuccess) { cudaGetLastError(); return DKV_ERR_CUDA; }
+  if (launch_tc(grid, st, maps, maps, p, none) != cudaSuccess) { cudaGetLastError(); return DKV_ERR_CUDA; }
   p.mode = tc::kEmit;
   p.idesc = make_idesc(128, p.nq16);
-  if (launch_tc(grid, st, maps, none, p) != cudaSuccess) { cudaGetLastError(); return DKV_ERR_CUDA; }
+  if (launch_tc(grid, st, maps, maps, none, p) != cudaSuccess) { cudaGetLastError(); return DKV_ERR_CUDA; }
   return DKV_OK;
 }
 

@@ -13,10 +13,8 @@
 // in two groups that alternate tiles, each warp one TMEM lane quadrant x half the columns.
 // Work is split evenly: the flattened (head, key tile) space for sweep 1 and the flattened
 // (head, prefix position) space for sweep 2 are cut into one contiguous slice per CTA.
-// One launch runs both sweeps of a group of layers back to back through the same pipeline: while the last thread blocks
-// finish a head's sweep 1, the others' copies and MMAs for sweep 2 are under way already; only the softmax warps wait, at a
-// head's start, until the parts of its statistics from all blocks are there (a counter per head, `done`).  That takes a
-// cooperative launch, and saves the launch, set-up and pipeline fill of a second one.
+// One launch runs up to two jobs back to back through the same pipeline (sweep 2 of one layer, then
+// sweep 1 of the next), so the fixed cost of a launch is paid once per layer.
 #pragma once
 #include <cuda.h>
 #include "common.cuh"
@@ -62,8 +60,6 @@ struct Params {
   int hkv;                 // KV heads per sample
   int* status;             // device status words; [0] = first error
   int stats_grid;          // CTAs of the launch that ran sweep 1 for this layer
-  unsigned int* done;      // null (sweep 1 is in an earlier launch, or not needed), or [heads] parts of a head that have arrived,
-                           // [heads] CTAs that have ended, [heads + 1] CTAs that have cleared their share of layer_hist.  Zero between launches
   int mode;                // kNone: nothing to do
   float out_scale;         // sweep 2: factor on the raw scores before pooling (1, or 1/(ws*G) for the window mean)
   int pool_avg;            // sweep 2: 0 = max-pool, 1 = average over the neighbours that exist
@@ -341,12 +337,13 @@ __host__ __device__ __forceinline__ int tile_owner(long long x, long long total,
 }
 
 // ------------------------------------------------------------------------------------------ kernel
-// job0, then job1, over the same layers; a job with mode kNone is skipped.
+// job0 uses maps0, job1 uses maps1; a job with mode kNone is skipped.
 // kFast: both jobs have exactly 128 window rows of 128 dims (ws*G = 128, D = 128, the shape of the 32/8-head models):
 // the row-block count, the chunk count and the k-step count are then compile-time constants.
 template <int NL, bool kFast>
 __global__ void __launch_bounds__(kThreads, 1)
-score_tc_kernel(const __grid_constant__ Maps<NL> maps, const __grid_constant__ Params job0, const __grid_constant__ Params job1) {
+score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ Maps<NL> maps1,
+                const __grid_constant__ Params job0, const __grid_constant__ Params job1) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* q_smem = smem;                              // [half][256 rows][128 B]
@@ -389,10 +386,6 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, const __grid_constant__ P
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
-  if (warp == 0 && lane == 0) {
-    auto prefetch = [](const CUtensorMap* m) { asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory"); };
-    prefetch(&maps.q[0]); prefetch(&maps.k[0]);
-  }
   pdl_launch();
   pdl_wait();
 
@@ -405,6 +398,7 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, const __grid_constant__ P
       for (int jb = 0; jb < 2 && ok; ++jb) {
         const Params& p = jb ? job1 : job0;
         if (p.mode == kNone) continue;
+        const Maps<NL>& maps = jb ? maps1 : maps0;
         const int halves = DIMS(p) / 64;
         const uint32_t tile_bytes = (uint32_t)halves * kHalfBytes;
         const int withhold = blockIdx.x == 0 ? p.withhold_tile : -1;
@@ -538,26 +532,8 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, const __grid_constant__ P
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
     int tile = 0;
     int hist_of = -1;                          // whose digits hist_s holds: layer * samples + sample of the job
-    // One thread waits until a counter that other CTAs raise has reached `n`, the others at the barrier.  Such a wait may
-    // follow another CTA's that has run out: that one reports (its limit is shorter).
-    auto wait_for = [&](const Params& p, unsigned int* counter, unsigned int n) {
-      if (sid == 0) {
-        const long long t0 = clock64();
-        while (*(volatile unsigned int*)counter < n && !*abort_flag) {
-          __nanosleep(64);
-          if (clock64() - t0 > 4 * p.wait_cycles) {
-            *abort_flag = 1;
-            if (atomicCAS(p.status, 0, 108) == 0) p.status[2] = (int)blockIdx.x;
-          }
-        }
-        __threadfence();
-      }
-      asm volatile("bar.sync 1, 512;" ::: "memory");
-    };
-    bool cleared = false;                      // every CTA has cleared its share of layer_hist
     // adds hist_s to the counters of `hist_of` and clears it; followed by a barrier before anything is counted again
     auto flush_hist = [&](const Params& p) {
-      if (p.done && !cleared) { cleared = true; wait_for(p, &p.done[p.heads + 1], gridDim.x); }
       unsigned int* to = p.layer_hist + (size_t)hist_of * kBins;
       for (int i = sid; i < kBins; i += kSoftmaxThreads) {
         const unsigned int n = hist_s[i];
@@ -569,11 +545,9 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, const __grid_constant__ P
       if (p.mode == kNone) continue;
       SegIter it(p, blockIdx.x, gridDim.x);
       Seg sg;
-      if (p.mode == kStats && p.layer_hist) {  // sweep 2 counts into them once every CTA has cleared its share (flush_hist)
+      if (p.mode == kStats && p.layer_hist) {  // sweep 2 of these layers, which counts, is in a later launch
         const int n = p.heads / p.hkv * kBins;
         for (int i = blockIdx.x * kSoftmaxThreads + sid; i < n; i += gridDim.x * kSoftmaxThreads) p.layer_hist[i] = 0;
-        asm volatile("bar.sync 1, 512;" ::: "memory");
-        if (sid == 0) { __threadfence(); atomicAdd(&p.done[p.heads + 1], 1u); }
       }
       const int tmask = NMBLK(p) == 1 ? 3 : 1, tshift = NMBLK(p) == 1 ? 2 : 1, scols = NMBLK(p) == 1 ? 128 : 256;
       const uint64_t scale22 = pack2(p.scale2, p.scale2);
@@ -659,7 +633,6 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, const __grid_constant__ P
             }
           }
           asm volatile("bar.sync 1, 512;" ::: "memory");
-          if (p.done && sid == 0) { __threadfence(); atomicAdd(&p.done[sg.bh], 1u); }
         } else {
           // ------------------------------------------------------------ sweep 2: one thread per key
           const int nb = sg.bh;
@@ -672,17 +645,17 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, const __grid_constant__ P
             // loads in flight each: a head of a one-layer job has some twenty parts, and read one after the other by one
             // thread they delayed the start of the job by 13 us
             const int rows = NMBLK(p) * 128, parts = kSoftmaxThreads / rows, r = sid & (rows - 1), part_ = sid / rows;
-            const float* lse_in = maps.lse[nb / p.hpl];
+            const float* lse_in = (jb ? maps1 : maps0).lse[nb / p.hpl];
             float m = -INFINITY, l = 0.f;
-            const long long total = (long long)p.heads * p.tph;
-            const int n = tile_owner((long long)(nb + 1) * p.tph - 1, total, p.stats_grid) - tile_owner((long long)nb * p.tph, total, p.stats_grid) + 1;
-            if (p.done) wait_for(p, &p.done[nb], (unsigned int)n);
             if (!lse_in && r < p.M) {
+              const long long total = (long long)p.heads * p.tph;
+              const int c_lo = tile_owner((long long)nb * p.tph, total, p.stats_grid);
+              const int n = tile_owner((long long)(nb + 1) * p.tph - 1, total, p.stats_grid) - c_lo + 1;
               const float2* st = p.stats + (size_t)nb * p.slots * p.m_stride + r;
               for (int c = part_; c < n; c += 4 * parts) {
                 float2 x[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) x[j] = c + j * parts < n ? __ldcg(&st[(size_t)(c + j * parts) * p.m_stride]) : make_float2(-INFINITY, 0.f);
+                for (int j = 0; j < 4; ++j) x[j] = c + j * parts < n ? st[(size_t)(c + j * parts) * p.m_stride] : make_float2(-INFINITY, 0.f);
                 const float mn = fmaxf(fmaxf(m, fmaxf(x[0].x, x[1].x)), fmaxf(x[2].x, x[3].x));
                 if (mn > -INFINITY) {
                   l *= fast_exp2(m - mn);
@@ -801,13 +774,6 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, const __grid_constant__ P
   }
   tc_fence_before();
   __syncthreads();
-  if (job1.done && warp == 0) {
-    // the last CTA to end clears the counters for the next launch
-    unsigned int ended = 0;
-    if (lane == 0) { __threadfence(); ended = atomicAdd(&job1.done[job1.heads], 1u); }
-    if (__shfl_sync(0xFFFFFFFFu, ended, 0) == gridDim.x - 1)
-      for (int i = lane; i < job1.heads + 2; i += 32) job1.done[i] = 0;
-  }
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
