@@ -197,19 +197,22 @@ EncodeTiledFn encode_tiled() {
   return fn;
 }
 
-// bf16 tensor [heads][rows][D] seen as (D, rows, heads); boxes of 64 columns x 128 rows, 128-byte swizzle,
+// bf16 tensor [heads][rows][D] seen as (D, rows, heads); boxes of 64 columns x `box_rows` rows, 128-byte swizzle,
 // rows past the end of a head read as zero.
-bool make_map(CUtensorMap* m, const void* base, int D, int rows, int heads) {
+bool make_map(CUtensorMap* m, const void* base, int D, int rows, int heads, int box_rows = 128) {
   EncodeTiledFn fn = encode_tiled();
   if (!fn) return false;
   const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)rows, (cuuint64_t)heads};
   const cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)rows * D * 2};
-  const cuuint32_t box[3] = {64, 128, 1};
+  const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+
+// Copies of the queries in sweep 1's 128-row operand (score_tc.cuh): as many as fit, up to four.
+int query_copies(int M) { return M <= 32 ? 4 : M <= 64 ? 2 : 1; }
 
 uint32_t make_idesc(int M, int N) {
   // fp32 accumulator, bf16 A and B, both K-major
@@ -230,7 +233,7 @@ bool make_job(dkv_ctx* c, int mode, int layer, int nl, const void* const* q, con
   const Shape& s = c->s;
   const int heads = s.Bt * s.Hkv;
   for (int i = 0; i < nl; ++i)
-    if (!make_map(&maps->q[i], q[i], s.D, s.M, heads) || !make_map(&maps->k[i], k[i], s.D, s.S, heads)) return false;
+    if (!make_map(&maps->q[i], q[i], s.D, s.M, heads, 128 / query_copies(s.M)) || !make_map(&maps->k[i], k[i], s.D, s.S, heads)) return false;
   for (int i = 0; i < nl; ++i) maps->lse[i] = lse ? lse[i] : nullptr;      // (entries past nl are never read)
   p->S = s.S; p->P = s.P; p->ws = s.ws; p->M = s.M; p->D = s.D; p->heads = nl * heads; p->half = s.pool / 2;
   p->nl = nl; p->hpl = heads;
@@ -257,22 +260,25 @@ bool make_job(dkv_ctx* c, int mode, int layer, int nl, const void* const* q, con
   return true;
 }
 
+// The scoring kernel for two jobs (either may be kNone) of the same shape: the specialised build for exactly 128 window rows
+// of 128 dims, builds with two or four copies of the queries for up to 64 or 32 window rows, the general one otherwise.
+template <int NL>
+auto score_kernel(int M, int D) {
+  return M == 128 && D == 128 ? tc::score_tc_kernel<NL, true, 1> : query_copies(M) == 4 ? tc::score_tc_kernel<NL, false, 4>
+       : query_copies(M) == 2 ? tc::score_tc_kernel<NL, false, 2> : tc::score_tc_kernel<NL, false, 1>;
+}
 cudaError_t set_score_attributes() {
-  for (const void* f : {(const void*)tc::score_tc_kernel<1, true>, (const void*)tc::score_tc_kernel<1, false>,
-                        (const void*)tc::score_tc_kernel<tc::kMaxGroup, true>, (const void*)tc::score_tc_kernel<tc::kMaxGroup, false>}) {
-    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes);
-    if (e != cudaSuccess) return e;
-  }
+  for (const int* s : (const int[][2]){{128, 128}, {32, 128}, {64, 128}, {256, 128}})
+    for (const void* f : {(const void*)score_kernel<1>(s[0], s[1]), (const void*)score_kernel<tc::kMaxGroup>(s[0], s[1])}) {
+      const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes);
+      if (e != cudaSuccess) return e;
+    }
   return cudaSuccess;
 }
-
-// The scoring kernel for two jobs (either may be kNone): the specialised build when every job has exactly 128 window
-// rows of 128 dims, the general one otherwise.
 template <int NL>
 cudaError_t launch_tc(int grid, cudaStream_t st, const tc::Maps<NL>& m0, const tc::Maps<NL>& m1, const tc::Params& j0, const tc::Params& j1) {
-  auto fast = [](const tc::Params& p) { return p.mode == tc::kNone || (p.M == 128 && p.D == 128); };
-  return launch_pdl(fast(j0) && fast(j1) ? tc::score_tc_kernel<NL, true> : tc::score_tc_kernel<NL, false>, dim3(grid), tc::kThreads,
-                    (size_t)tc::kSmemBytes, 1, st, m0, m1, j0, j1);
+  const tc::Params& j = j0.mode == tc::kNone ? j1 : j0;
+  return launch_pdl(score_kernel<NL>(j.M, j.D), dim3(grid), tc::kThreads, (size_t)tc::kSmemBytes, 1, st, m0, m1, j0, j1);
 }
 
 // Thread blocks of a scoring launch over `nl` layers: one an SM, fewer if there are fewer key tiles.
@@ -1058,7 +1064,7 @@ int dkv_score_static(const dkv_config* cfg, const void* q_win, const void* k, fl
   cudaStream_t st = as_stream(stream);
   tc::Maps<1> maps;
   maps.lse[0] = nullptr;
-  if (!make_map(&maps.q[0], q_win, D, M, heads) || !make_map(&maps.k[0], k, D, S, heads)) return DKV_ERR_CUDA;
+  if (!make_map(&maps.q[0], q_win, D, M, heads, 128 / query_copies(M)) || !make_map(&maps.k[0], k, D, S, heads)) return DKV_ERR_CUDA;
   if (cudaMemsetAsync(su.ptr, 0, 256, st) != cudaSuccess) return DKV_ERR_CUDA;   // status words start at zero
   tc::Params p, none;
   memset(&p, 0, sizeof p);

@@ -340,7 +340,10 @@ __host__ __device__ __forceinline__ int tile_owner(long long x, long long total,
 // job0 uses maps0, job1 uses maps1; a job with mode kNone is skipped.
 // kFast: both jobs have exactly 128 window rows of 128 dims (ws*G = 128, D = 128, the shape of the 32/8-head models):
 // the row-block count, the chunk count and the k-step count are then compile-time constants.
-template <int NL, bool kFast>
+// kCopies: with at most 128 / kCopies window rows (64 or 32) the queries lie kCopies times in the 128-row operand of sweep 1, and
+// every copy's tensor-memory lanes take a share of the keys: without that the lanes past the window rows spend as many
+// exponentials as the others.
+template <int NL, bool kFast, int kCopies>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ Maps<NL> maps1,
                 const __grid_constant__ Params job0, const __grid_constant__ Params job1) {
@@ -366,7 +369,8 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ 
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_flag = &abort_s;
-  auto NMBLK = [](const Params& p) { return kFast ? 1 : p.nmblk; };
+  constexpr int kRows = 128 / kCopies;                 // operand rows of one copy of the queries
+  auto NMBLK = [](const Params& p) { return kFast || kCopies > 1 ? 1 : p.nmblk; };
   auto DIMS = [](const Params& p) { return kFast ? 128 : p.D; };
 
   if (threadIdx.x == 0) {
@@ -418,8 +422,8 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ 
             if (ok) {
               mbar_expect_tx(QFULL, (uint32_t)(NMBLK(p) * halves) * kHalfBytes);
               for (int h = 0; h < halves; ++h)
-                for (int mb = 0; mb < NMBLK(p); ++mb)
-                  tma_load_3d(smem_u32(q_smem + h * (2 * kHalfBytes) + mb * kHalfBytes), q_map, QFULL, 64 * h, 128 * mb, hh);
+                for (int mb = 0; mb < NMBLK(p) * kCopies; ++mb)
+                  tma_load_3d(smem_u32(q_smem + h * (2 * kHalfBytes) + mb * kRows * 128), q_map, QFULL, 64 * h, kCopies > 1 ? 0 : 128 * mb, hh);
               ++nq;
             }
           }
@@ -554,6 +558,62 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ 
       while (it.next(sg)) {
         if (p.mode == kStats) {
           // ------------------------------------------------------------ sweep 1: (max, sum) per window row
+          if constexpr (kCopies > 1) {
+            constexpr int kCols = 64 / kCopies;                      // keys of a tile this warp takes
+            const int lrow = row & (kRows - 1), limit = p.P + lrow % p.ws, col = half * 64 + (row / kRows) * kCols;
+            float mx = -INFINITY, sum = 0.f;
+            const int tile0 = tile;
+            tile += sg.ntiles;
+            for (int i = (grp ^ tile0) & 1, tile_ = tile0 + i; i < sg.ntiles; i += 2, tile_ += 2) {
+              const int t = tile_ & 3, kb = sg.key0 + i * kTileKeys + col;
+              mbar_wait(TFULL(t), (tile_ >> 2) & 1, abort_flag, p.status, 106, p.wait_cycles);
+              tc_fence_after();
+              float xv[kCols];
+              if constexpr (kCols == 32) tc_ld32(lane_addr + (uint32_t)(t * 128 + col), xv); else tc_ld16(lane_addr + (uint32_t)(t * 128 + col), xv);
+              tc_wait_ld();
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(TEMPTY(t));
+              if (kb + kCols - 1 > p.P) {
+#pragma unroll
+                for (int e = 0; e < kCols; ++e) if (kb + e > limit) xv[e] = -INFINITY;
+              }
+              float cm = xv[0];
+#pragma unroll
+              for (int e = 1; e + 1 < kCols; e += 2) cm = fmax3(cm, xv[e], xv[e + 1]);
+              cm = fmaxf(cm, xv[kCols - 1]);
+              if (cm == -INFINITY) continue;
+              const float mnew = fmaxf(mx, cm * p.scale2);
+              if (mnew > mx) { sum *= fast_exp2(mx - mnew); mx = mnew; }
+              uint64_t s01 = 0ull, s23 = 0ull;
+              const uint64_t neg2 = pack2(-mx, -mx);
+#pragma unroll
+              for (int e = 0; e < kCols; e += 4) {
+                s01 = exp2_acc2(poly_pair(e / 2), s01, xv[e], xv[e + 1], scale22, neg2);
+                s23 = exp2_acc2(poly_pair(e / 2 + 1), s23, xv[e + 2], xv[e + 3], scale22, neg2);
+              }
+              float s0, s1, s2, s3;
+              unpack2(s01, s0, s1); unpack2(s23, s2, s3);
+              sum += (s0 + s1) + (s2 + s3);
+            }
+            // merge the column parts (4 warps x kCopies) and publish this CTA's statistics for the head
+            merge_s[part * 128 + row] = make_float2(mx, sum);
+            asm volatile("bar.sync 1, 512;" ::: "memory");
+            if (sid < p.M) {
+              const long long total = (long long)p.heads * p.tph;
+              const int slot = blockIdx.x - tile_owner((long long)sg.bh * p.tph, total, gridDim.x);
+              float m = -INFINITY, l = 0.f;
+#pragma unroll
+              for (int q = 0; q < 4 * kCopies; ++q) m = fmaxf(m, merge_s[q * kRows + sid].x);
+              if (m > -INFINITY) {
+#pragma unroll
+                for (int q = 0; q < 4 * kCopies; ++q) { const float2 o = merge_s[q * kRows + sid]; l += o.y * fast_exp2(o.x - m); }
+              }
+              p.stats[((size_t)sg.bh * p.slots + slot) * p.m_stride + sid] = make_float2(m, l);
+            }
+            asm volatile("bar.sync 1, 512;" ::: "memory");
+            continue;
+          }
           float mx[2] = {-INFINITY, -INFINITY}, sum[2] = {0.f, 0.f};
           const int limit0 = p.P + (row % p.ws), limit1 = p.P + ((row + 128) % p.ws);
           // this thread's tiles only: every other one, by the parity of the tile's number over the launch
