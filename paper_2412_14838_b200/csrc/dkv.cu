@@ -341,10 +341,12 @@ int do_select(dkv_ctx* c, int layer, int* sorted_out, int* rank_out, cudaStream_
     ProfScope ps(c, DKV_STEP_SELECT, 1, st);
     unsigned int* lh = c->d_layer_hist + (size_t)layer * s.Bt * kBins;
     DKV_CUDA(c, cudaMemsetAsync(lh, 0, sizeof(unsigned int) * s.Bt * kBins, st));
-    // a cluster a head while the heads leave SMs idle and a block's share is a few thousand positions at least
+    // A cluster a head from the length where its exchanges (about 2 us) cost less than the passes over the scores that it
+    // saves, while the heads leave half of the SMs idle: 4 blocks from 8192 positions, 8 from 24576 (a call, heads of
+    // 6300/10000/16352/32736 scores, 1 block: 12.3/14.3/16.4/22.6 us; 4: 12.3/12.3/14.3/14.4; 8 with 8 heads: 32736: 14.3;
+    // 8 with 18 heads: 17 to 18 at any length; 2 never pays).
     const int heads = s.Bt * s.Hkv;
-    int parts = 1;
-    while (parts < 8 && heads * parts * 2 <= c->n_sms && s.P > parts * 2 * kSelThreads) parts *= 2;
+    const int parts = s.P >= 24576 && heads * 16 <= c->n_sms ? 8 : s.P >= 8192 && heads * 8 <= c->n_sms ? 4 : 1;
     DKV_LAUNCH(c, launch_pdl(parts > 1 ? select_topk_kernel<true> : select_topk_kernel<false>, dim3(heads * parts), kSelThreads, select_smem(c->sel_cap),
                              parts, st, (const float*)(c->d_scores + (size_t)layer * layer_scores(s)), c->d_idx + (size_t)layer * layer_idx(s), lh, s.P,
                              s.Blc, c->sel_cap, c->d_count, s.Hkv, s.L, layer, parts));

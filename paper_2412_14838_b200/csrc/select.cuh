@@ -352,8 +352,8 @@ __device__ __forceinline__ int* select_head(const uint32_t* __restrict__ v, int 
 }
 
 // dkv_select_topk: the `keep` best of every head of one layer.  idx: [Bt*Hkv][keep], in order.  Adds the heads' digit
-// counts to layer_hist [Bt][2048] and records count[b][layer] = keep.  One block a head, or a cluster of `parts` blocks while
-// the heads leave SMs idle (8 heads of 16352: 14.8 -> 13 us).  grid Bt*Hkv*parts.
+// counts to layer_hist [Bt][2048] and records count[b][layer] = keep.  One block a head, or a cluster of `parts` blocks (the
+// launch says when).  grid Bt*Hkv*parts.
 template <bool kShared>
 __global__ void __launch_bounds__(kSelThreads, 2)
 select_topk_kernel(const float* __restrict__ scores, int* __restrict__ idx, unsigned int* __restrict__ layer_hist, int P,
