@@ -304,6 +304,7 @@ int launch_score(dkv_ctx* c, const ScoreGroup* e, ScoreGroup* s, const void* con
   if (s) s->grid = grid;
   if (e && !make_job(c, tc::kEmit, e->first, e->n, q + e->first, k + e->first, scores_out, e->buf, grid, e->grid, hist, &m0, &j0, lse ? lse + e->first : nullptr)) return DKV_ERR_CUDA;
   if (s && !make_job(c, tc::kStats, s->first, s->n, q + s->first, k + s->first, nullptr, s->buf, grid, grid, hist, &m1, &j1)) return DKV_ERR_CUDA;
+  j0.inputs_ready = e && !lse;               // sweep 1 of group `e` was in the launch before
   ProfScope ps(c, s ? DKV_STEP_SCORE_STATS : DKV_STEP_SCORE_EMIT, 1, st);
   DKV_LAUNCH(c, launch_tc(grid, st, e ? m0 : m1, s ? m1 : m0, j0, j1));
   return DKV_OK;

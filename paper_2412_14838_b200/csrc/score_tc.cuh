@@ -70,6 +70,7 @@ struct Params {
   long long wait_cycles;   // limit of every mbarrier wait, in clock64 ticks
   int retain_tiles;        // sweep 1: the last `retain_tiles` key tiles of a CTA's slice are kept in L2 for sweep 2, which starts
                            // with them; every other key tile of either sweep is marked to be evicted first (0: no marking)
+  int inputs_ready;        // first job: the launch before this one was a scoring launch that has waited for the inputs
   int withhold_tile;       // test hook: CTA 0 never loads its key tile number `withhold_tile` of this job (-1: off),
                            // so that the wait for it runs out and the timeout path can be exercised
 };
@@ -390,8 +391,16 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
-  pdl_launch();
-  pdl_wait();
+  // The launch before this one may have been sweep 1 over the same queries and keys (inputs_ready).  A launch that waits for
+  // its inputs lets the next one start only after that, so they are there: copies and MMAs begin at once, and only the
+  // warps that read sweep 1's statistics wait for its end (8 layers of 1K: 43.2 -> 41.0 us).
+  if (job0.inputs_ready) {
+    pdl_launch();
+    if (warp != 0 && warp != 1 && warp != kMmaWarp2) pdl_wait();
+  } else {
+    pdl_wait();
+    pdl_launch();
+  }
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
