@@ -1,0 +1,81 @@
+"""The sizes at which the launches of a selection, the budget updates and the host-buffer pass change their form."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import dynamickv as O
+from paper_2412_14838_b200 import binding as B
+from paper_2412_14838_b200 import build, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    B.load()
+
+
+# one block a head below 8192 positions or above 18 heads, four to 24575 positions or from 10 to 18 heads, else eight;
+# "same": more equal scores than the list holds
+@pytest.mark.parametrize("P,Hkv,Bl,kind", [(8191, 2, 100, "ties"), (8192, 1, 1, "ties"), (8193, 18, 333, "ties"), (8200, 19, 64, "ties"),
+                                           (24575, 3, 700, "ties"), (24576, 9, 64, "ties"), (24577, 10, 64, "ties"), (24609, 2, 4096, "ties"),
+                                           (9001, 2, 500, "same"), (30011, 1, 500, "same")])
+def test_select_of_one_layer(P, Hkv, Bl, kind):
+    w = synth.Workload("sel", 41, L=1, Hq=Hkv, Hkv=Hkv, D=64, Bt=1, S=P + 8, ws=8, pool=7, N=Bl, Bl=Bl, m=1, recipe="iid")
+    sc = synth.pooled_like_scores((1, Hkv, P), 7, seed=P, tie_fraction=0.2)
+    if kind == "same":
+        sc[...] = 0.25
+        sc[:, :, P - 100:P - 90] = 0.5
+    h = B.dkv_create(B.config_of(w))
+    try:
+        B.dkv_set_scores(h, 0, torch.from_numpy(sc).cuda())
+        idx = torch.empty((1, Hkv, w.Blc), dtype=torch.int32, device="cuda")
+        rank = torch.empty_like(idx)
+        B.dkv_select_topk(h, 0, idx, rank)
+        idx, rank = idx.cpu().numpy(), rank.cpu().numpy()
+    finally:
+        B.dkv_destroy(h)
+    for head in range(Hkv):
+        ref = O.select_topk(sc[0, head].astype(np.float64), Bl)
+        assert (idx[0, head] == ref["idx"]).all() and (rank[0, head] == ref["rank"]).all(), f"head {head}"
+
+
+@pytest.mark.parametrize("L,m", [(7, 1), (8, 1), (9, 1), (17, 2)])       # the updates of a pass run up to eight at a time
+def test_updates_of_a_pass_and_pageable_results(L, m):
+    w = synth.Workload("upd", 42, L=L, Hq=4, Hkv=2, D=64, Bt=2, S=333, ws=9, pool=3, N=20, Bl=60, m=m, recipe="sink")
+    bits = [{n: np.ascontiguousarray(a).view(np.int16) for n, a in synth.layer_inputs(w, l).items()} for l in range(L)]
+    q, k, v = ([torch.from_numpy(t[n]).cuda() for t in bits] for n in "qkv")
+    shape = (w.Bt, w.Hkv, w.Blc + w.ws, w.D)
+    kb, vb = ([torch.zeros(shape, dtype=torch.int16, device="cuda") for _ in range(L)] for _ in range(2))
+    h = B.dkv_create(B.config_of(w))
+    try:
+        B.dkv_run_prefill_pass(h, q, k, v, kb, vb)
+        torch.cuda.synchronize()
+        counts = np.zeros((w.Bt, L), dtype=np.int32)
+        B.dkv_get_counts(h, counts)
+        hist = []
+        for l in range(L):
+            sc = np.empty((w.Bt, w.Hkv, w.P), dtype=np.float32)
+            B.dkv_memcpy_to_host(h, sc, B.dkv_layer_views(h, l)[0], sc.nbytes)
+            hist.append(sc)
+        for b in range(w.Bt):
+            ref = np.full(L, w.Blc, dtype=np.int64)
+            for l in [n for n in range(1, L + 1) if n % m == 0 or n == L]:
+                ref = np.asarray(O.rebudget([hist[i][b].astype(np.float64) for i in range(l)], ref, w.N, w.Bl, L)["counts"])
+            assert counts[b].tolist() == ref.tolist()
+        out = [[np.zeros(shape, dtype=np.int16) for _ in range(L)] for _ in range(2)]        # not page-locked
+        again = np.zeros_like(counts)
+        B.dkv_run_prefill_pass_host(h, *([torch.from_numpy(t[n]) for t in bits] for n in "qkv"), out[0], out[1], again)
+        # single-layer launches cut the keys differently: scores differ in the last bits, so a row at a cut may differ
+        near = np.abs(again.astype(int) - counts).max()
+        assert near <= 1
+        for l in range(L):
+            for b in range(w.Bt):
+                n, p = int(min(counts[b, l], again[b, l])), int(again[b, l])
+                for got, want, src in ((out[0], kb, "k"), (out[1], vb, "v")):
+                    same = (got[l][b, :, :n] == want[l][b, :, :n].cpu().numpy()).all(axis=-1)
+                    assert same.mean() >= 0.98
+                    assert (got[l][b, :, p:p + w.ws] == bits[l][src][b, :, w.P:]).all()
+    finally:
+        B.dkv_destroy(h)
