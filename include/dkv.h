@@ -179,11 +179,10 @@ int dkv_compact_all(dkv_ctx* ctx, int32_t upto_layer, void* const* kb, void* con
  * after the last one if L % m != 0) rebudget and shrink all preceding layers.  Resets the context first.
  * q_win, k, v, kb, vb : HOST arrays of L device pointers (layouts as above).
  * All layers' tensors must be resident when the call is made: the scoring kernel is launched once per group of
- * consecutive layers (sweep 2 of one group, sweep 1 of the next), the steps that consume a layer's scores run
- * beside the following groups' scoring.  The results are those of the layer-by-layer loop.
- * The first call with a given set of pointers records the whole pass as a CUDA graph (on an internal stream
- * that forks from `stream` and rejoins it); later calls with the same pointers replay it, whatever the
- * buffers then contain.  The plain sequence of launches is used instead while dkv_profile is on, when
+ * consecutive layers (sweep 2 of one group, sweep 1 of the next); then all updates run together and every layer is
+ * selected and gathered once, with its final count.  The results are those of the layer-by-layer loop.
+ * The first call with a given set of pointers records the whole pass as a CUDA graph (on an internal stream);
+ * later calls with the same pointers replay it on `stream`, whatever the buffers then contain.  The plain sequence of launches is used instead while dkv_profile is on, when
  * `stream` is itself being captured, or if the capture fails. */
 int dkv_run_prefill_pass(dkv_ctx* ctx, const void* const* q_win, const void* const* k, const void* const* v,
                          void* const* kb, void* const* vb, void* stream);
@@ -203,7 +202,8 @@ int dkv_run_prefill_pass_lse(dkv_ctx* ctx, const void* const* q_win, const void*
  * kernels can address (cudaHostAlloc / cudaHostRegister) the gather reads those rows in place and the
  * rest of v never crosses the bus; pageable v is copied in full like k.  After the last update
  * the counts and, of every layer's kb/vb, the valid rows of every head (count + ws; the rest of the
- * fixed-stride host buffers is left untouched) are copied back.  Synchronises.
+ * fixed-stride host buffers is left untouched) are copied back: by one kernel that writes them in place where every
+ * kb[l] and vb[l] is page-locked and 16-byte aligned, else by strided copies.  Synchronises.
  * q_win, k, v, kb, vb : host arrays of L HOST pointers; counts_out : host int32 [Bt, L]. */
 int dkv_run_prefill_pass_host(dkv_ctx* ctx, const void* const* q_win, const void* const* k,
                               const void* const* v, void* const* kb, void* const* vb, int32_t* counts_out);

@@ -26,7 +26,7 @@ struct dkv_ctx {
   int device;
   // device state
   float* d_scores;      // [L][Bt][Hkv][P]  pooled scores, the history A^b
-  int* d_idx;           // [L][Bt][Hkv][Blc] kept positions, ascending
+  int* d_idx;           // [L][Bt][Hkv][Blc] kept positions, in buffer order
   int* d_count;         // [Bt][L] budget of each layer
   int* d_held;          // [Bt][L] rows the layer's buffers hold
   int* d_dbg;           // 3 x [Bt][L] : cnt, Z, Z' of the last update
@@ -640,8 +640,8 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
     c->pass_group = env_int("DKV_PASS_GROUP", (s.L + launches - 1) / launches, 1, tc::kMaxGroup);
     c->emit_backward = env_int("DKV_EMIT_FORWARD", 0, 0, 1) == 0;
     // Sweep 2 starts on the keys sweep 1 streamed last: that much of a job (4/7 of L2, 72 of 126 MB) is loaded with
-    // an evict-last policy, every other key tile and the gather's rows evict-first, so that neither the rest of the
-    // stream nor the side kernels' traffic pushes it out before it is read again.
+    // an evict-last policy, every other key tile and the gather's rows evict-first, so that the rest of the
+    // stream does not push it out before it is read again.
     int l2_bytes = 0;
     if (cudaDeviceGetAttribute(&l2_bytes, cudaDevAttrL2CacheSize, c->device) != cudaSuccess) l2_bytes = 0;
     c->retain_mb = c->emit_backward ? env_int("DKV_L2_RETAIN_MB", (int)(((long long)l2_bytes * 4 / 7) >> 20), 0, 1024) : 0;

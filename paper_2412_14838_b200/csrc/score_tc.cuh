@@ -14,7 +14,7 @@
 // Work is split evenly: the flattened (head, key tile) space for sweep 1 and the flattened
 // (head, prefix position) space for sweep 2 are cut into one contiguous slice per CTA.
 // One launch runs up to two jobs back to back through the same pipeline (sweep 2 of one layer, then
-// sweep 1 of the next), so the fixed cost of a launch is paid once per layer.
+// sweep 1 of the next; a job covers a group of layers), so the fixed cost of a launch is paid once per group.
 #pragma once
 #include <cuda.h>
 #include "common.cuh"
@@ -343,7 +343,7 @@ __host__ __device__ __forceinline__ int tile_owner(long long x, long long total,
 // the row-block count, the chunk count and the k-step count are then compile-time constants.
 // kCopies: with at most 128 / kCopies window rows (64 or 32) the queries lie kCopies times in the 128-row operand of sweep 1, and
 // every copy's tensor-memory lanes take a share of the keys: without that the lanes past the window rows spend as many
-// exponentials as the others.
+// exponentials as the others (a pass of four layers of 1K with 64 window rows: 45.1 -> 43.2 us).
 template <int NL, bool kFast, int kCopies>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ Maps<NL> maps1,
@@ -393,7 +393,7 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ 
   const uint32_t tmem_base = tmem_base_s;
   // The launch before this one may have been sweep 1 over the same queries and keys (inputs_ready).  A launch that waits for
   // its inputs lets the next one start only after that, so they are there: copies and MMAs begin at once, and only the
-  // warps that read sweep 1's statistics wait for its end (8 layers of 1K: 43.2 -> 41.0 us).
+  // warps that read sweep 1's statistics wait for its end (a pass of four layers of 1K: 43.1 -> 41.0 us).
   if (job0.inputs_ready) {
     pdl_launch();
     if (warp != 0 && warp != 1 && warp != kMmaWarp2) pdl_wait();
