@@ -417,8 +417,15 @@ int do_select_gather(dkv_ctx* c, const void* const* k, const void* const* v, voi
   PassPtrs ptrs;
   for (int l = 0; l < s.L; ++l) { ptrs.k[l] = k[l]; ptrs.v[l] = v[l]; ptrs.kb[l] = kb[l]; ptrs.vb[l] = vb[l]; }
   ProfScope ps(c, DKV_STEP_SELECT, 1, st);
-  DKV_LAUNCH(c, launch_pdl(select_gather_kernel, dim3(s.Bt * s.Hkv, s.L), kSelThreads, select_smem(c->sel_cap), 1, st, ptrs, (const float*)c->d_scores,
-                           c->d_idx, (const int*)c->d_count, c->d_held, s.P, s.ws, s.Blc, c->sel_cap, s.S, s.D * 2 / 16, s.Hkv, s.L));
+  // A cluster a head, as in do_select, while all blocks fit on the SMs at once, two to each: the blocks share the copying
+  // too.  Per pass with 1 / 4 / 8 blocks a head: 8 heads of 8160 58 / 51 / 51 us, of 32736 99 / 76 / 71; 32 heads 74 / 71 / 72 and
+  // 165 / 154 / 146; 64 heads 101 / 99 / 102 and 269 / 261 / 274; 8 to 64 heads of 4000: 47 to 69, the same with 4, slower with 8;
+  // 112 heads and more, which need two waves: slower.
+  const int heads = s.Bt * s.Hkv * s.L;
+  const int parts = s.P >= 24576 && heads * 4 <= c->n_sms ? 8 : s.P >= 6144 && heads * 2 <= c->n_sms ? 4 : 1;
+  DKV_LAUNCH(c, launch_pdl(parts > 1 ? select_gather_kernel<true> : select_gather_kernel<false>, dim3(s.Bt * s.Hkv * parts, s.L), kSelThreads,
+                           select_smem(c->sel_cap), parts, st, ptrs, (const float*)c->d_scores,
+                           c->d_idx, (const int*)c->d_count, c->d_held, s.P, s.ws, s.Blc, c->sel_cap, s.S, s.D * 2 / 16, s.Hkv, s.L, parts));
   return DKV_OK;
 }
 
@@ -681,7 +688,8 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
     const int most = (int)(select_smem(kMaxCountingList) > select_smem(DKV_MAX_LAYER_BUDGET) ? select_smem(kMaxCountingList) : select_smem(DKV_MAX_LAYER_BUDGET));
     TRY(cudaFuncSetAttribute(select_topk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     TRY(cudaFuncSetAttribute(select_topk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    TRY(cudaFuncSetAttribute(select_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRY(cudaFuncSetAttribute(select_gather_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRY(cudaFuncSetAttribute(select_gather_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     TRY(cudaFuncSetAttribute(sort_positions_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DKV_MAX_LAYER_BUDGET * 8));
   }
 #undef TRY

@@ -79,3 +79,33 @@ def test_updates_of_a_pass_and_pageable_results(L, m):
                     assert (got[l][b, :, p:p + w.ws] == bits[l][src][b, :, w.P:]).all()
     finally:
         B.dkv_destroy(h)
+
+
+# one block a head below 6144 positions or above 74 heads, four to 24575 positions or from 38 heads, else eight
+@pytest.mark.parametrize("P,L,Hkv,Bl", [(6143, 2, 3, 90), (6144, 2, 3, 90), (6177, 74, 1, 33), (6145, 25, 3, 33), (24575, 2, 2, 700), (24577, 37, 1, 40),
+                                        (24576, 19, 2, 40), (24601, 2, 1, 5000)])
+def test_select_and_gather_of_a_pass(P, L, Hkv, Bl):
+    w = synth.Workload("sg", 43, L=L, Hq=Hkv, Hkv=Hkv, D=64, Bt=1, S=P + 7, ws=7, pool=3, N=max(1, Bl // 2), Bl=Bl, m=4, recipe="iid")
+    g = torch.Generator(device="cuda").manual_seed(P)
+    rand = lambda heads, rows: [torch.randn((1, heads, rows, w.D), generator=g, device="cuda", dtype=torch.bfloat16) for _ in range(L)]
+    q, k, v = rand(w.Hq, w.ws), rand(Hkv, w.S), rand(Hkv, w.S)
+    k[0][:, 0, :P] = 0                                       # a head of equal scores
+    kb, vb = ([torch.zeros((1, Hkv, w.Blc + w.ws, w.D), dtype=torch.bfloat16, device="cuda") for _ in range(L)] for _ in range(2))
+    h = B.dkv_create(B.config_of(w))
+    try:
+        B.dkv_run_prefill_pass(h, q, k, v, kb, vb)
+        torch.cuda.synchronize()
+        counts = np.zeros((1, L), dtype=np.int32)
+        B.dkv_get_counts(h, counts)
+        for l in range(L):
+            n, sc = int(counts[0, l]), np.empty((Hkv, P), dtype=np.float32)
+            scores, idx = B.dkv_layer_views(h, l)
+            B.dkv_memcpy_to_host(h, sc, scores, sc.nbytes)
+            kept = B.read_device_i32(h, idx, (Hkv, w.Blc))[:, :n]
+            want = np.argsort(-sc, axis=1, kind="stable")[:, :n]
+            assert (kept == want).all(), f"layer {l}"
+            rows = torch.from_numpy(np.concatenate([want, np.tile(np.arange(P, w.S), (Hkv, 1))], axis=1)).cuda()
+            for src, buf in ((k, kb), (v, vb)):
+                assert torch.equal(buf[l][0, :, :n + w.ws], torch.gather(src[l][0], 1, rows[:, :, None].expand(-1, -1, w.D)))
+    finally:
+        B.dkv_destroy(h)
