@@ -418,14 +418,15 @@ int do_select_gather(dkv_ctx* c, const void* const* k, const void* const* v, voi
   for (int l = 0; l < s.L; ++l) { ptrs.k[l] = k[l]; ptrs.v[l] = v[l]; ptrs.kb[l] = kb[l]; ptrs.vb[l] = vb[l]; }
   ProfScope ps(c, DKV_STEP_SELECT, 1, st);
   // A cluster a head, as in do_select, while all blocks fit on the SMs at once, two to each: the blocks share the copying
-  // too.  Per pass with 1 / 4 / 8 blocks a head: 8 heads of 8160 58 / 51 / 51 us, of 32736 99 / 76 / 71; 32 heads 74 / 71 / 72 and
-  // 165 / 154 / 146; 64 heads 101 / 99 / 102 and 269 / 261 / 274; 8 to 64 heads of 4000: 47 to 69, the same with 4, slower with 8;
-  // 112 heads and more, which need two waves: slower.
+  // too, so that the line depends on the rows to copy as well (one costs about as much as 16 positions).  Per pass with
+  // 1 / 4 / 8 blocks a head and B^l = 128 | 1024: 8 heads of 6144 47 / 49 / 49 | 57 / 51 / 50 us, of 16352 55 / 54 / 55 | 67 / 58 / 57,
+  // of 32736 72 / 66 / 65 | 83 / 70 / 67; 32 heads of 16352 90 / 91 / 92 | 102 / 97 / 95; 64 heads of 6144 75 / 79 / 86 | 88 / 85 / 100, of
+  // 32736 234 / 233 / 264 | 248 / 237 / 260; 112 heads need two waves: slower.
   const int heads = s.Bt * s.Hkv * s.L;
-  const int parts = s.P >= 24576 && heads * 4 <= c->n_sms ? 8 : s.P >= 6144 && heads * 2 <= c->n_sms ? 4 : 1;
-  DKV_LAUNCH(c, launch_pdl(parts > 1 ? select_gather_kernel<true> : select_gather_kernel<false>, dim3(s.Bt * s.Hkv * parts, s.L), kSelThreads,
+  const int parts = s.P >= 24576 && heads * 4 <= c->n_sms ? 8 : s.P + 16 * s.Blc >= 20480 && heads * 2 <= c->n_sms ? 4 : 1;
+  DKV_LAUNCH(c, launch_pdl(parts > 1 ? select_gather_cluster_kernel : select_gather_kernel, dim3(s.Bt * s.Hkv * parts, s.L), kSelThreads,
                            select_smem(c->sel_cap), parts, st, ptrs, (const float*)c->d_scores,
-                           c->d_idx, (const int*)c->d_count, c->d_held, s.P, s.ws, s.Blc, c->sel_cap, s.S, s.D * 2 / 16, s.Hkv, s.L, parts));
+                           c->d_idx, (const int*)c->d_count, c->d_held, s.P, s.ws, s.Blc, c->sel_cap, s.S, s.D * 2 / 16, s.Hkv, s.L));
   return DKV_OK;
 }
 
@@ -688,8 +689,8 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
     const int most = (int)(select_smem(kMaxCountingList) > select_smem(DKV_MAX_LAYER_BUDGET) ? select_smem(kMaxCountingList) : select_smem(DKV_MAX_LAYER_BUDGET));
     TRY(cudaFuncSetAttribute(select_topk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     TRY(cudaFuncSetAttribute(select_topk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    TRY(cudaFuncSetAttribute(select_gather_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    TRY(cudaFuncSetAttribute(select_gather_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRY(cudaFuncSetAttribute(select_gather_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    TRY(cudaFuncSetAttribute(select_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     TRY(cudaFuncSetAttribute(sort_positions_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DKV_MAX_LAYER_BUDGET * 8));
   }
 #undef TRY

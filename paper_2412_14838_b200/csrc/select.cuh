@@ -373,32 +373,50 @@ select_topk_kernel(const float* __restrict__ scores, int* __restrict__ idx, unsi
 // the ws window rows of K and V into the layer's buffers.  Selecting and copying the final rows once replaces a
 // selection and copy of B^l rows per layer and a truncation per update: 32K prompt with B^l = 4 N: 71 MB of rows read
 // instead of 272, and no block of the scoring kernel gives way to it while keys are streamed.
-// One block a head, or a cluster of `parts` blocks, which share the selection and the copying.  grid (Bt*Hkv*parts, layers).
-template <bool kShared>
+// grid (Bt*Hkv, layers).
 __global__ void __launch_bounds__(kSelThreads, 2)
 select_gather_kernel(const __grid_constant__ PassPtrs ptrs, const float* __restrict__ scores, int* __restrict__ idx,
-                     const int* __restrict__ count, int* __restrict__ held, int P, int ws, int stride, int cap, int S, int vec, int Hkv, int L,
-                     int parts) {
+                     const int* __restrict__ count, int* __restrict__ held, int P, int ws, int stride, int cap, int S, int vec, int Hkv, int L) {
   extern __shared__ __align__(16) unsigned char dyn[];
-  const int bh = kShared ? blockIdx.x / parts : blockIdx.x, part = kShared ? blockIdx.x % parts : 0, heads = kShared ? gridDim.x / parts : gridDim.x;
+  const int bh = blockIdx.x, b = bh / Hkv, layer = blockIdx.y, tid = threadIdx.x;
+  const size_t head = (size_t)layer * gridDim.x + bh;
+  pdl_launch();
+  pdl_wait();
+  const int n = count[b * L + layer];
+  if (tid == 0 && bh % Hkv == 0) held[b * L + layer] = n;
+  const int* sel = nullptr;
+  if (n > 0) {
+    sel = select_head<false>(reinterpret_cast<const uint32_t*>(scores) + head * P, P, n, cap, dyn, nullptr, 0, 1);
+    for (int i = tid; i < n; i += kSelThreads) idx[head * stride + i] = sel[i];
+  }
+  gather_rows(static_cast<const uint4*>(ptrs.k[layer]), static_cast<const uint4*>(ptrs.v[layer]), static_cast<uint4*>(ptrs.kb[layer]),
+              static_cast<uint4*>(ptrs.vb[layer]), sel, n, bh, S, P, ws, stride + ws, vec, tid, kSelThreads, 0, 1);
+}
+
+// The same with a cluster a head, whose blocks share the selection and the copying.  grid (Bt*Hkv*cluster size, layers).
+__global__ void __launch_bounds__(kSelThreads, 2)
+select_gather_cluster_kernel(const __grid_constant__ PassPtrs ptrs, const float* __restrict__ scores, int* __restrict__ idx,
+                             const int* __restrict__ count, int* __restrict__ held, int P, int ws, int stride, int cap, int S, int vec, int Hkv,
+                             int L) {
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) unsigned char dyn[];
+  const int parts = cg::this_cluster().num_blocks(), part = blockIdx.x % parts, bh = blockIdx.x / parts;
   const int b = bh / Hkv, layer = blockIdx.y, tid = threadIdx.x;
-  const size_t head = (size_t)layer * heads + bh;
+  const size_t head = (size_t)layer * (gridDim.x / parts) + bh;
   pdl_launch();
   pdl_wait();
   const int n = count[b * L + layer];
   if (tid == 0 && part == 0 && bh % Hkv == 0) held[b * L + layer] = n;
   const int* sel = nullptr;
   if (n > 0) {
-    sel = select_head<kShared>(reinterpret_cast<const uint32_t*>(scores) + head * P, P, n, cap, dyn, nullptr, part, parts);
-    if constexpr (kShared) {                               // every block copies from the first one's list (it starts `dyn`)
-      cooperative_groups::this_cluster().sync();
-      sel = cooperative_groups::this_cluster().map_shared_rank(reinterpret_cast<int*>(dyn), 0);
-    }
+    select_head<true>(reinterpret_cast<const uint32_t*>(scores) + head * P, P, n, cap, dyn, nullptr, part, parts);
+    cg::this_cluster().sync();                             // the first block's list (at the start of `dyn`) is complete
+    sel = cg::this_cluster().map_shared_rank(reinterpret_cast<int*>(dyn), 0);
     for (int i = part * kSelThreads + tid; i < n; i += parts * kSelThreads) idx[head * stride + i] = sel[i];
   }
   gather_rows(static_cast<const uint4*>(ptrs.k[layer]), static_cast<const uint4*>(ptrs.v[layer]), static_cast<uint4*>(ptrs.kb[layer]),
               static_cast<uint4*>(ptrs.vb[layer]), sel, n, bh, S, P, ws, stride + ws, vec, tid, kSelThreads, part, parts);
-  if constexpr (kShared) cooperative_groups::this_cluster().sync();      // the list is read until here
+  cg::this_cluster().sync();                               // the list is read until here
 }
 
 // The positions idx[b,h,0..n) of one layer ascending (sorted_out) and the place each had in idx (rank_out), either

@@ -81,9 +81,10 @@ def test_updates_of_a_pass_and_pageable_results(L, m):
         B.dkv_destroy(h)
 
 
-# one block a head below 6144 positions or above 74 heads, four to 24575 positions or from 38 heads, else eight
-@pytest.mark.parametrize("P,L,Hkv,Bl", [(6143, 2, 3, 90), (6144, 2, 3, 90), (6177, 74, 1, 33), (6145, 25, 3, 33), (24575, 2, 2, 700), (24577, 37, 1, 40),
-                                        (24576, 19, 2, 40), (24601, 2, 1, 5000)])
+# one block a head where positions + 16 rows are below 20480 or heads are more than 74, else four, or eight from 24576
+# positions with up to 37 heads
+@pytest.mark.parametrize("P,L,Hkv,Bl", [(19583, 2, 3, 56), (19584, 2, 3, 56), (6177, 2, 2, 1001), (19951, 74, 1, 33), (19953, 25, 3, 33), (24575, 2, 2, 700),
+                                        (24577, 37, 1, 40), (24576, 19, 2, 40), (24601, 2, 1, 5000)])
 def test_select_and_gather_of_a_pass(P, L, Hkv, Bl):
     w = synth.Workload("sg", 43, L=L, Hq=Hkv, Hkv=Hkv, D=64, Bt=1, S=P + 7, ws=7, pool=3, N=max(1, Bl // 2), Bl=Bl, m=4, recipe="iid")
     g = torch.Generator(device="cuda").manual_seed(P)
