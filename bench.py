@@ -313,8 +313,8 @@ def run_gpu(args, w):
                 "launches_per_pass": score_launches, "scoring_ms_per_layer": score_ms / w.L,
                 "traffic": (ncu_traffic(w, score_launches) or {}).get("live_bytes_per_launch"),
                 "traffic_cold_cache": (ncu_traffic(w, score_launches) or {}).get("cold_bytes_per_launch"),
-                "traffic_note": "DRAM bytes of a full launch (sweep 2 of 4 layers + sweep 1 of the next 4); the first "
-                                "and last launch of a pass run one sweep only, so avg launches carry 8/9 of that",
+                "traffic_note": "DRAM bytes of a full launch (sweep 2 of a group of layers + sweep 1 of the next), null "
+                                "where no capture of this kernel source and grouping exists",
                 "whole_pass": {"algorithmic_bytes": w.algorithmic_bytes(),
                                "achieved_gbs": w.algorithmic_bytes() / (ms_per_step * 1e-3) / 1e9,
                                "frac_of_measured_peak": w.algorithmic_bytes() / (ms_per_step * 1e-3) / 1e9 / peak,
