@@ -393,7 +393,9 @@ decode_split_kernel(const __grid_constant__ DecodePtrs ptrs, const __grid_consta
     if (i0 < i1 && i1 == pairs) prefix_s[pairs] = at;
     __syncthreads();
   }
-  const int total = prefix_s[pairs], slices = gridDim.x * NW, own = blockIdx.x * NW + warp;
+  // no more slices than units: an empty slice would leave no part, and whoever merges a head counts on one from each
+  const int total = prefix_s[pairs], slices = min((int)gridDim.x * NW, total), own = blockIdx.x * NW + warp;
+  if (own >= slices) return;
   auto slice = [&](int c) { return (int)((long long)total * c / slices); };
   auto owner = [&](int u) { return (int)(((long long)(u + 1) * slices + total - 1) / total) - 1; };   // slice that holds u
   const int u1 = slice(own + 1), chunks = (a.GQ + QB - 1) / QB;

@@ -110,3 +110,32 @@ def test_select_and_gather_of_a_pass(P, L, Hkv, Bl):
                 assert torch.equal(buf[l][0, :, :n + w.ws], torch.gather(src[l][0], 1, rows[:, :, None].expand(-1, -1, w.D)))
     finally:
         B.dkv_destroy(h)
+
+
+# steps over many heads whose rows make fewer 16-row blocks than the launch has warps, about as many, and more
+@pytest.mark.parametrize("L,Bt,Hkv,G,D,N,nq", [(11, 2, 4, 1, 128, 73, 1), (16, 1, 4, 7, 128, 56, 1), (20, 1, 2, 2, 64, 4, 3), (19, 1, 2, 4, 128, 300, 4),
+                                               (12, 2, 4, 3, 64, 190, 1), (32, 1, 8, 4, 64, 64, 1)])
+def test_decoding_step_over_short_heads(L, Bt, Hkv, G, D, N, nq):
+    w = synth.Workload("dec", 44, L=L, Hq=G * Hkv, Hkv=Hkv, D=D, Bt=Bt, S=1205, ws=8, pool=3, N=N, Bl=2 * N, m=3, recipe="iid")
+    g = torch.Generator(device="cuda").manual_seed(N)
+    rand = lambda *shape: [torch.randn(shape, generator=g, device="cuda", dtype=torch.bfloat16) for _ in range(L)]
+    q, k, v = (rand(Bt, heads, rows, D) for heads, rows in ((w.Hq, w.ws), (Hkv, w.S), (Hkv, w.S)))
+    q = [x * (0.3 + l / L) for l, x in enumerate(q)]
+    kb, vb = ([torch.zeros((Bt, Hkv, w.Blc + w.ws, D), dtype=torch.bfloat16, device="cuda") for _ in range(L)] for _ in range(2))
+    h = B.dkv_create(B.config_of(w))
+    try:
+        B.dkv_run_prefill_pass(h, q, k, v, kb, vb)
+        counts = np.zeros((Bt, L), dtype=np.int32)
+        B.dkv_get_counts(h, counts)
+        for _ in range(2):                                   # the second call finds what the first has left
+            dq, out = rand(Bt, w.Hq, nq, D), [torch.zeros((Bt, w.Hq, nq, D), device="cuda") for _ in range(L)]
+            B.dkv_decode_attend(h, 0, L, nq, dq, kb, vb, out)
+            torch.cuda.synchronize()
+            for l in range(L):
+                for b in range(Bt):
+                    n = int(counts[b, l]) + w.ws
+                    kk, vv = (x[l][b, :, :n].double().repeat_interleave(G, dim=0) for x in (kb, vb))
+                    want = (dq[l][b].double() @ kk.transpose(1, 2) / D ** 0.5).softmax(-1) @ vv
+                    assert (out[l][b] - want).abs().max() <= 1e-5 * want.abs().max(), f"layer {l}, sample {b}"
+    finally:
+        B.dkv_destroy(h)
