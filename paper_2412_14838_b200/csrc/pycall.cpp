@@ -17,7 +17,7 @@
 
 namespace {
 
-constexpr int kMaxList = 4096;       // longest list of per-layer tensors taken without an allocation of its own
+constexpr Py_ssize_t kMaxList = 4096;       // longest list of per-layer tensors taken
 
 // Address of a torch tensor, an integer, None (NULL), or of anything with data_ptr() or a numpy-like .ctypes.data.
 bool address(PyObject* x, void** out) {
@@ -52,23 +52,29 @@ bool stream_of(PyObject* x, void** out) {
   return !PyErr_Occurred();
 }
 
-// The addresses of a sequence's items.
+// The addresses of a sequence's items.  The library reads one address a layer, whatever the length of the list: there
+// are never fewer than DKV_MAX_LAYERS entries, and a list that is too short ends in NULLs, which the library refuses.
 struct Addresses {
-  void* few[64] = {};              // a list that is too short ends in NULLs, which the library refuses
+  void* few[DKV_MAX_LAYERS] = {};
   void** p = few;
-  ~Addresses() { if (p != few) PyMem_Free(p); }
+  PyObject* items = nullptr;
+  ~Addresses() {
+    if (p != few) PyMem_Free(p);
+    Py_XDECREF(items);
+  }
   bool take(PyObject* seq) {
-    PyObject* f = PySequence_Fast(seq, "a sequence of tensors or addresses is expected");
-    if (!f) return false;
-    const Py_ssize_t n = PySequence_Fast_GET_SIZE(f);
-    if (n > 64) {
-      p = n <= kMaxList ? static_cast<void**>(PyMem_Malloc(sizeof(void*) * n)) : nullptr;
-      if (!p) { p = few; Py_DECREF(f); PyErr_SetString(PyExc_ValueError, "too many tensors"); return false; }
+    items = PySequence_Fast(seq, "a sequence of tensors or addresses is expected");
+    if (!items) return false;
+    const Py_ssize_t n = PySequence_Fast_GET_SIZE(items);
+    if (n > kMaxList) { PyErr_SetString(PyExc_ValueError, "too many tensors"); return false; }
+    if (n > DKV_MAX_LAYERS) {
+      void** more = static_cast<void**>(PyMem_Malloc(sizeof(void*) * n));
+      if (!more) { PyErr_NoMemory(); return false; }
+      p = more;
     }
-    bool ok = true;
-    for (Py_ssize_t i = 0; ok && i < n; ++i) ok = address(PySequence_Fast_GET_ITEM(f, i), &p[i]);
-    Py_DECREF(f);
-    return ok;
+    for (Py_ssize_t i = 0; i < n && i < PySequence_Fast_GET_SIZE(items); ++i)      // (an item's own code may shorten its list)
+      if (!address(PySequence_Fast_GET_ITEM(items, i), &p[i])) return false;
+    return true;
   }
 };
 

@@ -1,5 +1,8 @@
 """Argument conversion of the calls that go through native code; nothing reaches the device here."""
 import ctypes
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -35,3 +38,27 @@ def test_a_configuration_passes_by_address():
     with pytest.raises(binding.DkvError) as e:
         binding.dkv_score_static(cfg, torch.zeros(4), torch.zeros(4), torch.zeros(4), ctypes.c_void_p(0).value or 0)
     assert e.value.code == binding.DKV_ERR_INVALID_ARG
+
+
+# Stands in for the library in a child process: how many of the DKV_MAX_LAYERS addresses it may read are not NULL.
+STAND_IN = """
+int dkv_run_prefill_pass(void* ctx, const void* const* q, const void* const* k, const void* const* v, void* const* kb, void* const* vb,
+                         void* stream) {
+  int n = 0;
+  for (int i = 0; i < 128; ++i) n += q[i] != 0;
+  return n;
+}
+"""
+
+
+def test_lists_of_any_length_end_in_nulls(tmp_path):
+    (tmp_path / "stand_in.c").write_text(STAND_IN)
+    lib = str(tmp_path / "stand_in.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", lib, str(tmp_path / "stand_in.c")], check=True)
+    code = ("from paper_2412_14838_b200 import binding as B; B.load()\n"
+            "print([B._native().run_prefill_pass(0, [8] * n, [], [], [], [], 0) for n in (0, 1, 64, 65, 100, 127, 128, 200)])")
+    # fresh memory is filled with a pattern, so that an entry that was never written is not NULL by chance
+    env = dict(os.environ, LD_PRELOAD=lib, MALLOC_PERTURB_="90", PYTHONMALLOC="malloc")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    res = subprocess.run([sys.executable, "-c", code], cwd=root, env=env, capture_output=True, text=True, check=True)
+    assert res.stdout.strip() == "[0, 1, 64, 65, 100, 127, 128, 128]"
