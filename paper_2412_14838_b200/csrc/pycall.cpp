@@ -78,9 +78,11 @@ struct Addresses {
   }
 };
 
+// A 32-bit integer; one that does not fit is refused rather than cut to another layer or count.
 bool number(PyObject* x, int32_t* out) {
   const long v = PyLong_AsLong(x);
   if (v == -1 && PyErr_Occurred()) return false;
+  if (v != (int32_t)v) { PyErr_SetString(PyExc_OverflowError, "an integer does not fit 32 bits"); return false; }
   *out = (int32_t)v;
   return true;
 }

@@ -62,3 +62,15 @@ def test_lists_of_any_length_end_in_nulls(tmp_path):
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     res = subprocess.run([sys.executable, "-c", code], cwd=root, env=env, capture_output=True, text=True, check=True)
     assert res.stdout.strip() == "[0, 1, 64, 65, 100, 127, 128, 128]"
+
+
+@pytest.mark.parametrize("value", [2**31, 2**32, 2**32 + 1, -2**31 - 1, 2**70])
+def test_an_integer_that_does_not_fit_is_refused(value):
+    t = torch.zeros(4)
+    for call in (lambda: binding.dkv_select_topk(0, value, stream=0), lambda: binding.dkv_rebudget(0, value, stream=0),
+                 lambda: binding.dkv_decode_attend(0, 0, 1, value, [t], [t], [t], [t], stream=0)):
+        with pytest.raises(OverflowError):
+            call()
+    for fits in (2**31 - 1, -2**31):
+        with pytest.raises(binding.DkvError):                # reaches the library, which refuses the NULL context
+            binding.dkv_select_topk(0, fits, stream=0)
