@@ -3,12 +3,14 @@
 Every step of the path runs inside the CUDA library; this module converts torch tensors (or raw
 integer addresses) to pointers, passes the current CUDA stream, and raises ``DkvError`` on a
 non-zero return code.  The calls that a serving loop makes convert their arguments in native code
-(csrc/pycall.cpp, loaded as ``_dkv_pycall``), the others through ctypes.  There is no CPU fallback:
-``load()`` raises when the library is missing.
+(csrc/pycall.cpp, loaded as ``_dkv_pycall``), the others through ctypes.  The native half is linked with
+torch's libraries; a program without torch (arrays and addresses of its own, streams as integers) makes
+the same calls through ctypes alone.  There is no CPU fallback: ``load()`` raises when the library is missing.
 """
 from __future__ import annotations
 
 import ctypes
+import operator
 import os
 from typing import Optional, Sequence
 
@@ -41,7 +43,7 @@ class DkvError(RuntimeError):
 
 
 _lib = None
-_call = None                     # the native half, csrc/pycall.cpp
+_call = None                     # argument conversion: the native half, csrc/pycall.cpp, or _CtypesCalls without torch
 
 
 def load() -> ctypes.CDLL:
@@ -59,7 +61,7 @@ def load() -> ctypes.CDLL:
         "dkv_destroy": [vp],
         "dkv_reset": [vp, vp],
         "dkv_score": [vp, i32, vp, vp, vp, vp],
-        "dkv_score_static": [ctypes.POINTER(DkvConfig), vp, vp, vp, vp],
+        "dkv_score_static": [vp, vp, vp, vp, vp],
         "dkv_score_lse": [vp, i32, vp, vp, vp, vp, vp],
         "dkv_set_scores": [vp, i32, vp, vp],
         "dkv_select_topk": [vp, i32, vp, vp, vp],
@@ -95,10 +97,45 @@ def load() -> ctypes.CDLL:
         fn.restype = ctypes.c_int
     lib.dkv_strerror.restype = ctypes.c_char_p
     lib.dkv_launch_count.restype = ctypes.c_int64
-    import torch                 # noqa: F401  (the native half is linked with torch's libraries)
-    from . import _dkv_pycall
-    _lib, _call = lib, _dkv_pycall
+    try:
+        import torch             # noqa: F401  (the native half is linked with its libraries)
+    except ImportError:
+        call = _CtypesCalls(lib)
+    else:
+        from . import _dkv_pycall as call
+    _lib, _call = lib, call
     return lib
+
+
+class _CtypesCalls:
+    """The native half's functions for a program without torch: the same arguments, converted by ctypes."""
+
+    def __init__(self, lib: ctypes.CDLL):
+        self._lib = lib
+
+    def __getattr__(self, name):
+        fn = getattr(self._lib, "dkv_" + name)
+        takes_stream = name != "run_prefill_pass_host"
+
+        def call(*args):
+            if takes_stream and args[-1] is None:
+                raise TypeError("without torch there is no current stream: pass one (0: the legacy default stream)")
+            return fn(*[_argument(t, x) for t, x in zip(fn.argtypes, args, strict=True)])
+
+        return call
+
+
+def _argument(ctype, x):
+    """What ctypes takes for `x`: lists of tensors or addresses as an array with an entry for every layer the library
+    may read, NULL past the list's end; integers that fit 32 bits; addresses."""
+    if ctype is ctypes.c_int32:
+        x = operator.index(x)
+        if not -2**31 <= x < 2**31:
+            raise OverflowError("an integer does not fit 32 bits")
+        return x
+    if ctype is ctypes.POINTER(ctypes.c_void_p):
+        return (ctypes.c_void_p * max(len(x), 128))(*[_ptr(item) for item in x])
+    return x if ctype is ctypes.c_uint64 else _ptr(x)
 
 
 def _native():
@@ -122,6 +159,8 @@ def _ptr(x) -> Optional[int]:
         return x.data_ptr()
     if hasattr(x, "ctypes"):
         return x.ctypes.data
+    if hasattr(x, "cuda_stream"):
+        return x.cuda_stream
     raise TypeError(f"cannot take the address of {type(x)}")
 
 

@@ -1,10 +1,11 @@
 """Build libdkv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _dkv_pycall.so (the native half of
-binding.py: argument conversion) with the host compiler.
+binding.py: argument conversion; only where torch is installed, whose libraries it is linked with) with the host compiler.
 
 ``python -m paper_2412_14838_b200.build`` or ``build()``; nvcc cross-compiles without a GPU.
 """
 from __future__ import annotations
 
+import importlib.util
 import os
 import shutil
 import subprocess
@@ -57,7 +58,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         _run([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC", "-Xptxas", "-v" if verbose else "-O3",
               "-o", LIB] + [os.path.join(CSRC, s) for s in SOURCES], verbose)
-    if force or _stale(PYCALL, [PYCALL_SOURCE, HEADER]):
+    if importlib.util.find_spec("torch") and (force or _stale(PYCALL, [PYCALL_SOURCE, HEADER])):
         _build_pycall(verbose)
     return LIB
 

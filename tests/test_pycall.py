@@ -64,6 +64,39 @@ def test_lists_of_any_length_end_in_nulls(tmp_path):
     assert res.stdout.strip() == "[0, 1, 64, 65, 100, 127, 128, 128]"
 
 
+def test_a_program_without_torch_makes_the_same_calls(tmp_path):
+    (tmp_path / "stand_in.c").write_text(STAND_IN)
+    lib = str(tmp_path / "stand_in.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", lib, str(tmp_path / "stand_in.c")], check=True)
+    code = f"""
+import sys
+sys.modules["torch"] = None                                   # "import torch" fails
+import ctypes, numpy as np
+from paper_2412_14838_b200 import binding as B
+def raises(kind, call):
+    try: call()
+    except kind as e: return getattr(e, "code", 0)
+    raise AssertionError(kind)
+B.load()
+a = np.zeros(4, dtype=np.float32)
+cfg = B.make_config(4, 8, 2, 64, 1, 16, 16, 5, 64, 128, 2)     # S = ws: refused on the host
+refused = [lambda: B.dkv_decode_attend(0, 0, 1, 1, [a], [a], [a.ctypes.data], [a], stream=0), lambda: B.dkv_reset(0, 0),
+           lambda: B.dkv_run_prefill_pass_host(0, [a], [a], [a], [a], [None], None), lambda: B.dkv_score_static(cfg, a, a, a, 0),
+           lambda: B.dkv_memcpy_to_host(0, a, 8, a.nbytes, 0), lambda: B.dkv_rebudget(0, np.int64(1), stream=0)]
+assert [raises(B.DkvError, c) for c in refused] == [B.DKV_ERR_INVALID_ARG] * len(refused)
+raises(OverflowError, lambda: B.dkv_select_topk(0, 2**32, stream=0))
+raises(TypeError, lambda: B.dkv_reset(0))                      # no stream, no torch whose current one to take
+raises(TypeError, lambda: B.dkv_compact_all(0, 1, ["x"], [a], 0))
+seen = []
+stand_in = ctypes.CDLL({lib!r}).dkv_run_prefill_pass           # the converted list as the library sees it
+for n in (0, 1, 127, 128, 200):
+    seen.append(stand_in(None, B._argument(ctypes.POINTER(ctypes.c_void_p), [8] * n)))
+assert seen == [0, 1, 127, 128, 128], seen
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", code], cwd=root, check=True)
+
+
 @pytest.mark.parametrize("value", [2**31, 2**32, 2**32 + 1, -2**31 - 1, 2**70])
 def test_an_integer_that_does_not_fit_is_refused(value):
     t = torch.zeros(4)
