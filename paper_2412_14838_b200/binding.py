@@ -102,6 +102,10 @@ def load() -> ctypes.CDLL:
     except ImportError:
         call = _CtypesCalls(lib)
     else:
+        from . import build
+        if (was := build.pycall_built_for()) not in (None, build.torch_version()):
+            raise RuntimeError(f"_dkv_pycall.so was linked with torch {was}, installed is {build.torch_version()}: run "
+                               "`python -m paper_2412_14838_b200.build`")
         from . import _dkv_pycall as call
     _lib, _call = lib, call
     return lib

@@ -5,7 +5,7 @@ binding.py: argument conversion; only where torch is installed, whose libraries 
 """
 from __future__ import annotations
 
-import importlib.util
+import importlib.metadata
 import os
 import shutil
 import subprocess
@@ -16,6 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdkv.so")
 SOURCES = ["dkv.cu"]
 PYCALL = os.path.join(HERE, "_dkv_pycall.so")
+PYCALL_TORCH = PYCALL + ".torch"        # beside it: the torch version it was linked with
 PYCALL_SOURCE = os.path.join(CSRC, "pycall.cpp")
 HEADER = os.path.join(os.path.dirname(HERE), "include", "dkv.h")
 
@@ -25,6 +26,23 @@ def _nvcc() -> str:
         if cand and os.path.exists(cand):
             return cand
     raise RuntimeError("nvcc not found: libdkv.so cannot be built")
+
+
+def torch_version() -> str | None:
+    """The installed torch's version, None where there is none (without importing it, which takes seconds)."""
+    try:
+        return importlib.metadata.version("torch")
+    except importlib.metadata.PackageNotFoundError:
+        return None
+
+
+def pycall_built_for() -> str | None:
+    """The torch version that _dkv_pycall.so was linked with, if its build left a note."""
+    try:
+        with open(PYCALL_TORCH) as f:
+            return f.read().strip()
+    except FileNotFoundError:
+        return None
 
 
 def _stale(lib: str, deps) -> bool:
@@ -49,16 +67,18 @@ def _build_pycall(verbose: bool) -> None:
           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(f"-I{d}" for d in inc), PYCALL_SOURCE,
           "-o", PYCALL, f"-L{HERE}", "-l:libdkv.so", f"-L{root}/lib", "-ltorch_python", "-lc10", "-lc10_cuda",
           "-Wl,-rpath,$ORIGIN", f"-Wl,-rpath,{root}/lib"], verbose)
+    with open(PYCALL_TORCH, "w") as f:
+        f.write(torch_version() + "\n")
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile what is older than its sources; return the library's path."""
+    """Compile what is older than its sources, or linked with another torch; return the library's path."""
     kernels = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != os.path.basename(PYCALL_SOURCE)]
     if force or _stale(LIB, kernels + [HEADER]):
         _run([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC", "-Xptxas", "-v" if verbose else "-O3",
               "-o", LIB] + [os.path.join(CSRC, s) for s in SOURCES], verbose)
-    if importlib.util.find_spec("torch") and (force or _stale(PYCALL, [PYCALL_SOURCE, HEADER])):
+    if torch_version() and (force or _stale(PYCALL, [PYCALL_SOURCE, HEADER]) or pycall_built_for() != torch_version()):
         _build_pycall(verbose)
     return LIB
 

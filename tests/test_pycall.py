@@ -107,3 +107,19 @@ def test_an_integer_that_does_not_fit_is_refused(value):
     for fits in (2**31 - 1, -2**31):
         with pytest.raises(binding.DkvError):                # reaches the library, which refuses the NULL context
             binding.dkv_select_topk(0, fits, stream=0)
+
+
+def test_the_native_half_belongs_to_one_torch_version(monkeypatch, tmp_path):
+    built = []
+    note = tmp_path / "note"
+    monkeypatch.setattr(build, "PYCALL_TORCH", str(note))
+    monkeypatch.setattr(build, "_build_pycall", lambda verbose: (built.append(1), note.write_text(build.torch_version())))
+    note.write_text("1.0.0")                                   # linked with another version: rebuilt, and only then
+    build.build()
+    build.build()
+    assert built == [1]
+    note.write_text("1.0.0")
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "_call", None)
+    with pytest.raises(RuntimeError, match="linked with torch 1.0.0"):
+        binding.load()
