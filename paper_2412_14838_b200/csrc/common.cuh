@@ -27,7 +27,9 @@ __device__ __forceinline__ float fast_exp2(float x) {
 }
 
 // Programmatic dependent launch: the kernel may have been scheduled while its predecessor on the stream still ran;
-// nothing that a predecessor may have written is touched before pdl_wait.
+// nothing that a predecessor may have written is touched before pdl_wait.  Such memory is not read-only for the lifetime
+// of the grid: a kernel with pdl_wait takes its pointers without __restrict__ and reads with plain loads (no __ldg), which
+// the compiler may neither turn into non-coherent loads nor move above the wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

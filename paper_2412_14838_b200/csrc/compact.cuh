@@ -11,8 +11,8 @@ constexpr int kGatherRows = 4;      // rows per thread, all loads issued before 
 // One head's buffer rows: row r < n is source row sel[r] (shared or global memory), the ws window rows P .. S-1 follow.
 // 16 bytes of K and of V per thread and row, `threads` threads (a multiple of vec = 16-byte pieces per row); `part` of
 // `parts` sets of threads share the head.
-__device__ __forceinline__ void gather_rows(const uint4* __restrict__ k_src, const uint4* __restrict__ v_src, uint4* __restrict__ kb,
-                                            uint4* __restrict__ vb, const int* sel, int n, int bh, int S, int P, int ws,
+__device__ __forceinline__ void gather_rows(const uint4* k_src, const uint4* v_src, uint4* kb,
+                                            uint4* vb, const int* sel, int n, int bh, int S, int P, int ws,
                                             int row_stride /* rows per head in kb/vb */, int vec, int tid, int threads, int part, int parts) {
   const int per_pass = threads / vec, c = tid % vec, rows = n + ws;
   const size_t src0 = (size_t)bh * S * vec + c, dst0 = (size_t)bh * row_stride * vec + c;
@@ -39,9 +39,9 @@ __device__ __forceinline__ void gather_rows(const uint4* __restrict__ k_src, con
 // records held[b][layer] = n.  grid (row blocks, Bt*Hkv).
 constexpr int kGatherThreads = 256;
 __global__ void __launch_bounds__(kGatherThreads)
-gather_rows_kernel(const uint4* __restrict__ k_src, const uint4* __restrict__ v_src, uint4* __restrict__ kb,
-                   uint4* __restrict__ vb, const int* __restrict__ idx, const int* __restrict__ count, int sel_n, int idx_stride,
-                   int S, int P, int ws, int row_stride, int vec, int* __restrict__ held, int Hkv, int L, int layer) {
+gather_rows_kernel(const uint4* k_src, const uint4* v_src, uint4* kb,
+                   uint4* vb, const int* idx, const int* count, int sel_n, int idx_stride,
+                   int S, int P, int ws, int row_stride, int vec, int* held, int Hkv, int L, int layer) {
   const int bh = blockIdx.y, b = bh / Hkv;
   pdl_launch();
   pdl_wait();
@@ -64,7 +64,7 @@ struct PassPtrs {
 // copies for 32 layers, which have to wait for the counts, took 0.2 ms of 6.7 longer.)  Bound by the bus.
 // grid (row blocks of kGatherThreads / vec * kGatherRows, Bt*Hkv, layers).
 __global__ void __launch_bounds__(kGatherThreads)
-copy_valid_kernel(const __grid_constant__ PassPtrs ptrs, const int* __restrict__ held, int ws, int rows, int vec, int Hkv, int L) {
+copy_valid_kernel(const __grid_constant__ PassPtrs ptrs, const int* held, int ws, int rows, int vec, int Hkv, int L) {
   const int bh = blockIdx.y, layer = blockIdx.z, per_pass = kGatherThreads / vec, c = threadIdx.x % vec;
   pdl_launch();
   pdl_wait();
@@ -94,7 +94,7 @@ constexpr int kShrinkThreads = 256;
 // blocks, each block read completely before it is written.  The last block of a (layer, sample) to arrive (a ticket
 // each, zero between launches) records held[b][layer] = want: everyone has read the old value by then.
 __global__ void __launch_bounds__(kShrinkThreads)
-shrink_kernel(LayerPtrs ptrs, int layer0, const int* __restrict__ count, int* __restrict__ held, unsigned int* __restrict__ tickets,
+shrink_kernel(LayerPtrs ptrs, int layer0, const int* count, int* held, unsigned int* tickets,
               int Hkv, int L, int ws, int row_stride, int vec_per_row) {
   const int layer = layer0 + blockIdx.y;
   const int bh = blockIdx.x, b = bh / Hkv;

@@ -49,7 +49,7 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
 // The upper halves (bf16 by truncation) of two floats, `a` in the low half; and what truncation leaves of a float.
 __device__ __forceinline__ uint32_t pack_hi(float a, float b) { return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632); }
 __device__ __forceinline__ float rest_of(float a) { return a - __uint_as_float(__float_as_uint(a) & 0xFFFF0000u); }
-__device__ __forceinline__ uint4 ld_row16(const uint16_t* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
+__device__ __forceinline__ uint4 ld_row16(const uint16_t* p) { return *reinterpret_cast<const uint4*>(p); }
 
 // State of one warp: QB (8 or 16) queries against the rows it has seen.  Lane (g, t) = (lane / 4, lane % 4) holds
 // queries g (and g + 8), output dims 64*(j/8) + 16 t + {j%8, 8 + j%8}, j < D/8.

@@ -40,8 +40,8 @@ struct RbState {                   // per update and sample
 // grid (updates, Bt).  layer_hist: [L][Bt][2048].  state: [updates][Bt].  above: [updates][Bt][L] scores above the digit
 // per layer.  Clears cand_n [Bt]; fill > 0: count[b][.] starts at `fill` (a pass selects after the updates).
 __global__ void __launch_bounds__(1024)
-rb_locate_kernel(const __grid_constant__ RbBatch batch, const unsigned int* __restrict__ layer_hist, RbState* __restrict__ state,
-                 unsigned int* __restrict__ above, unsigned int* __restrict__ cand_n, int* __restrict__ count, int fill, int Bt,
+rb_locate_kernel(const __grid_constant__ RbBatch batch, const unsigned int* layer_hist, RbState* state,
+                 unsigned int* above, unsigned int* cand_n, int* count, int fill, int Bt,
                  int Hkv, int L, int P) {
   __shared__ unsigned int hist[kBins];
   __shared__ int sm_scan[33];
@@ -83,8 +83,8 @@ rb_locate_kernel(const __grid_constant__ RbBatch batch, const unsigned int* __re
 // (cand_stride pairs per sample); its order is arbitrary, only counts are taken from it.  Matches are parked in shared
 // memory, then the block reserves a range of the list with one atomic and copies them out.
 __global__ void __launch_bounds__(kRbThreads)
-rb_collect_kernel(const __grid_constant__ RbBatch batch, const float* __restrict__ scores, const RbState* __restrict__ state,
-                  uint2* __restrict__ cand, unsigned int* __restrict__ cand_n, int Bt, size_t per_layer /* Hkv*P */, size_t cand_stride) {
+rb_collect_kernel(const __grid_constant__ RbBatch batch, const float* scores, const RbState* state,
+                  uint2* cand, unsigned int* cand_n, int Bt, size_t per_layer /* Hkv*P */, size_t cand_stride) {
   __shared__ uint32_t parked[kRbChunk];
   __shared__ unsigned int wanted[kBins / 32];
   __shared__ unsigned int s_cnt, s_base;
@@ -133,9 +133,9 @@ rb_collect_kernel(const __grid_constant__ RbBatch batch, const float* __restrict
 // Z_i = floor(Bl*cnt_i/max cnt); Z'_i = floor(Z_i*N*L/sum Z); count_i = min(count_i, Z'_i).
 // grid (kRbCluster, updates, Bt).  dbg_*: [Bt][L], of update `shown` (-1: none).  counts_out (single updates only): a copy.
 __global__ void __launch_bounds__(1024)
-rb_finish_kernel(const __grid_constant__ RbBatch batch, const RbState* __restrict__ state, const unsigned int* __restrict__ above,
-                 const uint2* __restrict__ cand, const unsigned int* __restrict__ cand_n, size_t cand_stride, int* __restrict__ count,
-                 int* __restrict__ dbg_cnt, int* __restrict__ dbg_z, int* __restrict__ dbg_zp, int shown, int* __restrict__ counts_out,
+rb_finish_kernel(const __grid_constant__ RbBatch batch, const RbState* state, const unsigned int* above,
+                 const uint2* cand, const unsigned int* cand_n, size_t cand_stride, int* count,
+                 int* dbg_cnt, int* dbg_z, int* dbg_zp, int shown, int* counts_out,
                  int Bt, int L, int Bl, int N, int prorata, int minmax) {
   namespace cg = cooperative_groups;
   __shared__ unsigned int hist[kBins], total_hist[kBins];

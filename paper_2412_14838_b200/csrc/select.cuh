@@ -182,7 +182,7 @@ __host__ __device__ inline size_t select_smem(int cap) {
   return (size_t)cap * 8 * (cap <= kMaxCountingList ? 2 : 1) + sizeof(unsigned int) * kSortBins;
 }
 template <bool kShared>
-__device__ __forceinline__ int* select_head(const uint32_t* __restrict__ v, int P, int n, int cap, unsigned char* dyn, unsigned int* gh, int part,
+__device__ __forceinline__ int* select_head(const uint32_t* v, int P, int n, int cap, unsigned char* dyn, unsigned int* gh, int part,
                                             int parts) {
   namespace cg = cooperative_groups;
   __shared__ int sm_scan[33];
@@ -356,8 +356,8 @@ __device__ __forceinline__ int* select_head(const uint32_t* __restrict__ v, int 
 // launch says when).  grid Bt*Hkv*parts.
 template <bool kShared>
 __global__ void __launch_bounds__(kSelThreads, 2)
-select_topk_kernel(const float* __restrict__ scores, int* __restrict__ idx, unsigned int* __restrict__ layer_hist, int P,
-                   int keep, int cap, int* __restrict__ count, int Hkv, int L, int layer, int parts) {
+select_topk_kernel(const float* scores, int* idx, unsigned int* layer_hist, int P,
+                   int keep, int cap, int* count, int Hkv, int L, int layer, int parts) {
   extern __shared__ __align__(16) unsigned char dyn[];
   const int head = blockIdx.x / parts, b = head / Hkv;
   pdl_launch();
@@ -375,8 +375,8 @@ select_topk_kernel(const float* __restrict__ scores, int* __restrict__ idx, unsi
 // instead of 272, and no block of the scoring kernel gives way to it while keys are streamed.
 // grid (Bt*Hkv, layers).
 __global__ void __launch_bounds__(kSelThreads, 2)
-select_gather_kernel(const __grid_constant__ PassPtrs ptrs, const float* __restrict__ scores, int* __restrict__ idx,
-                     const int* __restrict__ count, int* __restrict__ held, int P, int ws, int stride, int cap, int S, int vec, int Hkv, int L) {
+select_gather_kernel(const __grid_constant__ PassPtrs ptrs, const float* scores, int* idx,
+                     const int* count, int* held, int P, int ws, int stride, int cap, int S, int vec, int Hkv, int L) {
   extern __shared__ __align__(16) unsigned char dyn[];
   const int bh = blockIdx.x, b = bh / Hkv, layer = blockIdx.y, tid = threadIdx.x;
   const size_t head = (size_t)layer * gridDim.x + bh;
@@ -395,8 +395,8 @@ select_gather_kernel(const __grid_constant__ PassPtrs ptrs, const float* __restr
 
 // The same with a cluster a head, whose blocks share the selection and the copying.  grid (Bt*Hkv*cluster size, layers).
 __global__ void __launch_bounds__(kSelThreads, 2)
-select_gather_cluster_kernel(const __grid_constant__ PassPtrs ptrs, const float* __restrict__ scores, int* __restrict__ idx,
-                             const int* __restrict__ count, int* __restrict__ held, int P, int ws, int stride, int cap, int S, int vec, int Hkv,
+select_gather_cluster_kernel(const __grid_constant__ PassPtrs ptrs, const float* scores, int* idx,
+                             const int* count, int* held, int P, int ws, int stride, int cap, int S, int vec, int Hkv,
                              int L) {
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char dyn[];

@@ -1,0 +1,53 @@
+"""Kernels that are resident while their predecessor still writes (programmatic dependent launch): nothing in their
+source may let the compiler treat what they read as read-only memory.  Read from the source; nothing runs."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2412_14838_b200", "csrc")
+
+
+def _source(name):
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"/\*.*?\*/", "", re.sub(r"//[^\n]*", "", text), flags=re.S)
+
+
+def _functions(text):
+    """(name, parameters, body) of every kernel and device function."""
+    for m in re.finditer(r"__(?:global|device)__[^;{}]*?(\w+)\s*\((?=[^)]*\))", text):
+        if m.group(1) == "__launch_bounds__":
+            m = re.compile(r"(\w+)\s*\(").search(text, text.index(")", m.end()) + 1)
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"(": 1, ")": -1}.get(text[i], 0)
+            i += 1
+        params, start = text[m.end():i - 1], text.find("{", i)
+        depth, j = 1, start + 1
+        while depth:
+            depth += {"{": 1, "}": -1}.get(text[j], 0)
+            j += 1
+        yield m.group(1), params, text[start:j]
+
+
+HEADERS = sorted(f for f in os.listdir(CSRC) if f.endswith(".cuh"))
+
+
+def test_every_kernel_launched_with_overlap_waits():
+    launched = set(re.findall(r"launch_pdl\((?:parts > 1 \? )?(\w+)", _source("dkv.cu"))) - {"void"}
+    assert {"rb_locate_kernel", "select_gather_cluster_kernel", "shrink_kernel", "decode_split_kernel"} <= launched
+    kernels = {n: body for f in HEADERS for n, _, body in _functions(_source(f))}
+    for name in launched - {"score_kernel"} | {"score_tc_kernel", "select_topk_kernel", "select_gather_kernel"}:
+        assert "pdl_wait();" in kernels[name], name
+
+
+@pytest.mark.parametrize("header", HEADERS)
+def test_no_read_of_such_a_kernel_is_marked_read_only(header):
+    text = _source(header)
+    assert not re.search(r"__ldg\s*\(|ld\.global\.(?:\w+\.)*nc|__ld(?:lu|cv)\s*\(", text)
+    functions = list(_functions(text))
+    waiting = [n for n, _, body in functions if "pdl_wait();" in body]
+    called = {n for n, _, _ in functions if any(re.search(rf"\b{n}\b", b) for m, _, b in functions if m in waiting)}
+    for name, params, _ in functions:
+        if name in waiting or name in called or not name.endswith("_kernel"):
+            assert "__restrict__" not in params, name
