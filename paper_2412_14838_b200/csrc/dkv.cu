@@ -449,14 +449,19 @@ int update_points(const Shape& s, int* l) {
   return n;
 }
 
-int do_reset(dkv_ctx* c, cudaStream_t st) {
-  const Shape& s = c->s;
-  DKV_CUDA(c, cudaMemsetAsync(c->d_count, 0, sizeof(int) * s.Bt * s.L, st));
-  DKV_CUDA(c, cudaMemsetAsync(c->d_held, 0, sizeof(int) * s.Bt * s.L, st));
-  DKV_CUDA(c, cudaMemsetAsync(c->d_dbg, 0, sizeof(int) * 3 * s.Bt * s.L, st));
+// What the host knows of the layers.
+void forget_layers(dkv_ctx* c) {
   memset(c->scored, 0, sizeof c->scored);
   memset(c->selected, 0, sizeof c->selected);
   memset(c->gathered, 0, sizeof c->gathered);
+}
+
+int do_reset(dkv_ctx* c, cudaStream_t st) {
+  const Shape& s = c->s;
+  forget_layers(c);
+  DKV_CUDA(c, cudaMemsetAsync(c->d_count, 0, sizeof(int) * s.Bt * s.L, st));
+  DKV_CUDA(c, cudaMemsetAsync(c->d_held, 0, sizeof(int) * s.Bt * s.L, st));
+  DKV_CUDA(c, cudaMemsetAsync(c->d_dbg, 0, sizeof(int) * 3 * s.Bt * s.L, st));
   return DKV_OK;
 }
 
@@ -792,6 +797,9 @@ int dkv_compact_all(dkv_ctx* c, int32_t upto_layer, void* const* kb, void* const
   return do_shrink(c, 0, upto_layer, kb, vb, as_stream(stream));
 }
 
+static int enqueue_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, const void* const* v,
+                        const float* const* lse, void* const* kb, void* const* vb, cudaStream_t st);
+
 static int run_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, const void* const* v,
                     const float* const* lse, void* const* kb, void* const* vb, void* stream) {
   if (!c || !q_win || !k || !v || !kb || !vb) return DKV_ERR_INVALID_ARG;
@@ -801,7 +809,21 @@ static int run_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, 
       return DKV_ERR_INVALID_ARG;
     if (lse && (!lse[l] || ((uintptr_t)lse[l] & 3))) return DKV_ERR_INVALID_ARG;
   }
+  // A pass overwrites every word of the counts, the held rows and the update's integers itself, so that the reset it begins
+  // with is needed on the device only if a launch is refused midway.
   cudaStream_t st = as_stream(stream);
+  forget_layers(c);
+  const int rc = enqueue_pass(c, q_win, k, v, lse, kb, vb, st);
+  if (rc) {
+    const int why = c->last_cuda;
+    do_reset(c, st);
+    c->last_cuda = why;
+  }
+  return rc;
+}
+
+static int enqueue_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, const void* const* v,
+                        const float* const* lse, void* const* kb, void* const* vb, cudaStream_t st) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusNone; }
   // per-step profiling needs its events between the launches; a caller that is capturing gets the plain calls

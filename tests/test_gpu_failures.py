@@ -6,6 +6,9 @@ tensor memory and ends, and the host reads DKV_ERR_TIMEOUT from dkv_last_status.
 out the harmless way: the copy of one key tile is simply never issued (dkv_debug_withhold_tile), with the
 wait limit set to about a millisecond.  Nothing traps, no address is invalid, the context stays usable.
 """
+import contextlib
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -93,3 +96,69 @@ def test_two_live_contexts_with_different_layer_budgets():
     finally:
         B.dkv_destroy(a)
         B.dkv_destroy(b)
+
+
+@contextlib.contextmanager
+def stream_that_refuses_work():
+    """A stream whose capture was invalidated: the runtime refuses every launch and copy on it, on the host, until the
+    capture is ended."""
+    rt = ctypes.CDLL("libcudart.so.12")
+    rt.cudaStreamEndCapture.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+    stream = torch.cuda.Stream()
+    handle = ctypes.c_void_p(stream.cuda_stream)
+    assert rt.cudaStreamBeginCapture(handle, 2) == 0
+    assert rt.cudaStreamSynchronize(handle) != 0               # not allowed in a capture
+    try:
+        yield stream
+    finally:
+        graph = ctypes.c_void_p()
+        assert rt.cudaStreamEndCapture(handle, ctypes.byref(graph)) != 0 and not graph.value
+        rt.cudaGetLastError()
+
+
+class _Pass:
+    """One prompt of the smallest workload on the device."""
+
+    def __init__(self):
+        self.w = w = synth.WORKLOADS["tiny"]
+        bits = [synth.layer_inputs(w, l) for l in range(w.L)]
+        self.q, self.k, self.v = ([_dev(t[n]) for t in bits] for n in ("q", "k", "v"))
+        shape = (w.Bt, w.Hkv, w.Blc + w.ws, w.D)
+        self.kb, self.vb = ([torch.zeros(shape, dtype=torch.int16, device="cuda") for _ in range(w.L)] for _ in range(2))
+        shape = (w.Bt, w.Hq, 1, w.D)
+        self.dq = [torch.randn(shape, device="cuda").to(torch.bfloat16) for _ in range(w.L)]
+        self.out = [torch.zeros(shape, device="cuda") for _ in range(w.L)]
+        self.lse = [torch.zeros((w.Bt, w.Hq, w.ws), device="cuda") for _ in range(w.L)]
+
+    def run(self, ctx, use, stream=None):
+        if use == "lse":
+            B.dkv_run_prefill_pass_lse(ctx, self.q, self.k, self.v, self.lse, self.kb, self.vb, stream)
+        else:
+            B.dkv_run_prefill_pass(ctx, self.q, self.k, self.v, self.kb, self.vb, stream)
+
+    def decode(self, ctx):
+        B.dkv_decode_attend(ctx, 0, self.w.L, 1, self.dq, self.kb, self.vb, self.out)
+        torch.cuda.synchronize()
+        return torch.stack(self.out).clone()
+
+
+@pytest.mark.parametrize("use", ["pass", "lse"])
+def test_a_pass_that_fails_midway_leaves_no_layer_of_the_pass_before(use):
+    p = _Pass()
+    ctx = B.dkv_create(B.config_of(p.w))
+    try:
+        p.run(ctx, use)
+        want = p.decode(ctx)
+        with stream_that_refuses_work() as stream:
+            with pytest.raises(B.DkvError) as e:
+                p.run(ctx, use, stream)
+            assert e.value.code == B.DKV_ERR_CUDA and B.dkv_last_cuda_error(ctx) != 0
+        for call in (lambda: p.decode(ctx), lambda: B.dkv_rebudget(ctx, p.w.L), lambda: B.dkv_select_topk(ctx, 0),
+                     lambda: B.dkv_compact_all(ctx, p.w.L, p.kb, p.vb)):
+            with pytest.raises(B.DkvError) as e:
+                call()
+            assert e.value.code == B.DKV_ERR_STATE
+        p.run(ctx, use)
+        assert torch.equal(p.decode(ctx), want)
+    finally:
+        B.dkv_destroy(ctx)
