@@ -84,28 +84,27 @@ namespace {
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// A failed call is reported once: the runtime keeps its code until it is read, and the next check after a launch would
+// otherwise take it for its own, in this context or another.
 int cuda_fail(dkv_ctx* c, cudaError_t e) {
   if (c) c->last_cuda = (int)e;
+  cudaGetLastError();
   return e == cudaErrorMemoryAllocation ? DKV_ERR_NOMEM : DKV_ERR_CUDA;
 }
 #define DKV_CUDA(ctx, call)                                   \
   do {                                                        \
     cudaError_t e__ = (call);                                 \
-    if (e__ != cudaSuccess) return cuda_fail((ctx), e__);     \
+    if (e__ != cudaSuccess) return cuda_fail(ctx, e__);       \
   } while (0)
-// After a launch: a launch error is reported once and cleared (cudaGetLastError), so that a refused launch
-// does not make every later call of every context fail.
 #define DKV_LAUNCH(ctx, call)                                 \
   do {                                                        \
-    cudaError_t e__ = (call);                                 \
-    if (e__ != cudaSuccess) { cudaGetLastError(); return cuda_fail((ctx), e__); } \
+    DKV_CUDA(ctx, call);                                      \
     (ctx)->launches++;                                        \
   } while (0)
 #define DKV_LAUNCHED(ctx)                                     \
   do {                                                        \
+    DKV_CUDA(ctx, cudaGetLastError());                        \
     (ctx)->launches++;                                        \
-    cudaError_t e__ = cudaGetLastError();                     \
-    if (e__ != cudaSuccess) return cuda_fail((ctx), e__);     \
   } while (0)
 
 // Event pair around one step's launches; read back by dkv_profile_read.
@@ -1065,17 +1064,19 @@ int dkv_score_static(const dkv_config* cfg, const void* q_win, const void* k, fl
   if (!q_win || !k || !scores_out || !aligned16(q_win) || !aligned16(k) || !aligned16(scores_out))
     return DKV_ERR_INVALID_ARG;
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return DKV_ERR_CUDA;
+  DKV_CUDA(nullptr, cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return DKV_ERR_CUDA;
   StaticSetup su;
   {
     std::lock_guard<std::mutex> lock(g_static_mutex);
     StaticSetup& g = g_static_setup[dev];
     if (!g.done) {                           // first call on this device
       void* ptr = nullptr;
-      if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess || !ptr) return DKV_ERR_CUDA;
+      DKV_CUDA(nullptr, cudaGetSymbolAddress(&ptr, g_static_scratch));
       int sms = 0;
-      if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return DKV_ERR_CUDA;
-      if (set_score_attributes() != cudaSuccess) return DKV_ERR_CUDA;
+      DKV_CUDA(nullptr, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+      if (!ptr || sms < 1) return DKV_ERR_CUDA;
+      DKV_CUDA(nullptr, set_score_attributes());
       g.ptr = static_cast<unsigned char*>(ptr);
       g.sms = sms;
       g.done = true;
@@ -1099,7 +1100,7 @@ int dkv_score_static(const dkv_config* cfg, const void* q_win, const void* k, fl
   tc::Maps<1> maps;
   maps.lse[0] = nullptr;
   if (!make_map(&maps.q[0], q_win, D, M, heads, 128 / query_copies(M)) || !make_map(&maps.k[0], k, D, S, heads)) return DKV_ERR_CUDA;
-  if (cudaMemsetAsync(su.ptr, 0, 256, st) != cudaSuccess) return DKV_ERR_CUDA;   // status words start at zero
+  DKV_CUDA(nullptr, cudaMemsetAsync(su.ptr, 0, 256, st));   // status words start at zero
   tc::Params p, none;
   memset(&p, 0, sizeof p);
   memset(&none, 0, sizeof none);
@@ -1120,10 +1121,10 @@ int dkv_score_static(const dkv_config* cfg, const void* q_win, const void* k, fl
   p.stats_grid = grid;
   p.mode = tc::kStats;
   p.idesc = make_idesc(128, 128);
-  if (launch_tc(grid, st, maps, maps, p, none) != cudaSuccess) { cudaGetLastError(); return DKV_ERR_CUDA; }
+  DKV_CUDA(nullptr, launch_tc(grid, st, maps, maps, p, none));
   p.mode = tc::kEmit;
   p.idesc = make_idesc(128, p.nq16);
-  if (launch_tc(grid, st, maps, maps, none, p) != cudaSuccess) { cudaGetLastError(); return DKV_ERR_CUDA; }
+  DKV_CUDA(nullptr, launch_tc(grid, st, maps, maps, none, p));
   return DKV_OK;
 }
 
@@ -1145,8 +1146,8 @@ int dkv_last_status(dkv_ctx* c, int32_t* host_status) {
 
 int dkv_static_last_status(int32_t* host_status) {
   if (!host_status) return DKV_ERR_INVALID_ARG;
-  if (cudaDeviceSynchronize() != cudaSuccess) return DKV_ERR_CUDA;
-  if (cudaMemcpyFromSymbol(host_status, g_static_scratch, sizeof(int) * 8) != cudaSuccess) return DKV_ERR_CUDA;
+  DKV_CUDA(nullptr, cudaDeviceSynchronize());
+  DKV_CUDA(nullptr, cudaMemcpyFromSymbol(host_status, g_static_scratch, sizeof(int) * 8));
   host_status[1] = 0;
   return host_status[0] == 0 ? DKV_OK : DKV_ERR_TIMEOUT;
 }

@@ -162,3 +162,23 @@ def test_a_pass_that_fails_midway_leaves_no_layer_of_the_pass_before(use):
         assert torch.equal(p.decode(ctx), want)
     finally:
         B.dkv_destroy(ctx)
+
+
+def test_a_refused_call_is_reported_once():
+    w = synth.WORKLOADS["tiny"]
+    a, b = B.dkv_create(B.config_of(w)), B.dkv_create(B.config_of(w))
+    d = torch.zeros(w.Bt * w.Hkv * w.S * w.D, device="cuda")
+    try:
+        with stream_that_refuses_work() as stream:
+            launched = B.dkv_launch_count(a)
+            for call in (lambda: B.dkv_select_positions(a, 0, 4, 4, stream), lambda: B.dkv_reset(a, stream),
+                         lambda: B.dkv_score_static(B.config_of(w), d, d, d, stream)):
+                with pytest.raises(B.DkvError) as e:
+                    call()
+                assert e.value.code == B.DKV_ERR_CUDA
+            assert B.dkv_launch_count(a) == launched
+        for ctx in (b, a):
+            B.dkv_select_positions(ctx, 0, 4, 4)
+    finally:
+        B.dkv_destroy(a)
+        B.dkv_destroy(b)
