@@ -877,14 +877,11 @@ int dkv_run_prefill_pass_lse(dkv_ctx* c, const void* const* q_win, const void* c
   return run_pass(c, q_win, k, v, lse, kb, vb, stream);
 }
 
-int dkv_run_prefill_pass_host(dkv_ctx* c, const void* const* q_win, const void* const* k, const void* const* v,
-                              void* const* kb, void* const* vb, int32_t* counts_out) {
-  if (!c || !q_win || !k || !v || !kb || !vb) return DKV_ERR_INVALID_ARG;
+// The host-buffer pass up to its results, on the context's own streams.
+static int host_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, const void* const* v, void* const* kb,
+                     void* const* vb, int32_t* counts_out) {
   const Shape& s = c->s;
-  for (int l = 0; l < s.L; ++l)
-    if (!q_win[l] || !k[l] || !v[l] || !kb[l] || !vb[l]) return DKV_ERR_INVALID_ARG;
-  int rc = ensure_staging(c);
-  if (rc) return rc;
+  int rc;
   cudaStream_t cp = c->st_copy, st = c->st_comp;
   if ((rc = do_reset(c, st))) return rc;
   // Only the kept rows of V are ever needed on the device (count + ws of S per head).  Where the caller's V is
@@ -954,6 +951,26 @@ int dkv_run_prefill_pass_host(dkv_ctx* c, const void* const* q_win, const void* 
   c->host_h2d = h2d; c->host_d2h = d2h;
   DKV_CUDA(c, cudaStreamSynchronize(cp));
   return DKV_OK;
+}
+
+int dkv_run_prefill_pass_host(dkv_ctx* c, const void* const* q_win, const void* const* k, const void* const* v,
+                              void* const* kb, void* const* vb, int32_t* counts_out) {
+  if (!c || !q_win || !k || !v || !kb || !vb) return DKV_ERR_INVALID_ARG;
+  for (int l = 0; l < c->s.L; ++l)
+    if (!q_win[l] || !k[l] || !v[l] || !kb[l] || !vb[l]) return DKV_ERR_INVALID_ARG;
+  int rc = ensure_staging(c);
+  if (!rc) rc = host_pass(c, q_win, k, v, kb, vb, counts_out);
+  if (rc && c->staged) {
+    // what was enqueued before the refused call still reads and writes the caller's buffers: it ends before the call does
+    const int why = c->last_cuda;
+    cudaStreamSynchronize(c->st_copy);
+    cudaStreamSynchronize(c->st_comp);
+    do_reset(c, c->st_comp);
+    cudaStreamSynchronize(c->st_comp);
+    cudaGetLastError();
+    c->last_cuda = why;
+  }
+  return rc;
 }
 
 int dkv_host_pass_bytes(dkv_ctx* c, int64_t* h2d, int64_t* d2h) {

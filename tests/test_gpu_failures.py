@@ -182,3 +182,37 @@ def test_a_refused_call_is_reported_once():
     finally:
         B.dkv_destroy(a)
         B.dkv_destroy(b)
+
+
+def test_a_host_buffer_pass_that_fails_midway_leaves_no_layer():
+    w = synth.WORKLOADS["tiny"]
+    p = _Pass()
+    pin = lambda tensors: [t.cpu().pin_memory() for t in tensors]
+    q, k, v, kb, vb = (pin(x) for x in (p.q, p.k, p.v, p.kb, p.vb))
+    counts, again = (np.zeros((w.Bt, w.L), dtype=np.int32) for _ in range(2))
+    rt = ctypes.CDLL("libcudart.so.12")
+    rt.cudaStreamEndCapture.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+    other, graph = ctypes.c_void_p(torch.cuda.Stream().cuda_stream), ctypes.c_void_p()
+    ctx = B.dkv_create(B.config_of(w))
+    try:
+        B.dkv_run_prefill_pass_host(ctx, q, k, v, kb, vb, counts)
+        # while another stream is captured in the strictest mode the runtime refuses some calls, the read of the counts
+        # into ordinary memory among them
+        assert rt.cudaStreamBeginCapture(other, 0) == 0
+        try:
+            with pytest.raises(B.DkvError) as e:
+                B.dkv_run_prefill_pass_host(ctx, q, k, v, kb, vb, again)
+            assert e.value.code == B.DKV_ERR_CUDA and B.dkv_last_cuda_error(ctx) != 0
+        finally:
+            rt.cudaStreamEndCapture(other, ctypes.byref(graph))
+            rt.cudaGetLastError()
+        for call in (lambda: B.dkv_rebudget(ctx, 1), lambda: p.decode(ctx)):
+            with pytest.raises(B.DkvError) as e:
+                call()
+            assert e.value.code == B.DKV_ERR_STATE
+        B.dkv_get_counts(ctx, again)
+        assert (again == 0).all()
+        B.dkv_run_prefill_pass_host(ctx, q, k, v, kb, vb, again)
+        assert (again == counts).all()
+    finally:
+        B.dkv_destroy(ctx)
