@@ -53,8 +53,8 @@ struct dkv_ctx {
   uint8_t scored[DKV_MAX_LAYERS], gathered[DKV_MAX_LAYERS];
   uint8_t selected[DKV_MAX_LAYERS];     // 1: by scores (dkv_select_topk), 2: by position (dkv_select_positions)
   int sel_n[DKV_MAX_LAYERS];            // positions selected per head: Blc, or what dkv_select_positions kept
-  // decoding over the compressed cache (allocated on first use, grown on demand)
-  float* d_dec_scratch;                 // parts of heads that lie in more than one block's slice
+  // decoding over the compressed cache
+  float* d_dec_scratch;                 // parts of heads that lie in more than one block's slice (allocated on first use, grown on demand)
   size_t dec_scratch_floats;
   unsigned int* d_dec_tickets;          // [L][Bt*Hkv], zero between launches
   long long launches;
@@ -499,10 +499,6 @@ int do_decode(dkv_ctx* c, int layer0, int nl, int nq, const void* const* q, cons
     if (split_grid > most) split_grid = (int)most;
     const int qb = GQ <= 8 ? 8 : 16;
     const size_t need = (size_t)split_grid * 4 * 2 * ((GQ + qb - 1) / qb) * (qb * s.D + qb * 2);
-    if (!c->d_dec_tickets) {
-      DKV_CUDA(c, cudaMalloc(&c->d_dec_tickets, sizeof(unsigned int) * s.L * BH));
-      DKV_CUDA(c, cudaMemset(c->d_dec_tickets, 0, sizeof(unsigned int) * s.L * BH));
-    }
     if (need > c->dec_scratch_floats) {
       if (c->d_dec_scratch) { DKV_CUDA(c, cudaDeviceSynchronize()); cudaFree(c->d_dec_scratch); c->d_dec_scratch = nullptr; c->dec_scratch_floats = 0; }
       DKV_CUDA(c, cudaMalloc(&c->d_dec_scratch, need * sizeof(float)));
@@ -687,6 +683,11 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   TRY(cudaMemset(c->d_count, 0, sizeof(int) * bl));
   TRY(cudaMemset(c->d_held, 0, sizeof(int) * bl));
   TRY(cudaMemset(c->d_dbg, 0, sizeof(int) * 3 * bl));
+  TRY(cudaMalloc(&c->d_dec_tickets, sizeof(unsigned int) * s.L * heads));
+  TRY(cudaMemset(c->d_dec_tickets, 0, sizeof(unsigned int) * s.L * heads));
+  // The words above are cleared on the legacy default stream, for which the first kernel of a caller's non-blocking stream
+  // does not wait.
+  TRY(cudaStreamSynchronize(cudaStreamLegacy));
   // The attributes belong to the functions, not to this context: always the most any valid configuration needs, so that
   // contexts do not undo each other.
   {
@@ -1156,7 +1157,10 @@ int dkv_last_status(dkv_ctx* c, int32_t* host_status) {
   if (!c || !host_status) return DKV_ERR_INVALID_ARG;
   DKV_CUDA(c, cudaDeviceSynchronize());
   DKV_CUDA(c, cudaMemcpy(host_status, c->d_status, sizeof(int) * 8, cudaMemcpyDeviceToHost));
-  if (host_status[0] != 0) DKV_CUDA(c, cudaMemset(c->d_status, 0, sizeof(int) * 8));   // reported once
+  if (host_status[0] != 0) {                   // reported once
+    DKV_CUDA(c, cudaMemset(c->d_status, 0, sizeof(int) * 8));
+    DKV_CUDA(c, cudaStreamSynchronize(cudaStreamLegacy));     // (as in dkv_create)
+  }
   host_status[1] = (int32_t)(c->launches & 0x7FFFFFFF);
   return host_status[0] == 0 ? DKV_OK : DKV_ERR_TIMEOUT;
 }

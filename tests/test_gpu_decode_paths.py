@@ -57,3 +57,28 @@ def test_decode_attention(L, Hkv, G, nq, D, Bt, ws, keep):
         assert all((a - b).abs().max() <= 3e-6 * b.abs().max() for a, b in zip(out, first))
     finally:
         B.dkv_destroy(ctx)
+
+
+def test_first_step_on_a_stream_that_does_not_wait_for_the_default_one():
+    L, Hkv, G, D, S, ws = 10, 8, 4, 128, 700, 8              # heads enough for the slices, which count arrivals
+    g = torch.Generator(device="cuda").manual_seed(7)
+    new = lambda *s: [torch.randn(s, generator=g, device="cuda").to(torch.bfloat16) for _ in range(L)]
+    q, k, v, dq = new(1, Hkv * G, ws, D), new(1, Hkv, S, D), new(1, Hkv, S, D), new(1, Hkv * G, 1, D)
+    kb, vb = ([torch.zeros((1, Hkv, 300 + ws, D), device="cuda", dtype=torch.bfloat16) for _ in range(L)] for _ in range(2))
+    out, again = ([torch.zeros((1, Hkv * G, 1, D), device="cuda") for _ in range(L)] for _ in range(2))
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ctx = B.dkv_create(B.make_config(L, Hkv * G, Hkv, D, 1, S, ws, 3, 100, 300, 2))
+    try:
+        torch.cuda._sleep(200_000_000)                       # the default stream is busy for a tenth of a second
+        B.dkv_run_prefill_pass(ctx, q, k, v, kb, vb, side)
+        B.dkv_decode_attend(ctx, 0, L, 1, dq, kb, vb, out, side)
+        side.synchronize()
+        first = [o.clone() for o in out]
+        torch.cuda.synchronize()
+        B.dkv_run_prefill_pass(ctx, q, k, v, kb, vb)
+        B.dkv_decode_attend(ctx, 0, L, 1, dq, kb, vb, again)
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) and a.abs().max() > 0 for a, b in zip(first, again))
+    finally:
+        B.dkv_destroy(ctx)
