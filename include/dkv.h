@@ -181,18 +181,17 @@ int dkv_compact_all(dkv_ctx* ctx, int32_t upto_layer, void* const* kb, void* con
  * All layers' tensors must be resident when the call is made: the scoring kernel is launched once per group of
  * consecutive layers (sweep 2 of one group, sweep 1 of the next); then all updates run together and every layer is
  * selected and gathered once, with its final count.  The results are those of the layer-by-layer loop.
- * The first call with a given set of pointers records the whole pass as a CUDA graph (on an internal stream);
- * later calls with the same pointers replay it on `stream`, whatever the buffers then contain.  The plain sequence of launches is used instead while dkv_profile is on, when
- * `stream` is itself being captured, or if the capture fails. */
+ * Nothing is kept from one call for the next: buffers not seen before cost what the same ones do.  The call may be
+ * captured into a CUDA graph of the caller's. */
 int dkv_run_prefill_pass(dkv_ctx* ctx, const void* const* q_win, const void* const* k, const void* const* v,
                          void* const* kb, void* const* vb, void* stream);
 
 /* Algorithm 1's loop when the caller's prefill attention kernel has already produced, for every layer, the
  * log-denominators of the window rows (see dkv_score_lse): every layer is scored in one sweep over its keys.
  * lse : HOST array of L device pointers, each fp32 [Bt, Hq, ws] (natural logarithm), 4-byte aligned.
- * Everything else as dkv_run_prefill_pass, including the recording of the pass as a CUDA graph.  (Section 4.3
- * notes that the scoring needs the window rows' attention probabilities explicitly, which a fused attention
- * kernel does not return; its log-denominators are what it does return.) */
+ * Everything else as dkv_run_prefill_pass.  (Section 4.3 notes that the scoring needs the window rows' attention
+ * probabilities explicitly, which a fused attention kernel does not return; its log-denominators are what it does
+ * return.) */
 int dkv_run_prefill_pass_lse(dkv_ctx* ctx, const void* const* q_win, const void* const* k, const void* const* v,
                              const float* const* lse, void* const* kb, void* const* vb, void* stream);
 

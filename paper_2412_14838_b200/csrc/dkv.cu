@@ -58,12 +58,6 @@ struct dkv_ctx {
   size_t dec_scratch_floats;
   unsigned int* d_dec_tickets;          // [L][Bt*Hkv], zero between launches
   long long launches;
-  // dkv_run_prefill_pass as a CUDA graph: captured on the first call with a set of pointers, replayed afterwards
-  bool use_graph;
-  cudaStream_t gstream;        // the graph is captured here
-  cudaGraphExec_t pass_exec;
-  std::vector<const void*>* pass_key;
-  long long pass_launches;
   int last_cuda;
   // optional per-step timing with CUDA events (dkv_profile)
   bool prof_on;
@@ -555,9 +549,6 @@ void free_all(dkv_ctx* c) {
   cudaFree(c->d_rb_state); cudaFree(c->d_rb_above); cudaFree(c->d_layer_hist); cudaFree(c->d_shrink_tickets);
   cudaFree(c->d_cand); cudaFree(c->d_cand_n); cudaFree(c->d_status); cudaFree(c->d_tc_stats);
   cudaFree(c->d_dec_scratch); cudaFree(c->d_dec_tickets);
-  if (c->pass_exec) cudaGraphExecDestroy(c->pass_exec);
-  delete c->pass_key;
-  if (c->gstream) cudaStreamDestroy(c->gstream);
   if (c->prof_recs) {
     for (ProfRec& r : *c->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     delete c->prof_recs;
@@ -674,10 +665,6 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   TRY(cudaMalloc(&c->d_cand_n, sizeof(unsigned int) * s.Bt));
   TRY(cudaMalloc(&c->d_tc_stats, sizeof(float2) * 3 * c->stats_rows * 256));
   TRY(set_score_attributes());
-  TRY(cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking));
-  c->pass_key = new (std::nothrow) std::vector<const void*>();
-  if (!c->pass_key) { free_all(c); delete c; return DKV_ERR_NOMEM; }
-  c->use_graph = env_int("DKV_NO_GRAPH", 0, 0, 1) == 0;
   TRY(cudaMalloc(&c->d_status, sizeof(int) * 8));
   TRY(cudaMemset(c->d_status, 0, sizeof(int) * 8));
   TRY(cudaMemset(c->d_count, 0, sizeof(int) * bl));
@@ -797,9 +784,6 @@ int dkv_compact_all(dkv_ctx* c, int32_t upto_layer, void* const* kb, void* const
   return do_shrink(c, 0, upto_layer, kb, vb, as_stream(stream));
 }
 
-static int enqueue_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, const void* const* v,
-                        const float* const* lse, void* const* kb, void* const* vb, cudaStream_t st);
-
 static int run_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, const void* const* v,
                     const float* const* lse, void* const* kb, void* const* vb, void* stream) {
   if (!c || !q_win || !k || !v || !kb || !vb) return DKV_ERR_INVALID_ARG;
@@ -813,58 +797,13 @@ static int run_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, 
   // with is needed on the device only if a launch is refused midway.
   cudaStream_t st = as_stream(stream);
   forget_layers(c);
-  const int rc = enqueue_pass(c, q_win, k, v, lse, kb, vb, st);
+  const int rc = do_pass(c, q_win, k, v, lse, kb, vb, st);
   if (rc) {
     const int why = c->last_cuda;
     do_reset(c, st);
     c->last_cuda = why;
   }
   return rc;
-}
-
-static int enqueue_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, const void* const* v,
-                        const float* const* lse, void* const* kb, void* const* vb, cudaStream_t st) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusNone; }
-  // per-step profiling needs its events between the launches; a caller that is capturing gets the plain calls
-  if (!c->use_graph || c->prof_on || cap != cudaStreamCaptureStatusNone) return do_pass(c, q_win, k, v, lse, kb, vb, st);
-
-  std::vector<const void*> key;
-  key.reserve(6 * (size_t)c->s.L);
-  for (int l = 0; l < c->s.L; ++l) {
-    key.push_back(q_win[l]); key.push_back(k[l]); key.push_back(v[l]); key.push_back(kb[l]); key.push_back(vb[l]);
-    key.push_back(lse ? lse[l] : nullptr);
-  }
-  if (!c->pass_exec || *c->pass_key != key) {
-    // first call with these buffers: record the whole pass
-    if (c->pass_exec) { cudaGraphExecDestroy(c->pass_exec); c->pass_exec = nullptr; }
-    const long long before = c->launches;
-    cudaGraph_t graph = nullptr;
-    DKV_CUDA(c, cudaStreamBeginCapture(c->gstream, cudaStreamCaptureModeThreadLocal));
-    const int rc = do_pass(c, q_win, k, v, lse, kb, vb, c->gstream);
-    const cudaError_t e = cudaStreamEndCapture(c->gstream, &graph);
-    if (rc != DKV_OK || e != cudaSuccess || !graph) {
-      if (graph) cudaGraphDestroy(graph);
-      cudaGetLastError();
-      c->launches = before;
-      c->use_graph = false;                         // not capturable here: run the plain calls from now on
-      return do_pass(c, q_win, k, v, lse, kb, vb, st);
-    }
-    c->pass_launches = c->launches - before;
-    c->launches = before;
-    const cudaError_t ei = cudaGraphInstantiate(&c->pass_exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (ei != cudaSuccess) {
-      cudaGetLastError();
-      c->pass_exec = nullptr; c->use_graph = false;
-      return do_pass(c, q_win, k, v, lse, kb, vb, st);
-    }
-    *c->pass_key = key;
-  }
-  DKV_CUDA(c, cudaGraphLaunch(c->pass_exec, st));
-  c->launches += c->pass_launches;
-  mark_pass_done(c);
-  return DKV_OK;
 }
 
 int dkv_run_prefill_pass(dkv_ctx* c, const void* const* q_win, const void* const* k, const void* const* v,
@@ -1176,7 +1115,6 @@ int dkv_static_last_status(int32_t* host_status) {
 int dkv_set_wait_limit(dkv_ctx* c, int64_t clock_ticks) {
   if (!c || clock_ticks < 1000) return DKV_ERR_INVALID_ARG;
   c->wait_cycles = clock_ticks;
-  if (c->pass_exec) { cudaGraphExecDestroy(c->pass_exec); c->pass_exec = nullptr; }   // recorded with the old limit
   return DKV_OK;
 }
 
@@ -1184,7 +1122,6 @@ int dkv_debug_withhold_tile(dkv_ctx* c, int32_t sweep, int32_t tile) {
   if (!c || (tile >= 0 && sweep != 1 && sweep != 2)) return DKV_ERR_INVALID_ARG;
   c->withhold_sweep = tile >= 0 ? sweep : -1;
   c->withhold_tile = tile >= 0 ? tile : -1;
-  if (c->pass_exec) { cudaGraphExecDestroy(c->pass_exec); c->pass_exec = nullptr; }
   return DKV_OK;
 }
 

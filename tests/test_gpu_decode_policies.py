@@ -153,7 +153,7 @@ def test_pass_scored_from_log_denominators_matches_oracle(name):
         check_properties(g)
         near = compare_full(g)          # the oracle's two-sweep pass: the same quantity up to the rounding of lse
         assert near <= 8
-        g.run()                          # replayed graph
+        g.run()                          # a second pass
         check_properties(g)
     finally:
         g.close()
