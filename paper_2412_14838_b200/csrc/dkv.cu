@@ -260,13 +260,11 @@ auto score_kernel(int M, int D) {
   return M == 128 && D == 128 ? tc::score_tc_kernel<NL, true, 1> : query_copies(M) == 4 ? tc::score_tc_kernel<NL, false, 4>
        : query_copies(M) == 2 ? tc::score_tc_kernel<NL, false, 2> : tc::score_tc_kernel<NL, false, 1>;
 }
-cudaError_t set_score_attributes() {
-  for (const int* s : (const int[][2]){{128, 128}, {32, 128}, {64, 128}, {256, 128}})
-    for (const void* f : {(const void*)score_kernel<1>(s[0], s[1]), (const void*)score_kernel<tc::kMaxGroup>(s[0], s[1])}) {
-      const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes);
-      if (e != cudaSuccess) return e;
-    }
-  return cudaSuccess;
+// The build's shared memory, per function and device: set before its first launch, and only for the builds that a caller can
+// reach, since each is loaded onto the device by it.
+template <int NL>
+cudaError_t set_score_attribute(int M, int D) {
+  return cudaFuncSetAttribute(score_kernel<NL>(M, D), cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes);
 }
 template <int NL>
 cudaError_t launch_tc(int grid, cudaStream_t st, const tc::Maps<NL>& m0, const tc::Maps<NL>& m1, const tc::Params& j0, const tc::Params& j1) {
@@ -664,7 +662,8 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   TRY(cudaMalloc(&c->d_cand, sizeof(uint2) * s.L * layer_scores(s)));
   TRY(cudaMalloc(&c->d_cand_n, sizeof(unsigned int) * s.Bt));
   TRY(cudaMalloc(&c->d_tc_stats, sizeof(float2) * 3 * c->stats_rows * 256));
-  TRY(set_score_attributes());
+  TRY(set_score_attribute<1>(s.M, s.D));
+  TRY(set_score_attribute<tc::kMaxGroup>(s.M, s.D));
   TRY(cudaMalloc(&c->d_status, sizeof(int) * 8));
   TRY(cudaMemset(c->d_status, 0, sizeof(int) * 8));
   TRY(cudaMemset(c->d_count, 0, sizeof(int) * bl));
@@ -1033,7 +1032,8 @@ int dkv_score_static(const dkv_config* cfg, const void* q_win, const void* k, fl
       int sms = 0;
       DKV_CUDA(nullptr, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
       if (!ptr || sms < 1) return DKV_ERR_CUDA;
-      DKV_CUDA(nullptr, set_score_attributes());
+      for (const int* m : (const int[][2]){{128, 128}, {32, 128}, {64, 128}, {256, 128}})      // later calls may have any shape
+        DKV_CUDA(nullptr, set_score_attribute<1>(m[0], m[1]));
       g.ptr = static_cast<unsigned char*>(ptr);
       g.sms = sms;
       g.done = true;
