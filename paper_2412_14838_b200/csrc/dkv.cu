@@ -542,6 +542,17 @@ int do_pass(dkv_ctx* c, const void* const* q, const void* const* k, const void* 
   return DKV_OK;
 }
 
+// All of it, or as much as there is of it.
+void free_staging(dkv_ctx* c) {
+  for (int i = 0; i < 2; ++i) {
+    for (void** p : {&c->st_q[i], &c->st_k[i], &c->st_v[i]}) { cudaFree(*p); *p = nullptr; }
+    for (cudaEvent_t* e : {&c->ev_copied[i], &c->ev_consumed[i]}) if (*e) { cudaEventDestroy(*e); *e = nullptr; }
+  }
+  for (int l = 0; l < c->s.L; ++l) for (void** p : {&c->st_kb[l], &c->st_vb[l]}) { cudaFree(*p); *p = nullptr; }
+  for (cudaStream_t* s : {&c->st_copy, &c->st_comp}) if (*s) { cudaStreamDestroy(*s); *s = nullptr; }
+  c->staged = false;
+}
+
 void free_all(dkv_ctx* c) {
   cudaFree(c->d_scores); cudaFree(c->d_idx); cudaFree(c->d_count); cudaFree(c->d_held); cudaFree(c->d_dbg);
   cudaFree(c->d_rb_state); cudaFree(c->d_rb_above); cudaFree(c->d_layer_hist); cudaFree(c->d_shrink_tickets);
@@ -551,18 +562,10 @@ void free_all(dkv_ctx* c) {
     for (ProfRec& r : *c->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     delete c->prof_recs;
   }
-  if (c->staged) {
-    for (int i = 0; i < 2; ++i) {
-      cudaFree(c->st_q[i]); cudaFree(c->st_k[i]); cudaFree(c->st_v[i]);
-      cudaEventDestroy(c->ev_copied[i]); cudaEventDestroy(c->ev_consumed[i]);
-    }
-    for (int l = 0; l < c->s.L; ++l) { cudaFree(c->st_kb[l]); cudaFree(c->st_vb[l]); }
-    cudaStreamDestroy(c->st_copy); cudaStreamDestroy(c->st_comp);
-  }
+  free_staging(c);
 }
 
-int ensure_staging(dkv_ctx* c) {
-  if (c->staged) return DKV_OK;
+int make_staging(dkv_ctx* c) {
   const Shape& s = c->s;
   for (int i = 0; i < 2; ++i) {
     DKV_CUDA(c, cudaMalloc(&c->st_q[i], layer_q_bytes(s)));
@@ -577,8 +580,15 @@ int ensure_staging(dkv_ctx* c) {
   }
   DKV_CUDA(c, cudaStreamCreateWithFlags(&c->st_copy, cudaStreamNonBlocking));
   DKV_CUDA(c, cudaStreamCreateWithFlags(&c->st_comp, cudaStreamNonBlocking));
-  c->staged = true;
   return DKV_OK;
+}
+
+int ensure_staging(dkv_ctx* c) {
+  if (c->staged) return DKV_OK;
+  const int rc = make_staging(c);
+  if (rc) free_staging(c);                     // a later call starts anew
+  c->staged = rc == DKV_OK;
+  return rc;
 }
 
 }  // namespace

@@ -216,3 +216,25 @@ def test_a_host_buffer_pass_that_fails_midway_leaves_no_layer():
         assert (again == counts).all()
     finally:
         B.dkv_destroy(ctx)
+
+
+def test_a_host_buffer_pass_that_finds_too_little_memory_keeps_none_of_it():
+    # two layers of keys and values in flight: 2 x 3 x 512 MB of staging
+    w = synth.Workload("staging", 73, L=2, Hq=8, Hkv=8, D=128, Bt=8, S=32768, ws=8, pool=3, N=16, Bl=32, m=1, recipe="iid")
+    some = torch.zeros(1 << 20, dtype=torch.uint8)            # never read: the call fails before it copies anything
+    counts = np.zeros((w.Bt, w.L), dtype=np.int32)
+    torch.cuda.empty_cache()
+    ctx = B.dkv_create(B.config_of(w))
+    free = torch.cuda.mem_get_info()[0]
+    taken = torch.empty(free - (900 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        before = torch.cuda.mem_get_info()[0]
+        for _ in range(3):
+            with pytest.raises(B.DkvError) as e:
+                B.dkv_run_prefill_pass_host(ctx, *[[some] * w.L] * 5, counts)
+            assert e.value.code == B.DKV_ERR_NOMEM
+        assert torch.cuda.mem_get_info()[0] > before - (64 << 20)
+    finally:
+        del taken
+        torch.cuda.empty_cache()
+        B.dkv_destroy(ctx)
