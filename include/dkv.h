@@ -55,7 +55,7 @@ extern "C" {
                                     t_i = (cnt_i - min)/(max - min), all 1 if every layer counts the same  */
 #define DKV_F_ALL          0x7u
 
-typedef struct dkv_ctx dkv_ctx;     /* opaque; owns score history, kept indices, ranks, counts, workspace */
+typedef struct dkv_ctx dkv_ctx;     /* opaque; owns score history, kept indices, counts, workspace */
 
 /* Problem statement of Algorithm 1 (its inputs r_max, m, wt, ws, S, d_k) plus the model shape. */
 typedef struct {
@@ -75,7 +75,10 @@ typedef struct {
 } dkv_config;
 
 /* Create a context for `cfg` on the current device (host call; allocates device memory:
- * score history 4*L*Bt*Hkv*P bytes, kept indices and ranks 8*L*Bt*Hkv*Bl' bytes, small workspaces).
+ * score history 4*L*Bt*Hkv*P bytes, candidates of the global top-K 8*L*Bt*Hkv*P, kept indices 4*L*Bt*Hkv*Bl', digit
+ * counts 8192*L*Bt, partial softmax statistics 6144 * (SM count + 64*Bt*Hkv), small workspaces; the
+ * staging of the host-buffer pass (q, k, v of two layers, kb, vb of all) and the decoding scratch come with the first
+ * call that needs them).
  * Errors: INVALID_ARG, UNSUPPORTED, NOMEM, CUDA.  On error *out is NULL. */
 int dkv_create(const dkv_config* cfg, dkv_ctx** out);
 /* Free everything the context owns (synchronises the device). */
@@ -198,8 +201,9 @@ int dkv_run_prefill_pass_lse(dkv_ctx* ctx, const void* const* q_win, const void*
 /* The same pass with all tensors in HOST memory (pinned memory recommended): each layer's q and k
  * are copied to device staging buffers owned by the context and processed; of v only the kept rows are
  * needed (Algorithm 1 gathers V_c at the selected indices), so where v[l] is page-locked memory that
- * kernels can address (cudaHostAlloc / cudaHostRegister) the gather reads those rows in place and the
- * rest of v never crosses the bus; pageable v is copied in full like k.  After the last update
+ * kernels can address (cudaHostAlloc / cudaHostRegister) the gather reads the Bl' best rows and the window in place and
+ * the rest of v never crosses the bus; pageable v is copied in full like k.  A buffer is page-locked as a whole or not
+ * at all.  After the last update
  * the counts and, of every layer's kb/vb, the valid rows of every head (count + ws; the rest of the
  * fixed-stride host buffers is left untouched) are copied back: by one kernel that writes them in place where every
  * kb[l] and vb[l] is page-locked and 16-byte aligned, else by strided copies.  Synchronises.

@@ -289,7 +289,8 @@ struct DecodeMerge {
 // Few heads (a step over one layer or a few): one cluster of gridDim.x blocks per head, its row blocks dealt out to
 // all warps of the cluster.  Every block pushes the pieces of its result into the shared memory of the block that
 // owns the piece, so one cluster barrier is all the merge waits for.  With 8 heads of 500 rows every warp has at most
-// one or two row blocks: a call is one round of loads plus the merge.
+// one or two row blocks: a call is one round of loads plus the merge.  It is the device that bounds a step made of such
+// calls: 5.4 us a call with the queue full (8 heads of about 500 rows), where the host needs 3.1.
 // grid (cluster size <= 8, Bt*Hkv, layers).
 template <int D, int QB, int NW>
 __global__ void __launch_bounds__(NW * 32)
@@ -358,10 +359,10 @@ decode_cluster_kernel(const __grid_constant__ DecodePtrs ptrs, const __grid_cons
 // into merging warps).  A head counts kDecHeadCost blocks more than it has: its set-up and its results.  A head that
 // lies in one slice is finished there; of the others every warp leaves its part in scratch, as it lies in its
 // registers, and the warp that arrives last for a head (a ticket per head) merges the parts in slice order.
-// Two blocks of four warps an SM: at 255 registers nothing spills; three at 168 were 8 % slower, and requesting the
-// next row block before the current one is worked on gains nothing here.  Measured (32 layers, caches colder than L2):
-// 33 us for four queries over 67 MB, 21 us for one over 47 MB of 1024 short heads, where the launch, the lengths'
-// prefix sums and two or three heads' load latencies per warp are most of the time.
+// Two blocks of four warps an SM: at the 255 registers that leaves (254 used at most) nothing spills; three at 168 were
+// 8 % slower, and requesting the next row block before the current one is worked on gains nothing here.  Measured (32
+// layers, caches colder than L2): 32 us for four queries over 67 MB, 21 us for one over 47 MB of 1024 short heads, where
+// the launch, the lengths' prefix sums and two or three heads' load latencies per warp are most of the time.
 // Dynamic shared memory: nl*Bt + 1 integers.
 constexpr int kDecHeadCost = 2;   // 1 to 4 measured: within 1 %, 3 and 4 slower for short heads
 template <int D, int QB, int NW>

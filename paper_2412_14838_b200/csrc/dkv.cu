@@ -480,7 +480,7 @@ int do_decode(dkv_ctx* c, int layer0, int nl, int nq, const void* const* q, cons
   a.scale2 = kLog2e / sqrtf((float)s.D);
   a.held = c->d_held; a.scratch = nullptr; a.tickets = nullptr;
   // A cluster per head while the heads alone leave SMs idle (as many blocks a head as fit one wave, at most the
-  // portable 8, and one row block a warp at least); equal slices of all rows once there is a head per SM or so.
+  // portable 8, and one row block a warp at least); equal slices of all rows from a head per four SMs on.
   int cluster = 1, split_grid = 0;
   const int warps = GQ <= 8 ? 8 : 4;
   while (cluster < 8 && heads * cluster * 2 <= c->n_sms && cluster * warps * kDecRowBlock < s.rows) cluster *= 2;

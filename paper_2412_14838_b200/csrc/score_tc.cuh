@@ -28,7 +28,6 @@ constexpr int kMmaWarp2 = 18;
 constexpr int kStages = 4;                 // K tiles in flight
 constexpr int kThreads = 608;              // warp 0: TMA, warps 1 and 18: MMA (even / odd tiles), warps 2..17: softmax
 constexpr int kSoftmaxThreads = 512;
-constexpr int kParts = 4;                  // softmax warps per TMEM lane quadrant: 2 tile groups x 2 column halves
 constexpr int kMaxSegTiles = 16;           // sweep 2: tiles per pooled segment
 // TMEM accumulator stages: four of 128 columns when the window rows fit one 128-row block (ws*G <= 128),
 // else two of 256.  A softmax group then always has a second accumulator being filled while it reads one.
