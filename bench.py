@@ -32,19 +32,18 @@ UNIT = "tokens/s"
 DEFAULT_WORKLOAD = "mistral32k"
 NOMINAL_HBM_GBS = 8000.0
 
-# DRAM traffic of one full scoring launch (dram__bytes_read.sum + dram__bytes_write.sum): sweep 2 of four layers
-# followed by sweep 1 of the next four, taken with ncu on the 8-layer cut of the mistral32k shape (same per-layer
-# shape and group size, so the figure needs no scaling; see profiles/score_tc_kernel_mistral32k_8layers.md).
-# "live" is a single-pass capture without ncu's cache flush, i.e. with whatever the previous launch left in L2, as
-# in a real pass; "cold" is the --set full capture, where every replay starts from flushed caches.  Both hold for
-# the kernel source they were measured on, for that per-layer shape and for four-layer groups only: any other
-# source hash, shape or grouping reports null.
+# DRAM traffic of one full scoring launch (dram__bytes_read.sum + dram__bytes_write.sum): sweep 2 of a group of layers
+# followed by sweep 1 of the next, taken with ncu on the 16-layer cut of the mistral32k shape (same per-layer shape and
+# group size, so the figure needs no scaling; see profiles/score_tc_kernel_mistral32k_16layers.md).  "live" is a
+# single-pass capture without ncu's cache flush, i.e. with whatever the previous launch left in L2, as in a real pass;
+# "cold" starts from flushed caches.  Both hold for the kernel source they were measured on, for that per-layer shape
+# and for groups of that many layers only: any other source hash, shape or grouping reports null.
 NCU_TRAFFIC = {
-    "kernel_sha256": "303acb3e0fa3bf64ba7b5cb1069bb408c1cc9088dab894f6a69887c302ea26de",
+    "kernel_sha256": "54a6664d8c8e2746ff04426daa3dea882238f1d62f30c823f6b0c26fcdbc2e1c",
     "shape": (8, 128, 1, 32768, 32),          # Hkv, D, Bt, S, ws
-    "layers_per_launch": 4,
-    "live_bytes_per_launch": 478_000_384 + 28_855_296,
-    "cold_bytes_per_launch": 540_321_280 + 6_633_728,
+    "layers_per_launch": 8,
+    "live_bytes_per_launch": 1_019_605_504 + 23_030_016,
+    "cold_bytes_per_launch": 1_081_276_416 + 9_970_944,
 }
 
 
@@ -60,8 +59,10 @@ def ncu_traffic(w, score_launches=None):
         return None
     g = NCU_TRAFFIC["layers_per_launch"]
     if w.L % g or score_launches is None or round(score_launches) != w.L // g + 1:
-        return None                             # the pass was not run in full four-layer groups
+        return None                             # the pass was not run in full groups of that many layers
     return NCU_TRAFFIC
+
+
 FALLBACK_HBM_GBS = 6650.0
 
 
