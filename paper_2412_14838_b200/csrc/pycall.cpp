@@ -19,10 +19,11 @@ namespace {
 
 constexpr Py_ssize_t kMaxList = 4096;       // longest list of per-layer tensors taken
 
-// Address of a torch tensor, an integer, None (NULL), or of anything with data_ptr() or a numpy-like .ctypes.data.
+// Address of a torch tensor, an integer, None (NULL), or of anything with data_ptr() (a tensor subclass may have its own)
+// or a numpy-like .ctypes.data.
 bool address(PyObject* x, void** out) {
   if (x == Py_None) { *out = nullptr; return true; }
-  if (THPVariable_Check(x)) { *out = THPVariable_Unpack(x).data_ptr(); return true; }
+  if (THPVariable_CheckExact(x)) { *out = THPVariable_Unpack(x).data_ptr(); return true; }
   PyObject* v = nullptr;
   if (PyLong_Check(x)) {
     v = x;

@@ -49,25 +49,42 @@ int dkv_run_prefill_pass(void* ctx, const void* const* q, const void* const* k, 
   return n;
 }
 """
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-def test_lists_of_any_length_end_in_nulls(tmp_path):
+@pytest.fixture
+def stand_in(tmp_path):
     (tmp_path / "stand_in.c").write_text(STAND_IN)
     lib = str(tmp_path / "stand_in.so")
     subprocess.run(["gcc", "-shared", "-fPIC", "-o", lib, str(tmp_path / "stand_in.c")], check=True)
+    return lib
+
+
+def test_lists_of_any_length_end_in_nulls(stand_in):
     code = ("from paper_2412_14838_b200 import binding as B; B.load()\n"
             "print([B._native().run_prefill_pass(0, [8] * n, [], [], [], [], 0) for n in (0, 1, 64, 65, 100, 127, 128, 200)])")
     # fresh memory is filled with a pattern, so that an entry that was never written is not NULL by chance
-    env = dict(os.environ, LD_PRELOAD=lib, MALLOC_PERTURB_="90", PYTHONMALLOC="malloc")
-    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    res = subprocess.run([sys.executable, "-c", code], cwd=root, env=env, capture_output=True, text=True, check=True)
+    env = dict(os.environ, LD_PRELOAD=stand_in, MALLOC_PERTURB_="90", PYTHONMALLOC="malloc")
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=env, capture_output=True, text=True, check=True)
     assert res.stdout.strip() == "[0, 1, 64, 65, 100, 127, 128, 128]"
 
 
-def test_a_program_without_torch_makes_the_same_calls(tmp_path):
-    (tmp_path / "stand_in.c").write_text(STAND_IN)
-    lib = str(tmp_path / "stand_in.so")
-    subprocess.run(["gcc", "-shared", "-fPIC", "-o", lib, str(tmp_path / "stand_in.c")], check=True)
+def test_a_tensor_subclass_gives_its_own_address(stand_in):
+    code = """
+import torch
+from paper_2412_14838_b200 import binding as B; B.load()
+class Elsewhere(torch.Tensor):
+    def data_ptr(self): return 0
+class Plain(torch.Tensor): pass
+t = torch.zeros(4)
+items = [t, t.as_subclass(Elsewhere), t.as_subclass(Plain), torch.nn.Parameter(t), t.as_subclass(Elsewhere)]
+print(B._native().run_prefill_pass(0, items, [], [], [], [], 0))
+"""
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, LD_PRELOAD=stand_in), capture_output=True, text=True, check=True)
+    assert res.stdout.strip() == "3"
+
+
+def test_a_program_without_torch_makes_the_same_calls(stand_in):
     code = f"""
 import sys
 sys.modules["torch"] = None                                   # "import torch" fails
@@ -88,13 +105,12 @@ raises(OverflowError, lambda: B.dkv_select_topk(0, 2**32, stream=0))
 raises(TypeError, lambda: B.dkv_reset(0))                      # no stream, no torch whose current one to take
 raises(TypeError, lambda: B.dkv_compact_all(0, 1, ["x"], [a], 0))
 seen = []
-stand_in = ctypes.CDLL({lib!r}).dkv_run_prefill_pass           # the converted list as the library sees it
+library = ctypes.CDLL({stand_in!r}).dkv_run_prefill_pass           # the converted list as the library sees it
 for n in (0, 1, 127, 128, 200):
-    seen.append(stand_in(None, B._argument(ctypes.POINTER(ctypes.c_void_p), [8] * n)))
+    seen.append(library(None, B._argument(ctypes.POINTER(ctypes.c_void_p), [8] * n)))
 assert seen == [0, 1, 127, 128, 128], seen
 """
-    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    subprocess.run([sys.executable, "-c", code], cwd=root, check=True)
+    subprocess.run([sys.executable, "-c", code], cwd=ROOT, check=True)
 
 
 @pytest.mark.parametrize("value", [2**31, 2**32, 2**32 + 1, -2**31 - 1, 2**70])
