@@ -75,8 +75,10 @@ typedef struct {
 } dkv_config;
 
 /* Create a context for `cfg` on the current device (host call; allocates device memory:
- * score history 4*L*Bt*Hkv*P bytes, candidates of the global top-K 8*L*Bt*Hkv*P, kept indices 4*L*Bt*Hkv*Bl', digit
- * counts 8192*L*Bt, partial softmax statistics 6144 * (SM count + 64*Bt*Hkv), small workspaces; the
+ * score history 4*L*Bt*Hkv*P bytes, candidates of the global top-K 8*L*Bt*Hkv*P (while a pass scores, its unpooled scores:
+ * at least 4 bytes per key of min(L, 32) layers, S rounded up to 128, twice that from 129 window rows on), kept indices
+ * 4*L*Bt*Hkv*Bl', digit counts 8192*L*Bt, partial softmax statistics 6144 * (SM count + 64*Bt*Hkv) and
+ * 16 * window rows * (SM count + min(L, 32)*Bt*Hkv), small workspaces; the
  * staging of the host-buffer pass (q, k, v of two layers, kb, vb of all) and the decoding scratch come with the first
  * call that needs them).
  * Errors: INVALID_ARG, UNSUPPORTED, NOMEM, CUDA.  On error *out is NULL. */
@@ -181,8 +183,8 @@ int dkv_compact_all(dkv_ctx* ctx, int32_t upto_layer, void* const* kb, void* con
 /* Algorithm 1's loop over all L layers: score, select, gather each layer; after every m-th layer (and
  * after the last one if L % m != 0) rebudget and shrink all preceding layers.  Resets the context first.
  * q_win, k, v, kb, vb : HOST arrays of L device pointers (layouts as above).
- * All layers' tensors must be resident when the call is made: the scoring kernel is launched once per group of
- * consecutive layers (sweep 2 of one group, sweep 1 of the next); then all updates run together and every layer is
+ * All layers' tensors must be resident when the call is made: a scoring launch covers a group of consecutive layers
+ * (up to 32); then all updates run together and every layer is
  * selected and gathered once, with its final count.  The results are those of the layer-by-layer loop.
  * Nothing is kept from one call for the next: buffers not seen before cost what the same ones do.  The call may be
  * captured into a CUDA graph of the caller's. */
@@ -290,7 +292,7 @@ int dkv_debug_withhold_tile(dkv_ctx* ctx, int32_t sweep, int32_t tile);
  * (DKV_STEP_*), the summed event time in milliseconds and the number of kernels covered since the
  * last read, then clears the sums.  ms, launches : host arrays of DKV_N_STEPS entries. */
 #define DKV_STEP_SCORE_STATS 0   /* sweep 1 of the scoring: softmax statistics per window row */
-#define DKV_STEP_SCORE_EMIT  1   /* sweep 2 of the scoring: per-token sums, pooled             */
+#define DKV_STEP_SCORE_EMIT  1   /* sweep 2 of the scoring: per-token sums, pooled (in a pass perhaps by a launch of its own) */
 #define DKV_STEP_SELECT      2
 #define DKV_STEP_GATHER      3
 #define DKV_STEP_REBUDGET    4

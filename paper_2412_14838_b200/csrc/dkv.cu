@@ -4,6 +4,7 @@
 #include <stdint.h>
 #include <stdlib.h>
 #include <string.h>
+#include <algorithm>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -13,10 +14,13 @@
 #include "compact.cuh"
 #include "decode.cuh"
 #include "rebudget.cuh"
+#include "score_sweep.cuh"
 #include "score_tc.cuh"
 #include "select.cuh"
 
 using namespace dkv;
+using sweep::pool_kernel;
+using sweep::score_sweep_kernel;
 
 struct ProfRec { cudaEvent_t a, b; int step; int launches; };
 
@@ -31,7 +35,8 @@ struct dkv_ctx {
   int* d_held;          // [Bt][L] rows the layer's buffers hold
   int* d_dbg;           // 3 x [Bt][L] : cnt, Z, Z' of the last update
   unsigned int* d_layer_hist; // [L][Bt][2048] digit histogram of every layer's scores (all heads of a sample)
-  uint2* d_cand;              // [Bt][L*Hkv*P] (score bits, layer) of the scores with the digit of a global top-K's threshold
+  uint2* d_cand;              // [Bt][L*Hkv*P] (score bits, layer) of the scores with the digit of a global top-K's threshold;
+                              // while a pass scores, its unpooled scores: float [layers of a launch][heads][planes][tiles * 128]
   unsigned int* d_cand_n;     // [Bt]
   RbState* d_rb_state;        // [kRbUpdates][Bt]
   unsigned int* d_rb_above;   // [kRbUpdates][Bt][L]
@@ -48,6 +53,9 @@ struct dkv_ctx {
   int retain_mb;        // MB of a sweep-1 job's keys (the end of every CTA's slice) marked to stay in L2 for sweep 2
   long long wait_cycles;   // limit of the scoring kernel's mbarrier waits (dkv_set_wait_limit)
   int withhold_sweep, withhold_tile;   // test hook of dkv_debug_withhold_tile (-1: off)
+  // passes scored by score_sweep.cuh
+  float2* d_stats;      // row sums of a head's segments
+  int planes, plane_rows;  // window rows of a head: planes of at most 128
   float2* d_tc_stats;   // [3][stats_rows][256]: partial softmax statistics, three jobs in rotation, each [heads][slots][256]
   // host state
   uint8_t scored[DKV_MAX_LAYERS], gathered[DKV_MAX_LAYERS];
@@ -301,6 +309,95 @@ int launch_score(dkv_ctx* c, const ScoreGroup* e, ScoreGroup* s, const void* con
   return DKV_OK;
 }
 
+// ---- scoring of a pass (score_sweep.cuh) ---------------------------------------------------------
+int tiles_per_head(const Shape& s) { return (s.S + tc::kTileKeys - 1) / tc::kTileKeys; }
+int row_blocks(const dkv_ctx* c) { return (c->plane_rows + 31) / 32 * 4; }              // the kernel's NB
+int most_layers(const dkv_ctx* c) { return c->s.L < tc::kMaxGroup ? c->s.L : tc::kMaxGroup; }
+// Segments a (head, plane) can have in a launch over nl layers: its share of the pipes, one cut at either end.
+int stats_places(const dkv_ctx* c, int nl) { return 2 * c->n_sms / (nl * c->s.Bt * c->s.Hkv * c->planes) + 2; }
+
+// Calls f with the kernel of this context's shape for one sweep, and its shared memory.
+template <int kSweep, typename F>
+cudaError_t with_sweep_kernel(int nb, F f) {
+  switch (nb) {
+    case 4: return f(score_sweep_kernel<4, kSweep>, (int)sweep::Shape1<4>::kSmem);
+    case 8: return f(score_sweep_kernel<8, kSweep>, (int)sweep::Shape1<8>::kSmem);
+    case 12: return f(score_sweep_kernel<12, kSweep>, (int)sweep::Shape1<12>::kSmem);
+    default: return f(score_sweep_kernel<16, kSweep>, (int)sweep::Shape1<16>::kSmem);
+  }
+}
+// The builds' shared memory, per function and device: set before their first launch, and only for the builds that a caller can
+// reach, since each is loaded onto the device by it.
+cudaError_t set_sweep_attributes(int nb) {
+  auto set = [](auto kernel, int smem) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
+  cudaError_t e = set(pool_kernel, 0);
+  if (e == cudaSuccess) e = with_sweep_kernel<sweep::kRowSums>(nb, set);
+  if (e == cudaSuccess) e = with_sweep_kernel<sweep::kKeySums>(nb, set);
+  return e != cudaSuccess ? e : with_sweep_kernel<sweep::kGivenSums>(nb, set);
+}
+
+// Which of the two scoring kernels takes a pass.  With the caller's normalisers it is always score_sweep.cuh, and for one layer at a
+// time always score_tc.cuh, which has a launch less and pools in it (a layer of 32K with normalisers 18.3 us a call, by sweeps 23.1;
+// without, 8 layers of 4K call by call 253-298 us against 278-328).  score_tc.cuh remains for 128 window rows of 128 dims, for
+// which it has a build, while an SM has few tiles (8 layers of 4K, 4 heads: 58 us against 65; 32 of 8K, 110 tiles an SM: 285 / 283;
+// 32 of 32K, 443: 1046 / 1024; 4 x 16K, 886: 2013 / 1955), and where planes of 32, 64, 96 or 128 rows leave many rows empty (224
+// rows, 28 layers of 16K: 423 / 454).
+bool pass_by_sweeps(const dkv_ctx* c) {
+  const Shape& s = c->s;
+  if (s.M == 128 && s.D == 128)
+    return (long long)s.L * s.Bt * s.Hkv * tiles_per_head(s) >= 200ll * c->n_sms;
+  return c->planes == 1 || c->planes * ((c->plane_rows + 31) / 32 * 32) - s.M <= 16;
+}
+
+// Scores of a pass's `nl` consecutive layers from `layer`, and their digits: row sums, key sums and pooling, or with the caller's
+// normalisers the last two.  q, k, lse (or null): the layers' pointers.
+int launch_sweeps(dkv_ctx* c, int layer, int nl, const void* const* q, const void* const* k, const float* const* lse, cudaStream_t st) {
+  const Shape& s = c->s;
+  const int heads = s.Bt * s.Hkv, nb = row_blocks(c), tph = tiles_per_head(s);
+  sweep::Layers maps;                        // only the first nl entries are filled in and read
+  for (int i = 0; i < nl; ++i) {
+    if (!make_map(&maps.q[i], q[i], s.D, s.M, heads, 8 * nb) || !make_map(&maps.k[i], k[i], s.D, s.S, heads)) return DKV_ERR_CUDA;
+    maps.lse[i] = lse ? lse[i] : nullptr;
+    maps.q_at[i] = static_cast<const uint4*>(q[i]); maps.k_at[i] = static_cast<const uint4*>(k[i]);
+  }
+  sweep::Args a;
+  memset(&a, 0, sizeof a);
+  a.S = s.S; a.P = s.P; a.ws = s.ws; a.M = s.M; a.D = s.D;
+  a.planes = c->planes; a.plane_rows = c->plane_rows;
+  a.tph = tph;
+  a.hpl = heads; a.vheads = nl * heads * c->planes;
+  a.scale2 = kLog2e / sqrtf((float)s.D);
+  a.post = (c->cfg.flags & DKV_F_WINDOW_MEAN) ? 1.0f / (float)s.M : 1.0f;
+  a.idesc = make_idesc(128, 8 * nb);         // columns past the window rows are zero logits
+  a.raw = reinterpret_cast<float*>(c->d_cand);
+  a.stats = c->d_stats; a.slots = stats_places(c, nl);
+  a.hist = c->d_layer_hist + (size_t)layer * s.Bt * kBins;
+  a.hist_n = nl * s.Bt * kBins;
+  a.status = c->d_status;
+  a.wait_cycles = c->wait_cycles;
+  const long long tiles = (long long)a.vheads * tph;
+  const dim3 grid((unsigned int)((tiles + 1) / 2 < c->n_sms ? (tiles + 1) / 2 : c->n_sms));
+  auto launch = [&](auto score_kernel, int smem) { return launch_pdl(score_kernel, grid, sweep::kOneThreads, (size_t)smem, 1, st, maps, a); };
+  if (!lse) {
+    a.withhold_tile = c->withhold_sweep == tc::kStats ? c->withhold_tile : -1;
+    ProfScope ps(c, DKV_STEP_SCORE_STATS, 1, st);
+    DKV_LAUNCH(c, (with_sweep_kernel<sweep::kRowSums>(nb, launch)));
+  }
+  a.withhold_tile = c->withhold_sweep == tc::kEmit ? c->withhold_tile : -1;
+  {
+    ProfScope ps(c, DKV_STEP_SCORE_EMIT, 1, st);
+    DKV_LAUNCH(c, lse ? (with_sweep_kernel<sweep::kGivenSums>(nb, launch)) : (with_sweep_kernel<sweep::kKeySums>(nb, launch)));
+  }
+  ProfScope ps(c, DKV_STEP_SCORE_EMIT, 1, st);
+  int seg = sweep::kPoolSeg;
+  while (seg > sweep::kPoolThreads && (long long)nl * heads * ((s.P + seg - 1) / seg) < 2 * c->n_sms) seg /= 2;
+  const int segs = (s.P + seg - 1) / seg;
+  DKV_LAUNCH(c, launch_pdl(pool_kernel, dim3(segs * nl * heads), sweep::kPoolThreads, 0, 1, st, (const float*)a.raw,
+                           c->d_scores + (size_t)layer * layer_scores(s), a.hist, s.P, tph * tc::kTileKeys, c->planes, s.pool / 2,
+                           (int)(c->cfg.pool_kind == 1), s.Hkv, seg, segs));
+  return DKV_OK;
+}
+
 // One layer on its own; lse: as for dkv_score_lse, or null.
 int do_score(dkv_ctx* c, int layer, const void* q, const void* k, const float* lse, float* scores_out, cudaStream_t st) {
   ScoreGroup g = {layer, 1, layer % 3, 0};
@@ -520,22 +617,22 @@ int do_decode(dkv_ctx* c, int layer0, int nl, int nq, const void* const* q, cons
 int do_pass(dkv_ctx* c, const void* const* q, const void* const* k, const void* const* v, const float* const* lse,
             void* const* kb, void* const* vb, cudaStream_t st) {
   const Shape& s = c->s;
-  int rc;
-  if (lse) DKV_CUDA(c, cudaMemsetAsync(c->d_layer_hist, 0, sizeof(unsigned int) * s.L * s.Bt * kBins, st));   // else sweep 1 does it
-  ScoreGroup prev = {}, cur = {};
-  for (int g = 0, done = 0; done < s.L || prev.n; ++g) {
-    cur.first = done; cur.n = s.L - done < c->pass_group ? s.L - done : c->pass_group; cur.buf = g % 3;
-    done += cur.n;
-    if (lse) {
-      if (!cur.n) break;
-      rc = launch_score<tc::kMaxGroup>(c, &cur, nullptr, q, k, lse, nullptr, true, st);
-    } else {
-      rc = launch_score<tc::kMaxGroup>(c, prev.n ? &prev : nullptr, cur.n ? &cur : nullptr, q, k, nullptr, nullptr, true, st);
+  const int most = most_layers(c);
+  int rc, l[DKV_MAX_LAYERS];
+  if (lse || pass_by_sweeps(c)) {
+    for (int i = 0; i < s.L; i += most) {
+      const int nl = s.L - i < most ? s.L - i : most;
+      if ((rc = launch_sweeps(c, i, nl, q + i, k + i, lse ? lse + i : nullptr, st))) return rc;
+    }
+  } else {
+    ScoreGroup prev = {}, cur = {};
+    for (int g = 0, done = 0; done < s.L || prev.n; ++g) {
+      cur.first = done; cur.n = s.L - done < c->pass_group ? s.L - done : c->pass_group; cur.buf = g % 3;
+      done += cur.n;
+      if ((rc = launch_score<tc::kMaxGroup>(c, prev.n ? &prev : nullptr, cur.n ? &cur : nullptr, q, k, nullptr, nullptr, true, st))) return rc;
       prev = cur;
     }
-    if (rc) return rc;
   }
-  int l[DKV_MAX_LAYERS];
   if ((rc = do_rebudget(c, l, update_points(s, l), s.Blc, nullptr, st))) return rc;
   if ((rc = do_select_gather(c, k, v, kb, vb, st))) return rc;
   mark_pass_done(c);
@@ -556,7 +653,7 @@ void free_staging(dkv_ctx* c) {
 void free_all(dkv_ctx* c) {
   cudaFree(c->d_scores); cudaFree(c->d_idx); cudaFree(c->d_count); cudaFree(c->d_held); cudaFree(c->d_dbg);
   cudaFree(c->d_rb_state); cudaFree(c->d_rb_above); cudaFree(c->d_layer_hist); cudaFree(c->d_shrink_tickets);
-  cudaFree(c->d_cand); cudaFree(c->d_cand_n); cudaFree(c->d_status); cudaFree(c->d_tc_stats);
+  cudaFree(c->d_cand); cudaFree(c->d_cand_n); cudaFree(c->d_status); cudaFree(c->d_tc_stats); cudaFree(c->d_stats);
   cudaFree(c->d_dec_scratch); cudaFree(c->d_dec_tickets);
   if (c->prof_recs) {
     for (ProfRec& r : *c->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
@@ -628,6 +725,8 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   s.m = cfg->update_interval;
   s.G = s.Hq / s.Hkv; s.P = s.S - s.ws; s.M = s.ws * s.G; s.Blc = s.Bl < s.P ? s.Bl : s.P; s.rows = s.Blc + s.ws;
   const int heads = s.Bt * s.Hkv;
+  c->planes = (s.M + 127) / 128;
+  c->plane_rows = c->planes == 1 ? s.M : ((s.M + c->planes - 1) / c->planes + 7) / 8 * 8;
   c->sel_cap = 1024;                                       // a quarter more than B^l for the rest of the threshold's digit
   while (c->sel_cap < s.Blc + s.Blc / 4 && c->sel_cap < DKV_MAX_LAYER_BUDGET) c->sel_cap <<= 1;
 
@@ -669,7 +768,13 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   TRY(cudaMalloc(&c->d_shrink_tickets, sizeof(unsigned int) * bl));
   TRY(cudaMemset(c->d_shrink_tickets, 0, sizeof(unsigned int) * bl));
   TRY(cudaMalloc(&c->d_layer_hist, sizeof(unsigned int) * s.L * s.Bt * kBins));
-  TRY(cudaMalloc(&c->d_cand, sizeof(uint2) * s.L * layer_scores(s)));
+  {
+    const int most = most_layers(c);
+    TRY(cudaMalloc(&c->d_cand, std::max(sizeof(uint2) * s.L * layer_scores(s), sizeof(float) * most * heads * c->planes * tiles_per_head(s) * tc::kTileKeys)));
+    // a launch over fewer layers than `most` (the last of a pass) has more segments a head, but no more in all
+    TRY(cudaMalloc(&c->d_stats, sizeof(float2) * c->plane_rows * (2 * c->n_sms + 2 * most * heads * c->planes)));
+    TRY(set_sweep_attributes(row_blocks(c)));
+  }
   TRY(cudaMalloc(&c->d_cand_n, sizeof(unsigned int) * s.Bt));
   TRY(cudaMalloc(&c->d_tc_stats, sizeof(float2) * 3 * c->stats_rows * 256));
   TRY(set_score_attribute<1>(s.M, s.D));

@@ -1,0 +1,92 @@
+"""Scoring of whole passes at the sizes where the sweeps change: window rows around their 32-row steps and the second plane, keys
+around a tile, heads that lie in one pipe's range and in many, logits that a row's reference cannot hold."""
+import pytest
+import torch
+
+from paper_2412_14838_b200 import binding as B
+from paper_2412_14838_b200 import build
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    B.load()
+
+
+def _scores(q, k, ws, pool):
+    """Eq. 1-2 in 64 bits: q [Bt, Hq, ws, D], k [Bt, Hkv, S, D] -> [Bt, Hkv, S - ws]."""
+    (Bt, Hkv, S, D), G = k.shape, q.shape[1] // k.shape[1]
+    t = q.double().view(Bt, Hkv, G * ws, D) @ k.double().transpose(-1, -2) / D ** 0.5
+    last = S - ws + torch.arange(ws, device="cuda").repeat(G)
+    t.masked_fill_(torch.arange(S, device="cuda") > last[:, None], -torch.inf)
+    return torch.nn.functional.max_pool1d(t.softmax(-1)[..., :S - ws].sum(2), pool, 1, pool // 2), t.logsumexp(-1).view(Bt, Hkv * G, ws)
+
+
+def _passes(L, Hkv, G, D, Bt, S, ws, pool, change=None, most=5e-5):
+    """Both kinds of pass; a score is a sum of 2^(t - lse): with |t| < 128 in 32 bits each is off by 2^-18 ln 2 at most, and the
+    instruction for 2^x and the sums add a few 2^-22."""
+    g = torch.Generator(device="cuda").manual_seed(S)
+    new = lambda *s: [torch.randn(s, generator=g, device="cuda").to(torch.bfloat16) for _ in range(L)]
+    q, k, v = new(Bt, G * Hkv, ws, D), new(Bt, Hkv, S, D), new(Bt, Hkv, S, D)
+    if change:
+        change(q, k)
+    P, rows = S - ws, min(8, S - ws) + ws
+    kb, vb = ([torch.zeros((Bt, Hkv, rows, D), device="cuda", dtype=torch.bfloat16) for _ in range(L)] for _ in range(2))
+    want, lse = zip(*(_scores(q[l], k[l], ws, pool) for l in range(L)))
+    lse = [x.float().contiguous() for x in lse]
+    h = B.dkv_create(B.make_config(L, G * Hkv, Hkv, D, Bt, S, ws, pool, 4, 8, 2))
+    try:
+        for run in (lambda: B.dkv_run_prefill_pass(h, q, k, v, kb, vb), lambda: B.dkv_run_prefill_pass_lse(h, q, k, v, lse, kb, vb)):
+            run()
+            for l in range(L):
+                got = torch.zeros((Bt, Hkv, P))
+                B.dkv_memcpy_to_host(h, got, B.dkv_layer_views(h, l)[0], got.numel() * 4)
+                off = (got.cuda().double() - want[l]).abs() / want[l].clamp_min(1e-25)
+                assert off.max() <= most, f"layer {l}: {off.max():.1e}"
+            assert B.dkv_last_status(h)[0] == B.DKV_OK
+    finally:
+        B.dkv_destroy(h)
+
+
+# (window rows G * ws: 1, 32, 33, 64, 65, 96, 97, 128, 130, 192, 256)
+@pytest.mark.parametrize("G,ws,D", [(1, 1, 64), (1, 32, 128), (3, 11, 64), (2, 32, 64), (5, 13, 128), (3, 32, 128), (1, 97, 64), (4, 32, 64),
+                                    (5, 26, 64), (6, 32, 128), (8, 32, 64)])
+def test_window_rows(G, ws, D):
+    _passes(2, 2, G, D, 1, 900, ws, 5)
+
+
+# the last tile full, with one key, with the prefix ending at its start; fewer tiles than pipes; heads in many pipes and many in one
+@pytest.mark.parametrize("L,Hkv,Bt,S,pool", [(1, 1, 1, 9, 1), (1, 1, 1, 128, 3), (1, 2, 1, 129, 7), (3, 1, 1, 136, 255), (2, 3, 2, 2049, 7),
+                                             (2, 1, 1, 20011, 3), (33, 6, 3, 257, 9), (2, 2, 1, 2056, 5)])
+def test_lengths(L, Hkv, Bt, S, pool):
+    _passes(L, Hkv, 2, 64, Bt, S, 8, pool)
+
+
+def test_a_call_of_128_rows_over_many_tiles():
+    _passes(32, 8, 4, 128, 2, 8200, 32, 7)
+
+
+def test_logits_that_are_far_above_the_first_key_of_a_segment():
+    def far(q, k):                                           # up to 200 above it: 2^288 times its exponential
+        q[0][:, :, :, 0], k[0][..., 0], k[0][:, 0, 700:705, 0] = 16.0, 0.0, 100.0
+    _passes(2, 2, 2, 64, 1, 2000, 8, 5, far, most=2e-4)      # |t| < 512: 2^-16 ln 2 and more
+
+
+def test_a_head_with_a_key_that_is_no_number_spoils_no_other():
+    g = torch.Generator(device="cuda").manual_seed(1)
+    new = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+    q, k = new(1, 6, 8, 64), new(1, 3, 700, 64)
+    k[0, 1, 300, 5] = torch.nan
+    kb = torch.zeros((1, 3, 16, 64), device="cuda", dtype=torch.bfloat16)
+    h = B.dkv_create(B.make_config(1, 6, 3, 64, 1, 700, 8, 3, 4, 8, 2))
+    try:
+        B.dkv_run_prefill_pass(h, [q], [k], [k], [kb], [kb.clone()])
+        got = torch.zeros((1, 3, 692))
+        B.dkv_memcpy_to_host(h, got, B.dkv_layer_views(h, 0)[0], got.numel() * 4)
+        want = _scores(q, k, 8, 3)[0].cpu()
+        assert got[0, 1].isnan().all()
+        assert ((got[0, ::2] - want[0, ::2]).abs() <= 5e-5 * want[0, ::2]).all()
+    finally:
+        B.dkv_destroy(h)
