@@ -181,6 +181,38 @@ __device__ __forceinline__ void bitonic_sort(unsigned long long* keys, int sort_
 __host__ __device__ inline size_t select_smem(int cap) {
   return (size_t)cap * 8 * (cap <= kMaxCountingList ? 2 : 1) + sizeof(unsigned int) * kSortBins;
 }
+// A block's share of a head's positions.
+template <bool kShared>
+__device__ __forceinline__ void select_share(int P, int part, int parts, int& lo, int& hi) {
+  const int share = kShared ? ((P + parts - 1) / parts + 31) & ~31 : P;
+  lo = min(P, part * share); hi = min(P, lo + share);
+}
+constexpr int kSelUnroll = 8;                              // scores a thread has in flight
+__device__ __forceinline__ unsigned int* select_bins(unsigned char* dyn, int cap) {
+  return reinterpret_cast<unsigned int*>(dyn + (size_t)cap * 8 * (cap <= kMaxCountingList ? 2 : 1));
+}
+// The first step, which does not depend on n: the share's digits are counted in `bins` [kBins].  Ends with a barrier.
+template <bool kShared>
+__device__ __forceinline__ void count_digits(const uint32_t* v, int P, unsigned int* bins, int part, int parts) {
+  const int tid = threadIdx.x;
+  int lo, hi;
+  select_share<kShared>(P, part, parts, lo, hi);
+  const int hi32 = lo + ((hi - lo + 31) & ~31);
+  for (int i = tid; i < kBins; i += kSelThreads) bins[i] = 0;
+  __syncthreads();
+  for (int p0 = lo + tid; p0 < hi32; p0 += kSelThreads * kSelUnroll) {
+    uint32_t u[kSelUnroll];
+#pragma unroll
+    for (int j = 0; j < kSelUnroll; ++j) { const int p = p0 + j * kSelThreads; u[j] = p < hi ? v[p] : 0u; }
+#pragma unroll
+    for (int j = 0; j < kSelUnroll; ++j) {
+      const int p = p0 + j * kSelThreads;
+      if (p < hi32) run_bump(bins, digit_of(u[j]), p < hi);   // warp-uniform: neighbours share digits after pooling
+    }
+  }
+  __syncthreads();
+}
+// The other steps; count_digits has been called.
 template <bool kShared>
 __device__ __forceinline__ int* select_head(const uint32_t* v, int P, int n, int cap, unsigned char* dyn, unsigned int* gh, int part,
                                             int parts) {
@@ -191,11 +223,11 @@ __device__ __forceinline__ int* select_head(const uint32_t* v, int P, int n, int
   const int tid = threadIdx.x, lane = tid & 31;
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(dyn);
   unsigned long long* sorted = keys + (cap <= kMaxCountingList ? cap : 0);
-  unsigned int* bins = reinterpret_cast<unsigned int*>(sorted + cap);
+  unsigned int* bins = select_bins(dyn, cap);
   unsigned int* sums = kShared ? bins + kBins : bins;      // the whole head's counts
-  constexpr int kUnroll = 8;                               // scores a thread has in flight
-  const int share = kShared ? ((P + parts - 1) / parts + 31) & ~31 : P;
-  const int lo = min(P, part * share), hi = min(P, lo + share), hi32 = lo + ((hi - lo + 31) & ~31);
+  int lo, hi;
+  select_share<kShared>(P, part, parts, lo, hi);
+  const int hi32 = lo + ((hi - lo + 31) & ~31);
   auto add_up = [&]() {                                    // bins of all blocks -> sums
     if constexpr (kShared) {
       cg::this_cluster().sync();
@@ -211,20 +243,7 @@ __device__ __forceinline__ int* select_head(const uint32_t* v, int P, int n, int
   };
 
   // 1: the digit of the n-th largest score
-  for (int i = tid; i < kBins; i += kSelThreads) bins[i] = 0;
-  if (tid == 0) { s_n = 0; s_max = 0; s_full = 0; }
-  __syncthreads();
-  for (int p0 = lo + tid; p0 < hi32; p0 += kSelThreads * kUnroll) {
-    uint32_t u[kUnroll];
-#pragma unroll
-    for (int j = 0; j < kUnroll; ++j) { const int p = p0 + j * kSelThreads; u[j] = p < hi ? v[p] : 0u; }
-#pragma unroll
-    for (int j = 0; j < kUnroll; ++j) {
-      const int p = p0 + j * kSelThreads;
-      if (p < hi32) run_bump(bins, digit_of(u[j]), p < hi);   // warp-uniform: neighbours share digits after pooling
-    }
-  }
-  __syncthreads();
+  if (tid == 0) { s_n = 0; s_max = 0; s_full = 0; }        // barriers follow before these are counted up
   if (gh) for (int i = tid; i < kBins; i += kSelThreads) { const unsigned int c = bins[i]; if (c) atomicAdd(&gh[i], c); }
   add_up();
   find_digit(sums, kBins, P, n, sm_scan, found);
@@ -256,12 +275,12 @@ __device__ __forceinline__ int* select_head(const uint32_t* v, int P, int n, int
     to_n = cg::this_cluster().map_shared_rank(&s_n, 0);
     to_max = cg::this_cluster().map_shared_rank(&s_max, 0);
   }
-  for (int p0 = lo + tid; p0 < hi32; p0 += kSelThreads * kUnroll) {
-    uint32_t u[kUnroll];
+  for (int p0 = lo + tid; p0 < hi32; p0 += kSelThreads * kSelUnroll) {
+    uint32_t u[kSelUnroll];
 #pragma unroll
-    for (int j = 0; j < kUnroll; ++j) { const int p = p0 + j * kSelThreads; u[j] = p < hi ? v[p] : 0u; }
+    for (int j = 0; j < kSelUnroll; ++j) { const int p = p0 + j * kSelThreads; u[j] = p < hi ? v[p] : 0u; }
 #pragma unroll
-    for (int j = 0; j < kUnroll; ++j) {
+    for (int j = 0; j < kSelUnroll; ++j) {
       const int p = p0 + j * kSelThreads;
       const bool take = p < hi && u[j] >= from;
       const unsigned int m = __ballot_sync(0xFFFFFFFFu, take);
@@ -363,8 +382,9 @@ select_topk_kernel(const float* scores, int* idx, unsigned int* layer_hist, int 
   pdl_launch();
   pdl_wait();
   if (threadIdx.x == 0 && blockIdx.x % (Hkv * parts) == 0) count[b * L + layer] = keep;
-  const int* sel = select_head<kShared>(reinterpret_cast<const uint32_t*>(scores) + (size_t)head * P, P, keep, cap, dyn,
-                                        layer_hist + (size_t)b * kBins, blockIdx.x % parts, parts);
+  const uint32_t* v = reinterpret_cast<const uint32_t*>(scores) + (size_t)head * P;
+  count_digits<kShared>(v, P, select_bins(dyn, cap), blockIdx.x % parts, parts);
+  const int* sel = select_head<kShared>(v, P, keep, cap, dyn, layer_hist + (size_t)b * kBins, blockIdx.x % parts, parts);
   if (sel) for (int i = threadIdx.x; i < keep; i += kSelThreads) idx[(size_t)head * keep + i] = sel[i];
 }
 
@@ -373,6 +393,8 @@ select_topk_kernel(const float* scores, int* idx, unsigned int* layer_hist, int 
 // the ws window rows of K and V into the layer's buffers.  Selecting and copying the final rows once replaces a
 // selection and copy of B^l rows per layer and a truncation per update: 32K prompt with B^l = 4 N: 71 MB of rows read
 // instead of 272, and no block of the scoring kernel gives way to it while keys are streamed.
+// The scores' digits are counted while the last update still runs (rb_finish_kernel; see rb_collect_kernel for why the scores
+// are complete by then): only launched right behind it.
 // grid (Bt*Hkv, layers).
 __global__ void __launch_bounds__(kSelThreads, 2)
 select_gather_kernel(const __grid_constant__ PassPtrs ptrs, const float* scores, int* idx,
@@ -380,13 +402,15 @@ select_gather_kernel(const __grid_constant__ PassPtrs ptrs, const float* scores,
   extern __shared__ __align__(16) unsigned char dyn[];
   const int bh = blockIdx.x, b = bh / Hkv, layer = blockIdx.y, tid = threadIdx.x;
   const size_t head = (size_t)layer * gridDim.x + bh;
-  pdl_launch();
+  const uint32_t* v = reinterpret_cast<const uint32_t*>(scores) + head * P;
+  count_digits<false>(v, P, select_bins(dyn, cap), 0, 1);
   pdl_wait();
+  pdl_launch();
   const int n = count[b * L + layer];
   if (tid == 0 && bh % Hkv == 0) held[b * L + layer] = n;
   const int* sel = nullptr;
   if (n > 0) {
-    sel = select_head<false>(reinterpret_cast<const uint32_t*>(scores) + head * P, P, n, cap, dyn, nullptr, 0, 1);
+    sel = select_head<false>(v, P, n, cap, dyn, nullptr, 0, 1);
     for (int i = tid; i < n; i += kSelThreads) idx[head * stride + i] = sel[i];
   }
   gather_rows(static_cast<const uint4*>(ptrs.k[layer]), static_cast<const uint4*>(ptrs.v[layer]), static_cast<uint4*>(ptrs.kb[layer]),
@@ -403,13 +427,15 @@ select_gather_cluster_kernel(const __grid_constant__ PassPtrs ptrs, const float*
   const int parts = cg::this_cluster().num_blocks(), part = blockIdx.x % parts, bh = blockIdx.x / parts;
   const int b = bh / Hkv, layer = blockIdx.y, tid = threadIdx.x;
   const size_t head = (size_t)layer * (gridDim.x / parts) + bh;
-  pdl_launch();
+  const uint32_t* v = reinterpret_cast<const uint32_t*>(scores) + head * P;
+  count_digits<true>(v, P, select_bins(dyn, cap), part, parts);
   pdl_wait();
+  pdl_launch();
   const int n = count[b * L + layer];
   if (tid == 0 && part == 0 && bh % Hkv == 0) held[b * L + layer] = n;
   const int* sel = nullptr;
   if (n > 0) {
-    select_head<true>(reinterpret_cast<const uint32_t*>(scores) + head * P, P, n, cap, dyn, nullptr, part, parts);
+    select_head<true>(v, P, n, cap, dyn, nullptr, part, parts);
     cg::this_cluster().sync();                             // the first block's list (at the start of `dyn`) is complete
     sel = cg::this_cluster().map_shared_rank(reinterpret_cast<int*>(dyn), 0);
     for (int i = part * kSelThreads + tid; i < n; i += parts * kSelThreads) idx[head * stride + i] = sel[i];
