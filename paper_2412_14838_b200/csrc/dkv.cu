@@ -262,10 +262,12 @@ bool make_job(dkv_ctx* c, int mode, int layer, int nl, const void* const* q, con
 }
 
 // The scoring kernel for two jobs (either may be kNone) of the same shape: the specialised build for exactly 128 window rows
-// of 128 dims, builds with two or four copies of the queries for up to 64 or 32 window rows, the general one otherwise.
+// of 128 dims, builds with two or four copies of the queries for up to 64 or 32 window rows, the general one otherwise.  Groups of
+// layers have 128 rows of 128 dims or more than 128 rows (pass_by_sweeps).
 template <int NL>
 auto score_kernel(int M, int D) {
-  return M == 128 && D == 128 ? tc::score_tc_kernel<NL, true, 1> : query_copies(M) == 4 ? tc::score_tc_kernel<NL, false, 4>
+  if constexpr (NL > 1) return M == 128 && D == 128 ? tc::score_tc_kernel<NL, true, 1> : tc::score_tc_kernel<NL, false, 1>;
+  else return M == 128 && D == 128 ? tc::score_tc_kernel<NL, true, 1> : query_copies(M) == 4 ? tc::score_tc_kernel<NL, false, 4>
        : query_copies(M) == 2 ? tc::score_tc_kernel<NL, false, 2> : tc::score_tc_kernel<NL, false, 1>;
 }
 // The build's shared memory, per function and device: set before its first launch, and only for the builds that a caller can
@@ -311,7 +313,7 @@ int launch_score(dkv_ctx* c, const ScoreGroup* e, ScoreGroup* s, const void* con
 
 // ---- scoring of a pass (score_sweep.cuh) ---------------------------------------------------------
 int tiles_per_head(const Shape& s) { return (s.S + tc::kTileKeys - 1) / tc::kTileKeys; }
-int row_blocks(const dkv_ctx* c) { return (c->plane_rows + 31) / 32 * 4; }              // the kernel's NB
+int row_blocks(const dkv_ctx* c) { return (c->plane_rows + 15) / 16 * 2; }              // the kernel's NB
 int most_layers(const dkv_ctx* c) { return c->s.L < tc::kMaxGroup ? c->s.L : tc::kMaxGroup; }
 // Segments a (head, plane) can have in a launch over nl layers: its share of the pipes, one cut at either end.
 int stats_places(const dkv_ctx* c, int nl) { return 2 * c->n_sms / (nl * c->s.Bt * c->s.Hkv * c->planes) + 2; }
@@ -320,9 +322,13 @@ int stats_places(const dkv_ctx* c, int nl) { return 2 * c->n_sms / (nl * c->s.Bt
 template <int kSweep, typename F>
 cudaError_t with_sweep_kernel(int nb, F f) {
   switch (nb) {
+    case 2: return f(score_sweep_kernel<2, kSweep>, (int)sweep::Shape1<2>::kSmem);
     case 4: return f(score_sweep_kernel<4, kSweep>, (int)sweep::Shape1<4>::kSmem);
+    case 6: return f(score_sweep_kernel<6, kSweep>, (int)sweep::Shape1<6>::kSmem);
     case 8: return f(score_sweep_kernel<8, kSweep>, (int)sweep::Shape1<8>::kSmem);
+    case 10: return f(score_sweep_kernel<10, kSweep>, (int)sweep::Shape1<10>::kSmem);
     case 12: return f(score_sweep_kernel<12, kSweep>, (int)sweep::Shape1<12>::kSmem);
+    case 14: return f(score_sweep_kernel<14, kSweep>, (int)sweep::Shape1<14>::kSmem);
     default: return f(score_sweep_kernel<16, kSweep>, (int)sweep::Shape1<16>::kSmem);
   }
 }
@@ -340,13 +346,13 @@ cudaError_t set_sweep_attributes(int nb) {
 // time always score_tc.cuh, which has a launch less and pools in it (a layer of 32K with normalisers 18.3 us a call, by sweeps 23.1;
 // without, 8 layers of 4K call by call 253-298 us against 278-328).  score_tc.cuh remains for 128 window rows of 128 dims, for
 // which it has a build, while an SM has few tiles (8 layers of 4K, 4 heads: 58 us against 65; 32 of 8K, 110 tiles an SM: 285 / 283;
-// 32 of 32K, 443: 1046 / 1024; 4 x 16K, 886: 2013 / 1955), and where planes of 32, 64, 96 or 128 rows leave many rows empty (224
-// rows, 28 layers of 16K: 423 / 454).
+// 32 of 32K, 443: 1046 / 1024; 4 x 16K, 886: 2013 / 1955), and for more than 128 rows (two planes, whose pooling takes a launch)
+// while an SM has at most two tiles (4 layers of 1K, 4 heads, 224 rows, 128 tiles in all: 48.3 / 50.2; 8 of 2K, 512 tiles:
+// 60.8 / 58.7; 28 of 16K: 388 / 364 in bursts and the same, 408-418, at the power cap; 16 of 16K, 4 heads of 64, 140 rows: 207 / 168).
 bool pass_by_sweeps(const dkv_ctx* c) {
   const Shape& s = c->s;
-  if (s.M == 128 && s.D == 128)
-    return (long long)s.L * s.Bt * s.Hkv * tiles_per_head(s) >= 200ll * c->n_sms;
-  return c->planes == 1 || c->planes * ((c->plane_rows + 31) / 32 * 32) - s.M <= 16;
+  const long long tiles = (long long)s.L * s.Bt * s.Hkv * tiles_per_head(s);
+  return tiles >= (s.M == 128 && s.D == 128 ? 200ll : c->planes > 1 ? 2ll : 0ll) * c->n_sms;
 }
 
 // Scores of a pass's `nl` consecutive layers from `layer`, and their digits: row sums, key sums and pooling, or with the caller's
@@ -737,8 +743,8 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
     c->n_sms = sms > 0 ? sms : 1;
     c->stats_rows = (size_t)c->n_sms + 2 * tc::kMaxGroup * heads;
     // Layers per scoring launch of the pass: enough that a thread block has about 110 tiles a sweep.  A launch costs some 8 us
-    // (fill, drain, statistics) whatever it does: 32 layers of 8K in launches of 8 / 16 / 32 layers take 299 / 290 / 286 us,
-    // 28 layers of 16K with 224 window rows 449 / 414 / 406; at 32K eight layers are as good as more.
+    // (fill, drain, statistics) whatever it does: 32 layers of 8K in launches of 8 / 16 / 32 layers take 299 / 290 / 286 us;
+    // at 32K eight layers are as good as more.
     const long long tiles = (long long)heads * ((s.S + tc::kTileKeys - 1) / tc::kTileKeys), want = (110ll * c->n_sms + tiles - 1) / tiles;
     int g = want < s.L ? (int)want : s.L;
     if (g > tc::kMaxGroup) g = tc::kMaxGroup;
@@ -778,7 +784,7 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   TRY(cudaMalloc(&c->d_cand_n, sizeof(unsigned int) * s.Bt));
   TRY(cudaMalloc(&c->d_tc_stats, sizeof(float2) * 3 * c->stats_rows * 256));
   TRY(set_score_attribute<1>(s.M, s.D));
-  TRY(set_score_attribute<tc::kMaxGroup>(s.M, s.D));
+  if (!pass_by_sweeps(c)) TRY(set_score_attribute<tc::kMaxGroup>(s.M, s.D));
   TRY(cudaMalloc(&c->d_status, sizeof(int) * 8));
   TRY(cudaMemset(c->d_status, 0, sizeof(int) * 8));
   TRY(cudaMemset(c->d_count, 0, sizeof(int) * bl));

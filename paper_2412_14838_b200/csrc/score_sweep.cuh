@@ -4,7 +4,8 @@
 // known when a head's last key has been seen, so the keys are swept twice (once where the caller has the log-denominators).
 //
 //   tile      128 keys of one head: logits^T = K . Q_win^T on the tensor cores, one TMEM lane a key, one column a window row
-//             (at most 128 rows; up to 256 rows are two PLANES whose sums are added by pool_kernel).
+//             (at most 128 rows, rounded up to 16; up to 256 rows are two PLANES whose sums are added by pool_kernel).  With rows
+//             rounded up to 32, 72 and 224 rows cost more: 14 layers of 3 x 5003 131.4 us, now 124.0; 28 of 16K 454 before, 390.
 //   pipes     a block has two, each with its own contiguous range of the tiles, in SEGMENTS of one head, its own slots, copies,
 //             MMAs, accumulator stages and eight warps for exponentials.
 //   warps     0-7 and 8-15 exponentials of either pipe, 16 and 17 its copies, 18 and 19 its MMAs, 20 and 21 log-denominators of
@@ -24,7 +25,7 @@
 // about 10 in all beside its tiles, most of it instructions that are fetched for the first time: with the loops unrolled over
 // a whole tile it took 15, and with two streams of long loops (row sums in one pipe, key sums in the other) a tile took twice as long.
 //
-// Against score_tc.cuh (us a pass): 14 layers of 3 x 5003, 6 heads of 64, 72 rows 166 -> 138; 16 layers of 16K, 4 heads of 64,
+// Against score_tc.cuh (us a pass): 14 layers of 3 x 5003, 6 heads of 64, 72 rows 166 -> 131; 16 layers of 16K, 4 heads of 64,
 // 32 / 96 / 128 / 192 rows 118 / 149 / 155 / 220 -> 107 / 123 / 139 / 186; 28 of 2 x 2K, 4 heads of 128, 96 / 192 / 256 rows
 // 114 / 153 / 162 -> 102 / 138 / 151; 32 layers of 32K, 8 heads of 128, with log-denominators 572 -> 530-554.
 #pragma once
@@ -46,15 +47,16 @@ enum Sweep { kRowSums, kKeySums, kGivenSums };       // kGivenSums: key sums wit
 
 constexpr int kSlots = 3, kSlotBytes = 2 * kHalfBytes;      // of a pipe: queries, two tiles of keys
 
-// NB: 8-column blocks of window rows (4, 8, 12 or 16)
+// NB: 8-column blocks of window rows (even, at most 16)
 template <int NB>
 struct Shape1 {
   static constexpr int kCols = 8 * NB;                                      // accumulator columns of a tile
-  static constexpr int kPer = NB <= 8 ? 4 : 2;                              // accumulator stages of a pipe
+  static constexpr int kPer = NB <= 8 ? 4 : 2;                              // accumulator stages of a pipe,
+  static constexpr int kStage = (kCols + 31) / 32 * 32;                     // this many columns apart
   static constexpr int kQBytes = kCols * 128;                               // window rows x 64 dims
   static constexpr int kPipeBars = 2 * kSlots + 2 * kPer + 5, kBars = 2 * kPipeBars + 1;
   static constexpr int kSmem = 1024 + 2 * kSlots * kSlotBytes + 2 * 4 * kCols * 8 + 3 * 2 * kCols * 4 + kBars * 8;
-  static_assert(kSmem + 1024 <= 227 * 1024 && 2 * kPer * kCols <= 512, "shared and tensor memory of an SM");
+  static_assert(kSmem + 1024 <= 227 * 1024 && 2 * kPer * kStage <= 512, "shared and tensor memory of an SM");
 };
 
 struct Args {
@@ -82,11 +84,19 @@ struct Layers {                                // by layer of the launch
 };
 
 // ------------------------------------------------------------------------------------------ PTX
-// N = 2, 4 or 8 blocks of 8 columns x 16 lanes.  Register 4 b + 2 i + j: block b, lane (key) laneid / 4 + 8 i, column 2 (laneid % 4) + j.
+// N = 1 to 8 blocks of 8 columns x 16 lanes (N that are no power of two by several loads).  Register 4 b + 2 i + j: block b, lane (key) laneid / 4 + 8 i, column 2 (laneid % 4) + j.
 template <int N>
 __device__ __forceinline__ void ld_block(uint32_t a, float* v) {
   uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  if constexpr (N == 2)
+  if constexpr (N > 4 && N < 8) {
+    ld_block<4>(a, v);
+    ld_block<N - 4>(a + 32, v + 16);
+  } else if constexpr (N == 3) {
+    ld_block<2>(a, v);
+    ld_block<1>(a + 16, v + 8);
+  } else if constexpr (N == 1)
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+  else if constexpr (N == 2)
     asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(a));
   else if constexpr (N == 4)
@@ -146,7 +156,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
 score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ Args a) {
   using C = Shape1<NB>;
   constexpr bool kRows = kSweep == kRowSums;
-  constexpr int kCols = C::kCols, kPer = C::kPer;
+  constexpr int kCols = C::kCols, kPer = C::kPer, kStage = C::kStage;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);     // [2 pipes][kSlots][half][128][128 B]
   float* sum_s = reinterpret_cast<float*>(ring + 2 * kSlots * kSlotBytes);  // [2 pipes][4 quads][kCols] a segment's row sums
@@ -248,7 +258,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     // Row sums: a warp has 32 lanes (keys) x half of the columns, 16 lanes at a time.  Key sums: 16 lanes x all columns, four blocks at a time.
     constexpr int kHalf = NB / 2, kSet = 4;
     const int c0 = kRows ? half * kHalf * 8 : 0, first = quad * 32 + (kRows ? 0 : half * 16);
-    const uint32_t addr = tmem_base + ((uint32_t)first << 16) + (uint32_t)(pipe * kPer * kCols + c0);
+    const uint32_t addr = tmem_base + ((uint32_t)first << 16) + (uint32_t)(pipe * kPer * kStage + c0);
     const int col2 = c0 + 2 * (lane & 3), key = first + (lane >> 2);        // the thread's keys: key, key + 8 (, key + 16, key + 24)
     if (kSweep != kKeySums) for (int i = blockIdx.x * (kSoftWarps * 32) + threadIdx.x; i < a.hist_n; i += grid * (kSoftWarps * 32)) a.hist[i] = 0;
     Ring st(kPer, 0);
@@ -272,12 +282,12 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           if (!ok) break;
           tc_fence_after();
           const bool masked = (sg.t0 + t + 1) * kTile - 1 > a.P;            // row r sees keys 0 .. P + r % ws
-          const uint32_t at = addr + (uint32_t)(st.s * kCols);
+          const uint32_t at = addr + (uint32_t)(st.s * kStage);
 #pragma unroll 1
           for (int h = 0; h < 2; ++h) {
             float x[4 * kHalf];
             const uint32_t from = at + (uint32_t)(h << 20);                 // 16 lanes on
-            if constexpr (kHalf == 6) { ld_block<4>(from, x); ld_block<2>(from + 32, x + 16); } else { ld_block<kHalf>(from, x); }
+            ld_block<kHalf>(from, x);
             tc_wait_ld();
             if (h) {
               tc_fence_before();
@@ -321,11 +331,18 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, 4));
           if (!(lane & 4)) *reinterpret_cast<uint64_t*>(&my_sum[8 * (b + (lane >> 3))]) = u;
         }
-        if constexpr (kHalf % 4) {
-          uint64_t u = swap(16, sum[kHalf - 2], sum[kHalf - 1]);
+        if constexpr (kHalf & 2) {
+          constexpr int b = kHalf & ~3;
+          uint64_t u = swap(16, sum[b], sum[b + 1]);
           u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, 8));
           u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, 4));
-          if (!(lane & 12)) *reinterpret_cast<uint64_t*>(&my_sum[8 * (kHalf - 2 + (lane >> 4))]) = u;
+          if (!(lane & 12)) *reinterpret_cast<uint64_t*>(&my_sum[8 * (b + (lane >> 4))]) = u;
+        }
+        if constexpr (kHalf & 1) {
+          uint64_t u = sum[kHalf - 1];
+#pragma unroll
+          for (int o = 16; o >= 4; o >>= 1) u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, o));
+          if (lane < 4) *reinterpret_cast<uint64_t*>(&my_sum[8 * (kHalf - 1)]) = u;
         }
       } else {
         const float* my_c = c_s + (2 * pipe + slot) * kCols + col2;
@@ -335,25 +352,28 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           if (!ok) break;
           tc_fence_after();
           uint64_t sum[4] = {0ull, 0ull, 0ull, 0ull};   // over the columns so far, by key and parity of the block
-          const uint32_t at = addr + (uint32_t)(st.s * kCols);
-#pragma unroll 1
-          for (int b0 = 0; b0 < NB; b0 += kSet) {
-            float x[4 * kSet];
-            ld_block<kSet>(at + (uint32_t)(8 * b0), x);
-            uint64_t c[kSet];
+          const uint32_t at = addr + (uint32_t)(st.s * kStage);
+          auto blocks = [&](auto count, int b0) {
+            constexpr int kN = decltype(count)::value;
+            float x[4 * kN];
+            ld_block<kN>(at + (uint32_t)(8 * b0), x);
+            uint64_t c[kN];
 #pragma unroll
-            for (int b = 0; b < kSet; ++b) c[b] = *reinterpret_cast<const uint64_t*>(&my_c[8 * (b0 + b)]);
+            for (int b = 0; b < kN; ++b) c[b] = *reinterpret_cast<const uint64_t*>(&my_c[8 * (b0 + b)]);
             tc_wait_ld();
-            if (b0 + kSet == NB) {
+            if (b0 + kN == NB) {
               tc_fence_before();
               __syncwarp();
               if (lane == 0) mbar_arrive(TEMPTY(st.s));
             }
 #pragma unroll
-            for (int b = 0; b < kSet; ++b)
+            for (int b = 0; b < kN; ++b)
 #pragma unroll
               for (int j = 0; j < 2; ++j) sum[2 * j + (b & 1)] = exp2_acc2(false, sum[2 * j + (b & 1)], x[4 * b + 2 * j], x[4 * b + 2 * j + 1], scale22, c[b]);
-          }
+          };
+#pragma unroll 1
+          for (int b0 = 0; b0 + kSet <= NB; b0 += kSet) blocks(std::integral_constant<int, kSet>(), b0);
+          if constexpr (NB % kSet) blocks(std::integral_constant<int, NB % kSet>(), NB - NB % kSet);
           st.next();
           // over all columns; a lane pair ends with one key
           float s0, s1, u, v;
@@ -464,7 +484,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           ok = wait(FULL(s), kr.ph, 104) && wait(TEMPTY(st.s), st.ph, 105);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t d = tmem_base + (uint32_t)((pipe * kPer + st.s) * kCols), k_lo = q_lo + ((uint32_t)(s * kSlotBytes) >> 4);
+          const uint32_t d = tmem_base + (uint32_t)((pipe * kPer + st.s) * kStage), k_lo = q_lo + ((uint32_t)(s * kSlotBytes) >> 4);
           if (a.D == 128) {
             tc_mma_x8<(kHalfBytes >> 4), (kHalfBytes >> 4)>(d, k_lo, q_lo, hi, a.idesc);
           } else {

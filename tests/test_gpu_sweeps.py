@@ -90,3 +90,10 @@ def test_a_head_with_a_key_that_is_no_number_spoils_no_other():
         assert ((got[0, ::2] - want[0, ::2]).abs() <= 5e-5 * want[0, ::2]).all()
     finally:
         B.dkv_destroy(h)
+
+
+# the builds are 16 window rows apart: 16, 17, 48, 49, 80, 81, 112, 113 rows, two planes of 72 and of 112, and of 88 with 16 empty ones
+@pytest.mark.parametrize("G,ws,D", [(1, 16, 64), (1, 17, 128), (3, 16, 128), (7, 7, 64), (5, 16, 64), (3, 27, 128), (7, 16, 128), (1, 113, 64),
+                                    (5, 28, 128), (7, 32, 64), (7, 24, 128)])
+def test_window_rows_around_sixteens(G, ws, D):
+    _passes(2, 2, G, D, 1, 900, ws, 5)
