@@ -558,8 +558,8 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
 // ------------------------------------------------------------------------------------------ pooling
 // Eq. 2's pooling of the unpooled scores (the sum over a head's planes), and the digits of the result for the updates.
 // raw: [heads * planes][raw_stride].  scores: [heads][P].  layer_hist: [layers][samples][kBins] counters that a sweep before has cleared.  grid heads * segs, segs = ceil(P / seg), seg
-// (a multiple of the threads, kPoolSeg at most): as many as give every SM two blocks.  Bound by the L2: 32 layers of 32K, 67 MB
-// in and out, take 13 us.
+// (a multiple of the threads, kPoolSeg at most): as many as give every SM two blocks.  Bound by instructions (neighbours,
+// digits, counters), not by memory: 16 layers of 32K, 17 MB in from L2 and as much out, take 22 us where a copy of it takes 5.
 constexpr int kPoolThreads = 256, kPoolSeg = 2048;
 __global__ void __launch_bounds__(kPoolThreads)
 pool_kernel(const float* raw, float* scores, unsigned int* layer_hist, int P, int raw_stride, int planes, int half, int avg, int hkv, int seg, int segs) {
