@@ -150,6 +150,17 @@ __device__ __forceinline__ float dot8(uint4 a, uint4 b, float s) {       // + ei
   return s;
 }
 
+// A sum of 2^64 or more hands its exponent to its reference.  Parts are added relative to the largest reference, whose own sum is at
+// least 1: with sums below 2^64 no number of them reaches infinity, and what is lost where a factor is below the smallest normal
+// float (2^-126) is below 2^-62 of the result.
+__device__ __forceinline__ void lower_sum(float& ref, float& sum) {
+  if (sum >= 0x1p64f && sum < INFINITY) {
+    const int e = (__float_as_int(sum) >> 23) - 127;
+    sum = __int_as_float(__float_as_int(sum) - (e << 23));
+    ref += (float)e;
+  }
+}
+
 // ------------------------------------------------------------------------------------------ kernel
 template <int NB, int kSweep>
 __global__ void __launch_bounds__(kOneThreads, 1)
@@ -532,6 +543,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           for (int w = 0; w < 4; ++w) {
             m[w] = ref_s[(pipe * 4 + w) * kCols + row];
             l[w] = sum_s[(pipe * 4 + w) * kCols + row];
+            lower_sum(m[w], l[w]);
             if (l[w] != 0.f) top = fmaxf(top, m[w]);    // (0: no key of this quad counts for the row)
           }
 #pragma unroll

@@ -74,6 +74,28 @@ def test_logits_that_are_far_above_the_first_key_of_a_segment():
     _passes(2, 2, 2, 64, 1, 2000, 8, 5, far, most=2e-4)      # |t| < 512: 2^-16 ln 2 and more
 
 
+# One key of every 128 a little less than 88.7 nats (128 bits) above the others: the sums of the segments are finite, and would
+# not be together.  |t| < 256: 2^-17 ln 2 a factor.
+@pytest.mark.parametrize("nats", [82.0, 83.5, 84.0, 87.0, 88.5, 89.0, 95.0])
+@pytest.mark.parametrize("L,Hkv,S", [(1, 1, 32768), (1, 3, 4999), (40, 8, 520)])    # a head in 256 segments, in 40, in one or two
+def test_sums_of_segments_that_no_float_can_hold_together(L, Hkv, S, nats):
+    def far(q, k):
+        for x, y in zip(q, k):
+            x[..., 0], y[..., 0], y[:, 0, 5::128, 0] = 16.0, 0.0, nats / 2
+    _passes(L, Hkv, 1, 64, 1, S, 8, 5, far, most=1e-4)
+
+
+# A sum of nearly 2^128 relative to its own reference, and another part whose reference is 126.6 bits above that one, so that the
+# factor between them is below the smallest normal float; in another quarter of the tile, and in another segment.
+@pytest.mark.parametrize("at", [32, 3 * 128])
+def test_a_large_sum_beside_a_large_reference(at):
+    def far(q, k):
+        q[0][...], k[0][...] = 0.0, 0.0
+        q[0][..., :2] = 16.0
+        k[0][:, :, 5, 0], k[0][:, :, at, 0], k[0][:, :, at, 1] = 44.25, 43.5, 0.375      # 88.5 and 87.75 nats
+    _passes(1, 1, 1, 64, 1, 2056, 8, 1, far, most=1e-4)
+
+
 def test_a_head_with_a_key_that_is_no_number_spoils_no_other():
     g = torch.Generator(device="cuda").manual_seed(1)
     new = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
