@@ -228,7 +228,6 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
   };
   auto row0_of = [&](int vh) { return (vh & (a.planes - 1)) * a.plane_rows; };
   auto wait = [&](uint32_t bar, uint32_t parity, int code) { return mbar_wait(bar, parity, abort_flag, a.status, code, a.wait_cycles); };
-  auto give_registers = [] { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs)); };
   const long long tiles = (long long)a.vheads * a.tph;
   // Minus the log-denominators of rows [r, r + 16) of a (head, plane), two lanes a row -> to[]: from the parts that the head's
   // segments have left, four in flight a lane, or the caller's.
@@ -259,6 +258,8 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     if (!(lane & 1)) to[row] = c;
   };
 
+  // The warps of a warpgroup have to change their registers by the same instruction: here, before the roles part.
+  if (warp >= kSoftWarps) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
   if (warp < kSoftWarps) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftRegs));
     // ------------------------------------------------------------------ exponentials and sums
@@ -436,7 +437,6 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
       }
     }
   } else if (warp < kMmaWarp) {
-    give_registers();
     // ------------------------------------------------------------------ copies
     if (lane == 0) {
       const int halves = a.D / 64;
@@ -479,7 +479,6 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
         for (int s = 0; s < kSlots; ++s) if (used >> s & 1u) mbar_drain(FULL(s), parity >> s & 1u);
     }
   } else if (warp < kRowWarp) {
-    give_registers();
     // ------------------------------------------------------------------ MMAs
     if (lane == 0) {
       const uint64_t desc = smem_desc(smem_u32(ring + pipe * kSlots * kSlotBytes));
@@ -515,7 +514,6 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
       }
     }
   } else if (warp < kPublishWarp) {
-    give_registers();
     // ------------------------------------------------------------------ log-denominators of the segments but the first
     Segs sg(a, 2 * blockIdx.x + pipe, 2 * grid);
     for (int i = 0; !kRows && sg.next(); ++i) {
@@ -528,7 +526,6 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
       if (lane == 0) mbar_arrive(CFULL(slot));
     }
   } else {
-    give_registers();
     // ------------------------------------------------------------------ a segment's row sums -> the rows' counters
     if constexpr (kRows) {
       Segs sg(a, 2 * blockIdx.x + pipe, 2 * grid);

@@ -51,3 +51,16 @@ def test_no_read_of_such_a_kernel_is_marked_read_only(header):
     for name, params, _ in functions:
         if name in waiting or name in called or not name.endswith("_kernel"):
             assert "__restrict__" not in params, name
+
+
+def test_a_warpgroup_changes_its_registers_by_one_instruction():
+    """setmaxnreg has to be the same instruction for all warps of a warpgroup, and a block's shares no more than it was launched with."""
+    text = _source("score_sweep.cuh")
+    kernel = {n: body for n, _, body in _functions(text)}["score_sweep_kernel"]
+    changes = re.findall(r"if \(warp (<|>=) kSoftWarps\) \{?\s*asm volatile\(\"setmaxnreg\.(inc|dec)\.", kernel)
+    assert sorted(changes) == [("<", "inc"), (">=", "dec")] and text.count("setmaxnreg") == 2
+    value = {n: int(v) for n, v in re.findall(r"\b(k\w+) = (\d+)\b", text)}
+    soft, warps = value["kSoftWarps"], value["kWarps"]
+    assert soft % 4 == 0 and warps % 4 == 0
+    at_launch = 65536 // (warps * 32) // 8 * 8
+    assert soft * value["kSoftRegs"] + (warps - soft) * value["kOtherRegs"] <= warps * at_launch
