@@ -54,7 +54,7 @@ struct Shape1 {
   static constexpr int kPer = NB <= 8 ? 4 : 2;                              // accumulator stages of a pipe,
   static constexpr int kStage = (kCols + 31) / 32 * 32;                     // this many columns apart
   static constexpr int kQBytes = kCols * 128;                               // window rows x 64 dims
-  static constexpr int kPipeBars = 2 * kSlots + 2 * kPer + 5, kBars = 2 * kPipeBars + 1;
+  static constexpr int kPipeBars = 2 * kSlots + 2 * kPer + 6, kBars = 2 * kPipeBars;
   static constexpr int kSmem = 1024 + 2 * kSlots * kSlotBytes + 2 * 4 * kCols * 8 + 3 * 2 * kCols * 4 + kBars * 8;
   static_assert(kSmem + 1024 <= 227 * 1024 && 2 * kPer * kStage <= 512, "shared and tensor memory of an SM");
 };
@@ -188,7 +188,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
   auto CFULL = [&](int i) { return pbar + 8u * (2 * kSlots + 2 * kPer + i); };        // references or log-denominators are there
   auto CEMPTY = [&](int i) { return pbar + 8u * (2 * kSlots + 2 * kPer + 2 + i); };   // the segment is done (row sums are in sum_s)
   const uint32_t SUMFREE = pbar + 8u * (2 * kSlots + 2 * kPer + 4);         // row sums have been read
-  const uint32_t DRAIN = bar0 + 8u * (2 * C::kPipeBars);
+  const uint32_t DRAIN = pbar + 8u * (2 * kSlots + 2 * kPer + 5);           // all MMAs have ended
   volatile int* abort_flag = &abort_s;
 
   if (threadIdx.x == 0) {
@@ -198,9 +198,8 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
       for (int s = 0; s < 2 * kSlots + kPer; ++s) mbar_init(b + 8u * s, 1);             // FULL, EMPTY, TFULL
       for (int s = 0; s < kPer; ++s) mbar_init(b + 8u * (2 * kSlots + kPer + s), kLaneWarps);
       for (int i = 0; i < 2; ++i) { mbar_init(b + 8u * (2 * kSlots + 2 * kPer + i), 1); mbar_init(b + 8u * (2 * kSlots + 2 * kPer + 2 + i), kLaneWarps); }
-      mbar_init(b + 8u * (2 * kSlots + 2 * kPer + 4), 1);
+      for (int i = 4; i < 6; ++i) mbar_init(b + 8u * (2 * kSlots + 2 * kPer + i), 1);
     }
-    mbar_init(DRAIN, 2);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == kMmaWarp) {
@@ -227,6 +226,8 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     return a.stats + ((size_t)vh * a.slots + place) * a.plane_rows;
   };
   auto row0_of = [&](int vh) { return (vh & (a.planes - 1)) * a.plane_rows; };
+  // What whole warps wait for they go on without once a wait has run out, as no wait blocks any more then: whether it had come is for
+  // each lane to see, and lanes that left a loop alone would be missing from its next shuffle.  Single lanes stop.
   auto wait = [&](uint32_t bar, uint32_t parity, int code) { return mbar_wait(bar, parity, abort_flag, a.status, code, a.wait_cycles); };
   const long long tiles = (long long)a.vheads * a.tph;
   // Minus the log-denominators of rows [r, r + 16) of a (head, plane), two lanes a row -> to[]: from the parts that the head's
@@ -281,17 +282,15 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
       } else if (i == 0) {                              // the first segment's are needed soon: 16 rows a warp
         if (16 * part < kCols) fill(c_s + 2 * pipe * kCols, sg.vh, 16 * part);
         asm volatile("bar.sync %0, 256;" ::"r"(1 + pipe) : "memory");
-      } else if (!wait(CFULL(slot), i >> 1 & 1, 106)) {
-        break;
+      } else {
+        wait(CFULL(slot), i >> 1 & 1, 106);
       }
-      bool ok = true;
       if constexpr (kRows) {
         uint64_t c[kHalf], sum[kHalf];                  // minus the references; sums over the thread's keys so far, by columns
 #pragma unroll
         for (int b = 0; b < kHalf; ++b) c[b] = sum[b] = 0ull;
         for (int t = 0; t < sg.n; ++t) {
-          ok = wait(TFULL(st.s), st.ph, 106);
-          if (!ok) break;
+          wait(TFULL(st.s), st.ph, 106);
           tc_fence_after();
           const bool masked = (sg.t0 + t + 1) * kTile - 1 > a.P;            // row r sees keys 0 .. P + r % ws
           const uint32_t at = addr + (uint32_t)(st.s * kStage);
@@ -329,10 +328,9 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           }
           st.next();
         }
-        if (!ok) break;
         // Over the 8 lanes that have a column's keys: halves are exchanged, so that a lane ends with one pair of columns of four blocks.
         auto swap = [&](int o, uint64_t lo_v, uint64_t hi_v) { return add2(lane & o ? hi_v : lo_v, __shfl_xor_sync(0xFFFFFFFFu, lane & o ? lo_v : hi_v, o)); };
-        if (!wait(SUMFREE, (i & 1) ^ 1, 106)) break;
+        wait(SUMFREE, (i & 1) ^ 1, 106);
         float* my_sum = sum_s + (pipe * 4 + quad) * kCols + col2;
         if (lane < 4)
 #pragma unroll
@@ -360,8 +358,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
         const float* my_c = c_s + (2 * pipe + slot) * kCols + col2;
         float* raw = a.raw + ((size_t)sg.vh * a.tph + sg.t0) * kTile + key + (lane & 1) * 8;
         for (int t = 0; t < sg.n; ++t, raw += kTile) {
-          ok = wait(TFULL(st.s), st.ph, 106);
-          if (!ok) break;
+          wait(TFULL(st.s), st.ph, 106);
           tc_fence_after();
           uint64_t sum[4] = {0ull, 0ull, 0ull, 0ull};   // over the columns so far, by key and parity of the block
           const uint32_t at = addr + (uint32_t)(st.s * kStage);
@@ -398,7 +395,6 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           r += __shfl_xor_sync(0xFFFFFFFFu, r, 2);
           if (!(lane & 2)) *raw = r * a.post;
         }
-        if (!ok) break;
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(CEMPTY(slot));
@@ -475,8 +471,9 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           kr.next();
         }
       }
-      if (!ok || *abort_flag)       // copies that may still be on their way must land before this block's shared memory is given up
-        for (int s = 0; s < kSlots; ++s) if (used >> s & 1u) mbar_drain(FULL(s), parity >> s & 1u);
+      // Copies land before this block's shared memory is given up, and MMAs (below) end before its tensor memory is, whenever another
+      // warp's wait has run out.
+      for (int s = 0; s < kSlots; ++s) if (used >> s & 1u) mbar_drain(FULL(s), parity >> s & 1u);
     }
   } else if (warp < kRowWarp) {
     // ------------------------------------------------------------------ MMAs
@@ -508,17 +505,15 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
         }
         if (ok) tc_commit(EMPTY(0));
       }
-      if (!ok || *abort_flag) {     // the MMAs end before tensor memory is given up
-        tc_commit(DRAIN);
-        mbar_drain(DRAIN, 0);
-      }
+      tc_commit(DRAIN);
+      mbar_drain(DRAIN, 0);
     }
   } else if (warp < kPublishWarp) {
     // ------------------------------------------------------------------ log-denominators of the segments but the first
     Segs sg(a, 2 * blockIdx.x + pipe, 2 * grid);
     for (int i = 0; !kRows && sg.next(); ++i) {
       const int slot = i & 1;
-      if (!wait(CEMPTY(slot), (i >> 1 & 1) ^ 1, 107)) break;                // the segment before last is done with its own
+      wait(CEMPTY(slot), (i >> 1 & 1) ^ 1, 107);                            // the segment before last is done with its own
       if (i > 0)
 #pragma unroll 1
         for (int r = 0; r < kCols; r += 16) fill(c_s + (2 * pipe + slot) * kCols, sg.vh, r);
@@ -532,7 +527,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
       for (int i = 0; sg.next(); ++i) {
         const int rows = min(a.M - row0_of(sg.vh), a.plane_rows);
         float2* to = sums_of(sg.vh, pipe);
-        if (!wait(CEMPTY(i & 1), i >> 1 & 1, 107)) break;
+        wait(CEMPTY(i & 1), i >> 1 & 1, 107);
 #pragma unroll 1
         for (int row = lane; row < rows; row += 32) {
           float m[4], l[4], top = -INFINITY, sum = 0.f;

@@ -62,6 +62,43 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(sweep):
         B.dkv_destroy(ctx)
 
 
+# A pipe with one tile and pipes with five, in which the copy after the withheld tile waits for its slot; with a limit of a millisecond,
+# and with the shortest one, which any wait may exceed.
+@pytest.mark.parametrize("use,sweep", [("pass", 1), ("pass", 2), ("lse", 2)])
+@pytest.mark.parametrize("S,tile,limit", [(300, 0, 2_000_000), (6200, 0, 2_000_000), (6200, 3, 2_000_000), (6200, 3, 1000)])
+def test_a_wait_that_runs_out_in_a_pass_is_reported_and_the_context_stays_usable(use, sweep, S, tile, limit):
+    L, Hkv, G, D, ws = 4, 8, 2, 64, 16
+    g = torch.Generator(device="cuda").manual_seed(S)
+    new = lambda *s: [torch.randn(s, generator=g, device="cuda").to(torch.bfloat16) for _ in range(L)]
+    q, k, v = new(1, G * Hkv, ws, D), new(1, Hkv, S, D), new(1, Hkv, S, D)
+    kb, vb = ([torch.zeros((1, Hkv, 64 + ws, D), device="cuda", dtype=torch.bfloat16) for _ in range(L)] for _ in range(2))
+    hidden = torch.arange(S, device="cuda") > (S - ws + torch.arange(ws, device="cuda")).repeat(G)[:, None]
+    logits = [(a.double().view(1, Hkv, G * ws, D) @ b.double().transpose(-1, -2) / D ** 0.5).masked_fill(hidden, -torch.inf) for a, b in zip(q, k)]
+    lse = [t.logsumexp(-1).view(1, Hkv * G, ws).float().contiguous() for t in logits]
+    want = [t.softmax(-1)[..., :S - ws].sum(2).cpu() for t in logits]
+    ctx = B.dkv_create(B.make_config(L, G * Hkv, Hkv, D, 1, S, ws, 1, 32, 64, 2))
+    run = (lambda: B.dkv_run_prefill_pass_lse(ctx, q, k, v, lse, kb, vb)) if use == "lse" else (lambda: B.dkv_run_prefill_pass(ctx, q, k, v, kb, vb))
+    try:
+        for _ in range(3):
+            B.dkv_set_wait_limit(ctx, limit)
+            B.dkv_debug_withhold_tile(ctx, sweep, tile)
+            run()
+            code, status = B.dkv_last_status(ctx)
+            assert code == B.DKV_ERR_TIMEOUT and 101 <= status[0] <= 107, f"{code} {status}"
+            assert limit == 1000 or status[2] == 0
+            assert B.dkv_last_status(ctx)[0] == B.DKV_OK
+            B.dkv_debug_withhold_tile(ctx, 0, -1)
+            B.dkv_set_wait_limit(ctx, 4_000_000_000)
+            run()
+            assert B.dkv_last_status(ctx)[0] == B.DKV_OK
+            for l in range(L):
+                got = torch.zeros((1, Hkv, S - ws))
+                B.dkv_memcpy_to_host(ctx, got, B.dkv_layer_views(ctx, l)[0], got.numel() * 4)
+                assert ((got - want[l]).abs() <= 5e-5 * want[l]).all()
+    finally:
+        B.dkv_destroy(ctx)
+
+
 def test_wait_limit_and_hook_arguments_are_checked():
     ctx = B.dkv_create(B.config_of(synth.WORKLOADS["tiny"]))
     try:
