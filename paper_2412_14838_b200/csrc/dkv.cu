@@ -364,7 +364,6 @@ int launch_sweeps(dkv_ctx* c, int layer, int nl, const void* const* q, const voi
   for (int i = 0; i < nl; ++i) {
     if (!make_map(&maps.q[i], q[i], s.D, s.M, heads, 8 * nb) || !make_map(&maps.k[i], k[i], s.D, s.S, heads)) return DKV_ERR_CUDA;
     maps.lse[i] = lse ? lse[i] : nullptr;
-    maps.q_at[i] = static_cast<const uint4*>(q[i]); maps.k_at[i] = static_cast<const uint4*>(k[i]);
   }
   sweep::Args a;
   memset(&a, 0, sizeof a);

@@ -17,7 +17,9 @@
 //
 // Row sums are e = 2^(t - m) with m the logit of the first key that the warp has seen in the segment: as that key counts with
 // e = 1, no maximum is searched, and a sum only fails where another logit is 127 bits above it (or is infinite, or a NaN).  It is
-// infinite or a NaN then, and the block computes that row of its segment again without tensor cores, from its maximum.
+// infinite or a NaN then, and the pipe sweeps that segment twice more when it has come to its end, for the largest logits and for
+// sums relative to them (a pass of 32 layers of 32K, 8 heads of 128, 128 rows: 0.83 ms, with one such head 1.12, with all of them
+// 3.15; by the ordinary cores, row by row on the block that had the segment, 18.8 and 70).
 //
 // What bounds it: a tile takes an SM 0.7 (row sums) and 0.8 us (key sums), 5.9-6.8 TB/s, near the 6.5 of a copy, in the launches
 // of eight layers of 32K; a whole pass over 32K runs at the power limit, 0.95 us a tile.  The softmax loops bound what is in L2:
@@ -79,7 +81,6 @@ struct Args {
 
 struct Layers {                                // by layer of the launch
   CUtensorMap q[kMaxGroup], k[kMaxGroup];
-  const uint4 *q_at[kMaxGroup], *k_at[kMaxGroup];      // what they describe
   const float* lse[kMaxGroup];
 };
 
@@ -106,24 +107,20 @@ __device__ __forceinline__ void ld_block(uint32_t a, float* v) {
     asm volatile("tcgen05.ld.sync.aligned.16x256b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]) : "r"(a));
 }
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
 
 // ------------------------------------------------------------------------------------------ order of work
-// The segments of one pipe: its range of the tiles, cut at the heads.
+// The segments of a range of the tiles: the range cut at the heads.
 struct Segs {
   int g, end, tph;                              // what is left of the range
   int vh, t0, n;                                // the segment: (head, plane), first tile, tiles
-  __device__ Segs(const Args& a, int pipe, int pipes) : tph(a.tph), t0(0), n(0) {
-    const long long tiles = (long long)a.vheads * a.tph;
-    g = (int)(tiles * pipe / pipes); end = (int)(tiles * (pipe + 1) / pipes);
+  __device__ Segs(int g_, int end_, int tph_) : g(g_), end(end_), tph(tph_), n(0) {
     vh = g / tph;
     t0 = g - vh * tph;
     --vh;                                       // next() begins with it
   }
+  // those of one pipe
+  __device__ Segs(const Args& a, int pipe, int pipes)
+      : Segs((int)((long long)a.vheads * a.tph * pipe / pipes), (int)((long long)a.vheads * a.tph * (pipe + 1) / pipes), a.tph) {}
   __device__ bool next() {
     if (g >= end) return false;
     if (n) t0 = 0;
@@ -139,16 +136,6 @@ struct Ring {
   __device__ Ring(int n_, int ph_) : s(0), ph(ph_), n(n_) {}
   __device__ void next() { if (++s == n) { s = 0; ph ^= 1; } }
 };
-
-__device__ __forceinline__ float dot8(uint4 a, uint4 b, float s) {       // + eight products of bf16 pairs
-  const uint32_t x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    s = fmaf(__uint_as_float(x[i] << 16), __uint_as_float(y[i] << 16), s);
-    s = fmaf(__uint_as_float(x[i] & 0xFFFF0000u), __uint_as_float(y[i] & 0xFFFF0000u), s);
-  }
-  return s;
-}
 
 // A sum of 2^64 or more hands its exponent to its reference.  Parts are added relative to the largest reference, whose own sum is at
 // least 1: with sums below 2^64 no number of them reaches infinity, and what is lost where a factor is below the smallest normal
@@ -176,7 +163,8 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
   int* last_s = reinterpret_cast<int*>(c_s + 4 * kCols);                    // [2][kCols] last key that a plane's row sees
   uint64_t* bars = reinterpret_cast<uint64_t*>(last_s + 2 * kCols);
   __shared__ uint32_t tmem_base_s;
-  __shared__ int abort_s, redo_s;
+  __shared__ int abort_s;
+  __shared__ int again_s[2][2];                 // a pipe's tiles from the first to the last segment with a sum that is not finite
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grid = gridDim.x;
   const int pipe = warp < kSoftWarps ? warp / kLaneWarps : warp & 1;
   const uint32_t bar0 = smem_u32(bars), pbar = bar0 + 8u * (pipe * C::kPipeBars);
@@ -192,7 +180,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
   volatile int* abort_flag = &abort_s;
 
   if (threadIdx.x == 0) {
-    abort_s = redo_s = 0;
+    abort_s = 0;
     for (int p = 0; p < 2; ++p) {
       const uint32_t b = bar0 + 8u * (p * C::kPipeBars);
       for (int s = 0; s < 2 * kSlots + kPer; ++s) mbar_init(b + 8u * s, 1);             // FULL, EMPTY, TFULL
@@ -206,6 +194,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::);
   }
+  if (kRows && threadIdx.x < 4) again_s[threadIdx.x >> 1][threadIdx.x & 1] = 0;
   if (kRows && threadIdx.x < 2 * kCols) last_s[threadIdx.x] = a.P + (threadIdx.x / kCols * a.plane_rows + threadIdx.x % kCols) % a.ws;
   tc_fence_before();
   __syncthreads();
@@ -230,6 +219,22 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
   // each lane to see, and lanes that left a loop alone would be missing from its next shuffle.  Single lanes stop.
   auto wait = [&](uint32_t bar, uint32_t parity, int code) { return mbar_wait(bar, parity, abort_flag, a.status, code, a.wait_cycles); };
   const long long tiles = (long long)a.vheads * a.tph;
+  // Row sums: all warps of the block meet after the pipes' segments, and those of a pipe with a sum that is not finite go round a second
+  // time, over its segments from the first to the last such one.
+  auto second_round = [&](Segs& sg) {
+    __syncwarp();
+    asm volatile("bar.sync 3, %0;" ::"n"(kOneThreads) : "memory");
+    if (!again_s[pipe][1]) return false;
+    sg = Segs(again_s[pipe][0], again_s[pipe][1], a.tph);
+    return true;
+  };
+  // f(segments, round) for each round, in two copies: what only the second round does, in the way of the first, made a pass of four
+  // layers of 1K 0.4 to 1 us longer (of 38).
+  auto rounds = [&](auto f) {
+    Segs sg(a, 2 * blockIdx.x + pipe, 2 * grid);
+    f(sg, std::integral_constant<int, 0>());
+    if constexpr (kRows) if (second_round(sg)) f(sg, std::integral_constant<int, 1>());
+  };
   // Minus the log-denominators of rows [r, r + 16) of a (head, plane), two lanes a row -> to[]: from the parts that the head's
   // segments have left, four in flight a lane, or the caller's.
   auto fill = [&](float* to, int vh, int r) {
@@ -275,180 +280,180 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     const int col2 = c0 + 2 * (lane & 3), key = first + (lane >> 2);        // the thread's keys: key, key + 8 (, key + 16, key + 24)
     if (kSweep != kKeySums) for (int i = blockIdx.x * (kSoftWarps * 32) + threadIdx.x; i < a.hist_n; i += grid * (kSoftWarps * 32)) a.hist[i] = 0;
     Ring st(kPer, 0);
-    Segs sg(a, 2 * blockIdx.x + pipe, 2 * grid);
-    for (int i = 0; sg.next(); ++i) {
-      const int slot = i & 1;
-      if (kRows) {
-      } else if (i == 0) {                              // the first segment's are needed soon: 16 rows a warp
-        if (16 * part < kCols) fill(c_s + 2 * pipe * kCols, sg.vh, 16 * part);
-        asm volatile("bar.sync %0, 256;" ::"r"(1 + pipe) : "memory");
-      } else {
-        wait(CFULL(slot), i >> 1 & 1, 106);
-      }
-      if constexpr (kRows) {
-        uint64_t c[kHalf], sum[kHalf];                  // minus the references; sums over the thread's keys so far, by columns
+    int i = 0;                                          // segments so far
+    rounds([&](Segs& sg, auto round_) {
+      constexpr int round = decltype(round_)::value;
+      for (; sg.next(); ++i) {
+        const int slot = i & 1;
+        if (kRows) {
+        } else if (i == 0) {                              // the first segment's are needed soon: 16 rows a warp
+          if (16 * part < kCols) fill(c_s + 2 * pipe * kCols, sg.vh, 16 * part);
+          asm volatile("bar.sync %0, 256;" ::"r"(1 + pipe) : "memory");
+        } else {
+          wait(CFULL(slot), i >> 1 & 1, 106);
+        }
+        if constexpr (kRows) {
+          uint64_t c[kHalf], sum[kHalf];                  // minus the references; sums over the thread's keys so far, by columns
 #pragma unroll
-        for (int b = 0; b < kHalf; ++b) c[b] = sum[b] = 0ull;
-        for (int t = 0; t < sg.n; ++t) {
-          wait(TFULL(st.s), st.ph, 106);
-          tc_fence_after();
-          const bool masked = (sg.t0 + t + 1) * kTile - 1 > a.P;            // row r sees keys 0 .. P + r % ws
-          const uint32_t at = addr + (uint32_t)(st.s * kStage);
-#pragma unroll 1
-          for (int h = 0; h < 2; ++h) {
-            float x[4 * kHalf];
-            const uint32_t from = at + (uint32_t)(h << 20);                 // 16 lanes on
-            ld_block<kHalf>(from, x);
+          for (int b = 0; b < kHalf; ++b) c[b] = sum[b] = 0ull;
+          auto mask = [&](float (&x)[4 * kHalf], int t, int h) {              // row r sees keys 0 .. P + r % ws
+            if ((sg.t0 + t + 1) * kTile - 1 <= a.P) return;
+            const int *last = last_s + (sg.vh & (a.planes - 1)) * kCols + col2, k0 = (sg.t0 + t) * kTile + key + 16 * h;
+#pragma unroll
+            for (int b = 0; b < kHalf; ++b) {
+              const int2 to = *reinterpret_cast<const int2*>(&last[8 * b]);
+              x[4 * b] = k0 > to.x ? -INFINITY : x[4 * b]; x[4 * b + 1] = k0 > to.y ? -INFINITY : x[4 * b + 1];
+              x[4 * b + 2] = k0 + 8 > to.x ? -INFINITY : x[4 * b + 2]; x[4 * b + 3] = k0 + 8 > to.y ? -INFINITY : x[4 * b + 3];
+            }
+          };
+          auto read = [&](float (&x)[4 * kHalf], int h) {                     // the tile's lanes 16 h on
+            ld_block<kHalf>(addr + (uint32_t)(st.s * kStage + (h << 20)), x);
             tc_wait_ld();
             if (h) {
               tc_fence_before();
               __syncwarp();
               if (lane == 0) mbar_arrive(TEMPTY(st.s));
             }
-            if (t + h == 0) {
-#pragma unroll
-              for (int b = 0; b < kHalf; ++b) {
-                const float r0 = __shfl_sync(0xFFFFFFFFu, x[4 * b], lane & 3), r1 = __shfl_sync(0xFFFFFFFFu, x[4 * b + 1], lane & 3);
-                c[b] = pack2(r0 * -a.scale2, r1 * -a.scale2);
-              }
-            }
-            if (masked) {
-              const int *last = last_s + (sg.vh & (a.planes - 1)) * kCols + col2, k0 = (sg.t0 + t) * kTile + key + 16 * h;
-#pragma unroll
-              for (int b = 0; b < kHalf; ++b) {
-                const int2 to = *reinterpret_cast<const int2*>(&last[8 * b]);
-                x[4 * b] = k0 > to.x ? -INFINITY : x[4 * b]; x[4 * b + 1] = k0 > to.y ? -INFINITY : x[4 * b + 1];
-                x[4 * b + 2] = k0 + 8 > to.x ? -INFINITY : x[4 * b + 2]; x[4 * b + 3] = k0 + 8 > to.y ? -INFINITY : x[4 * b + 3];
-              }
-            }
-#pragma unroll
-            for (int b = 0; b < kHalf; ++b)
-#pragma unroll
-              for (int j = 0; j < 2; ++j) sum[b] = exp2_acc2(false, sum[b], x[4 * b + 2 * j], x[4 * b + 2 * j + 1], scale22, c[b]);
-          }
-          st.next();
-        }
-        // Over the 8 lanes that have a column's keys: halves are exchanged, so that a lane ends with one pair of columns of four blocks.
-        auto swap = [&](int o, uint64_t lo_v, uint64_t hi_v) { return add2(lane & o ? hi_v : lo_v, __shfl_xor_sync(0xFFFFFFFFu, lane & o ? lo_v : hi_v, o)); };
-        wait(SUMFREE, (i & 1) ^ 1, 106);
-        float* my_sum = sum_s + (pipe * 4 + quad) * kCols + col2;
-        if (lane < 4)
-#pragma unroll
-          for (int b = 0; b < kHalf; ++b) *reinterpret_cast<uint64_t*>(&ref_s[(pipe * 4 + quad) * kCols + col2 + 8 * b]) = c[b] ^ 0x8000000080000000ull;
-#pragma unroll
-        for (int b = 0; b + 4 <= kHalf; b += 4) {
-          uint64_t u = swap(8, swap(16, sum[b], sum[b + 2]), swap(16, sum[b + 1], sum[b + 3]));
-          u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, 4));
-          if (!(lane & 4)) *reinterpret_cast<uint64_t*>(&my_sum[8 * (b + (lane >> 3))]) = u;
-        }
-        if constexpr (kHalf & 2) {
-          constexpr int b = kHalf & ~3;
-          uint64_t u = swap(16, sum[b], sum[b + 1]);
-          u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, 8));
-          u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, 4));
-          if (!(lane & 12)) *reinterpret_cast<uint64_t*>(&my_sum[8 * (b + (lane >> 4))]) = u;
-        }
-        if constexpr (kHalf & 1) {
-          uint64_t u = sum[kHalf - 1];
-#pragma unroll
-          for (int o = 16; o >= 4; o >>= 1) u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, o));
-          if (lane < 4) *reinterpret_cast<uint64_t*>(&my_sum[8 * (kHalf - 1)]) = u;
-        }
-      } else {
-        const float* my_c = c_s + (2 * pipe + slot) * kCols + col2;
-        float* raw = a.raw + ((size_t)sg.vh * a.tph + sg.t0) * kTile + key + (lane & 1) * 8;
-        for (int t = 0; t < sg.n; ++t, raw += kTile) {
-          wait(TFULL(st.s), st.ph, 106);
-          tc_fence_after();
-          uint64_t sum[4] = {0ull, 0ull, 0ull, 0ull};   // over the columns so far, by key and parity of the block
-          const uint32_t at = addr + (uint32_t)(st.s * kStage);
-          auto blocks = [&](auto count, int b0) {
-            constexpr int kN = decltype(count)::value;
-            float x[4 * kN];
-            ld_block<kN>(at + (uint32_t)(8 * b0), x);
-            uint64_t c[kN];
-#pragma unroll
-            for (int b = 0; b < kN; ++b) c[b] = *reinterpret_cast<const uint64_t*>(&my_c[8 * (b0 + b)]);
-            tc_wait_ld();
-            if (b0 + kN == NB) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(TEMPTY(st.s));
-            }
-#pragma unroll
-            for (int b = 0; b < kN; ++b)
-#pragma unroll
-              for (int j = 0; j < 2; ++j) sum[2 * j + (b & 1)] = exp2_acc2(false, sum[2 * j + (b & 1)], x[4 * b + 2 * j], x[4 * b + 2 * j + 1], scale22, c[b]);
           };
+          if constexpr (round > 0) {                      // the largest logits
+            float m[2 * kHalf];
+#pragma unroll
+            for (int b = 0; b < 2 * kHalf; ++b) m[b] = -INFINITY;
+            for (int t = 0; t < sg.n; ++t) {
+              wait(TFULL(st.s), st.ph, 106);
+              tc_fence_after();
 #pragma unroll 1
-          for (int b0 = 0; b0 + kSet <= NB; b0 += kSet) blocks(std::integral_constant<int, kSet>(), b0);
-          if constexpr (NB % kSet) blocks(std::integral_constant<int, NB % kSet>(), NB - NB % kSet);
-          st.next();
-          // over all columns; a lane pair ends with one key
-          float s0, s1, u, v;
-          unpack2(add2(sum[0], sum[1]), u, v);
-          s0 = u + v;
-          unpack2(add2(sum[2], sum[3]), u, v);
-          s1 = u + v;
-          const bool h = lane & 1;
-          float r = (h ? s1 : s0) + __shfl_xor_sync(0xFFFFFFFFu, h ? s0 : s1, 1);
-          r += __shfl_xor_sync(0xFFFFFFFFu, r, 2);
-          if (!(lane & 2)) *raw = r * a.post;
-        }
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(CEMPTY(slot));
-    }
-    if constexpr (kRows) {
-      // rows whose sums are not finite, one a warp: 30 times the time of a sweep where every row of every head is such a row
-      asm volatile("bar.sync 3, 576;" ::: "memory");
-#pragma unroll 1
-      for (int p = redo_s ? 0 : 2; p < 2; ++p) {
-        for (Segs sr(a, 2 * blockIdx.x + p, 2 * grid); sr.next();) {
-          const int head = sr.vh >> (a.planes - 1), layer = head / a.hpl, hh = head - layer * a.hpl, row0 = row0_of(sr.vh), vec = a.D / 8;
-          float2* to = sums_of(sr.vh, p);
-          const uint4* k = maps.k_at[layer] + (size_t)hh * a.S * vec;
-          for (int row = warp; row < min(a.M - row0, a.plane_rows); row += kSoftWarps) {
-            if (to[row].y < INFINITY) continue;
-            const uint4* q = maps.q_at[layer] + ((size_t)hh * a.M + row0 + row) * vec;
-            const int end = min(a.P + (row0 + row) % a.ws + 1, (sr.t0 + sr.n) * kTile);
-            float m = -INFINITY, l = 0.f;
-            for (int j = sr.t0 * kTile + lane; j < end; j += 32) {
-              float s = 0.f;
-              for (int i = 0; i < vec; ++i) s = dot8(q[i], k[(size_t)j * vec + i], s);
-              s *= a.scale2;
-              const float top = fmaxf(m, s);
-              l = (l == 0.f ? 0.f : l * fast_exp2(m - top)) + (s == -INFINITY ? 0.f : fast_exp2(s - top));
-              m = top;
+              for (int h = 0; h < 2; ++h) {
+                float x[4 * kHalf];
+                read(x, h);
+                mask(x, t, h);
+#pragma unroll
+                for (int b = 0; b < 2 * kHalf; ++b) m[b] = fmax3(m[b], x[2 * b - b % 2], x[2 * b - b % 2 + 2]);
+              }
+              st.next();
             }
-            float top = m;
 #pragma unroll
-            for (int o = 16; o; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
-            l = l == 0.f ? 0.f : l * fast_exp2(m - top);
+            for (int b = 0; b < 2 * kHalf; ++b) {
 #pragma unroll
-            for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
-            if (lane == 0) to[row] = make_float2(top, l);
+              for (int o = 4; o <= 16; o <<= 1) m[b] = fmaxf(m[b], __shfl_xor_sync(0xFFFFFFFFu, m[b], o));
+              m[b] = m[b] == -INFINITY ? 0.f : m[b] * -a.scale2;              // (no key of this warp counts for the row)
+            }
+#pragma unroll
+            for (int b = 0; b < kHalf; ++b) c[b] = pack2(m[2 * b], m[2 * b + 1]);
+          }
+          for (int t = 0; t < sg.n; ++t) {
+            wait(TFULL(st.s), st.ph, 106);
+            tc_fence_after();
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {
+              float x[4 * kHalf];
+              read(x, h);
+              if (t + h + round == 0) {
+#pragma unroll
+                for (int b = 0; b < kHalf; ++b) {
+                  const float r0 = __shfl_sync(0xFFFFFFFFu, x[4 * b], lane & 3), r1 = __shfl_sync(0xFFFFFFFFu, x[4 * b + 1], lane & 3);
+                  c[b] = pack2(r0 * -a.scale2, r1 * -a.scale2);
+                }
+              }
+              mask(x, t, h);
+#pragma unroll
+              for (int b = 0; b < kHalf; ++b)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) sum[b] = exp2_acc2(false, sum[b], x[4 * b + 2 * j], x[4 * b + 2 * j + 1], scale22, c[b]);
+            }
+            st.next();
+          }
+          // Over the 8 lanes that have a column's keys: halves are exchanged, so that a lane ends with one pair of columns of four blocks.
+          auto swap = [&](int o, uint64_t lo_v, uint64_t hi_v) { return add2(lane & o ? hi_v : lo_v, __shfl_xor_sync(0xFFFFFFFFu, lane & o ? lo_v : hi_v, o)); };
+          wait(SUMFREE, (i & 1) ^ 1, 106);
+          float* my_sum = sum_s + (pipe * 4 + quad) * kCols + col2;
+          if (lane < 4)
+#pragma unroll
+            for (int b = 0; b < kHalf; ++b) *reinterpret_cast<uint64_t*>(&ref_s[(pipe * 4 + quad) * kCols + col2 + 8 * b]) = c[b] ^ 0x8000000080000000ull;
+#pragma unroll
+          for (int b = 0; b + 4 <= kHalf; b += 4) {
+            uint64_t u = swap(8, swap(16, sum[b], sum[b + 2]), swap(16, sum[b + 1], sum[b + 3]));
+            u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, 4));
+            if (!(lane & 4)) *reinterpret_cast<uint64_t*>(&my_sum[8 * (b + (lane >> 3))]) = u;
+          }
+          if constexpr (kHalf & 2) {
+            constexpr int b = kHalf & ~3;
+            uint64_t u = swap(16, sum[b], sum[b + 1]);
+            u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, 8));
+            u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, 4));
+            if (!(lane & 12)) *reinterpret_cast<uint64_t*>(&my_sum[8 * (b + (lane >> 4))]) = u;
+          }
+          if constexpr (kHalf & 1) {
+            uint64_t u = sum[kHalf - 1];
+#pragma unroll
+            for (int o = 16; o >= 4; o >>= 1) u = add2(u, __shfl_xor_sync(0xFFFFFFFFu, u, o));
+            if (lane < 4) *reinterpret_cast<uint64_t*>(&my_sum[8 * (kHalf - 1)]) = u;
+          }
+        } else {
+          const float* my_c = c_s + (2 * pipe + slot) * kCols + col2;
+          float* raw = a.raw + ((size_t)sg.vh * a.tph + sg.t0) * kTile + key + (lane & 1) * 8;
+          for (int t = 0; t < sg.n; ++t, raw += kTile) {
+            wait(TFULL(st.s), st.ph, 106);
+            tc_fence_after();
+            uint64_t sum[4] = {0ull, 0ull, 0ull, 0ull};   // over the columns so far, by key and parity of the block
+            const uint32_t at = addr + (uint32_t)(st.s * kStage);
+            auto blocks = [&](auto count, int b0) {
+              constexpr int kN = decltype(count)::value;
+              float x[4 * kN];
+              ld_block<kN>(at + (uint32_t)(8 * b0), x);
+              uint64_t c[kN];
+#pragma unroll
+              for (int b = 0; b < kN; ++b) c[b] = *reinterpret_cast<const uint64_t*>(&my_c[8 * (b0 + b)]);
+              tc_wait_ld();
+              if (b0 + kN == NB) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(TEMPTY(st.s));
+              }
+#pragma unroll
+              for (int b = 0; b < kN; ++b)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) sum[2 * j + (b & 1)] = exp2_acc2(false, sum[2 * j + (b & 1)], x[4 * b + 2 * j], x[4 * b + 2 * j + 1], scale22, c[b]);
+            };
+#pragma unroll 1
+            for (int b0 = 0; b0 + kSet <= NB; b0 += kSet) blocks(std::integral_constant<int, kSet>(), b0);
+            if constexpr (NB % kSet) blocks(std::integral_constant<int, NB % kSet>(), NB - NB % kSet);
+            st.next();
+            // over all columns; a lane pair ends with one key
+            float s0, s1, u, v;
+            unpack2(add2(sum[0], sum[1]), u, v);
+            s0 = u + v;
+            unpack2(add2(sum[2], sum[3]), u, v);
+            s1 = u + v;
+            const bool h = lane & 1;
+            float r = (h ? s1 : s0) + __shfl_xor_sync(0xFFFFFFFFu, h ? s0 : s1, 1);
+            r += __shfl_xor_sync(0xFFFFFFFFu, r, 2);
+            if (!(lane & 2)) *raw = r * a.post;
           }
         }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(CEMPTY(slot));
       }
-    }
+    });
   } else if (warp < kMmaWarp) {
     // ------------------------------------------------------------------ copies
-    if (lane == 0) {
-      const int halves = a.D / 64;
-      const uint64_t first = l2_policy_evict_first();
-      const bool once = a.planes == 1;                                      // the sweep reads the keys once
-      const uint32_t slot0 = smem_u32(ring + pipe * kSlots * kSlotBytes);
-      Ring kr(2, 1);
-      unsigned int used = 0, parity = 0;                                    // slots with a copy of this block's, its phase
-      int n = 0, qph = 1;
-      bool ok = true;
-      auto arm = [&](int s, int ph, int bytes) {
-        mbar_expect_tx(FULL(s), (uint32_t)bytes);
-        used |= 1u << s;
-        parity = (parity & ~(1u << s)) | (unsigned int)(ph ^ 1) << s;
-      };
-      for (Segs sg(a, 2 * blockIdx.x + pipe, 2 * grid); ok && sg.next();) {
+    const int halves = a.D / 64;
+    const uint64_t first = l2_policy_evict_first();
+    const bool once = a.planes == 1;                                      // the sweep reads the keys once
+    const uint32_t slot0 = smem_u32(ring + pipe * kSlots * kSlotBytes);
+    Ring kr(2, 1);
+    unsigned int used = 0, parity = 0;                                    // slots with a copy of this block's, its phase
+    int n = 0, qph = 1;
+    bool ok = true;
+    auto arm = [&](int s, int ph, int bytes) {
+      mbar_expect_tx(FULL(s), (uint32_t)bytes);
+      used |= 1u << s;
+      parity = (parity & ~(1u << s)) | (unsigned int)(ph ^ 1) << s;
+    };
+    rounds([&](Segs& sg, auto round_) {
+      constexpr int round = decltype(round_)::value;
+      if (lane) return;
+      while (ok && sg.next()) {
         const int head = sg.vh >> (a.planes - 1), layer = head / a.hpl, hh = head - layer * a.hpl;
         const CUtensorMap* k_map = &maps.k[layer];
         ok = wait(EMPTY(0), qph, 101);
@@ -456,7 +461,8 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
         arm(0, qph, halves * C::kQBytes);
         for (int h = 0; h < halves; ++h) tma_load_3d(slot0 + h * kHalfBytes, &maps.q[layer], FULL(0), 64 * h, row0_of(sg.vh), hh);
         qph ^= 1;
-        for (int t = 0, row = sg.t0 * kTile; t < sg.n; ++t, ++n, row += kTile) {
+        for (int u = round ? -sg.n : 0; u < sg.n; ++u, ++n) {
+          const int row = (sg.t0 + (u < 0 ? u + sg.n : u)) * kTile;
           const int s = 1 + kr.s;
           ok = wait(EMPTY(s), kr.ph, 102);
           if (!ok) break;
@@ -474,19 +480,21 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
       // Copies land before this block's shared memory is given up, and MMAs (below) end before its tensor memory is, whenever another
       // warp's wait has run out.
       for (int s = 0; s < kSlots; ++s) if (used >> s & 1u) mbar_drain(FULL(s), parity >> s & 1u);
-    }
+    });
   } else if (warp < kRowWarp) {
     // ------------------------------------------------------------------ MMAs
-    if (lane == 0) {
-      const uint64_t desc = smem_desc(smem_u32(ring + pipe * kSlots * kSlotBytes));
-      const uint32_t hi = (uint32_t)(desc >> 32), q_lo = (uint32_t)desc;
-      Ring kr(2, 0), st(kPer, 1);
-      int qph = 0;
-      bool ok = true;
-      for (Segs sg(a, 2 * blockIdx.x + pipe, 2 * grid); ok && sg.next();) {
+    const uint64_t desc = smem_desc(smem_u32(ring + pipe * kSlots * kSlotBytes));
+    const uint32_t hi = (uint32_t)(desc >> 32), q_lo = (uint32_t)desc;
+    Ring kr(2, 0), st(kPer, 1);
+    int qph = 0;
+    bool ok = true;
+    rounds([&](Segs& sg, auto round_) {
+      constexpr int round = decltype(round_)::value;
+      if (lane) return;
+      while (ok && sg.next()) {
         ok = wait(FULL(0), qph, 103);
         qph ^= 1;
-        for (int t = 0; ok && t < sg.n; ++t) {
+        for (int u = round ? -sg.n : 0; ok && u < sg.n; ++u) {
           const int s = 1 + kr.s;
           ok = wait(FULL(s), kr.ph, 104) && wait(TEMPTY(st.s), st.ph, 105);
           if (!ok) break;
@@ -506,48 +514,60 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
         if (ok) tc_commit(EMPTY(0));
       }
       tc_commit(DRAIN);
-      mbar_drain(DRAIN, 0);
-    }
+      mbar_drain(DRAIN, round);
+    });
   } else if (warp < kPublishWarp) {
     // ------------------------------------------------------------------ log-denominators of the segments but the first
-    Segs sg(a, 2 * blockIdx.x + pipe, 2 * grid);
-    for (int i = 0; !kRows && sg.next(); ++i) {
-      const int slot = i & 1;
-      wait(CEMPTY(slot), (i >> 1 & 1) ^ 1, 107);                            // the segment before last is done with its own
-      if (i > 0)
+    int i = 0;
+    rounds([&](Segs& sg, auto) {
+      for (; !kRows && sg.next(); ++i) {
+        const int slot = i & 1;
+        wait(CEMPTY(slot), (i >> 1 & 1) ^ 1, 107);                            // the segment before last is done with its own
+        if (i > 0)
 #pragma unroll 1
-        for (int r = 0; r < kCols; r += 16) fill(c_s + (2 * pipe + slot) * kCols, sg.vh, r);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(CFULL(slot));
-    }
+          for (int r = 0; r < kCols; r += 16) fill(c_s + (2 * pipe + slot) * kCols, sg.vh, r);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(CFULL(slot));
+      }
+    });
   } else {
     // ------------------------------------------------------------------ a segment's row sums -> the rows' counters
     if constexpr (kRows) {
+      int i = 0;
       Segs sg(a, 2 * blockIdx.x + pipe, 2 * grid);
-      for (int i = 0; sg.next(); ++i) {
-        const int rows = min(a.M - row0_of(sg.vh), a.plane_rows);
-        float2* to = sums_of(sg.vh, pipe);
-        wait(CEMPTY(i & 1), i >> 1 & 1, 107);
+      int round = 0;
+      do {
+        for (; sg.next(); ++i) {
+          const int rows = min(a.M - row0_of(sg.vh), a.plane_rows);
+          float2* to = sums_of(sg.vh, pipe);
+          bool finite = true;
+          wait(CEMPTY(i & 1), i >> 1 & 1, 107);
 #pragma unroll 1
-        for (int row = lane; row < rows; row += 32) {
-          float m[4], l[4], top = -INFINITY, sum = 0.f;
+          for (int row = lane; row < rows; row += 32) {
+            float m[4], l[4], top = -INFINITY, sum = 0.f;
 #pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            m[w] = ref_s[(pipe * 4 + w) * kCols + row];
-            l[w] = sum_s[(pipe * 4 + w) * kCols + row];
-            lower_sum(m[w], l[w]);
-            if (l[w] != 0.f) top = fmaxf(top, m[w]);    // (0: no key of this quad counts for the row)
+            for (int w = 0; w < 4; ++w) {
+              m[w] = ref_s[(pipe * 4 + w) * kCols + row];
+              l[w] = sum_s[(pipe * 4 + w) * kCols + row];
+              lower_sum(m[w], l[w]);
+              if (l[w] != 0.f) top = fmaxf(top, m[w]);    // (0: no key of this quad counts for the row)
+            }
+#pragma unroll
+            for (int w = 0; w < 4; ++w) sum += l[w] == 0.f ? 0.f : l[w] * fast_exp2(m[w] - top);
+            finite = finite && sum < INFINITY;
+            to[row] = make_float2(top, sum);
           }
-#pragma unroll
-          for (int w = 0; w < 4; ++w) sum += l[w] == 0.f ? 0.f : l[w] * fast_exp2(m[w] - top);
-          if (!(sum < INFINITY)) { sum = NAN; redo_s = 1; }
-          to[row] = make_float2(top, sum);
+          finite = __all_sync(0xFFFFFFFFu, finite);
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(SUMFREE);
+            if (!round && !finite) {
+              if (!again_s[pipe][1]) again_s[pipe][0] = sg.g - sg.n;
+              again_s[pipe][1] = sg.g;
+            }
+          }
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(SUMFREE);
-      }
-      __threadfence_block();
-      asm volatile("bar.arrive 3, 576;" ::: "memory");
+      } while (!round++ && second_round(sg));
     }
   }
   tc_fence_before();

@@ -74,6 +74,56 @@ def test_logits_that_are_far_above_the_first_key_of_a_segment():
     _passes(2, 2, 2, 64, 1, 2000, 8, 5, far, most=2e-4)      # |t| < 512: 2^-16 ln 2 and more
 
 
+# Such logits in some heads only, first and last ones of a pipe's range among them: two planes, four accumulator stages and two, heads
+# in many pipes, many heads in one, several hundred (head, plane) pairs.
+@pytest.mark.parametrize("L,Hkv,G,D,Bt,S,ws", [(2, 2, 7, 128, 1, 2000, 32), (3, 2, 4, 64, 1, 20011, 32), (33, 6, 2, 64, 3, 257, 8),
+                                               (33, 3, 5, 64, 2, 200, 26), (1, 1, 1, 64, 1, 128, 3), (4, 8, 3, 128, 1, 6200, 27)])
+@pytest.mark.parametrize("every", [1, 5])
+def test_heads_with_logits_beyond_their_references(L, Hkv, G, D, Bt, S, ws, every):
+    def far(q, k):
+        n = 0
+        for x, y in zip(q, k):
+            x[..., 0] = 16.0
+            for b in range(Bt):
+                for h in range(Hkv):
+                    y[b, h, :, 0] = 0.0
+                    if n % every == 0:
+                        y[b, h, S // 3::37, 0] = 100.0
+                        y[b, h, S // 2::53, 0] = -100.0
+                    n += 1
+    _passes(L, Hkv, G, D, Bt, S, ws, 5, far, most=2e-4)
+
+
+@pytest.mark.parametrize("bad", [1, 64])
+def test_a_head_with_such_logits_costs_a_few_sweeps_of_its_own(bad):
+    L, Hkv, S, ws, D = 8, 8, 32768, 32, 128
+    g = torch.Generator(device="cuda").manual_seed(1)
+    new = lambda *s: [torch.randn(s, generator=g, device="cuda").to(torch.bfloat16) for _ in range(L)]
+    q, k = new(1, 3 * Hkv, ws, D), new(1, Hkv, S, D)
+    kb, vb = ([torch.zeros((1, Hkv, 8 + ws, D), device="cuda", dtype=torch.bfloat16) for _ in range(L)] for _ in range(2))
+    h = B.dkv_create(B.make_config(L, 3 * Hkv, Hkv, D, 1, S, ws, 5, 4, 8, 2))
+
+    def time():
+        best = 1e9
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            B.dkv_run_prefill_pass(h, q, k, k, kb, vb)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+    try:
+        time()
+        clean = time()
+        for i in range(bad):
+            k[i // Hkv][0, i % Hkv, 100, 0] = torch.nan
+        assert time() <= 4 * clean                           # two more sweeps for the row sums, which are less than half of a pass
+        assert B.dkv_last_status(h)[0] == B.DKV_OK
+    finally:
+        B.dkv_destroy(h)
+
+
 # One key of every 128 a little less than 88.7 nats (128 bits) above the others: the sums of the segments are finite, and would
 # not be together.  |t| < 256: 2^-17 ln 2 a factor.
 @pytest.mark.parametrize("nats", [82.0, 83.5, 84.0, 87.0, 88.5, 89.0, 95.0])
