@@ -278,7 +278,8 @@ int dkv_last_status(dkv_ctx* ctx, int32_t* host_status);
  * above ([1] is 0).  Synchronises the current device; DKV_OK or DKV_ERR_TIMEOUT.  The next dkv_score_static
  * call clears the words. */
 int dkv_static_last_status(int32_t* host_status);
-/* Limit of every wait inside the scoring kernel, in SM clock ticks (default 4e9, about 2 s; at least 1000).
+/* Limit of every wait inside the scoring kernels, in SM clock ticks (default 4e9, about 2 s; at least 1000); where one part of a
+ * thread block waits for another to finish with several key tiles, the limit for each of them.
  * A wait that runs out makes its thread block stop issuing work, finish, and record the failure for
  * dkv_last_status.  Applies to launches made after the call. */
 int dkv_set_wait_limit(dkv_ctx* ctx, int64_t clock_ticks);

@@ -380,6 +380,7 @@ int launch_sweeps(dkv_ctx* c, int layer, int nl, const void* const* q, const voi
   a.hist_n = nl * s.Bt * kBins;
   a.status = c->d_status;
   a.wait_cycles = c->wait_cycles;
+  a.segment_cycles = c->wait_cycles > INT64_MAX / (2 * tph) ? INT64_MAX : c->wait_cycles * (2 * tph);      // a segment swept twice
   const long long tiles = (long long)a.vheads * tph;
   const dim3 grid((unsigned int)((tiles + 1) / 2 < c->n_sms ? (tiles + 1) / 2 : c->n_sms));
   auto launch = [&](auto score_kernel, int smem) { return launch_pdl(score_kernel, grid, sweep::kOneThreads, (size_t)smem, 1, st, maps, a); };

@@ -75,7 +75,7 @@ struct Args {
   unsigned int* hist;           // null, or counters to clear
   int hist_n;
   int* status;
-  long long wait_cycles;
+  long long wait_cycles, segment_cycles;      // limits of a wait, for a tile and for a segment
   int withhold_tile;            // test hook: block 0 never loads its tile of this number (-1: off)
 };
 
@@ -218,6 +218,8 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
   // What whole warps wait for they go on without once a wait has run out, as no wait blocks any more then: whether it had come is for
   // each lane to see, and lanes that left a loop alone would be missing from its next shuffle.  Single lanes stop.
   auto wait = [&](uint32_t bar, uint32_t parity, int code) { return mbar_wait(bar, parity, abort_flag, a.status, code, a.wait_cycles); };
+  // for a segment of the warps with the exponentials
+  auto wait_segment = [&](uint32_t bar, uint32_t parity) { mbar_wait(bar, parity, abort_flag, a.status, 107, a.segment_cycles); };
   const long long tiles = (long long)a.vheads * a.tph;
   // Row sums: all warps of the block meet after the pipes' segments, and those of a pipe with a sum that is not finite go round a second
   // time, over its segments from the first to the last such one.
@@ -522,7 +524,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     rounds([&](Segs& sg, auto) {
       for (; !kRows && sg.next(); ++i) {
         const int slot = i & 1;
-        wait(CEMPTY(slot), (i >> 1 & 1) ^ 1, 107);                            // the segment before last is done with its own
+        wait_segment(CEMPTY(slot), (i >> 1 & 1) ^ 1);                            // the segment before last is done with its own
         if (i > 0)
 #pragma unroll 1
           for (int r = 0; r < kCols; r += 16) fill(c_s + (2 * pipe + slot) * kCols, sg.vh, r);
@@ -541,7 +543,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           const int rows = min(a.M - row0_of(sg.vh), a.plane_rows);
           float2* to = sums_of(sg.vh, pipe);
           bool finite = true;
-          wait(CEMPTY(i & 1), i >> 1 & 1, 107);
+          wait_segment(CEMPTY(i & 1), i >> 1 & 1);
 #pragma unroll 1
           for (int row = lane; row < rows; row += 32) {
             float m[4], l[4], top = -INFINITY, sum = 0.f;

@@ -99,6 +99,27 @@ def test_a_wait_that_runs_out_in_a_pass_is_reported_and_the_context_stays_usable
         B.dkv_destroy(ctx)
 
 
+@pytest.mark.parametrize("use", ["pass", "lse"])
+def test_the_limit_is_for_a_tile_and_not_for_a_head(use):
+    """Two heads of 65536 keys to a pipe, some 700 us, of 2 us a tile: a limit of 80 us is far from any wait for a tile."""
+    L, Hkv, D, S, ws = 8, 74, 64, 65536, 16
+    q, k = ([torch.randn((1, Hkv, n, D), device="cuda").to(torch.bfloat16) for _ in range(1)] * L for n in (ws, S))
+    kb, vb = ([torch.zeros((1, Hkv, 8 + ws, D), device="cuda", dtype=torch.bfloat16) for _ in range(L)] for _ in range(2))
+    lse = [torch.zeros((1, Hkv, ws), device="cuda")] * L
+    ctx = B.dkv_create(B.make_config(L, Hkv, Hkv, D, 1, S, ws, 5, 4, 8, 2))
+    try:
+        B.dkv_set_wait_limit(ctx, 150_000)
+        for _ in range(2):
+            if use == "lse":
+                B.dkv_run_prefill_pass_lse(ctx, q, k, k, lse, kb, vb)
+            else:
+                B.dkv_run_prefill_pass(ctx, q, k, k, kb, vb)
+            code, status = B.dkv_last_status(ctx)
+            assert code == B.DKV_OK, status
+    finally:
+        B.dkv_destroy(ctx)
+
+
 def test_wait_limit_and_hook_arguments_are_checked():
     ctx = B.dkv_create(B.config_of(synth.WORKLOADS["tiny"]))
     try:
