@@ -200,7 +200,8 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   // Key sums follow row sums over the same queries and keys, and row sums let them start only after their own wait for the inputs:
-  // copies and MMAs begin at once, and the other warps wait for the end of the row sums.
+  // copies and MMAs begin at once, and the other warps wait for the end of the row sums.  So do copies and MMAs before the first of
+  // their own waits that needs those warps: the limit is not for the time that another launch takes.
   if (kSweep == kKeySums) {
     pdl_launch();
     if (warp < kCopyWarp || warp >= kRowWarp) pdl_wait();
@@ -463,7 +464,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
         arm(0, qph, halves * C::kQBytes);
         for (int h = 0; h < halves; ++h) tma_load_3d(slot0 + h * kHalfBytes, &maps.q[layer], FULL(0), 64 * h, row0_of(sg.vh), hh);
         qph ^= 1;
-        for (int u = round ? -sg.n : 0; u < sg.n; ++u, ++n) {
+        for (int u = round ? -sg.n : 0; u < sg.n; ++u) {
           const int row = (sg.t0 + (u < 0 ? u + sg.n : u)) * kTile;
           const int s = 1 + kr.s;
           ok = wait(EMPTY(s), kr.ph, 102);
@@ -477,6 +478,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
             else for (int h = 0; h < halves; ++h) tma_load_3d(dst + h * kHalfBytes, k_map, FULL(s), 64 * h, row, hh);
           }
           kr.next();
+          if (++n == kPer + 1 && kSweep == kKeySums) pdl_wait();            // (the queries' slot may be waited for next)
         }
       }
       // Copies land before this block's shared memory is given up, and MMAs (below) end before its tensor memory is, whenever another
@@ -512,6 +514,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           tc_commit(TFULL(st.s));
           kr.next();
           st.next();
+          if (kSweep == kKeySums && st.s == 0) pdl_wait();                  // all stages have been used
         }
         if (ok) tc_commit(EMPTY(0));
       }

@@ -120,6 +120,33 @@ def test_the_limit_is_for_a_tile_and_not_for_a_head(use):
         B.dkv_destroy(ctx)
 
 
+def test_the_limit_does_not_count_the_wait_for_the_launch_before():
+    """The key sums of a pass start on the SMs whose row sums have ended.  One head whose logits are far above its first key keeps
+    two blocks for some 250 us longer (its row sums are computed again): the others wait, and their limit of 80 us or so stands for
+    what they wait for themselves."""
+    L, Hkv, D, S, ws = 32, 8, 64, 32768, 16
+    g = torch.Generator(device="cuda").manual_seed(3)
+    new = lambda *s: [torch.randn(s, generator=g, device="cuda").to(torch.bfloat16) for _ in range(L)]
+    q, k = new(1, Hkv, ws, D), new(1, Hkv, S, D)
+    q[5][:, 3, :, 0], k[5][:, 3, :, 0], k[5][:, 3, 70::999, 0] = 16.0, 0.0, 100.0
+    kb, vb = ([torch.zeros((1, Hkv, 8 + ws, D), device="cuda", dtype=torch.bfloat16) for _ in range(L)] for _ in range(2))
+    ctx = B.dkv_create(B.make_config(L, Hkv, Hkv, D, 1, S, ws, 5, 4, 8, 2))
+    scores = []
+    try:
+        for limit in (4_000_000_000, 150_000, 150_000):
+            B.dkv_set_wait_limit(ctx, limit)
+            B.dkv_run_prefill_pass(ctx, q, k, k, kb, vb)
+            code, status = B.dkv_last_status(ctx)
+            assert code == B.DKV_OK, f"limit {limit}: {status}"
+            got = torch.zeros((L, Hkv, S - ws))
+            for l in range(L):
+                B.dkv_memcpy_to_host(ctx, got[l], B.dkv_layer_views(ctx, l)[0], got[l].numel() * 4)
+            scores.append(got)
+        assert all(torch.equal(x, scores[0]) for x in scores)
+    finally:
+        B.dkv_destroy(ctx)
+
+
 def test_wait_limit_and_hook_arguments_are_checked():
     ctx = B.dkv_create(B.config_of(synth.WORKLOADS["tiny"]))
     try:
