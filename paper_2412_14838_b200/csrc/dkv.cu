@@ -333,12 +333,12 @@ cudaError_t with_sweep_kernel(int nb, F f) {
   }
 }
 // The builds' shared memory, per function and device: set before their first launch, and only for the builds that a caller can
-// reach, since each is loaded onto the device by it.
-cudaError_t set_sweep_attributes(int nb) {
+// reach, since each is loaded onto the device by it.  all: passes without the caller's normalisers too (pass_by_sweeps).
+cudaError_t set_sweep_attributes(int nb, bool all) {
   auto set = [](auto kernel, int smem) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
   cudaError_t e = set(pool_kernel, 0);
-  if (e == cudaSuccess) e = with_sweep_kernel<sweep::kRowSums>(nb, set);
-  if (e == cudaSuccess) e = with_sweep_kernel<sweep::kKeySums>(nb, set);
+  if (e == cudaSuccess && all) e = with_sweep_kernel<sweep::kRowSums>(nb, set);
+  if (e == cudaSuccess && all) e = with_sweep_kernel<sweep::kKeySums>(nb, set);
   return e != cudaSuccess ? e : with_sweep_kernel<sweep::kGivenSums>(nb, set);
 }
 
@@ -779,7 +779,7 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
     TRY(cudaMalloc(&c->d_cand, std::max(sizeof(uint2) * s.L * layer_scores(s), sizeof(float) * most * heads * c->planes * tiles_per_head(s) * tc::kTileKeys)));
     // a launch over fewer layers than `most` (the last of a pass) has more segments a head, but no more in all
     TRY(cudaMalloc(&c->d_stats, sizeof(float2) * c->plane_rows * (2 * c->n_sms + 2 * most * heads * c->planes)));
-    TRY(set_sweep_attributes(row_blocks(c)));
+    TRY(set_sweep_attributes(row_blocks(c), pass_by_sweeps(c)));
   }
   TRY(cudaMalloc(&c->d_cand_n, sizeof(unsigned int) * s.Bt));
   TRY(cudaMalloc(&c->d_tc_stats, sizeof(float2) * 3 * c->stats_rows * 256));

@@ -13,7 +13,7 @@ CHILD = """
 import sys, torch
 from paper_2412_14838_b200 import binding as B
 B.load()
-static, *shapes = eval(sys.argv[1])
+use, *shapes = eval(sys.argv[1])
 for Hq, Hkv, D, ws in shapes:                               # ws * Hq / Hkv window rows
     L, S = 3, 900
     g = torch.Generator(device="cuda").manual_seed(ws)
@@ -26,9 +26,17 @@ for Hq, Hkv, D, ws in shapes:                               # ws * Hq / Hkv wind
     logits.masked_fill_(torch.arange(S, device="cuda") > (S - ws + torch.arange(ws, device="cuda"))[:, None], float("-inf"))
     want = logits.softmax(-1)[..., :S - ws].sum(2).view(1, Hkv, -1, S - ws).sum(2)
     close = lambda x: ((x - want).abs().max() <= 1e-4 * want.max()).item()
-    if static:
+    if use == "static":
         B.dkv_score_static(cfg, q[0], k[0], one)
         assert close(one), "static"
+    elif use == "lse":
+        ctx = B.dkv_create(cfg)
+        lse = [logits.logsumexp(-1).float().contiguous()] * L
+        B.dkv_run_prefill_pass_lse(ctx, q, k, v, lse, kb, vb)
+        B.dkv_memcpy_to_host(ctx, host := torch.zeros(one.shape), B.dkv_layer_views(ctx, 0)[0], host.numel() * 4)
+        assert close(host.cuda()), "pass with log-denominators"
+        assert B.dkv_last_status(ctx)[0] == B.DKV_OK
+        B.dkv_destroy(ctx)
     else:
         ctx = B.dkv_create(cfg)
         B.dkv_score(ctx, 0, q[0], k[0], one)
@@ -43,7 +51,7 @@ print("ok")
 SHAPES = [(4, 2, 64, 16), (8, 2, 128, 16), (6, 2, 128, 32), (8, 2, 128, 32), (8, 2, 64, 32), (14, 2, 128, 32)]   # 32 .. 224 window rows
 
 
-@pytest.mark.parametrize("case", [(False, s) for s in SHAPES] + [(True, *SHAPES)], ids=str)
+@pytest.mark.parametrize("case", [(u, s) for u in ("pass", "lse") for s in SHAPES] + [("static", *SHAPES)], ids=str)
 def test_first_call_of_a_process(case):
     res = subprocess.run([sys.executable, "-c", CHILD, repr(case)], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert res.returncode == 0 and res.stdout.strip() == "ok", res.stderr[-2000:]
