@@ -54,7 +54,7 @@ struct dkv_ctx {
   long long wait_cycles;   // limit of the scoring kernel's mbarrier waits (dkv_set_wait_limit)
   int withhold_sweep, withhold_tile;   // test hook of dkv_debug_withhold_tile (-1: off)
   // passes scored by score_sweep.cuh
-  float2* d_stats;      // row sums of a head's segments
+  float2* d_stats;      // row sums of a head's segments (null where only passes with given log-denominators are)
   int planes, plane_rows;  // window rows of a head: planes of at most 128
   float2* d_tc_stats;   // [3][stats_rows][256]: partial softmax statistics, three jobs in rotation, each [heads][slots][256]
   // host state
@@ -741,7 +741,6 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
     int sms = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     c->n_sms = sms > 0 ? sms : 1;
-    c->stats_rows = (size_t)c->n_sms + 2 * tc::kMaxGroup * heads;
     // Layers per scoring launch of the pass: enough that a thread block has about 110 tiles a sweep.  A launch costs some 8 us
     // (fill, drain, statistics) whatever it does: 32 layers of 8K in launches of 8 / 16 / 32 layers take 299 / 290 / 286 us;
     // at 32K eight layers are as good as more.
@@ -750,6 +749,8 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
     if (g > tc::kMaxGroup) g = tc::kMaxGroup;
     const int launches = (s.L + g - 1) / g;
     c->pass_group = env_int("DKV_PASS_GROUP", (s.L + launches - 1) / launches, 1, tc::kMaxGroup);
+    // (stats_slots of a job's heads; score_tc.cuh's jobs are single layers where passes are scored by score_sweep.cuh)
+    c->stats_rows = (size_t)c->n_sms + 2 * (size_t)(pass_by_sweeps(c) ? 1 : c->pass_group) * heads;
     c->emit_backward = env_int("DKV_EMIT_FORWARD", 0, 0, 1) == 0;
     // Sweep 2 starts on the keys sweep 1 streamed last: that much of a job (4/7 of L2, 72 of 126 MB) is loaded with
     // an evict-last policy, every other key tile and the gather's rows evict-first, so that the rest of the
@@ -777,8 +778,8 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   {
     const int most = most_layers(c);
     TRY(cudaMalloc(&c->d_cand, std::max(sizeof(uint2) * s.L * layer_scores(s), sizeof(float) * most * heads * c->planes * tiles_per_head(s) * tc::kTileKeys)));
-    // a launch over fewer layers than `most` (the last of a pass) has more segments a head, but no more in all
-    TRY(cudaMalloc(&c->d_stats, sizeof(float2) * c->plane_rows * (2 * c->n_sms + 2 * most * heads * c->planes)));
+    // Row sums; a launch over fewer layers than `most` (the last of a pass) has more segments a head, but no more in all.
+    if (pass_by_sweeps(c)) TRY(cudaMalloc(&c->d_stats, sizeof(float2) * c->plane_rows * (2 * c->n_sms + 2 * most * heads * c->planes)));
     TRY(set_sweep_attributes(row_blocks(c), pass_by_sweeps(c)));
   }
   TRY(cudaMalloc(&c->d_cand_n, sizeof(unsigned int) * s.Bt));

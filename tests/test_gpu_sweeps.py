@@ -169,3 +169,33 @@ def test_a_head_with_a_key_that_is_no_number_spoils_no_other():
                                     (5, 28, 128), (7, 32, 64), (7, 24, 128)])
 def test_window_rows_around_sixteens(G, ws, D):
     _passes(2, 2, G, D, 1, 900, ws, 5)
+
+
+def test_a_context_of_many_heads_takes_no_statistics_for_groups_of_layers():
+    L, Bt, Hkv, S, ws, D = 32, 32, 8, 264, 8, 64
+    P = S - ws
+    cfg = B.make_config(L, Hkv, Hkv, D, Bt, S, ws, 3, 4, 8, 2)
+    B.dkv_destroy(B.dkv_create(cfg))                         # loads the kernels
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    h = B.dkv_create(cfg)
+    try:
+        # scores and candidates (4 and 8 bytes a position), unpooled scores and histograms; the rest is below 16 MB
+        known = L * Bt * (Hkv * P * 4 + max(Hkv * P * 8, Hkv * 384 * 4) + 2048 * 4)
+        assert free - torch.cuda.mem_get_info()[0] <= known + (24 << 20)
+        g = torch.Generator(device="cuda").manual_seed(7)
+        for l in range(5):                                   # three sets of statistics in turn
+            q, k = (torch.randn((Bt, Hkv, n, D), generator=g, device="cuda").to(torch.bfloat16) for n in (ws, S))
+            got = torch.zeros((Bt, Hkv, P), device="cuda")
+            B.dkv_score(h, l, q, k, got)
+            want = _scores(q, k, ws, 3)[0]
+            assert ((got - want).abs() <= 5e-5 * want).all()
+    finally:
+        B.dkv_destroy(h)
+
+
+# As many segments in a pipe as a prompt of one tile a head can have: 40000 samples of 8 heads, far logits in all.
+def test_a_thousand_segments_of_one_tile():
+    def far(q, k):
+        q[0][..., 0], k[0][..., 0], k[0][:, :, 3, 0] = 16.0, 0.0, 100.0
+    _passes(1, 8, 1, 64, 40000, 16, 1, 1, far, most=2e-4)
