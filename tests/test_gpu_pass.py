@@ -233,17 +233,21 @@ def test_pass_with_ragged_shape_and_final_partial_block():
         g.close()
 
 
-@pytest.mark.parametrize("group,taper,streams", [(1, 0, 1), (3, 0, 2), (8, 0, 4), (4, 1, 3)])
-def test_pass_is_the_same_however_the_layers_are_grouped(group, taper, streams, monkeypatch):
-    # The pass scores several layers per launch; the group size, a ragged last group, update points that fall
-    # inside a group (m = 2 with groups of 3) and the number of select streams are scheduling only.
+@pytest.mark.parametrize("group", [1, 3, 8, 4])
+def test_pass_is_the_same_however_the_layers_are_grouped(group, monkeypatch):
+    # A short pass with 128 window rows of 128 dims scores several layers per launch, sweep 2 of one group with sweep 1 of the
+    # next; the group size, a ragged last group and update points that fall inside a group (m = 2 with groups of 3) are
+    # scheduling only.
     monkeypatch.setenv("DKV_PASS_GROUP", str(group))
-    monkeypatch.setenv("DKV_PASS_TAPER", str(taper))
-    monkeypatch.setenv("DKV_SIDE_STREAMS", str(streams))
-    w = synth.Workload("grouppass", 52, L=7, Hq=8, Hkv=2, D=128, Bt=2, S=2100, ws=8, pool=5, N=24, Bl=64, m=2,
+    w = synth.Workload("grouppass", 52, L=7, Hq=8, Hkv=2, D=128, Bt=2, S=2100, ws=32, pool=5, N=24, Bl=64, m=2,
                        recipe="sink")
-    g = GpuPass(w).run()            # the context reads the overrides when it is created
+    g = GpuPass(w).run()            # the context reads the override when it is created
     try:
+        groups = -(-w.L // group)
+        if groups > 1:                                       # launches of a pass: one a group and one more, three for the updates
+            before = B.dkv_launch_count(g.h)
+            B.dkv_run_prefill_pass(g.h, g.q, g.k, g.v, g.kb, g.vb)
+            assert B.dkv_launch_count(g.h) - before == groups + 1 + 3 + 1
         check_properties(g)
         compare_full(g)
         B.dkv_run_prefill_pass(g.h, g.q, g.k, g.v, g.kb, g.vb)      # a second pass gives the same again
