@@ -75,8 +75,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """Compile what is older than its sources, or linked with another torch; return the library's path."""
     kernels = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != os.path.basename(PYCALL_SOURCE)]
     if force or _stale(LIB, kernels + [HEADER]):
+        # uncompressed: unpacking the device code takes the first dkv_create of a process 7 ms and more (10 -> 17-30)
         _run([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-              "-shared", "-Xcompiler", "-fPIC", "-Xptxas", "-v" if verbose else "-O3",
+              "-shared", "-Xcompiler", "-fPIC", "--no-compress", "-Xptxas", "-v" if verbose else "-O3",
               "-o", LIB] + [os.path.join(CSRC, s) for s in SOURCES], verbose)
     if torch_version() and (force or _stale(PYCALL, [PYCALL_SOURCE, HEADER]) or pycall_built_for() != torch_version()):
         _build_pycall(verbose)

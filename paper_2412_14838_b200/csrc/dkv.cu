@@ -313,6 +313,7 @@ int launch_score(dkv_ctx* c, const ScoreGroup* e, ScoreGroup* s, const void* con
 
 // ---- scoring of a pass (score_sweep.cuh) ---------------------------------------------------------
 int tiles_per_head(const Shape& s) { return (s.S + tc::kTileKeys - 1) / tc::kTileKeys; }
+bool long_heads(const dkv_ctx* c) { return tiles_per_head(c->s) > sweep::kRowTiles; }
 int row_blocks(const dkv_ctx* c) { return (c->plane_rows + 15) / 16 * 2; }              // the kernel's NB
 int most_layers(const dkv_ctx* c) { return c->s.L < tc::kMaxGroup ? c->s.L : tc::kMaxGroup; }
 // Segments a (head, plane) can have in a launch over nl layers: its share of the pipes, one cut at either end.
@@ -334,10 +335,10 @@ cudaError_t with_sweep_kernel(int nb, F f) {
 }
 // The builds' shared memory, per function and device: set before their first launch, and only for the builds that a caller can
 // reach, since each is loaded onto the device by it.  all: passes without the caller's normalisers too (pass_by_sweeps).
-cudaError_t set_sweep_attributes(int nb, bool all) {
+cudaError_t set_sweep_attributes(int nb, bool all, bool long_rows) {
   auto set = [](auto kernel, int smem) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
   cudaError_t e = set(pool_kernel, 0);
-  if (e == cudaSuccess && all) e = with_sweep_kernel<sweep::kRowSums>(nb, set);
+  if (e == cudaSuccess && all) e = long_rows ? with_sweep_kernel<sweep::kLongRowSums>(nb, set) : with_sweep_kernel<sweep::kRowSums>(nb, set);
   if (e == cudaSuccess && all) e = with_sweep_kernel<sweep::kKeySums>(nb, set);
   return e != cudaSuccess ? e : with_sweep_kernel<sweep::kGivenSums>(nb, set);
 }
@@ -387,7 +388,7 @@ int launch_sweeps(dkv_ctx* c, int layer, int nl, const void* const* q, const voi
   if (!lse) {
     a.withhold_tile = c->withhold_sweep == tc::kStats ? c->withhold_tile : -1;
     ProfScope ps(c, DKV_STEP_SCORE_STATS, 1, st);
-    DKV_LAUNCH(c, (with_sweep_kernel<sweep::kRowSums>(nb, launch)));
+    DKV_LAUNCH(c, long_heads(c) ? (with_sweep_kernel<sweep::kLongRowSums>(nb, launch)) : (with_sweep_kernel<sweep::kRowSums>(nb, launch)));
   }
   a.withhold_tile = c->withhold_sweep == tc::kEmit ? c->withhold_tile : -1;
   {
@@ -780,7 +781,7 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
     TRY(cudaMalloc(&c->d_cand, std::max(sizeof(uint2) * s.L * layer_scores(s), sizeof(float) * most * heads * c->planes * tiles_per_head(s) * tc::kTileKeys)));
     // Row sums; a launch over fewer layers than `most` (the last of a pass) has more segments a head, but no more in all.
     if (pass_by_sweeps(c)) TRY(cudaMalloc(&c->d_stats, sizeof(float2) * c->plane_rows * (2 * c->n_sms + 2 * most * heads * c->planes)));
-    TRY(set_sweep_attributes(row_blocks(c), pass_by_sweeps(c)));
+    TRY(set_sweep_attributes(row_blocks(c), pass_by_sweeps(c), long_heads(c)));
   }
   TRY(cudaMalloc(&c->d_cand_n, sizeof(unsigned int) * s.Bt));
   TRY(cudaMalloc(&c->d_tc_stats, sizeof(float2) * 3 * c->stats_rows * 256));

@@ -31,6 +31,7 @@
 // 32 / 96 / 128 / 192 rows 118 / 149 / 155 / 220 -> 107 / 123 / 139 / 186; 28 of 2 x 2K, 4 heads of 128, 96 / 192 / 256 rows
 // 114 / 153 / 162 -> 102 / 138 / 151; 32 layers of 32K, 8 heads of 128, with log-denominators 572 -> 530-554.
 #pragma once
+#include <limits.h>
 #include <type_traits>
 #include "score_tc.cuh"
 
@@ -45,7 +46,14 @@ constexpr int kSoftWarps = 16, kCopyWarp = 16, kMmaWarp = 18, kRowWarp = 20, kPu
 constexpr int kWarps = 24, kOneThreads = kWarps * 32;
 // Registers a thread: 80 at launch; the four warpgroups with the exponentials take what the other two give (4 x 96 + 2 x 48 = 6 x 80).
 constexpr int kSoftRegs = 96, kOtherRegs = 48;
-enum Sweep { kRowSums, kKeySums, kGivenSums };       // kGivenSums: key sums with the caller's log-denominators
+// kGivenSums: key sums with the caller's log-denominators; kLongRowSums: row sums of heads with more than kRowTiles tiles
+enum Sweep { kRowSums, kKeySums, kGivenSums, kLongRowSums };
+
+// Tiles whose row sums a thread adds one after the other, four additions each; longer segments are cut there and their parts added by
+// the warps that publish them.  296 heads of 262144 keys, logits of standard deviation 3: error of the scores (2-norm) 6.9e-6 uncut,
+// 8.7e-7 cut (score_tc.cuh 1.2e-6); of 32768 keys 9.2e-7.  A build of its own, as the cut in that of shorter heads made a pass of
+// four layers of 1K 0.7 us longer (39.5 -> 40.2).
+constexpr int kRowTiles = 256;
 
 constexpr int kSlots = 3, kSlotBytes = 2 * kHalfBytes;      // of a pipe: queries, two tiles of keys
 
@@ -109,7 +117,8 @@ __device__ __forceinline__ void ld_block(uint32_t a, float* v) {
 }
 
 // ------------------------------------------------------------------------------------------ order of work
-// The segments of a range of the tiles: the range cut at the heads.
+// The segments of a range of the tiles: the range cut at the heads, and after kMost tiles of one.
+template <int kMost>
 struct Segs {
   int g, end, tph;                              // what is left of the range
   int vh, t0, n;                                // the segment: (head, plane), first tile, tiles
@@ -123,9 +132,13 @@ struct Segs {
       : Segs((int)((long long)a.vheads * a.tph * pipe / pipes), (int)((long long)a.vheads * a.tph * (pipe + 1) / pipes), a.tph) {}
   __device__ bool next() {
     if (g >= end) return false;
-    if (n) t0 = 0;
-    ++vh;
-    n = min(tph - t0, end - g);
+    if (kMost < INT_MAX && n && t0 + n < tph) {
+      t0 += n;
+    } else {
+      if (n) t0 = 0;
+      ++vh;
+    }
+    n = min(min(tph - t0, kMost), end - g);
     g += n;
     return true;
   }
@@ -153,7 +166,7 @@ template <int NB, int kSweep>
 __global__ void __launch_bounds__(kOneThreads, 1)
 score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ Args a) {
   using C = Shape1<NB>;
-  constexpr bool kRows = kSweep == kRowSums;
+  constexpr bool kLong = kSweep == kLongRowSums, kRows = kSweep == kRowSums || kLong;
   constexpr int kCols = C::kCols, kPer = C::kPer, kStage = C::kStage;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);     // [2 pipes][kSlots][half][128][128 B]
@@ -222,19 +235,20 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
   // for a segment of the warps with the exponentials
   auto wait_segment = [&](uint32_t bar, uint32_t parity) { mbar_wait(bar, parity, abort_flag, a.status, 107, a.segment_cycles); };
   const long long tiles = (long long)a.vheads * a.tph;
+  using Segments = Segs<kLong ? kRowTiles : INT_MAX>;
   // Row sums: all warps of the block meet after the pipes' segments, and those of a pipe with a sum that is not finite go round a second
   // time, over its segments from the first to the last such one.
-  auto second_round = [&](Segs& sg) {
+  auto second_round = [&](Segments& sg) {
     __syncwarp();
     asm volatile("bar.sync 3, %0;" ::"n"(kOneThreads) : "memory");
     if (!again_s[pipe][1]) return false;
-    sg = Segs(again_s[pipe][0], again_s[pipe][1], a.tph);
+    sg = Segments(again_s[pipe][0], again_s[pipe][1], a.tph);
     return true;
   };
   // f(segments, round) for each round, in two copies: what only the second round does, in the way of the first, made a pass of four
   // layers of 1K 0.4 to 1 us longer (of 38).
   auto rounds = [&](auto f) {
-    Segs sg(a, 2 * blockIdx.x + pipe, 2 * grid);
+    Segments sg(a, 2 * blockIdx.x + pipe, 2 * grid);
     f(sg, std::integral_constant<int, 0>());
     if constexpr (kRows) if (second_round(sg)) f(sg, std::integral_constant<int, 1>());
   };
@@ -284,7 +298,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     if (kSweep != kKeySums) for (int i = blockIdx.x * (kSoftWarps * 32) + threadIdx.x; i < a.hist_n; i += grid * (kSoftWarps * 32)) a.hist[i] = 0;
     Ring st(kPer, 0);
     int i = 0;                                          // segments so far
-    rounds([&](Segs& sg, auto round_) {
+    rounds([&](Segments& sg, auto round_) {
       constexpr int round = decltype(round_)::value;
       for (; sg.next(); ++i) {
         const int slot = i & 1;
@@ -453,7 +467,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
       used |= 1u << s;
       parity = (parity & ~(1u << s)) | (unsigned int)(ph ^ 1) << s;
     };
-    rounds([&](Segs& sg, auto round_) {
+    rounds([&](Segments& sg, auto round_) {
       constexpr int round = decltype(round_)::value;
       if (lane) return;
       while (ok && sg.next()) {
@@ -492,7 +506,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     Ring kr(2, 0), st(kPer, 1);
     int qph = 0;
     bool ok = true;
-    rounds([&](Segs& sg, auto round_) {
+    rounds([&](Segments& sg, auto round_) {
       constexpr int round = decltype(round_)::value;
       if (lane) return;
       while (ok && sg.next()) {
@@ -524,7 +538,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
   } else if (warp < kPublishWarp) {
     // ------------------------------------------------------------------ log-denominators of the segments but the first
     int i = 0;
-    rounds([&](Segs& sg, auto) {
+    rounds([&](Segments& sg, auto) {
       for (; !kRows && sg.next(); ++i) {
         const int slot = i & 1;
         wait_segment(CEMPTY(slot), (i >> 1 & 1) ^ 1);                            // the segment before last is done with its own
@@ -539,10 +553,13 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     // ------------------------------------------------------------------ a segment's row sums -> the rows' counters
     if constexpr (kRows) {
       int i = 0;
-      Segs sg(a, 2 * blockIdx.x + pipe, 2 * grid);
-      int round = 0;
+      Segments sg(a, 2 * blockIdx.x + pipe, 2 * grid);
+      int round = 0, part = 0;                            // first tile of what the pipe has of the head
       do {
-        for (; sg.next(); ++i) {
+        for (int vh = -1; sg.next(); ++i) {
+          const bool more = kLong && sg.vh == vh;
+          vh = sg.vh;
+          if (!more) part = sg.g - sg.n;
           const int rows = min(a.M - row0_of(sg.vh), a.plane_rows);
           float2* to = sums_of(sg.vh, pipe);
           bool finite = true;
@@ -559,6 +576,12 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
             }
 #pragma unroll
             for (int w = 0; w < 4; ++w) sum += l[w] == 0.f ? 0.f : l[w] * fast_exp2(m[w] - top);
+            if (more) {
+              const float2 before = to[row];
+              const float most = fmaxf(top, before.x);
+              sum = (sum == 0.f ? 0.f : sum * fast_exp2(top - most)) + before.y * fast_exp2(before.x - most);
+              top = most;
+            }
             finite = finite && sum < INFINITY;
             to[row] = make_float2(top, sum);
           }
@@ -567,7 +590,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           if (lane == 0) {
             mbar_arrive(SUMFREE);
             if (!round && !finite) {
-              if (!again_s[pipe][1]) again_s[pipe][0] = sg.g - sg.n;
+              if (!again_s[pipe][1]) again_s[pipe][0] = part;
               again_s[pipe][1] = sg.g;
             }
           }

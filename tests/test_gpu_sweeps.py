@@ -199,3 +199,34 @@ def test_a_thousand_segments_of_one_tile():
     def far(q, k):
         q[0][..., 0], k[0][..., 0], k[0][:, :, 3, 0] = 16.0, 0.0, 100.0
     _passes(1, 8, 1, 64, 40000, 16, 1, 1, far, most=2e-4)
+
+
+# Heads of 2048 tiles, each on one pipe or two.  What a pipe adds one key after the other is 256 tiles: 1024 additions of a thread,
+# each off by 2^-25 of the sum in the mean, is 1e-6 of it and less for the 64 such sums of a row; logits of |t| < 64 are off by 2^-19
+# and 2^-20 in the mean.  (Added to the end of the head, 8192 of them, the largest mean error of a head was 5.4e-6.)
+@pytest.mark.parametrize("far", [False, True])
+def test_the_error_of_a_row_sum_does_not_grow_with_the_prompt(far):
+    Bt, Hkv, S, ws, D = 37, 4, 262144, 8, 64
+    P = S - ws
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q = (3 * torch.randn((Bt, Hkv, ws, D), generator=g, device="cuda")).to(torch.bfloat16)
+    k = torch.empty((Bt, Hkv, S, D), device="cuda", dtype=torch.bfloat16)
+    for x in k:
+        x.normal_(generator=g)
+    if far:                                                  # in a later part of some heads, and only there
+        q[3:5, ..., 0], k[3:5, ..., 0], k[3:5, :, 150000, 0] = 16.0, 0.0, 60.0
+    kb = torch.zeros((Bt, Hkv, 8 + ws, D), device="cuda", dtype=torch.bfloat16)
+    h = B.dkv_create(B.make_config(1, Hkv, Hkv, D, Bt, S, ws, 1, 4, 8, 2))
+    try:
+        B.dkv_run_prefill_pass(h, [q], [k], [k], [kb], [kb.clone()])
+        got = torch.zeros((Bt, Hkv, P))
+        B.dkv_memcpy_to_host(h, got, B.dkv_layer_views(h, 0)[0], got.numel() * 4)
+        for b in range(Bt):
+            want = _scores(q[b:b + 1], k[b:b + 1], ws, 1)[0][0]
+            off = (got[b].cuda().double() - want) / want.clamp_min(1e-25)
+            if far and 3 <= b < 5:                           # |t| < 256
+                assert off.abs().max() <= 1e-4
+            else:
+                assert off.mean(-1).abs().max() <= 2.5e-6, f"sample {b}: {off.mean(-1).abs().max():.1e}"
+    finally:
+        B.dkv_destroy(h)
