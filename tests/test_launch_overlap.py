@@ -64,3 +64,40 @@ def test_a_warpgroup_changes_its_registers_by_one_instruction():
     assert soft % 4 == 0 and warps % 4 == 0
     at_launch = 65536 // (warps * 32) // 8 * 8
     assert soft * value["kSoftRegs"] + (warps - soft) * value["kOtherRegs"] <= warps * at_launch
+
+
+def test_kernels_that_early_readers_count_on_start_them_after_their_own_wait():
+    """What kernels before the predecessor wrote is complete before a kernel's own wait only if the predecessor has waited itself
+    before it lets its successor start."""
+    kernels = {n: body for f in HEADERS for n, _, body in _functions(_source(f))}
+
+    def order(body):
+        return re.findall(r"\b(pdl_wait|pdl_launch)\(\);", body)
+
+    for name in ("rb_locate_kernel", "rb_collect_kernel", "rb_finish_kernel"):
+        assert order(kernels[name]) == ["pdl_wait", "pdl_launch"], name
+        head = kernels[name][:kernels[name].index("pdl_launch();")]
+        assert head.count("{") - head.count("}") == 1, f"{name}: the order holds for every thread"
+    sweep = kernels["score_sweep_kernel"]
+    key_sums = sweep.index("if (kSweep == kKeySums) {")
+    row_sums = sweep.index("} else {", key_sums)
+    assert order(sweep[row_sums:sweep.index("}", row_sums + 1)]) == ["pdl_wait", "pdl_launch"]
+    assert order(sweep[:key_sums]) == []
+    source = _source("dkv.cu")
+
+    def launches(function):
+        body = source[source.index(f"int {function}("):]
+        return re.findall(r"\b(rb_\w+_kernel|select_gather\w*_kernel|pool_kernel|score_kernel)\b", body[:body.index("\n}")])
+
+    # the early readers' predecessors are these
+    assert launches("do_rebudget") == ["rb_locate_kernel", "rb_collect_kernel", "rb_finish_kernel"]
+    assert launches("launch_sweeps").count("pool_kernel") == 1
+    body = source[source.index("int do_pass("):]
+    assert re.search(r"do_rebudget\(.*\n\s*if \(\(rc = do_select_gather\(", body[:body.index("\n}")])
+
+
+def test_the_scoring_kernel_of_passes_is_launched_with_overlap_and_waits():
+    body = _source("dkv.cu")
+    assert re.search(r"auto launch = \[&\]\(auto score_kernel, int smem\) \{ return launch_pdl\(score_kernel,", body)
+    kernels = {n: b for n, _, b in _functions(_source("score_sweep.cuh"))}
+    assert kernels["score_sweep_kernel"].count("pdl_wait();") >= 4 and "pdl_wait();" in kernels["pool_kernel"]
