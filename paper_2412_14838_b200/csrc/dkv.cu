@@ -733,7 +733,7 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
   s.G = s.Hq / s.Hkv; s.P = s.S - s.ws; s.M = s.ws * s.G; s.Blc = s.Bl < s.P ? s.Bl : s.P; s.rows = s.Blc + s.ws;
   const int heads = s.Bt * s.Hkv;
   c->planes = (s.M + 127) / 128;
-  c->plane_rows = c->planes == 1 ? s.M : ((s.M + c->planes - 1) / c->planes + 7) / 8 * 8;
+  c->plane_rows = c->planes == 1 ? s.M : (s.M + 31) / 32 * 16;
   c->sel_cap = 1024;                                       // a quarter more than B^l for the rest of the threshold's digit
   while (c->sel_cap < s.Blc + s.Blc / 4 && c->sel_cap < DKV_MAX_LAYER_BUDGET) c->sel_cap <<= 1;
 

@@ -71,7 +71,7 @@ struct Shape1 {
 
 struct Args {
   int S, P, ws, M, D;
-  int planes, plane_rows;       // 1 or 2; window rows of a plane (the second may have fewer)
+  int planes, plane_rows;       // 1 or 2; window rows of a plane: of two the first plane_rows and the last
   int tph;                      // tiles of a head
   int hpl, vheads;              // heads of a layer; (head, plane) pairs of the launch
   float scale2;                 // log2(e) / sqrt(D)
@@ -208,7 +208,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::);
   }
   if (kRows && threadIdx.x < 4) again_s[threadIdx.x >> 1][threadIdx.x & 1] = 0;
-  if (kRows && threadIdx.x < 2 * kCols) last_s[threadIdx.x] = a.P + (threadIdx.x / kCols * a.plane_rows + threadIdx.x % kCols) % a.ws;
+  if (kRows && threadIdx.x < 2 * kCols) last_s[threadIdx.x] = a.P + (threadIdx.x / kCols * (a.M - a.plane_rows) + threadIdx.x % kCols) % a.ws;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -228,7 +228,9 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     const int place = 2 * blockIdx.x + p - tile_owner((long long)vh * a.tph, (long long)a.vheads * a.tph, 2 * grid);
     return a.stats + ((size_t)vh * a.slots + place) * a.plane_rows;
   };
-  auto row0_of = [&](int vh) { return (vh & (a.planes - 1)) * a.plane_rows; };
+  // A plane's first row.  Of two planes neither has a column without a row: what both have (fewer than 32 rows) counts in the first.  An
+  // empty column's logits are 0 times a key, which is no number where the key is infinite.
+  auto row0_of = [&](int vh) { return (vh & (a.planes - 1)) * (a.M - a.plane_rows); };
   // What whole warps wait for they go on without once a wait has run out, as no wait blocks any more then: whether it had come is for
   // each lane to see, and lanes that left a loop alone would be missing from its next shuffle.  Single lanes stop.
   auto wait = [&](uint32_t bar, uint32_t parity, int code) { return mbar_wait(bar, parity, abort_flag, a.status, code, a.wait_cycles); };
@@ -256,7 +258,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
   // segments have left, four in flight a lane, or the caller's.
   auto fill = [&](float* to, int vh, int r) {
     const int head = vh >> (a.planes - 1), layer = head / a.hpl, row0 = row0_of(vh), row = r + (lane >> 1);
-    const bool in = row < min(a.M - row0, a.plane_rows);
+    const bool in = row < a.plane_rows && (row0 == 0 || row0 + row >= a.plane_rows);
     float c = -INFINITY;
     if constexpr (kSweep == kKeySums) {
       const int n = tile_owner((long long)(vh + 1) * a.tph - 1, tiles, 2 * grid) - tile_owner((long long)vh * a.tph, tiles, 2 * grid) + 1;
@@ -560,12 +562,11 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
           const bool more = kLong && sg.vh == vh;
           vh = sg.vh;
           if (!more) part = sg.g - sg.n;
-          const int rows = min(a.M - row0_of(sg.vh), a.plane_rows);
           float2* to = sums_of(sg.vh, pipe);
           bool finite = true;
           wait_segment(CEMPTY(i & 1), i >> 1 & 1);
 #pragma unroll 1
-          for (int row = lane; row < rows; row += 32) {
+          for (int row = lane; row < a.plane_rows; row += 32) {
             float m[4], l[4], top = -INFINITY, sum = 0.f;
 #pragma unroll
             for (int w = 0; w < 4; ++w) {

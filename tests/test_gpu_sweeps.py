@@ -1,4 +1,4 @@
-"""Scoring of whole passes at the sizes where the sweeps change: window rows around their 32-row steps and the second plane, keys
+"""Scoring of whole passes at the sizes where the sweeps change: window rows around their 16-row steps and the second plane, keys
 around a tile, heads that lie in one pipe's range and in many, logits that a row's reference cannot hold."""
 import pytest
 import torch
@@ -24,9 +24,9 @@ def _scores(q, k, ws, pool):
     return torch.nn.functional.max_pool1d(t.softmax(-1)[..., :S - ws].sum(2), pool, 1, pool // 2), t.logsumexp(-1).view(Bt, Hkv * G, ws)
 
 
-def _passes(L, Hkv, G, D, Bt, S, ws, pool, change=None, most=5e-5):
+def _passes(L, Hkv, G, D, Bt, S, ws, pool, change=None, most=5e-5, sweeps=False):
     """Both kinds of pass; a score is a sum of 2^(t - lse): with |t| < 128 in 32 bits each is off by 2^-18 ln 2 at most, and the
-    instruction for 2^x and the sums add a few 2^-22."""
+    instruction for 2^x and the sums add a few 2^-22.  sweeps: the pass has to be scored by row sums, key sums and pooling."""
     g = torch.Generator(device="cuda").manual_seed(S)
     new = lambda *s: [torch.randn(s, generator=g, device="cuda").to(torch.bfloat16) for _ in range(L)]
     q, k, v = new(Bt, G * Hkv, ws, D), new(Bt, Hkv, S, D), new(Bt, Hkv, S, D)
@@ -38,6 +38,12 @@ def _passes(L, Hkv, G, D, Bt, S, ws, pool, change=None, most=5e-5):
     lse = [x.float().contiguous() for x in lse]
     h = B.dkv_create(B.make_config(L, G * Hkv, Hkv, D, Bt, S, ws, pool, 4, 8, 2))
     try:
+        if sweeps:
+            B.dkv_profile(h, True)
+            B.dkv_run_prefill_pass(h, q, k, v, kb, vb)
+            scoring = B.dkv_profile_read(h)
+            B.dkv_profile(h, False)
+            assert (scoring["score_stats"][1], scoring["score_emit"][1]) == (-(-L // 32), 2 * -(-L // 32))
         for run in (lambda: B.dkv_run_prefill_pass(h, q, k, v, kb, vb), lambda: B.dkv_run_prefill_pass_lse(h, q, k, v, lse, kb, vb)):
             run()
             for l in range(L):
@@ -230,3 +236,15 @@ def test_the_error_of_a_row_sum_does_not_grow_with_the_prompt(far):
                 assert off.mean(-1).abs().max() <= 2.5e-6, f"sample {b}: {off.mean(-1).abs().max():.1e}"
     finally:
         B.dkv_destroy(h)
+
+
+def _masked(q, k):                                           # keys that no query sees: logits of minus infinity, first ones of heads too
+    for x, y in zip(q, k):
+        x[..., 0] = x[..., 0].abs() + 1
+        y[:, 0, :300, 0], y[..., 5::7, 0] = -torch.inf, -torch.inf
+
+
+# two planes of 80 rows and 64, and of 112; and one
+@pytest.mark.parametrize("G,ws,D", [(9, 16, 64), (7, 32, 128), (4, 32, 64), (1, 16, 64)])
+def test_keys_at_minus_infinity_count_for_nothing(G, ws, D):
+    _passes(20, 2, G, D, 1, 1000, ws, 1, _masked, sweeps=True)
