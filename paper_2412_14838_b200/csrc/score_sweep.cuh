@@ -580,7 +580,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
             if (more) {
               const float2 before = to[row];
               const float most = fmaxf(top, before.x);
-              sum = (sum == 0.f ? 0.f : sum * fast_exp2(top - most)) + before.y * fast_exp2(before.x - most);
+              sum = (sum == 0.f ? 0.f : sum * fast_exp2(top - most)) + (before.y == 0.f ? 0.f : before.y * fast_exp2(before.x - most));
               top = most;
             }
             finite = finite && sum < INFINITY;

@@ -248,3 +248,25 @@ def _masked(q, k):                                           # keys that no quer
 @pytest.mark.parametrize("G,ws,D", [(9, 16, 64), (7, 32, 128), (4, 32, 64), (1, 16, 64)])
 def test_keys_at_minus_infinity_count_for_nothing(G, ws, D):
     _passes(20, 2, G, D, 1, 1000, ws, 1, _masked, sweeps=True)
+
+
+def test_parts_of_a_long_head_at_minus_infinity():
+    """Heads of 1024 tiles, about one to a pipe, whose first two parts of 256 tiles hold no key that counts."""
+    L, Hkv, S, ws, D = 32, 8, 131072, 16, 64
+    P, masked = S - ws, 66000
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q, k = (torch.randn((1, Hkv, n, D), generator=g, device="cuda").to(torch.bfloat16) for n in (ws, S))
+    q[..., 0], k[:, :, :masked, 0] = q[..., 0].abs() + 1, -torch.inf
+    kb, vb = ([torch.zeros((1, Hkv, 8 + ws, D), device="cuda", dtype=torch.bfloat16) for _ in range(L)] for _ in range(2))
+    h = B.dkv_create(B.make_config(L, Hkv, Hkv, D, 1, S, ws, 1, 4, 8, 32))
+    try:
+        B.dkv_run_prefill_pass(h, [q] * L, [k] * L, [k] * L, kb, vb)
+        want = _scores(q, k, ws, 1)[0]
+        got = torch.zeros((1, Hkv, P))
+        for l in range(L):
+            B.dkv_memcpy_to_host(h, got, B.dkv_layer_views(h, l)[0], got.numel() * 4)
+            assert (got[..., :masked] == 0).all()
+            assert ((got.cuda() - want).abs() <= 5e-5 * want).all()
+        assert B.dkv_last_status(h)[0] == B.DKV_OK
+    finally:
+        B.dkv_destroy(h)
