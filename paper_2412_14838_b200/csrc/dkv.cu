@@ -378,7 +378,7 @@ int launch_sweeps(dkv_ctx* c, int layer, int nl, const void* const* q, const voi
   a.raw = reinterpret_cast<float*>(c->d_cand);
   a.stats = c->d_stats; a.slots = stats_places(c, nl);
   a.hist = c->d_layer_hist + (size_t)layer * s.Bt * kBins;
-  a.hist_n = nl * s.Bt * kBins;
+  a.hist_n = (size_t)nl * s.Bt * kBins;
   a.status = c->d_status;
   a.wait_cycles = c->wait_cycles;
   a.segment_cycles = c->wait_cycles > INT64_MAX / (2 * tph) ? INT64_MAX : c->wait_cycles * (2 * tph);      // a segment swept twice

@@ -81,7 +81,7 @@ struct Args {
   float2* stats;                // [vheads][slots][plane_rows] (m, sum) of a head's segments
   int slots;
   unsigned int* hist;           // null, or counters to clear
-  int hist_n;
+  size_t hist_n;
   int* status;
   long long wait_cycles, segment_cycles;      // limits of a wait, for a tile and for a segment
   int withhold_tile;            // test hook: block 0 never loads its tile of this number (-1: off)
@@ -297,7 +297,7 @@ score_sweep_kernel(const __grid_constant__ Layers maps, const __grid_constant__ 
     const int c0 = kRows ? half * kHalf * 8 : 0, first = quad * 32 + (kRows ? 0 : half * 16);
     const uint32_t addr = tmem_base + ((uint32_t)first << 16) + (uint32_t)(pipe * kPer * kStage + c0);
     const int col2 = c0 + 2 * (lane & 3), key = first + (lane >> 2);        // the thread's keys: key, key + 8 (, key + 16, key + 24)
-    if (kSweep != kKeySums) for (int i = blockIdx.x * (kSoftWarps * 32) + threadIdx.x; i < a.hist_n; i += grid * (kSoftWarps * 32)) a.hist[i] = 0;
+    if (kSweep != kKeySums) for (size_t n = blockIdx.x * (kSoftWarps * 32) + threadIdx.x; n < a.hist_n; n += grid * (kSoftWarps * 32)) a.hist[n] = 0;
     Ring st(kPer, 0);
     int i = 0;                                          // segments so far
     rounds([&](Segments& sg, auto round_) {

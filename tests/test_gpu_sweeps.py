@@ -1,8 +1,10 @@
 """Scoring of whole passes at the sizes where the sweeps change: window rows around their 16-row steps and the second plane, keys
 around a tile, heads that lie in one pipe's range and in many, logits that a row's reference cannot hold."""
+import numpy as np
 import pytest
 import torch
 
+from oracle import dynamickv as O
 from paper_2412_14838_b200 import binding as B
 from paper_2412_14838_b200 import build
 
@@ -268,5 +270,32 @@ def test_parts_of_a_long_head_at_minus_infinity():
             assert (got[..., :masked] == 0).all()
             assert ((got.cuda() - want).abs() <= 5e-5 * want).all()
         assert B.dkv_last_status(h)[0] == B.DKV_OK
+    finally:
+        B.dkv_destroy(h)
+
+
+def test_digit_counters_beyond_31_bits():
+    """32 layers of 32768 samples have 2^31 counters, which every pass has to clear: counts of a pass after others."""
+    L, Bt, S, ws, D, N, Bl = 32, 32768, 12, 1, 64, 4, 8
+    P = S - ws
+    g = torch.Generator(device="cuda").manual_seed(1)
+    new = lambda *s: torch.randn(s, generator=g, device="cuda").to(torch.bfloat16)
+    k, q = new(Bt, 1, S, D), [new(Bt, 1, ws, D) for _ in range(L)]
+    lse = [torch.full((Bt, 1, ws), 3.0, device="cuda")] * L
+    kb, vb = ([torch.zeros((Bt, 1, Bl + ws, D), device="cuda", dtype=torch.bfloat16) for _ in range(L)] for _ in range(2))
+    h = B.dkv_create(B.make_config(L, 1, 1, D, Bt, S, ws, 1, N, Bl, L))
+    try:
+        for run in (lambda q: B.dkv_run_prefill_pass_lse(h, q, [k] * L, [k] * L, lse, kb, vb), lambda q: B.dkv_run_prefill_pass(h, q, [k] * L, [k] * L, kb, vb)):
+            run(q[::-1])
+            run(q)
+            assert B.dkv_last_status(h)[0] == B.DKV_OK
+            counts = torch.zeros((Bt, L), dtype=torch.int32)
+            B.dkv_get_counts(h, counts)
+            scores = torch.zeros((L, Bt, 1, P))
+            for l in range(L):
+                B.dkv_memcpy_to_host(h, scores[l], B.dkv_layer_views(h, l)[0], scores[l].numel() * 4)
+            for b in (0, 1, Bt // 2 - 1, Bt // 2, Bt - 1):
+                want = O.rebudget([x.numpy() for x in scores[:, b]], [Bl] * L, N, Bl, L)["counts"]
+                assert np.array_equal(counts[b], want), f"sample {b}"
     finally:
         B.dkv_destroy(h)
