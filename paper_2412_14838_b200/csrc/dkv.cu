@@ -301,7 +301,8 @@ int launch_score(dkv_ctx* c, const ScoreGroup* e, ScoreGroup* s, const void* con
   tc::Params j0, j1;
   memset(&j0, 0, sizeof j0); memset(&j1, 0, sizeof j1);
   j0.mode = j1.mode = tc::kNone;
-  const int most = e && (!s || e->n > s->n) ? e->n : s->n, grid = score_grid(c, most);
+  // No more blocks than sweep 1 has tiles, whatever sweep 2 has: a block without a tile would leave a gap among its head's statistics.
+  const int grid = score_grid(c, (s ? s : e)->n);
   if (s) s->grid = grid;
   if (e && !make_job(c, tc::kEmit, e->first, e->n, q + e->first, k + e->first, scores_out, e->buf, grid, e->grid, hist, &m0, &j0, lse ? lse + e->first : nullptr)) return DKV_ERR_CUDA;
   if (s && !make_job(c, tc::kStats, s->first, s->n, q + s->first, k + s->first, nullptr, s->buf, grid, grid, hist, &m1, &j1)) return DKV_ERR_CUDA;

@@ -299,3 +299,10 @@ def test_digit_counters_beyond_31_bits():
                 assert np.array_equal(counts[b], want), f"sample {b}"
     finally:
         B.dkv_destroy(h)
+
+
+# Passes of 128 rows of 128 dims that are scored by groups of layers, the last group smaller (25, 25, 25, 22 layers; 26, 26, 26, 23;
+# 17, 16), with fewer tiles than SMs.  The fourth group's statistics go where the first one's were.
+@pytest.mark.parametrize("L,S", [(97, 500), (101, 500), (101, 896), (33, 896)])
+def test_last_group_with_fewer_tiles_than_the_one_before(L, S):
+    _passes(L, 1, 4, 128, 1, S, 32, 5)
