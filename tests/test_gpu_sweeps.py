@@ -306,3 +306,19 @@ def test_digit_counters_beyond_31_bits():
 @pytest.mark.parametrize("L,S", [(97, 500), (101, 500), (101, 896), (33, 896)])
 def test_last_group_with_fewer_tiles_than_the_one_before(L, S):
     _passes(L, 1, 4, 128, 1, S, 32, 5)
+
+
+# enough tiles (two an SM) for passes of two planes: 129 to 256 rows, planes that share rows and planes that do not, all of one size
+# of the builds and of the largest; without and with logits whose sums have to be computed again, in either plane
+@pytest.mark.parametrize("far", [False, True])
+@pytest.mark.parametrize("G,ws,D", [(1, 129, 64), (5, 26, 64), (5, 28, 128), (9, 16, 64), (7, 24, 128), (6, 32, 64), (7, 32, 128), (3, 75, 64),
+                                    (8, 32, 128), (8, 32, 64)])
+def test_two_planes(G, ws, D, far):
+    def change(q, k):
+        for n, (x, y) in enumerate(zip(q, k)):
+            x[..., 0], y[..., 0] = 0.0, 0.0
+            if n % 3 == 0:                                   # in this layer for the last query head, which is in the second plane
+                x[:, -1, :, 0], y[:, -1, 500::61, 0] = 16.0, 100.0
+            elif n % 3 == 1:                                 # for the first query head of a key head
+                x[:, ::G, :, 0], y[:, 0, 500::61, 0] = 16.0, 100.0
+    _passes(20, 2, G, D, 1, 1000, ws, 5, change if far else None, most=2e-4 if far else 5e-5, sweeps=True)
