@@ -356,7 +356,7 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ 
   float* raw_s = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(nlse_s) + kMiscBytes);   // [half][kMaxSegTiles * 128]
   uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(raw_s) + kRawBytes);
   unsigned int* hist_s = reinterpret_cast<unsigned int*>(bars + 32);   // [kBins] digits of the scores of one layer and sample (sweep 2)
-  // barriers: full[kStages], empty[kStages], tmem_full[4], tmem_empty[4], q_full, drain[2]
+  // barriers: full[kStages], empty[kStages], tmem_full[4], tmem_empty[4], q_full, drain[2], q_seen
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_s;
   const uint32_t bar0 = smem_u32(bars);
@@ -366,6 +366,7 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ 
   auto TEMPTY = [&](int t) { return bar0 + 8u * (2 * kStages + 4 + t); };
   const uint32_t QFULL = bar0 + 8u * (2 * kStages + 8);
   auto DRAIN = [&](int i) { return bar0 + 8u * (2 * kStages + 9 + i); };   // one per MMA issuer, used after an abort only
+  const uint32_t QSEEN = bar0 + 8u * (2 * kStages + 11);                   // both issuers have seen a head's queries
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_flag = &abort_s;
@@ -377,7 +378,7 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ 
     abort_s = 0;
     for (int s = 0; s < kStages; ++s) { mbar_init(FULL(s), 1); mbar_init(EMPTY(s), 1); }
     for (int t = 0; t < 4; ++t) { mbar_init(TFULL(t), 1); mbar_init(TEMPTY(t), 8); }
-    mbar_init(QFULL, 1);
+    mbar_init(QFULL, 1); mbar_init(QSEEN, 2);
     mbar_init(DRAIN(0), 1); mbar_init(DRAIN(1), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -424,7 +425,9 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ 
           const CUtensorMap* q_map = &maps.q[sg.bh / p.hpl];
           const CUtensorMap* k_map = &maps.k[sg.bh / p.hpl];
           if (sg.new_head) {
-            // every MMA that read the previous queries must have finished: the last tile of either issuer
+            // both issuers must have seen the previous queries (QFULL may not begin another phase before), and every MMA that read
+            // them must have finished: the last tile of either issuer
+            if (nq > 0) ok = mbar_wait(QSEEN, (nq - 1) & 1, abort_flag, p.status, 101, p.wait_cycles);
             for (int last = tile - 1; last >= 0 && last >= tile - 2; --last)
               ok = ok && mbar_wait(EMPTY(last % kStages), (last / kStages) & 1, abort_flag, p.status, 101, p.wait_cycles);
             if (ok) {
@@ -472,7 +475,7 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ 
       const uint64_t kdesc0 = smem_desc(smem_u32(k_smem)), qdesc0 = smem_desc(smem_u32(q_smem));
       const uint32_t kq_lo[2] = {(uint32_t)kdesc0, (uint32_t)qdesc0}, desc_hi = (uint32_t)(kdesc0 >> 32);
       int tile = 0, nq = 0;
-      bool q_wait = false;
+      bool q_ok = true;
       for (int jb = 0; jb < 2; ++jb) {
         const Params& p = jb ? job1 : job0;
         if (p.mode == kNone) continue;
@@ -481,20 +484,20 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps0, const __grid_constant__ 
         SegIter it(p, blockIdx.x, gridDim.x);
         Seg sg;
         while (it.next(sg)) {
-          // the wait for a head's queries is taken at this issuer's first tile of the head (it may have none)
-          if (sg.new_head) { q_wait = true; ++nq; }
+          // Every head's queries are waited for, also those of a head with one tile, which is the other issuer's: with a phase left out,
+          // the wait for the next one would be over by the parity of the one before it.
+          if (sg.new_head) {
+            q_ok = mbar_wait(QFULL, nq & 1, abort_flag, p.status, 103, p.wait_cycles);
+            if (q_ok) mbar_arrive(QSEEN);
+            ++nq;
+          }
           // this thread's tiles only: every other one, by the parity of the tile's number over the launch
           const int tile0 = tile;
           tile += sg.ntiles;
           for (int i = (which ^ tile0) & 1, tile_ = tile0 + i; i < sg.ntiles; i += 2, tile_ += 2) {
             const int tile = tile_;
-            bool ok = true;
-            if (q_wait) {
-              q_wait = false;
-              ok = mbar_wait(QFULL, (nq - 1) & 1, abort_flag, p.status, 103, p.wait_cycles);
-            }
             const int s = tile % kStages, n = tile / kStages, t = tile & tmask, nt = tile >> tshift;
-            ok = ok && mbar_wait(FULL(s), n & 1, abort_flag, p.status, 104, p.wait_cycles);
+            bool ok = q_ok && mbar_wait(FULL(s), n & 1, abort_flag, p.status, 104, p.wait_cycles);
             ok = ok && mbar_wait(TEMPTY(t), (nt & 1) ^ 1, abort_flag, p.status, 105, p.wait_cycles);
             if (!ok) continue;                           // nothing more is issued once a wait has run out
             tc_fence_after();

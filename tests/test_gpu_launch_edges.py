@@ -146,3 +146,56 @@ def test_decoding_step_over_short_heads(L, Bt, Hkv, G, D, N, nq):
                     assert (out[l][b] - want).abs().max() <= 1e-5 * want.abs().max(), f"layer {l}, sample {b}"
     finally:
         B.dkv_destroy(h)
+
+
+# Heads of one key tile, or of one in sweep 2 and few in sweep 1: the two MMA issuers of score_tc.cuh take tiles in turn, so that either
+# has none of many heads.  Calls for one layer, all builds; scores are the same in every call.
+@pytest.mark.parametrize("G,ws,D", [(1, 16, 64), (2, 32, 64), (3, 32, 128), (4, 32, 128), (7, 32, 128), (8, 32, 64)])
+@pytest.mark.parametrize("S,Bt,lse", [(100, 64, False), (100, 64, True), (130, 32, False), (300, 3, False)])
+def test_heads_of_one_tile(G, ws, D, S, Bt, lse):
+    Hkv, pool, P = 8, 5, S - ws
+    g = torch.Generator(device="cuda").manual_seed(S)
+    q, k = (torch.randn(n, generator=g, device="cuda").to(torch.bfloat16) for n in ((Bt, G * Hkv, ws, D), (Bt, Hkv, S, D)))
+    t = q.double().view(Bt, Hkv, G * ws, D) @ k.double().transpose(-1, -2) / D ** 0.5
+    last = P + torch.arange(ws, device="cuda").repeat(G)
+    t.masked_fill_(torch.arange(S, device="cuda") > last[:, None], -torch.inf)
+    want = torch.nn.functional.max_pool1d(t.softmax(-1)[..., :P].sum(2), pool, 1, pool // 2)
+    given = t.logsumexp(-1).view(Bt, Hkv * G, ws).float().contiguous()
+    h = B.dkv_create(B.make_config(1, G * Hkv, Hkv, D, Bt, S, ws, pool, 4, 8, 1))
+    try:
+        first = None
+        for _ in range(20):
+            got = torch.zeros((Bt, Hkv, P), device="cuda")
+            if lse:
+                B.dkv_score_lse(h, 0, q, k, given, got)
+            else:
+                B.dkv_score(h, 0, q, k, got)
+            first = got if first is None else first
+            assert torch.equal(got, first)
+        assert ((first - want).abs() <= 5e-5 * want).all()       # |t| < 128 in 32 bits: 2^-18 ln 2, and the sums
+        assert B.dkv_last_status(h)[0] == B.DKV_OK
+    finally:
+        B.dkv_destroy(h)
+
+
+def test_a_pass_over_heads_of_one_tile():
+    L, Hkv, G, D, Bt, S, ws, pool = 32, 8, 4, 128, 8, 100, 32, 5
+    g = torch.Generator(device="cuda").manual_seed(1)
+    new = lambda *s: [torch.randn(s, generator=g, device="cuda").to(torch.bfloat16) for _ in range(L)]
+    q, k = new(Bt, G * Hkv, ws, D), new(Bt, Hkv, S, D)
+    kb, vb = ([torch.zeros((Bt, Hkv, 8 + ws, D), device="cuda", dtype=torch.bfloat16) for _ in range(L)] for _ in range(2))
+    h = B.dkv_create(B.make_config(L, G * Hkv, Hkv, D, Bt, S, ws, pool, 4, 8, 4))
+    try:
+        for _ in range(20):
+            B.dkv_run_prefill_pass(h, q, k, k, kb, vb)
+        last = S - ws + torch.arange(ws, device="cuda").repeat(G)
+        for l in range(L):
+            t = q[l].double().view(Bt, Hkv, G * ws, D) @ k[l].double().transpose(-1, -2) / D ** 0.5
+            t.masked_fill_(torch.arange(S, device="cuda") > last[:, None], -torch.inf)
+            want = torch.nn.functional.max_pool1d(t.softmax(-1)[..., :S - ws].sum(2), pool, 1, pool // 2).cpu()
+            got = torch.zeros((Bt, Hkv, S - ws))
+            B.dkv_memcpy_to_host(h, got, B.dkv_layer_views(h, l)[0], got.numel() * 4)
+            assert ((got - want).abs() <= 5e-5 * want).all(), f"layer {l}"
+        assert B.dkv_last_status(h)[0] == B.DKV_OK
+    finally:
+        B.dkv_destroy(h)
