@@ -32,35 +32,41 @@ UNIT = "tokens/s"
 DEFAULT_WORKLOAD = "mistral32k"
 NOMINAL_HBM_GBS = 8000.0
 
-# DRAM traffic of one full scoring launch (dram__bytes_read.sum + dram__bytes_write.sum): sweep 2 of a group of layers
-# followed by sweep 1 of the next, taken with ncu on the 16-layer cut of the mistral32k shape (same per-layer shape and
-# group size, so the figure needs no scaling; see profiles/score_tc_kernel_mistral32k_16layers.md).  "live" is a
-# single-pass capture without ncu's cache flush, i.e. with whatever the previous launch left in L2, as in a real pass;
-# "cold" starts from flushed caches.  Both hold for the kernel source they were measured on, for that per-layer shape
-# and for groups of that many layers only: any other source hash, shape or grouping reports null.
+# DRAM traffic of the scoring of one pass (dram__bytes_read.sum + dram__bytes_write.sum of its row sums, key sums and
+# pooling), taken with ncu on the mistral32k shape: a single-pass capture without ncu's cache flush, i.e. with whatever the
+# launch before left in L2, as in a real pass (profiles/launch_list_mistral32k.md).  It holds for the sources it was
+# measured on, that shape and those launches only: any other reports null.
 NCU_TRAFFIC = {
-    "kernel_sha256": "54a6664d8c8e2746ff04426daa3dea882238f1d62f30c823f6b0c26fcdbc2e1c",
-    "shape": (8, 128, 1, 32768, 32),          # Hkv, D, Bt, S, ws
-    "layers_per_launch": 8,
-    "live_bytes_per_launch": 1_019_605_504 + 23_030_016,
-    "cold_bytes_per_launch": 1_081_276_416 + 9_970_944,
+    "kernel_sha256": "f8dcf01dda56855071ea1b9e6383ee3c4cd53f0e912c4cfe9833b8bd7f1e6d32",
+    "shape": (32, 8, 128, 1, 32768, 32),      # L, Hkv, D, Bt, S, ws
+    "score_launches": 3, "emit_launches": 2,  # row sums | key sums and pooling
+    "layers_per_launch": 32,
+    "live_bytes": 2_155_917_056 + 16_113_152 + 2_147_659_008 + 26_908_416 + 264_704 + 22_253_824,
 }
 
 
-def ncu_traffic(w, score_launches=None):
+def scoring_sha256():
+    """Of the kernels that score a pass."""
     import hashlib
-    src = os.path.join(ROOT, "paper_2412_14838_b200", "csrc", "score_tc.cuh")
+    sha = hashlib.sha256()
+    for name in ("score_sweep.cuh", "score_tc.cuh"):
+        with open(os.path.join(ROOT, "paper_2412_14838_b200", "csrc", name), "rb") as f:
+            sha.update(f.read())
+    return sha.hexdigest()
+
+
+def ncu_traffic(w, score_launches=None, emit_launches=None):
+    """The capture, if it is of this shape and of a pass of these launches: how many it made of sweep 2 says which kernel
+    scored it (two, with the pooling, or one beside those that begin with sweep 1)."""
+    c = NCU_TRAFFIC
+    if (w.L, w.Hkv, w.D, w.Bt, w.S, w.ws) != c["shape"] or None in (score_launches, emit_launches):
+        return None
+    if (round(score_launches), round(emit_launches)) != (c["score_launches"], c["emit_launches"]):
+        return None
     try:
-        with open(src, "rb") as f:
-            sha = hashlib.sha256(f.read()).hexdigest()
+        return c if scoring_sha256() == c["kernel_sha256"] else None
     except OSError:
         return None
-    if sha != NCU_TRAFFIC["kernel_sha256"] or (w.Hkv, w.D, w.Bt, w.S, w.ws) != NCU_TRAFFIC["shape"]:
-        return None
-    g = NCU_TRAFFIC["layers_per_launch"]
-    if w.L % g or score_launches is None or round(score_launches) != w.L // g + 1:
-        return None                             # the pass was not run in full groups of that many layers
-    return NCU_TRAFFIC
 
 
 FALLBACK_HBM_GBS = 6650.0
@@ -299,10 +305,11 @@ def run_gpu(args, w):
     B.dkv_profile(ctx, False)
     peaks, peak_kind = measured_peaks()
     peak = float(peaks["hbm_gbs"])
-    # the scoring kernel: every launch sweeps a group of layers (sweep 2 of one group, sweep 1 of the next), so
-    # the algorithmic bytes of a launch are the pass's K bytes over the launches of a pass
+    # the scoring: its launches (row sums, key sums, pooling; or sweeps of groups of layers) share the pass's K bytes equally
     score_ms = (prof["score_stats"][0] + prof["score_emit"][0]) / prof_steps
     score_launches = (prof["score_stats"][1] + prof["score_emit"][1]) / prof_steps
+    emit_launches = prof["score_emit"][1] / prof_steps
+    traffic = ncu_traffic(w, score_launches, emit_launches)
     score_launch_ms = score_ms / score_launches
     k_bytes = w.k_bytes_per_layer()
     launch_bytes = k_bytes * w.L / score_launches
@@ -312,10 +319,9 @@ def run_gpu(args, w):
                 "unit": "GB/s", "frac": achieved / peak,
                 "algorithmic_bytes_per_launch": launch_bytes, "avg_launch_ms": score_launch_ms,
                 "launches_per_pass": score_launches, "scoring_ms_per_layer": score_ms / w.L,
-                "traffic": (ncu_traffic(w, score_launches) or {}).get("live_bytes_per_launch"),
-                "traffic_cold_cache": (ncu_traffic(w, score_launches) or {}).get("cold_bytes_per_launch"),
-                "traffic_note": "DRAM bytes of a full launch (sweep 2 of a group of layers + sweep 1 of the next), null "
-                                "where no capture of this kernel source and grouping exists",
+                "traffic": traffic and traffic["live_bytes"] / score_launches,
+                "traffic_note": "DRAM bytes of the pass's scoring launches, row sums, key sums and pooling, over their number; null "
+                                "where no capture of these sources, this shape and these launches exists",
                 "whole_pass": {"algorithmic_bytes": w.algorithmic_bytes(),
                                "achieved_gbs": w.algorithmic_bytes() / (ms_per_step * 1e-3) / 1e9,
                                "frac_of_measured_peak": w.algorithmic_bytes() / (ms_per_step * 1e-3) / 1e9 / peak,

@@ -72,3 +72,18 @@ def test_ncu_traffic_is_tied_to_kernel_source_and_shape(monkeypatch):
     assert bench.ncu_traffic(synth.WORKLOADS["tiny"], 2) is None
     monkeypatch.setitem(bench.NCU_TRAFFIC, "kernel_sha256", "0" * 64)
     assert bench.ncu_traffic(w, w.L // layers + 1) is None
+
+
+def test_ncu_traffic_is_that_of_the_kernels_that_scored(monkeypatch):
+    """A cut of the workload, or a pass scored by groups of layers, may take as many launches as the captured one."""
+    import bench
+    from paper_2412_14838_b200 import synth
+    w = synth.WORKLOADS["mistral32k"]
+    c = bench.NCU_TRAFFIC
+    n, emit = c["score_launches"], c["emit_launches"]
+    monkeypatch.setitem(c, "kernel_sha256", bench.scoring_sha256())              # as for the sources that were measured
+    assert bench.ncu_traffic(w, n, emit) is c
+    assert 2 * w.L * w.k_bytes_per_layer() <= c["live_bytes"] <= 2.2 * w.L * w.k_bytes_per_layer()     # both sweeps read K from HBM
+    assert bench.ncu_traffic(w, n, 1) is None                                    # two groups of 16 layers, sweep 2 once on its own
+    assert bench.ncu_traffic(w.with_(L=16), n, emit) is None
+    assert bench.ncu_traffic(w, n + 1, emit) is None
