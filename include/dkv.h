@@ -77,8 +77,9 @@ typedef struct {
 /* Create a context for `cfg` on the current device (host call; allocates device memory:
  * score history 4*L*Bt*Hkv*P bytes, candidates of the global top-K 8*L*Bt*Hkv*P (while a pass scores, its unpooled scores:
  * at least 4 bytes per key of min(L, 32) layers, S rounded up to 128, twice that from 129 window rows on), kept indices
- * 4*L*Bt*Hkv*Bl', digit counts 8192*L*Bt, partial softmax statistics 6144 * (SM count + 64*Bt*Hkv) and
- * 16 * window rows * (SM count + min(L, 32)*Bt*Hkv), small workspaces; the
+ * 4*L*Bt*Hkv*Bl', digit counts 8192*L*Bt, partial softmax statistics 6144 * (SM count + 2*Bt*Hkv) and
+ * about 16 * window rows * (SM count + min(L, 32)*Bt*Hkv), or, where short passes are scored in groups of g <= 32 layers,
+ * 6144 * (SM count + 2*g*Bt*Hkv); small workspaces; the
  * staging of the host-buffer pass (q, k, v of two layers, kb, vb of all) and the decoding scratch come with the first
  * call that needs them).
  * Errors: INVALID_ARG, UNSUPPORTED, NOMEM, CUDA.  On error *out is NULL. */
@@ -284,7 +285,8 @@ int dkv_static_last_status(int32_t* host_status);
  * dkv_last_status.  Applies to launches made after the call. */
 int dkv_set_wait_limit(dkv_ctx* ctx, int64_t clock_ticks);
 /* Test hook for the path above: in the launches that follow, thread block 0 never loads its key tile number
- * `tile` (0-based, per launch) of scoring sweep `sweep` (1 = statistics, 2 = emit), so the wait for that
+ * `tile` (0-based, per launch; where a block works on two ranges of tiles at once, as it may in a pass, of
+ * the first range) of scoring sweep `sweep` (1 = statistics, 2 = emit), so the wait for that
  * tile runs out after the wait limit.  tile < 0 switches the hook off.  Nothing else is disturbed: no
  * invalid address, no trap. */
 int dkv_debug_withhold_tile(dkv_ctx* ctx, int32_t sweep, int32_t tile);

@@ -344,7 +344,9 @@ cudaError_t set_sweep_attributes(int nb, bool all, bool long_rows) {
   return e != cudaSuccess ? e : with_sweep_kernel<sweep::kGivenSums>(nb, set);
 }
 
-// Which of the two scoring kernels takes a pass.  With the caller's normalisers it is always score_sweep.cuh, and for one layer at a
+// Which of the two scoring kernels takes a pass.  With the caller's normalisers it is always score_sweep.cuh (128 rows of 128 dims, whole
+// passes against the library that scored them with score_tc.cuh: 4 layers of 700 keys 32.5 -> 30.1 us, 8 of 4K 42.5 -> 37.0, 32 of 1K /
+// 4K / 16K 60 / 96 / 247 -> 51 / 85 / 221), and for one layer at a
 // time always score_tc.cuh, which has a launch less and pools in it (a layer of 32K with normalisers 18.3 us a call, by sweeps 23.1;
 // without, 8 layers of 4K call by call 253-298 us against 278-328).  score_tc.cuh remains for 128 window rows of 128 dims, for
 // which it has a build, while an SM has few tiles (8 layers of 4K, 4 heads: 58 us against 65; 32 of 8K, 110 tiles an SM: 285 / 283;
@@ -614,9 +616,10 @@ int do_decode(dkv_ctx* c, int layer0, int nl, int nq, const void* const* q, cons
 }
 
 // Algorithm 1's loop, one chain of launches on `st`.
-//   scoring   launch g runs sweep 2 of layer group g-1 and then sweep 1 of group g (a group = up to `pass_group` layers, so
-//             that the fixed cost of a launch is paid once per group) on all SMs; sweep 2 also counts the scores' digits.
-//             With `lse` (the window rows' log-denominators of every layer) launch g runs sweep 2 of group g only.
+//   scoring   by score_sweep.cuh, up to 32 layers at a time: row sums, key sums, pooling; with `lse` (the window rows'
+//             log-denominators of every layer) the last two.  Or by score_tc.cuh (pass_by_sweeps): launch g runs sweep 2 of layer
+//             group g-1 and then sweep 1 of group g (a group = up to `pass_group` layers, so that the fixed cost of a launch is
+//             paid once per group).  Either counts the scores' digits.
 //   updates   all of Eq. 4-6's updates together: their order does not matter, a layer's count is the minimum over them
 //             and nothing reads an intermediate one.
 //   select, gather   with the final counts.
@@ -743,7 +746,7 @@ int dkv_create(const dkv_config* cfg, dkv_ctx** out) {
     int sms = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     c->n_sms = sms > 0 ? sms : 1;
-    // Layers per scoring launch of the pass: enough that a thread block has about 110 tiles a sweep.  A launch costs some 8 us
+    // Layers per scoring launch of a pass that score_tc.cuh scores: enough that a thread block has about 110 tiles a sweep.  A launch costs some 8 us
     // (fill, drain, statistics) whatever it does: 32 layers of 8K in launches of 8 / 16 / 32 layers take 299 / 290 / 286 us;
     // at 32K eight layers are as good as more.
     const long long tiles = (long long)heads * ((s.S + tc::kTileKeys - 1) / tc::kTileKeys), want = (110ll * c->n_sms + tiles - 1) / tiles;

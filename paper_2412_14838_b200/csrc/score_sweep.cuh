@@ -4,8 +4,8 @@
 // known when a head's last key has been seen, so the keys are swept twice (once where the caller has the log-denominators).
 //
 //   tile      128 keys of one head: logits^T = K . Q_win^T on the tensor cores, one TMEM lane a key, one column a window row
-//             (at most 128 rows, rounded up to 16; up to 256 rows are two PLANES whose sums are added by pool_kernel).  With rows
-//             rounded up to 32, 72 and 224 rows cost more: 14 layers of 3 x 5003 131.4 us, now 124.0; 28 of 16K 454 before, 390.
+//             (at most 128 rows, rounded up to 16; up to 256 rows are two PLANES whose sums are added by pool_kernel).  Rounded up
+//             to 32, 72 and 224 rows cost more: 14 layers of 3 x 5003 131.4 us against 124.0, 28 of 16K 454 against 390.
 //   pipes     a block has two, each with its own contiguous range of the tiles, in SEGMENTS of one head, its own slots, copies,
 //             MMAs, accumulator stages and eight warps for exponentials.
 //   warps     0-7 and 8-15 exponentials of either pipe, 16 and 17 its copies, 18 and 19 its MMAs, 20 and 21 log-denominators of
@@ -23,13 +23,15 @@
 //
 // What bounds it: a tile takes an SM 0.7 (row sums) and 0.8 us (key sums), 5.9-6.8 TB/s, near the 6.5 of a copy, in the launches
 // of eight layers of 32K; a whole pass over 32K runs at the power limit, 0.95 us a tile.  The softmax loops bound what is in L2:
-// 0.45 us a tile against 0.54 for the special-function unit at the same clock.  A launch takes 5 us to its first logits and
+// 32 layers of 16K that share one K, 8 heads of 128, 128 rows, take 0.69 us a tile for the row sums, of which the special-function
+// unit alone needs 0.55 (1024 clocks of 1.8-1.9 GHz); from HBM 0.76.  A launch takes 5 us to its first logits and
 // about 10 in all beside its tiles, most of it instructions that are fetched for the first time: with the loops unrolled over
 // a whole tile it took 15, and with two streams of long loops (row sums in one pipe, key sums in the other) a tile took twice as long.
 //
 // Against score_tc.cuh (us a pass): 14 layers of 3 x 5003, 6 heads of 64, 72 rows 166 -> 131; 16 layers of 16K, 4 heads of 64,
 // 32 / 96 / 128 / 192 rows 118 / 149 / 155 / 220 -> 107 / 123 / 139 / 186; 28 of 2 x 2K, 4 heads of 128, 96 / 192 / 256 rows
-// 114 / 153 / 162 -> 102 / 138 / 151; 32 layers of 32K, 8 heads of 128, with log-denominators 572 -> 530-554.
+// 114 / 153 / 162 -> 102 / 138 / 151; 32 layers of 32K, 8 heads of 128, with log-denominators 572 -> 530-554.  28 layers of 16K, 4 heads
+// of 128, 224 rows: 415-423 -> 388-422, mostly at the power limit, where they are equal.
 #pragma once
 #include <limits.h>
 #include <type_traits>
