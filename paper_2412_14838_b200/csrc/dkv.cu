@@ -353,9 +353,14 @@ cudaError_t set_sweep_attributes(int nb, bool all, bool long_rows) {
 // 32 of 32K, 443: 1046 / 1024; 4 x 16K, 886: 2013 / 1955), and for more than 128 rows (two planes, whose pooling takes a launch)
 // while an SM has at most two tiles (4 layers of 1K, 4 heads, 224 rows, 128 tiles in all: 48.3 / 50.2; 8 of 2K, 512 tiles:
 // 60.8 / 58.7; 28 of 16K: 388 / 364 in bursts and the same, 408-418, at the power cap; 16 of 16K, 4 heads of 64, 140 rows: 207 / 168).
+// So do 208 rows and more over heads of two tiles whose scored positions, with their neighbours in the pooling, fill one: sweep 2 of
+// score_tc.cuh reads that one only.  32 layers of B samples of 8 heads of 130 keys (score_tc.cuh / sweeps), B = 3, 4, 8: 224 rows of 128 dims
+// 110 / 104, 133 / 137, 228 / 240; 256 rows of 128 dims 112 / 110, 135 / 143, 233 / 251 (150 keys); 256 of 64 dims B = 6, 8 179 / 177, 222 / 238.  With
+// fewer rows or longer heads the sweeps are faster again: 192 rows 225 / 221, 224 rows of 160 keys, B = 6, 193 / 186.
 bool pass_by_sweeps(const dkv_ctx* c) {
   const Shape& s = c->s;
   const long long tiles = (long long)s.L * s.Bt * s.Hkv * tiles_per_head(s);
+  if (s.M >= 208 && tiles_per_head(s) == 2 && s.P + s.pool / 2 * 2 <= tc::kTileKeys && tiles >= (s.D == 128 ? 12ll : 24ll) * c->n_sms) return false;
   return tiles >= (s.M == 128 && s.D == 128 ? 200ll : c->planes > 1 ? 2ll : 0ll) * c->n_sms;
 }
 

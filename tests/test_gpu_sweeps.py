@@ -322,3 +322,24 @@ def test_two_planes(G, ws, D, far):
             elif n % 3 == 1:                                 # for the first query head of a key head
                 x[:, ::G, :, 0], y[:, 0, 500::61, 0] = 16.0, 100.0
     _passes(20, 2, G, D, 1, 1000, ws, 5, change if far else None, most=2e-4 if far else 5e-5, sweeps=True)
+
+
+# At the line where score_tc.cuh takes passes of more than 207 rows over heads of two tiles, one of them without a scored position
+# (samples: fewest that it takes, one less; a row less; one position more).
+@pytest.mark.parametrize("G,ws,D,Bt,S,sweeps", [(8, 26, 128, 7, 150, False), (8, 26, 128, 6, 150, True), (9, 23, 128, 7, 147, True), (8, 32, 128, 7, 156, False),
+                                                (8, 32, 128, 7, 157, True), (8, 32, 64, 14, 130, False), (8, 32, 64, 13, 130, True)])
+def test_many_short_heads_of_many_rows(G, ws, D, Bt, S, sweeps):
+    L, Hkv, pool = 16, 8, 5                                   # 256 tiles a sample
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert sms == 148, "the samples are for 148 SMs"
+    _passes(L, Hkv, G, D, Bt, S, ws, pool, sweeps=sweeps)
+    if not sweeps:
+        q, k = (torch.randn((Bt, n, m, D), device="cuda").to(torch.bfloat16) for n, m in ((G * Hkv, ws), (Hkv, S)))
+        kb, vb = ([torch.zeros((Bt, Hkv, 8 + ws, D), device="cuda", dtype=torch.bfloat16) for _ in range(L)] for _ in range(2))
+        h = B.dkv_create(B.make_config(L, G * Hkv, Hkv, D, Bt, S, ws, pool, 4, 8, 2))
+        try:
+            before = B.dkv_launch_count(h)
+            B.dkv_run_prefill_pass(h, [q] * L, [k] * L, [k] * L, kb, vb)
+            assert B.dkv_launch_count(h) - before == 2 + 3 + 1       # sweep 1, sweep 2, the updates, selection
+        finally:
+            B.dkv_destroy(h)
